@@ -235,7 +235,10 @@ int moss_sample_estimate(moss_graph *g, int k, uint64_t budget, uint64_t seed, v
 /* Counts of samples first..first+count-1 of one method: counts_dev (device,
  * 22 uint64) receives [0] = collisions (no CIS) and [i] = samples of class i
  * (MOSS_METHOD_MOSS4MIN: its (class, c) slots).  Asynchronous on stream.
- * Shards of a sample range sum exactly. */
+ * Shards of a sample range sum exactly.  A call of 2^22 ids or more behind the
+ * edge filter may borrow up to 12 bytes per id (at most 805 MB) of device
+ * scratch from the library's pool, returned on the stream; without it (no
+ * memory, stream capture) the same counts come from the slower path. */
 int moss_sample_counts(moss_graph *g, int method, uint64_t first, uint64_t count, uint64_t seed,
                        void *stream, uint64_t *counts_dev);
 

@@ -751,6 +751,20 @@ static int sample_into(moss_graph *g, int method, uint64_t first, uint64_t count
         return MOSS_OK;
     }
     if (count > max_chunk) return fail(MOSS_EOVERFLOW, "count above %llu per call", (unsigned long long)max_chunk);
+    // a large call behind the filter is grouped (the same counts) when its
+    // scratch can be had; not under capture, where the call allocates nothing
+    const uint64_t scratch_bytes = classes ? 0 : group_bytes(method, dv, g->order != nullptr, count);
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusActive;
+    if (scratch_bytes && cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone) {
+        void *scratch = nullptr;
+        if (pool_alloc(g->device, &scratch, scratch_bytes, s) == cudaSuccess) {
+            const cudaError_t e = launch_counts_grouped(method, dv, first, count, seed, g->partials, scratch, counts_dev, s);
+            cudaFreeAsync(scratch, s);
+            MOSS_CUDA(e, "grouped sample kernels");
+            return MOSS_OK;
+        }
+        cudaGetLastError();   // no memory: the general path
+    }
     MOSS_CUDA(launch_counts(method, dv, first, count, seed, g->partials, classes, verts, counts_dev, s),
               "sample kernels");
     return MOSS_OK;

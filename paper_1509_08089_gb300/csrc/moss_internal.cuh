@@ -197,6 +197,11 @@ __host__ __device__ inline uint64_t mulhi64(uint64_t a, uint64_t b) {
 
 // floor(x * m / 2^64): a uniform index in [0, m) from a 64-bit word
 __device__ __forceinline__ uint64_t word_index(uint64_t x, uint64_t m) { return __umul64hi(x, m); }
+// the same for m < 2^32: two 32 x 32 -> 64 products instead of four
+__device__ __forceinline__ uint32_t word_index32(uint64_t x, uint32_t m) {
+    const uint64_t lo = (uint64_t)(uint32_t)x * m;
+    return (uint32_t)(((uint64_t)(uint32_t)(x >> 32) * m + (lo >> 32)) >> 32);
+}
 
 // ------------------------------------------------------------ warp scans --
 __device__ __forceinline__ uint64_t shfl_up64(uint64_t v, int d) { return __shfl_up_sync(0xffffffffu, v, d); }
@@ -391,9 +396,19 @@ void upload_luts(const uint8_t *lut4, const uint8_t *lut5, const uint8_t *lutc);
 cudaError_t launch_counts(int method, const DevGraph &g, uint64_t first, uint64_t count, uint64_t seed,
                           uint64_t *partials, uint8_t *classes, uint32_t *verts, uint64_t *counts_dev,
                           cudaStream_t s);
+// what follows the sampler launch of one chunk: Path-5's redraw stages and the reduce
+cudaError_t launch_tail(int method, const DevGraph &g, uint64_t first, uint64_t count, uint64_t seed,
+                        uint64_t *partials, int blocks, uint64_t *counts_dev, bool accumulate, cudaStream_t s);
 int sample_blocks(int method, int device);   // the most blocks any variant of a sampler launches
 int sample_launch_blocks(int method, int device, const DevGraph &g);   // blocks of the variant g uses
 int sample_rows(int method, int device);     // partial-count rows launch_counts needs
+
+// moss_group.cu: large calls behind the filter, the sample ids grouped by their first vertex
+void upload_luts_group(const uint8_t *lut4, const uint8_t *lut5, const uint8_t *lutc);
+// scratch of a grouped call; 0 when the call is not one to group
+uint64_t group_bytes(int method, const DevGraph &g, bool degree_order, uint64_t count);
+cudaError_t launch_counts_grouped(int method, const DevGraph &g, uint64_t first, uint64_t count, uint64_t seed,
+                                  uint64_t *partials, void *scratch, uint64_t *counts_dev, cudaStream_t s);
 
 // moss_finalize.cu
 struct FinalizeIn {
