@@ -5,8 +5,10 @@
 #include <cstdio>
 #include <cstring>
 #include <atomic>
+#include <memory>
 #include <mutex>
 #include <new>
+#include <vector>
 
 #include "../../include/moss.h"
 #include "moss_internal.cuh"
@@ -188,6 +190,74 @@ int ensure_luts(int device) {
 
 }  // namespace
 
+// ------------------------------------------------------------ host staging --
+// Totals and status flags as one record, so that one copy reads them back.
+struct DevStatus {
+    DevTotals tot;
+    uint32_t flags[2];
+};
+
+// Page-locked host memory of one graph: kernels write results straight into
+// it and totals are copied to it without staging (a copy into ordinary memory
+// costs the caller about 10 us each).
+struct Pinned {
+    moss_result res;
+    double cov[kSlots * kSlots];
+    DevStatus status;
+};
+
+namespace {
+// Slots of page-locked memory, kPinBatch per allocation (one costs tens of
+// us); an allocation with no slot in use is given back unless it is the only
+// one, so what is held follows the number of graphs alive.
+constexpr int kPinBatch = 32;
+struct PinBatch {
+    Pinned *mem = nullptr;
+    uint32_t used = 0;   // bit i: slot i taken
+};
+std::mutex g_pin_mutex;
+std::vector<PinBatch> g_pins;
+
+Pinned *pin_take() {
+    std::lock_guard<std::mutex> lk(g_pin_mutex);
+    for (PinBatch &b : g_pins)
+        for (int i = 0; i < kPinBatch; ++i)
+            if (!(b.used >> i & 1u)) {
+                b.used |= 1u << i;
+                return b.mem + i;
+            }
+    try {
+        g_pins.reserve(g_pins.size() + 1);
+    } catch (...) {
+        return nullptr;
+    }
+    PinBatch b;
+    if (cudaHostAlloc(reinterpret_cast<void **>(&b.mem), kPinBatch * sizeof(Pinned),
+                      cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    b.used = 1;
+    g_pins.push_back(b);
+    return b.mem;
+}
+
+void pin_give(Pinned *p) {
+    if (!p) return;
+    std::lock_guard<std::mutex> lk(g_pin_mutex);
+    for (size_t k = 0; k < g_pins.size(); ++k) {
+        PinBatch &b = g_pins[k];
+        if (p < b.mem || p >= b.mem + kPinBatch) continue;
+        b.used &= ~(1u << (p - b.mem));
+        if (!b.used && g_pins.size() > 1) {
+            cudaFreeHost(b.mem);
+            g_pins.erase(g_pins.begin() + k);
+        }
+        return;
+    }
+}
+}  // namespace
+
 // ------------------------------------------------------------ graph object --
 struct moss_graph {
     int device = 0;
@@ -230,7 +300,8 @@ struct moss_graph {
     uint32_t *hub_bits = nullptr;
     uint32_t *hub_list = nullptr;
     uint32_t *order = nullptr;   // input id of each internal vertex (MOSS_ORDER_DEGREE), else null
-    moss_result res_host{};      // host staging of the result
+    Pinned *pin = nullptr;       // what the device hands back (null: res_host through a copy)
+    moss_result res_host{};
     uint32_t flags_host[2] = {0, 0};
 };
 
@@ -245,6 +316,7 @@ void release(moss_graph *g) {
     if (g->filter) cudaFreeAsync(g->filter, 0);
     if (g->hub_mem) cudaFreeAsync(g->hub_mem, 0);
     if (g->min_arena) cudaFreeAsync(g->min_arena, 0);
+    pin_give(g->pin);
     delete g;
 }
 
@@ -360,10 +432,25 @@ struct Carver {
     }
 };
 
-int read_flags(moss_graph *g, cudaStream_t s) {
-    MOSS_CUDA(cudaMemcpyAsync(g->flags_host, g->flags, 2 * sizeof(uint32_t), cudaMemcpyDeviceToHost, s),
-              "reading status");
+// totals and status flags of the work queued on s (waits for it)
+int read_status(moss_graph *g, cudaStream_t s) {
+    DevStatus here;
+    DevStatus *to = g->pin ? &g->pin->status : &here;
+    MOSS_CUDA(cudaMemcpyAsync(to, g->tot, sizeof(DevStatus), cudaMemcpyDeviceToHost, s), "reading totals");
     MOSS_CUDA(cudaStreamSynchronize(s), "synchronising stream");
+    g->tot_h = to->tot;
+    memcpy(g->flags_host, to->flags, sizeof(to->flags));
+    return MOSS_OK;
+}
+
+// where a kernel on s leaves the result, and its arrival in *out (waits for s)
+moss_result *result_target(moss_graph *g) { return g->pin ? &g->pin->res : g->res_dev; }
+int read_result(moss_graph *g, cudaStream_t s, moss_result *out) {
+    if (!g->pin)
+        MOSS_CUDA(cudaMemcpyAsync(&g->res_host, g->res_dev, sizeof(moss_result), cudaMemcpyDeviceToHost, s),
+                  "reading result");
+    MOSS_CUDA(cudaStreamSynchronize(s), "synchronising stream");
+    if (out) memcpy(out, g->pin ? &g->pin->res : &g->res_host, sizeof(moss_result));
     return MOSS_OK;
 }
 
@@ -438,6 +525,7 @@ int moss_graph_load_csr_order(const void *row_ptr, int row_ptr_is_64, const uint
                                 : (n >= (1u << 14) ? MOSS_VERTEX_SPLIT_MID : MOSS_VERTEX_ONE_LEVEL);
     g->vsplit_min = n >= (1u << 20) ? MOSS_VERTEX_SPLIT_DEFAULT : MOSS_VERTEX_ONE_LEVEL;
     g->nnz = nnz;
+    g->pin = pin_take();
     void *rp_dev = nullptr;
     void *oscratch = nullptr;   // renumbering scratch (released before return)
     const size_t rp_bytes = (size_t)(n + 1ULL) * (row_ptr_is_64 ? 8 : 4);
@@ -475,12 +563,15 @@ int moss_graph_load_csr_order(const void *row_ptr, int row_ptr_is_64, const uint
                 g->gam[l] = c.take<u128>(n);
                 g->seed[l] = c.take<uint4>(2 * (uint64_t)n);
             }
-            g->tot = c.take<DevTotals>(1);
-            g->partials = c.take<uint64_t>((uint64_t)prow * kSlots + (uint64_t)slot_partial_rows(n) * 6 * 2);
+            {
+                DevStatus *st = c.take<DevStatus>(1);
+                g->tot = &st->tot;
+                g->flags = st->flags;
+            }
+            g->partials = c.take<uint64_t>(2 * (uint64_t)prow * kSlots + (uint64_t)slot_partial_rows(n) * 6 * 2);
             g->counts = c.take<uint64_t>(2 * kSlots);
             g->res_dev = c.take<moss_result>(1);
             g->cov_dev = c.take<double>(kSlots * kSlots);
-            g->flags = c.take<uint32_t>(2);
             g->defer = c.take<uint32_t>(kDeferChunk / 32);
             rp_dev = c.take<uint8_t>(rp_bytes);
             if (ordered) g->order = c.take<uint32_t>(n);
@@ -525,8 +616,7 @@ int moss_graph_load_csr_order(const void *row_ptr, int row_ptr_is_64, const uint
              "slot kernels");
         STEP(launch_totals(tp, slot_partial_rows(n), g->tot, s), "totals kernel");
     }
-    STEP(cudaMemcpyAsync(&g->tot_h, g->tot, sizeof(DevTotals), cudaMemcpyDeviceToHost, s), "reading totals");
-    rc = read_flags(g, s);
+    rc = read_status(g, s);
     if (rc) goto fail_out;
     if (!g->flags_host[0] && g->flags_host[1] != nnz) g->flags_host[0] |= kErrAsym;
     if (g->flags_host[0]) {
@@ -687,8 +777,7 @@ int moss_build_tables(moss_graph *g, unsigned k_mask, void *stream) {
     if (e == cudaSuccess) e = eh != cudaSuccess ? eh : ev;
     if (e != cudaSuccess) return cuda_fail(e, "table kernels");
     if (rc) return rc;
-    MOSS_CUDA(cudaMemcpyAsync(&g->tot_h, g->tot, sizeof(DevTotals), cudaMemcpyDeviceToHost, s), "reading totals");
-    rc = read_flags(g, s);
+    rc = read_status(g, s);
     if (rc) return rc;
     if (g->flags_host[0] & kErrOverflow) return fail(MOSS_EOVERFLOW, "a vertex weight total times n exceeds 2^128");
     g->built = 1u << 3;
@@ -735,8 +824,10 @@ int moss_vertex_levels(const moss_graph *g, int which, uint32_t *nheavy, uint64_
     return MOSS_OK;
 }
 
+// with `pending` the reduce of the (last chunk's) rows is left to the caller
 static int sample_into(moss_graph *g, int method, uint64_t first, uint64_t count, uint64_t seed, cudaStream_t s,
-                       uint64_t *counts_dev, uint8_t *classes, uint32_t *verts) {
+                       uint64_t *partials, uint64_t *counts_dev, uint8_t *classes, uint32_t *verts,
+                       CountRows *pending = nullptr) {
     if (method < 0 || method >= kMethods) return fail(MOSS_EINVAL, "method %d", method);
     if (!method_ready(g, method)) return fail(MOSS_ESTATE, "tables for method %d not built", method);
     if (count > 0 && g->tot_h.gamma[method] == 0)
@@ -747,7 +838,8 @@ static int sample_into(moss_graph *g, int method, uint64_t first, uint64_t count
     // per-warp 32-bit counters: keep each launch below 2^31 samples per warp
     const uint64_t max_chunk = (uint64_t)blocks * 8 * (1ULL << 31);
     if (count == 0) {
-        MOSS_CUDA(cudaMemsetAsync(counts_dev, 0, kSlots * sizeof(uint64_t), s), "clearing counts");
+        if (pending) *pending = CountRows{};
+        else MOSS_CUDA(cudaMemsetAsync(counts_dev, 0, kSlots * sizeof(uint64_t), s), "clearing counts");
         return MOSS_OK;
     }
     if (count > max_chunk) return fail(MOSS_EOVERFLOW, "count above %llu per call", (unsigned long long)max_chunk);
@@ -758,14 +850,15 @@ static int sample_into(moss_graph *g, int method, uint64_t first, uint64_t count
     if (scratch_bytes && cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone) {
         void *scratch = nullptr;
         if (pool_alloc(g->device, &scratch, scratch_bytes, s) == cudaSuccess) {
-            const cudaError_t e = launch_counts_grouped(method, dv, first, count, seed, g->partials, scratch, counts_dev, s);
+            const cudaError_t e = launch_counts_grouped(method, dv, first, count, seed, partials, scratch, counts_dev, s,
+                                                        pending);
             cudaFreeAsync(scratch, s);
             MOSS_CUDA(e, "grouped sample kernels");
             return MOSS_OK;
         }
         cudaGetLastError();   // no memory: the general path
     }
-    MOSS_CUDA(launch_counts(method, dv, first, count, seed, g->partials, classes, verts, counts_dev, s),
+    MOSS_CUDA(launch_counts(method, dv, first, count, seed, partials, classes, verts, counts_dev, s, pending),
               "sample kernels");
     return MOSS_OK;
 }
@@ -774,7 +867,8 @@ int moss_sample_counts(moss_graph *g, int method, uint64_t first, uint64_t count
                        uint64_t *counts_dev) {
     if (!g || !counts_dev) return fail(MOSS_EINVAL, "NULL argument");
     DeviceGuard dg(g->device);
-    return sample_into(g, method, first, count, seed, static_cast<cudaStream_t>(stream), counts_dev, nullptr, nullptr);
+    return sample_into(g, method, first, count, seed, static_cast<cudaStream_t>(stream), g->partials, counts_dev, nullptr,
+                       nullptr);
 }
 
 int moss_sample_records(moss_graph *g, int method, uint64_t first, uint64_t count, uint64_t seed, void *stream,
@@ -782,7 +876,7 @@ int moss_sample_records(moss_graph *g, int method, uint64_t first, uint64_t coun
     if (!g || !classes_dev) return fail(MOSS_EINVAL, "NULL argument");
     DeviceGuard dg(g->device);
     const cudaStream_t s = static_cast<cudaStream_t>(stream);
-    const int rc = sample_into(g, method, first, count, seed, s, g->counts, classes_dev, verts_dev);
+    const int rc = sample_into(g, method, first, count, seed, s, g->partials, g->counts, classes_dev, verts_dev);
     if (rc || !g->order || !verts_dev) return rc;
     // vertex words of the records back to input ids (MOSS-4 and MOSS-4Min: the first four)
     MOSS_CUDA(launch_map_records(verts_dev, count, method == 1 || method == 2 ? 5 : 4, g->order, g->n, s),
@@ -790,16 +884,19 @@ int moss_sample_records(moss_graph *g, int method, uint64_t first, uint64_t coun
     return MOSS_OK;
 }
 
-static int finalize_from_device(moss_graph *g, int k, const uint64_t K[2], cudaStream_t s, moss_result *out) {
-    FinalizeIn in;
-    in.k = k;
-    in.K[0] = K[0];
-    in.K[1] = K[1];
-    MOSS_CUDA(launch_finalize(in, g->counts, g->tot, g->res_dev, s), "finalize kernel");
-    MOSS_CUDA(cudaMemcpyAsync(&g->res_host, g->res_dev, sizeof(moss_result), cudaMemcpyDeviceToHost, s), "reading result");
-    MOSS_CUDA(cudaStreamSynchronize(s), "synchronising stream");
-    memcpy(out, &g->res_host, sizeof(moss_result));
-    return MOSS_OK;
+// Both sub-methods of an estimate (ids from 0) up to their rows of counts:
+// in one launch when they are small enough (same counts).
+static int sample_both(moss_graph *g, int ma, uint64_t ka, int mb, uint64_t kb, uint64_t seed, cudaStream_t s,
+                       CountRows *a, CountRows *b) {
+    const bool mix = ma == MOSS_METHOD_MOSS4;
+    if (pair_fits(mix, ka, kb)) {
+        MOSS_CUDA(launch_pair(mix, view(g), ka, kb, seed, g->partials, a, b, s), "sample kernels");
+        return MOSS_OK;
+    }
+    const int rc = sample_into(g, ma, 0, ka, seed, s, g->partials, g->counts, nullptr, nullptr, a);
+    if (rc) return rc;
+    return sample_into(g, mb, 0, kb, seed, s, g->partials + (uint64_t)g->partial_rows * kSlots, g->counts + kSlots,
+                       nullptr, nullptr, b);
 }
 
 int moss_sample_estimate(moss_graph *g, int k, uint64_t budget, uint64_t seed, void *stream, moss_result *out) {
@@ -807,31 +904,65 @@ int moss_sample_estimate(moss_graph *g, int k, uint64_t budget, uint64_t seed, v
     if (k != 4 && k != 5) return fail(MOSS_EINVAL, "k must be 4 or 5 (got %d)", k);
     DeviceGuard dg(g->device);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    uint64_t K[2] = {0, 0};
+    FinalizeIn in;
+    in.k = k;
+    in.K[0] = in.K[1] = 0;
+    CountRows a, b;
     int rc;
     if (k == 4) {
         if (!method_ready(g, 0)) return fail(MOSS_ESTATE, "tables for k=4 not built");
-        K[0] = g->tot_h.gamma[0] ? budget : 0;
-        MOSS_CUDA(cudaMemsetAsync(g->counts + kSlots, 0, kSlots * sizeof(uint64_t), s), "clearing counts");
-        if ((rc = sample_into(g, 0, 0, K[0], seed, s, g->counts, nullptr, nullptr))) return rc;
+        in.K[0] = g->tot_h.gamma[0] ? budget : 0;
+        if ((rc = sample_into(g, 0, 0, in.K[0], seed, s, g->partials, g->counts, nullptr, nullptr, &a))) return rc;
     } else {
         if (!method_ready(g, 1) || !method_ready(g, 2)) return fail(MOSS_ESTATE, "tables for k=5 not built");
-        K[0] = g->tot_h.gamma[1] ? budget / 2 : 0;
-        K[1] = g->tot_h.gamma[2] ? budget - budget / 2 : 0;
-        if ((rc = sample_into(g, 1, 0, K[0], seed, s, g->counts, nullptr, nullptr))) return rc;
-        if ((rc = sample_into(g, 2, 0, K[1], seed, s, g->counts + kSlots, nullptr, nullptr))) return rc;
+        in.K[0] = g->tot_h.gamma[1] ? budget / 2 : 0;
+        in.K[1] = g->tot_h.gamma[2] ? budget - budget / 2 : 0;
+        if ((rc = sample_both(g, 1, in.K[0], 2, in.K[1], seed, s, &a, &b))) return rc;
     }
-    return finalize_from_device(g, k, K, s, out);
+    MOSS_CUDA(launch_reduce_finalize(in, a, b, g->tot, result_target(g), s), "finalize kernel");
+    return read_result(g, s, out);
+}
+
+// Counts handed in by the caller: host memory travels as a kernel argument,
+// device memory is read where it is copied to.
+static int counts_arg(moss_graph *g, const uint64_t *hits, cudaStream_t s, HitsArg *arg) {
+    cudaPointerAttributes pa;
+    const bool known = cudaPointerGetAttributes(&pa, hits) == cudaSuccess;
+    if (!known) cudaGetLastError();
+    arg->dev = nullptr;
+    if (!known || pa.type == cudaMemoryTypeUnregistered || pa.type == cudaMemoryTypeHost) {
+        memcpy(arg->h, hits, sizeof(arg->h));
+        return MOSS_OK;
+    }
+    MOSS_CUDA(cudaMemcpyAsync(g->counts, hits, sizeof(arg->h), cudaMemcpyDefault, s), "copying counts");
+    arg->dev = g->counts;
+    return MOSS_OK;
+}
+
+static int finalize_given(moss_graph *g, const FinalizeIn &in, const uint64_t *hits, cudaStream_t s, double *cov_host,
+                          moss_result *out) {
+    HitsArg arg;
+    const int rc = counts_arg(g, hits, s, &arg);
+    if (rc) return rc;
+    double *cov = cov_host ? (g->pin ? g->pin->cov : g->cov_dev) : nullptr;
+    MOSS_CUDA(launch_finalize(in, arg, g->tot, result_target(g), cov, s), "finalize kernel");
+    if (cov_host && !g->pin)
+        MOSS_CUDA(cudaMemcpyAsync(cov_host, g->cov_dev, sizeof(g->pin->cov), cudaMemcpyDeviceToHost, s),
+                  "reading covariance");
+    const int rr = read_result(g, s, out);
+    if (!rr && cov_host && g->pin) memcpy(cov_host, g->pin->cov, sizeof(g->pin->cov));
+    return rr;
 }
 
 int moss_finalize(moss_graph *g, int k, const uint64_t *K, const uint64_t *hits, void *stream, moss_result *out) {
     if (!g || !K || !hits || !out) return fail(MOSS_EINVAL, "NULL argument");
     if (k != 4 && k != 5) return fail(MOSS_EINVAL, "k must be 4 or 5 (got %d)", k);
     DeviceGuard dg(g->device);
-    cudaStream_t s = static_cast<cudaStream_t>(stream);
-    MOSS_CUDA(cudaMemcpyAsync(g->counts, hits, 2 * kSlots * sizeof(uint64_t), cudaMemcpyDefault, s), "copying counts");
-    uint64_t KK[2] = {K[0], k == 4 ? 0 : K[1]};
-    return finalize_from_device(g, k, KK, s, out);
+    FinalizeIn in;
+    in.k = k;
+    in.K[0] = K[0];
+    in.K[1] = k == 4 ? 0 : K[1];
+    return finalize_given(g, in, hits, static_cast<cudaStream_t>(stream), nullptr, out);
 }
 
 int moss_covariance(moss_graph *g, int k, const uint64_t *K, const uint64_t *hits, void *stream, double *cov_host,
@@ -839,20 +970,11 @@ int moss_covariance(moss_graph *g, int k, const uint64_t *K, const uint64_t *hit
     if (!g || !K || !hits || !cov_host) return fail(MOSS_EINVAL, "NULL argument");
     if (k != 4 && k != 5) return fail(MOSS_EINVAL, "k must be 4 or 5 (got %d)", k);
     DeviceGuard dg(g->device);
-    cudaStream_t s = static_cast<cudaStream_t>(stream);
-    MOSS_CUDA(cudaMemcpyAsync(g->counts, hits, 2 * kSlots * sizeof(uint64_t), cudaMemcpyDefault, s), "copying counts");
     FinalizeIn in;
     in.k = k;
     in.K[0] = K[0];
     in.K[1] = k == 4 ? 0 : K[1];
-    MOSS_CUDA(launch_covariance(in, g->counts, g->tot, g->res_dev, g->cov_dev, s), "covariance kernel");
-    MOSS_CUDA(cudaMemcpyAsync(cov_host, g->cov_dev, kSlots * kSlots * sizeof(double), cudaMemcpyDeviceToHost, s),
-              "reading covariance");
-    MOSS_CUDA(cudaMemcpyAsync(&g->res_host, g->res_dev, sizeof(moss_result), cudaMemcpyDeviceToHost, s),
-              "reading result");
-    MOSS_CUDA(cudaStreamSynchronize(s), "synchronising stream");
-    if (out) memcpy(out, &g->res_host, sizeof(moss_result));
-    return MOSS_OK;
+    return finalize_given(g, in, hits, static_cast<cudaStream_t>(stream), cov_host, out);
 }
 
 int moss_sample_estimate_min(moss_graph *g, uint64_t budget, uint64_t budget_min, uint64_t seed, void *stream,
@@ -867,15 +989,11 @@ int moss_sample_estimate_min(moss_graph *g, uint64_t budget, uint64_t budget_min
     in.mix = 1;
     in.K[0] = g->tot_h.gamma[0] ? budget : 0;
     in.K[1] = g->tot_h.gamma[3] ? budget_min : 0;
-    int rc;
-    if ((rc = sample_into(g, MOSS_METHOD_MOSS4, 0, in.K[0], seed, s, g->counts, nullptr, nullptr))) return rc;
-    if ((rc = sample_into(g, MOSS_METHOD_MOSS4MIN, 0, in.K[1], seed, s, g->counts + kSlots, nullptr, nullptr)))
-        return rc;
-    MOSS_CUDA(launch_finalize(in, g->counts, g->tot, g->res_dev, s), "finalize kernel");
-    MOSS_CUDA(cudaMemcpyAsync(&g->res_host, g->res_dev, sizeof(moss_result), cudaMemcpyDeviceToHost, s), "reading result");
-    MOSS_CUDA(cudaStreamSynchronize(s), "synchronising stream");
-    memcpy(out, &g->res_host, sizeof(moss_result));
-    return MOSS_OK;
+    CountRows a, b;
+    const int rc = sample_both(g, MOSS_METHOD_MOSS4, in.K[0], MOSS_METHOD_MOSS4MIN, in.K[1], seed, s, &a, &b);
+    if (rc) return rc;
+    MOSS_CUDA(launch_reduce_finalize(in, a, b, g->tot, result_target(g), s), "finalize kernel");
+    return read_result(g, s, out);
 }
 
 int moss_finalize_min(moss_graph *g, const uint64_t *K, const uint64_t *hits, void *stream, double *cov_host,
@@ -883,25 +1001,12 @@ int moss_finalize_min(moss_graph *g, const uint64_t *K, const uint64_t *hits, vo
     if (!g || !K || !hits || !out) return fail(MOSS_EINVAL, "NULL argument");
     if (!(g->built >> 5 & 1u)) return fail(MOSS_ESTATE, "MOSS-4Min tables not built (Gamma-check unknown)");
     DeviceGuard dg(g->device);
-    cudaStream_t s = static_cast<cudaStream_t>(stream);
-    MOSS_CUDA(cudaMemcpyAsync(g->counts, hits, 2 * kSlots * sizeof(uint64_t), cudaMemcpyDefault, s), "copying counts");
     FinalizeIn in;
     in.k = 4;
     in.mix = 1;
     in.K[0] = K[0];
     in.K[1] = K[1];
-    if (cov_host) {
-        MOSS_CUDA(launch_covariance(in, g->counts, g->tot, g->res_dev, g->cov_dev, s), "covariance kernel");
-        MOSS_CUDA(cudaMemcpyAsync(cov_host, g->cov_dev, kSlots * kSlots * sizeof(double), cudaMemcpyDeviceToHost, s),
-                  "reading covariance");
-    } else {
-        MOSS_CUDA(launch_finalize(in, g->counts, g->tot, g->res_dev, s), "finalize kernel");
-    }
-    MOSS_CUDA(cudaMemcpyAsync(&g->res_host, g->res_dev, sizeof(moss_result), cudaMemcpyDeviceToHost, s),
-              "reading result");
-    MOSS_CUDA(cudaStreamSynchronize(s), "synchronising stream");
-    memcpy(out, &g->res_host, sizeof(moss_result));
-    return MOSS_OK;
+    return finalize_given(g, in, hits, static_cast<cudaStream_t>(stream), cov_host, out);
 }
 
 int moss_graph_stats(const moss_graph *g, moss_stats *out) {

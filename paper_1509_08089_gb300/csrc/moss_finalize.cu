@@ -46,12 +46,30 @@ __device__ __forceinline__ double warp_sum_d(double v) {
     return v;
 }
 
+// Row `row` of the covariance matrix, lane i its column i: c between sampled
+// classes, c2 in column 2 and its mirror in row 2, zeros elsewhere; row 2
+// itself holds its variance (when have2) and the zeros of what is no class.
+__device__ __forceinline__ void cov_row(double *cov, int row, int i, bool sampled, bool row_sampled, double c,
+                                        double c2, bool have2, double var2) {
+    if (i >= kSlots) return;
+    if (row == 2) {
+        if (i == 2) cov[2 * kSlots + 2] = have2 ? var2 : 0.0;
+        else if (!sampled) cov[2 * kSlots + i] = 0.0;
+    } else if (row_sampled) {
+        cov[row * kSlots + i] = i == 2 ? c2 : c;
+        if (i == 2) cov[2 * kSlots + row] = c2;
+    } else {
+        cov[row * kSlots + i] = 0.0;
+    }
+}
+
 // MOSS-5 with one warp: lane i is class i (1..21); the sums over classes
 // (the eta_2 identity, its variance, the concentrations) are warp sums.
 // hits0/hits1: counts of the two sub-methods (either may be null); cov
-// (nullable, 22 x 22 row-major) receives the covariance matrix.
+// (nullable, 22 x 22 row-major) receives row `row` of the covariance matrix,
+// and its mirror in row 2 (cov_row).
 __device__ void finalize5_warp(const FinalizeIn &in, const uint64_t *hits0, const uint64_t *hits1,
-                               const DevTotals *tot, moss_result *out, double *cov) {
+                               const DevTotals *tot, moss_result *out, double *cov, int row) {
     const int i = threadIdx.x & 31;
     const bool cls = i >= 1 && i <= 21;
     const double G0 = u128_to_double(tot->gamma[1]), G1 = u128_to_double(tot->gamma[2]);
@@ -109,7 +127,7 @@ __device__ void finalize5_warp(const FinalizeIn &in, const uint64_t *hits0, cons
         var = v2;
     }
     const double t = warp_sum_d(cls ? est : 0.0);         // concentrations (Sec. 6.3)
-    if (i < kSlots) {
+    if (out && i < kSlots) {
         out->hits[0][i] = h0;
         out->hits[1][i] = h1;
         out->est[i] = est;
@@ -118,7 +136,7 @@ __device__ void finalize5_warp(const FinalizeIn &in, const uint64_t *hits0, cons
         out->lambda[1][i] = a1;
         out->conc[i] = (cls && t != 0.0) ? est / t : 0.0;
     }
-    if (i == 0) {
+    if (out && i == 0) {
         out->k = 5;
         out->n_classes = 21;
         out->K[0] = in.K[0];
@@ -127,35 +145,26 @@ __device__ void finalize5_warp(const FinalizeIn &in, const uint64_t *hits0, cons
         out->triangles_var = 0.0;
     }
     if (cov) {
-        // lane j fills column j; Cov(eta_i, eta_j) = -plug_i plug_j sum_l a_i a_j / K_l
-        // off the diagonal, and row/column 2 from the linear identity
-        const bool colj = cls && i != 2;
+        // Cov(eta_r, eta_i) = -plug_r plug_i sum_l a_r a_i / K_l off the diagonal
+        const bool sampled = cls && i != 2, rowr = row >= 1 && row <= 21 && row != 2;
         const double c0 = a0 * plug, c1 = a1 * plug;
-        double c2 = 0.0;
-        for (int r = 0; r < kSlots; ++r) {
-            const double c0r = __shfl_sync(0xffffffffu, c0, r), c1r = __shfl_sync(0xffffffffu, c1, r);
-            const bool rowr = r >= 1 && r <= 21 && r != 2;
-            double c = 0.0;
-            if (rowr && colj) {
-                if (r == i) {
-                    c = var;
-                } else {
-                    if (av0) c -= c0r * c0 / K0;
-                    if (av1) c -= c1r * c1 / K1;
-                }
+        const double c0r = __shfl_sync(0xffffffffu, c0, row), c1r = __shfl_sync(0xffffffffu, c1, row);
+        double c = 0.0;
+        if (rowr && sampled) {
+            if (i == row) {
+                c = var;
+            } else {
+                if (av0) c -= c0r * c0 / K0;
+                if (av1) c -= c1r * c1 / K1;
             }
-            if (i < kSlots && r != 2) cov[r * kSlots + i] = c;
-            if (rowr && kPhi5[r - 1][2] > 0) c2 -= kPhi5[r - 1][2] * c;
         }
-        __syncwarp();
-        if (colj) {
-            cov[2 * kSlots + i] = c2;
-            cov[i * kSlots + 2] = c2;
-        } else if (i == 2) {
-            cov[2 * kSlots + 2] = var;
-        } else if (i < kSlots) {
-            cov[2 * kSlots + i] = 0.0;
+        // eta_2's linear identity: Cov(eta_2, eta_r) = -sum phi^(3)_j Cov(eta_j, eta_r)
+        double c2 = 0.0;
+        for (int j = 1; j <= 21; ++j) {
+            const double cj = __shfl_sync(0xffffffffu, c, j);
+            if (j != 2 && kPhi5[j - 1][2] > 0) c2 -= kPhi5[j - 1][2] * cj;
         }
+        cov_row(cov, row, i, sampled, rowr, c, c2, true, var);
     }
 }
 
@@ -163,9 +172,12 @@ __device__ void finalize5_warp(const FinalizeIn &in, const uint64_t *hits0, cons
 // class i (1..6); the eta_2 identity, its variance and the covariances are
 // formed on every lane from the values of classes 4, 5, 6 gathered by
 // shuffles, in the order the formulas are written; the concentrations' sum
-// is a warp sum.
+// is a warp sum.  The divisions, the slow part (FP64 runs at 1/64 of the FP32
+// rate: about 1 us each in a dependent chain), are spread over the lanes: a
+// lane per (class, c) slot of MOSS-4Min and per term of n_2's variance (one
+// lane did 24 divisions in turn before, 52 us for the mix from a cold start).
 __device__ void finalize4_warp(const FinalizeIn &in, const uint64_t *hits0, const uint64_t *hits1,
-                               const DevTotals *tot, moss_result *out, double *cov) {
+                               const DevTotals *tot, moss_result *out, double *cov, int row) {
     const int i = threadIdx.x & 31;
     const bool cls = i >= 1 && i <= 6, mix = in.mix != 0;
     const double G = u128_to_double(tot->gamma[0]), Gm = mix ? u128_to_double(tot->gamma[3]) : 0.0;
@@ -182,15 +194,19 @@ __device__ void finalize4_warp(const FinalizeIn &in, const uint64_t *hits0, cons
     const int first = i == 3 ? 0 : (i == 5 ? 4 : 10), nslot = i == 3 ? 4 : (i == 5 ? 6 : (i == 6 ? 12 : 0));
     const bool s1 = av1 && nslot > 0;
     double em = 0.0, h = 0.0;
-    if (s1) {
+    if (av1) {   // warp-uniform: lane l holds slot l's hits over its c and c^2
+        const int c = i < 4 ? i + 1 : (i < 10 ? i - 3 : i - 9);
+        const double ma = (double)h1 / c, mb = (double)h1 / (c * c);
         double sa = 0.0, sb = 0.0;
-        for (int c = 1; c <= nslot; ++c) {
-            const double m = (double)hits1[first + c - 1];
-            sa += m / c;
-            sb += m / (c * c);
+        for (int k = 0; k < 12; ++k) {
+            const double x = __shfl_sync(0xffffffffu, ma, first + k), y = __shfl_sync(0xffffffffu, mb, first + k);
+            if (k < nslot) {
+                sa += x;
+                sb += y;
+            }
         }
-        em = Gm / (2.0 * Km) * sa;
-        h = sa > 0 ? sb / sa : (i == 6 ? 1.0 / 3.0 : 1.0);
+        if (s1) em = Gm / (2.0 * Km) * sa;
+        if (s1) h = sa > 0 ? sb / sa : (i == 6 ? 1.0 / 3.0 : 1.0);
     }
     double est = 0.0, var = 0.0, plug = 0.0, a0 = 0.0, a1 = 0.0;
     if (s0 != s1) {
@@ -235,24 +251,23 @@ __device__ void finalize4_warp(const FinalizeIn &in, const uint64_t *hits0, cons
             const double s = E[4] + 2.0 * E[5] + 4.0 * E[6];
             v2 = (E[4] / P[4] + 4.0 * E[5] / P[5] + 16.0 * E[6] / P[6] - s * s) / K;
         }
-    } else if (av0 || av1) {
-        for (int r = 4; r <= 6; ++r)
-            for (int c = 4; c <= 6; ++c) {
-                double cv = Vv[r];
-                if (r != c) {
-                    cv = 0.0;
-                    if (av0) cv -= B0[r] * B0[c] / K;
-                    if (av1) cv -= B1[r] * B1[c] / Km;
-                }
-                v2 += coef[r] * coef[c] * cv;
-            }
+    } else if (av0 || av1) {   // lane 3 (r - 4) + c - 4 forms the term of classes r, c
+        const int l = i < 9 ? i : 0, r = 4 + l / 3, c = 4 + l % 3;
+        auto of = [](const double (&x)[7], int k) { return k == 4 ? x[4] : (k == 5 ? x[5] : x[6]); };
+        double cv = of(Vv, r);
+        if (r != c) {
+            cv = 0.0;
+            if (av0) cv -= of(B0, r) * of(B0, c) / K;
+            if (av1) cv -= of(B1, r) * of(B1, c) / Km;
+        }
+        for (int k = 0; k < 9; ++k) v2 += coef[4 + k / 3] * coef[4 + k % 3] * __shfl_sync(0xffffffffu, cv, k);
     }
     if (i == 2) {
         est = est2;
         var = v2;
     }
     const double t = warp_sum_d(cls ? est : 0.0);          // concentrations (Sec. 6.3)
-    if (i < kSlots) {
+    if (out && i < kSlots) {
         out->hits[0][i] = h0;
         out->hits[1][i] = h1;
         out->est[i] = est;
@@ -261,29 +276,25 @@ __device__ void finalize4_warp(const FinalizeIn &in, const uint64_t *hits0, cons
         out->lambda[1][i] = mix ? a1 : 0.0;
         out->conc[i] = (cls && t != 0.0) ? est / t : 0.0;
     }
-    if (i == 0) {
+    if (out && i == 0) {
         out->k = 4;
         out->n_classes = 6;
         out->K[0] = mix ? (av0 ? in.K[0] : 0) : in.K[0];
         out->K[1] = mix ? (av1 ? in.K[1] : 0) : in.K[1];
-        out->triangles = av0 ? (double)h0 * G / (6.0 * K) : 0.0;
-        out->triangles_var = av0 ? out->triangles / K * (G / 6.0 - out->triangles) : 0.0;
+        const double tri = av0 ? (double)h0 * G / (6.0 * K) : 0.0;
+        out->triangles = tri;
+        out->triangles_var = av0 ? tri / K * (G / 6.0 - tri) : 0.0;
     }
     if (cov) {
-        // lane j fills column j: Cov(n_i, n_j) = -sum_l b_i b_j / K_l off the
-        // diagonal (b = a^(l) plug; -n_i n_j / K for MOSS-4 alone), row and
-        // column 2 from the linear identity
-        for (int r = 0; r < kSlots; ++r)
-            if (i < kSlots) cov[r * kSlots + i] = 0.0;
-        __syncwarp();
-        const bool colj = cls && i != 2 && (mix || av0);
+        // Cov(n_r, n_i) = -sum_l b_r b_i / K_l off the diagonal (b = a^(l) plug;
+        // -n_r n_i / K for MOSS-4 alone)
+        const bool have = mix || av0;
+        const bool sampled = cls && i != 2, rowr = row >= 1 && row <= 6 && row != 2;
         const double b0 = mix ? a0 * plug : est, b1 = a1 * plug;
-        double c2 = 0.0;
-        for (int r = 1; r <= 6; ++r) {
-            const double b0r = __shfl_sync(0xffffffffu, b0, r), b1r = __shfl_sync(0xffffffffu, b1, r);
-            if (r == 2 || !colj) continue;
-            double c = 0.0;
-            if (r == i) {
+        const double b0r = __shfl_sync(0xffffffffu, b0, row), b1r = __shfl_sync(0xffffffffu, b1, row);
+        double c = 0.0;
+        if (have && rowr && sampled) {
+            if (i == row) {
                 c = var;
             } else if (mix) {
                 if (av0) c -= b0r * b0 / K;
@@ -291,39 +302,56 @@ __device__ void finalize4_warp(const FinalizeIn &in, const uint64_t *hits0, cons
             } else {
                 c = -b0r * b0 / K;
             }
-            cov[r * kSlots + i] = c;
-            if (r >= 4) {
-                if (mix) c2 -= coef[r] * c;
-                else c2 += coef[r] * c;
-            }
         }
-        __syncwarp();
-        if (colj) {
-            if (!mix) c2 = -c2;
-            cov[2 * kSlots + i] = c2;
-            cov[i * kSlots + 2] = c2;
-        } else if (i == 2 && (mix || av0)) {
-            cov[2 * kSlots + 2] = v2;
-        }
+        double c2 = 0.0;   // n_2's linear identity (eq. 2)
+        for (int j = 4; j <= 6; ++j) c2 -= coef[j] * __shfl_sync(0xffffffffu, c, j);
+        cov_row(cov, row, i, sampled, rowr, c, c2, have, v2);
     }
 }
 
-// called by a whole warp: a lane per class
+// called by a whole warp: a lane per class; out and cov are nullable
 __device__ void finalize_any(const FinalizeIn &in, const uint64_t *hits0, const uint64_t *hits1,
-                             const DevTotals *tot, moss_result *out, double *cov = nullptr) {
-    if (in.k == 5 && !in.mix) finalize5_warp(in, hits0, hits1, tot, out, cov);
-    else finalize4_warp(in, hits0, hits1, tot, out, cov);
+                             const DevTotals *tot, moss_result *out, double *cov = nullptr, int row = 0) {
+    if (in.k == 5 && !in.mix) finalize5_warp(in, hits0, hits1, tot, out, cov, row);
+    else finalize4_warp(in, hits0, hits1, tot, out, cov, row);
 }
 
-// one warp
-__global__ void k_covariance(FinalizeIn in, const uint64_t *hits, const DevTotals *tot, moss_result *out,
-                             double *cov) {
-    finalize_any(in, hits, hits + kSlots, tot, out, cov);
+// A block of one warp; with cov a block per row: every block finalizes (so
+// nothing passes between them) and writes its row, block 0 also the result.
+// One warp walking the 22 rows took 51 us, all of it FP64 division latency.
+__global__ void k_finalize(FinalizeIn in, const __grid_constant__ HitsArg hits, const DevTotals *tot, moss_result *out,
+                           double *cov) {
+    const int row = blockIdx.x;
+    const uint64_t *h = hits.dev ? hits.dev : hits.h;
+    finalize_any(in, h, h + kSlots, tot, row == 0 ? out : nullptr, cov, row);
 }
 
-// one warp
-__global__ void k_finalize(FinalizeIn in, const uint64_t *hits, const DevTotals *tot, moss_result *out) {
-    finalize_any(in, hits, hits + kSlots, tot, out);
+// The counts of both sub-methods from their rows (thread t adds slot t %
+// kSlots of every 32nd row from row t / kSlots, the rows of both together),
+// then the finalize on the first warp: one launch for two reduces and a
+// finalize.
+__global__ void __launch_bounds__(32 * kSlots) k_reduce_finalize(FinalizeIn in, CountRows a, CountRows b,
+                                                                 const DevTotals *tot, moss_result *out) {
+    __shared__ uint64_t part[2][32][kSlots];
+    __shared__ uint64_t hits[2][kSlots];
+    const int c = threadIdx.x % kSlots, r0 = threadIdx.x / kSlots;
+    uint64_t s0 = 0, s1 = 0;
+#pragma unroll 4
+    for (int r = r0; r < a.n; r += 32) s0 += a.rows[(uint64_t)r * kSlots + c];
+#pragma unroll 4
+    for (int r = r0; r < b.n; r += 32) s1 += b.rows[(uint64_t)r * kSlots + c];
+    part[0][r0][c] = s0;
+    part[1][r0][c] = s1;
+    __syncthreads();
+    if (threadIdx.x < 2 * kSlots) {
+        const int m = threadIdx.x / kSlots;
+        const uint64_t *base = m ? b.base : a.base;
+        uint64_t t = base ? base[c] : 0;
+        for (int r = 0; r < 32; ++r) t += part[m][r][c];
+        hits[m][c] = t;
+    }
+    __syncthreads();
+    if (threadIdx.x < 32) finalize_any(in, hits[0], hits[1], tot, out);
 }
 
 // one warp per request of a batch
@@ -340,15 +368,15 @@ __global__ void k_finalize_batch(const BatchRequest *reqs, int nreq, const uint6
 
 }  // namespace
 
-cudaError_t launch_finalize(const FinalizeIn &in, const uint64_t *hits_dev, const DevTotals *tot, void *result_dev,
+cudaError_t launch_finalize(const FinalizeIn &in, const HitsArg &hits, const DevTotals *tot, void *result, double *cov,
                             cudaStream_t s) {
-    k_finalize<<<1, 32, 0, s>>>(in, hits_dev, tot, static_cast<moss_result *>(result_dev));
+    k_finalize<<<cov ? kSlots : 1, 32, 0, s>>>(in, hits, tot, static_cast<moss_result *>(result), cov);
     return cudaGetLastError();
 }
 
-cudaError_t launch_covariance(const FinalizeIn &in, const uint64_t *hits_dev, const DevTotals *tot, void *result_dev,
-                              double *cov_dev, cudaStream_t s) {
-    k_covariance<<<1, 32, 0, s>>>(in, hits_dev, tot, static_cast<moss_result *>(result_dev), cov_dev);
+cudaError_t launch_reduce_finalize(const FinalizeIn &in, const CountRows &a, const CountRows &b, const DevTotals *tot,
+                                   void *result_dev, cudaStream_t s) {
+    k_reduce_finalize<<<1, 32 * kSlots, 0, s>>>(in, a, b, tot, static_cast<moss_result *>(result_dev));
     return cudaGetLastError();
 }
 

@@ -298,7 +298,8 @@ uint64_t group_bytes(int method, const DevGraph &g, bool degree_order, uint64_t 
 }
 
 cudaError_t launch_counts_grouped(int method, const DevGraph &g, uint64_t first, uint64_t count, uint64_t seed,
-                                  uint64_t *partials, void *scratch, uint64_t *counts_dev, cudaStream_t s) {
+                                  uint64_t *partials, void *scratch, uint64_t *counts_dev, cudaStream_t s,
+                                  CountRows *pending) {
     const bool philox = g.rng == kRngPhilox;
     const int sms = current_sms(), blocks = sms * (philox ? group_blocks<kRngPhilox>() : group_blocks<kRngSplitMix>());
     const uint64_t chunk = std::min(count, kGroupChunk);
@@ -307,7 +308,9 @@ cudaError_t launch_counts_grouped(int method, const DevGraph &g, uint64_t first,
         const uint32_t len = (uint32_t)std::min(chunk, count - c0);
         cudaError_t e = philox ? run_method<kRngPhilox>(method, g, first + c0, len, seed, w, partials, sms, blocks, s)
                                : run_method<kRngSplitMix>(method, g, first + c0, len, seed, w, partials, sms, blocks, s);
-        if (e == cudaSuccess) e = launch_tail(method, g, first + c0, len, seed, partials, blocks, counts_dev, c0 > 0, s);
+        if (e == cudaSuccess)
+            e = launch_tail(method, g, first + c0, len, seed, partials, blocks, nullptr, nullptr, counts_dev, c0 > 0, s,
+                            c0 + len == count ? pending : nullptr);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;

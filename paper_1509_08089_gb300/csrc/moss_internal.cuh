@@ -393,12 +393,26 @@ void upload_luts(const uint8_t *lut4, const uint8_t *lut5, const uint8_t *lutc);
 // entries); partials holds sample_rows(method) rows of 22 uint64.  Path-5 runs
 // in chunks of kDeferChunk ids: a launch that defers the samples whose first
 // sigma attempt collides, one that redoes them, and a reduce that accumulates.
+// With `pending` the last chunk's reduce is left to the caller, who gets its
+// rows (and counts_dev as the base to add when earlier chunks are in it).
+struct CountRows {
+    const uint64_t *rows = nullptr;   // n rows of kSlots partial counts
+    int n = 0;
+    const uint64_t *base = nullptr;   // kSlots counts to add, or null
+};
 cudaError_t launch_counts(int method, const DevGraph &g, uint64_t first, uint64_t count, uint64_t seed,
                           uint64_t *partials, uint8_t *classes, uint32_t *verts, uint64_t *counts_dev,
-                          cudaStream_t s);
+                          cudaStream_t s, CountRows *pending = nullptr);
 // what follows the sampler launch of one chunk: Path-5's redraw stages and the reduce
 cudaError_t launch_tail(int method, const DevGraph &g, uint64_t first, uint64_t count, uint64_t seed,
-                        uint64_t *partials, int blocks, uint64_t *counts_dev, bool accumulate, cudaStream_t s);
+                        uint64_t *partials, int blocks, uint8_t *classes, uint32_t *verts, uint64_t *counts_dev,
+                        bool accumulate, cudaStream_t s, CountRows *pending);
+// Both sub-methods of an estimate (T-5 and Path-5, or MOSS-4 and MOSS-4Min
+// when mix) in one launch, ids from 0; false when the budgets are too large
+// for it to pay.  Rows as launch_counts' pending ones.
+bool pair_fits(bool mix, uint64_t count_a, uint64_t count_b);
+cudaError_t launch_pair(bool mix, const DevGraph &g, uint64_t count_a, uint64_t count_b, uint64_t seed,
+                        uint64_t *partials, CountRows *a, CountRows *b, cudaStream_t s);
 int sample_blocks(int method, int device);   // the most blocks any variant of a sampler launches
 int sample_launch_blocks(int method, int device, const DevGraph &g);   // blocks of the variant g uses
 int sample_rows(int method, int device);     // partial-count rows launch_counts needs
@@ -408,7 +422,8 @@ void upload_luts_group(const uint8_t *lut4, const uint8_t *lut5, const uint8_t *
 // scratch of a grouped call; 0 when the call is not one to group
 uint64_t group_bytes(int method, const DevGraph &g, bool degree_order, uint64_t count);
 cudaError_t launch_counts_grouped(int method, const DevGraph &g, uint64_t first, uint64_t count, uint64_t seed,
-                                  uint64_t *partials, void *scratch, uint64_t *counts_dev, cudaStream_t s);
+                                  uint64_t *partials, void *scratch, uint64_t *counts_dev, cudaStream_t s,
+                                  CountRows *pending);
 
 // moss_finalize.cu
 struct FinalizeIn {
@@ -416,10 +431,17 @@ struct FinalizeIn {
     int mix = 0;      // k = 4 only: MOSS-4 (K[0], hits[0]) with MOSS-4Min (K[1], hits[1])
     uint64_t K[2];
 };
-cudaError_t launch_finalize(const FinalizeIn &in, const uint64_t *hits_dev, const DevTotals *tot,
-                            void *result_dev, cudaStream_t s);
-cudaError_t launch_covariance(const FinalizeIn &in, const uint64_t *hits_dev, const DevTotals *tot,
-                              void *result_dev, double *cov_dev, cudaStream_t s);
+// counts given by the caller: kSlots of each sub-method in dev, or by value
+struct HitsArg {
+    const uint64_t *dev;
+    uint64_t h[2 * kSlots];
+};
+// result (and, with cov, the 22 x 22 covariance matrix) of given counts
+cudaError_t launch_finalize(const FinalizeIn &in, const HitsArg &hits, const DevTotals *tot, void *result, double *cov,
+                            cudaStream_t s);
+// the counts of both sub-methods summed from their rows, and the finalize
+cudaError_t launch_reduce_finalize(const FinalizeIn &in, const CountRows &a, const CountRows &b, const DevTotals *tot,
+                                   void *result_dev, cudaStream_t s);
 
 // ---------------------------------------------------------------- batches --
 // One task = one sub-method of one request: sample ids [first, first+count)

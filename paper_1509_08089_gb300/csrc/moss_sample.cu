@@ -345,6 +345,52 @@ __global__ void k_reduce(const uint64_t *partials, int blocks, uint64_t *out, in
     }
 }
 
+// T-5 and Path-5 (or, MIX, MOSS-4 and MOSS-4Min) samples 0.. in one launch:
+// the first blocks_a blocks draw the first method's, the rest the second's,
+// each leaving a row of counts.  A small estimate is launches and latency, so
+// its two sub-methods share the chip and Path-5 redraws in line (two more
+// launches otherwise, each a few long dependent chains).
+template <bool MIX, bool HASH, int PM, int RNG>
+__global__ void __launch_bounds__(kThreads, 4)
+    k_sample_pair(DevGraph g, uint32_t blocks_a, uint64_t count_a, uint64_t count_b, uint64_t seed,
+                  uint64_t *partials) {
+    __shared__ uint8_t lut[MIX ? 64 : kLut];
+    __shared__ uint8_t lutc[MIX ? 4096 : 1];
+    __shared__ uint32_t hist[kWarps][kSlots];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int i = threadIdx.x; i < (MIX ? 64 : kLut); i += kThreads) lut[i] = MIX ? g_lut4[i] : g_lut5[i];
+    if (MIX)
+        for (int i = threadIdx.x; i < 4096; i += kThreads) lutc[i] = g_lutc[i];
+    for (int i = threadIdx.x; i < kWarps * kSlots; i += kThreads) (&hist[0][0])[i] = 0;
+    __syncthreads();
+    const bool second = blockIdx.x >= blocks_a;   // block-uniform
+    const uint32_t block = second ? blockIdx.x - blocks_a : blockIdx.x;
+    const uint64_t count = second ? count_b : count_a;
+    const uint64_t stride = (uint64_t)(second ? gridDim.x - blocks_a : blocks_a) * kThreads;
+    for (uint64_t base = ((uint64_t)block * kWarps + warp) * 32; base < count; base += stride) {
+        const uint64_t i = base + lane;
+        int cls = kSlots;
+        if (i < count) {
+            if (!second) {
+                cls = MIX ? sample_moss4<RNG, HASH, PM>(g, lut, seed, i).cls : sample_t5<RNG, HASH, PM>(g, lut, seed, i).cls;
+            } else if (MIX) {
+                const Sample sm = sample_min<RNG, HASH, PM>(g, lut, lutc, seed, i);
+                cls = min_slot(sm.cls, sm.v[4]);
+            } else {
+                cls = sample_path5<RNG, HASH, 3, PM>(g, lut, seed, i).cls;
+            }
+        }
+        const uint32_t peers = __match_any_sync(0xffffffffu, cls);
+        if (cls < kSlots && lane == __ffs(peers) - 1) atomicAdd(&hist[warp][cls], (uint32_t)__popc(peers));
+    }
+    __syncthreads();
+    if (threadIdx.x < kSlots) {
+        uint64_t sum = 0;
+        for (int w = 0; w < kWarps; ++w) sum += hist[w][threadIdx.x];
+        partials[(uint64_t)blockIdx.x * kSlots + threadIdx.x] = sum;
+    }
+}
+
 // the probe variant of a launch: 0 list search, 1 hashed set, 2 filter in
 // front of it, 3 hashed set with two-level vertex tables (kPmStream)
 int probe_variant(int method, const DevGraph &g) {
@@ -507,16 +553,25 @@ int sample_rows(int method, int device) {
 }
 
 cudaError_t launch_tail(int method, const DevGraph &g, uint64_t first, uint64_t count, uint64_t seed,
-                        uint64_t *partials, int blocks, uint64_t *counts_dev, bool accumulate, cudaStream_t s) {
+                        uint64_t *partials, int blocks, uint8_t *classes, uint32_t *verts, uint64_t *counts_dev,
+                        bool accumulate, cudaStream_t s, CountRows *pending) {
     int dev = 0, rows = blocks;
     cudaGetDevice(&dev);
     if (method == 2) {
-        const int d1 = defer_blocks(dev, 1), d2 = min(defer_blocks(dev, 2), d1);
+        // no more blocks than there are windows of the bitmap for their warps;
+        // the fallback stage adds into the first rows of the second-attempt stage
+        const uint64_t windows = (count + 1024ull * kWarps - 1) / (1024ull * kWarps);
+        const int d1 = (int)std::min<uint64_t>(defer_blocks(dev, 1), windows);
+        const int d2 = (int)std::min<uint64_t>(defer_blocks(dev, 2), d1);
         uint64_t *drows = partials + (uint64_t)blocks * kSlots;
         cudaError_t e;
-        if ((e = launch_deferred<1>(g, first, count, seed, drows, d1, nullptr, nullptr, s)) != cudaSuccess) return e;
-        if ((e = launch_deferred<2>(g, first, count, seed, drows, d2, nullptr, nullptr, s)) != cudaSuccess) return e;
+        if ((e = launch_deferred<1>(g, first, count, seed, drows, d1, classes, verts, s)) != cudaSuccess) return e;
+        if ((e = launch_deferred<2>(g, first, count, seed, drows, d2, classes, verts, s)) != cudaSuccess) return e;
         rows += d1;
+    }
+    if (pending) {
+        *pending = CountRows{partials, rows, accumulate ? counts_dev : nullptr};
+        return cudaSuccess;
     }
     k_reduce<<<1, 32 * kSlots, 0, s>>>(partials, rows, counts_dev, accumulate ? 1 : 0);
     return cudaGetLastError();
@@ -524,31 +579,74 @@ cudaError_t launch_tail(int method, const DevGraph &g, uint64_t first, uint64_t 
 
 cudaError_t launch_counts(int method, const DevGraph &g, uint64_t first, uint64_t count, uint64_t seed,
                           uint64_t *partials, uint8_t *classes, uint32_t *verts, uint64_t *counts_dev,
-                          cudaStream_t s) {
+                          cudaStream_t s, CountRows *pending) {
     int dev = 0;
     cudaGetDevice(&dev);
-    const int blocks = sample_launch_blocks(method, dev, g);
-    cudaError_t e;
-    if (method != 2) {
-        if ((e = launch_sample(method, g, first, count, seed, partials, blocks, classes, verts, s)) != cudaSuccess)
-            return e;
-        k_reduce<<<1, 32 * kSlots, 0, s>>>(partials, blocks, counts_dev, 0);
-        return cudaGetLastError();
-    }
-    // the fallback stage adds into the first rows of the second-attempt stage
-    const int d1 = defer_blocks(dev, 1), d2 = min(defer_blocks(dev, 2), d1);
-    for (uint64_t c0 = 0; c0 < count; c0 += kDeferChunk) {
-        const uint64_t len = count - c0 < kDeferChunk ? count - c0 : kDeferChunk;
+    const uint64_t chunk = method == 2 ? kDeferChunk : count;
+    for (uint64_t c0 = 0; c0 < count; c0 += chunk) {
+        const uint64_t len = std::min(chunk, count - c0);
+        // a block per 256 ids at most: every block leaves a row to add up
+        const int blocks = (int)std::min<uint64_t>(sample_launch_blocks(method, dev, g), (len + kThreads - 1) / kThreads);
         uint8_t *cl = classes ? classes + c0 : nullptr;
         uint32_t *vt = verts ? verts + 5 * c0 : nullptr;
-        uint64_t *drows = partials + (uint64_t)blocks * kSlots;
-        if ((e = launch_sample(2, g, first + c0, len, seed, partials, blocks, cl, vt, s)) != cudaSuccess) return e;
-        if ((e = launch_deferred<1>(g, first + c0, len, seed, drows, d1, cl, vt, s)) != cudaSuccess) return e;
-        if ((e = launch_deferred<2>(g, first + c0, len, seed, drows, d2, cl, vt, s)) != cudaSuccess) return e;
-        k_reduce<<<1, 32 * kSlots, 0, s>>>(partials, blocks + d1, counts_dev, c0 > 0 ? 1 : 0);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        cudaError_t e = launch_sample(method, g, first + c0, len, seed, partials, blocks, cl, vt, s);
+        if (e == cudaSuccess)
+            e = launch_tail(method, g, first + c0, len, seed, partials, blocks, cl, vt, counts_dev, c0 > 0, s,
+                            c0 + len == count ? pending : nullptr);
+        if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
+}
+
+// ----------------------------------------------------------- small estimates --
+namespace {
+
+constexpr int kPairBlocks = 4;   // resident blocks per SM (Path-5 with its redraws in line)
+
+template <bool MIX, int RNG>
+cudaError_t launch_pair_rng(const DevGraph &g, int blocks, int blocks_a, uint64_t count_a, uint64_t count_b,
+                            uint64_t seed, uint64_t *partials, cudaStream_t s) {
+    if (!g.hash) k_sample_pair<MIX, false, kPmPlain, RNG><<<blocks, kThreads, 0, s>>>(g, blocks_a, count_a, count_b, seed, partials);
+    else if (g.filter) k_sample_pair<MIX, true, kPmFilter, RNG><<<blocks, kThreads, 0, s>>>(g, blocks_a, count_a, count_b, seed, partials);
+    else k_sample_pair<MIX, true, kPmPlain, RNG><<<blocks, kThreads, 0, s>>>(g, blocks_a, count_a, count_b, seed, partials);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+// At four resident blocks per SM against the single launches' six, the pair
+// stops paying once the chip is full for long: k = 5 (us, two sampler launches
+// and two redraw stages -> one launch, 8k-edge graph / 2M-edge mesh / 1M-edge
+// power-law graph): budget 1e5 93 -> 42 / 94 -> 47 / 79 -> 44, 2e6 160 -> 128 /
+// 245 -> 203 / 155 -> 132, 5e6 269 -> 256 / 439 -> 431 / 267 -> 264, 1e7 455 ->
+// 466 / 766 -> 796 / 450 -> 485; the mix, which saves one launch, 1e5 52 -> 45 /
+// 54 -> 45 / 53 -> 45, 1e6 78 -> 68 / 119 -> 116 / 86 -> 79, 2e6 101 -> 92 / 167
+// -> 178 / 111 -> 109.
+bool pair_fits(bool mix, uint64_t count_a, uint64_t count_b) {
+    const uint64_t most = mix ? 1ull << 19 : 1ull << 21;
+    return count_a <= most && count_b <= most;
+}
+
+cudaError_t launch_pair(bool mix, const DevGraph &g, uint64_t count_a, uint64_t count_b, uint64_t seed,
+                        uint64_t *partials, CountRows *a, CountRows *b, cudaStream_t s) {
+    *a = *b = CountRows{};
+    if (count_a + count_b == 0) return cudaSuccess;
+    // a block per 256 ids, or the resident blocks split in proportion
+    const uint64_t most = (uint64_t)current_sms() * kPairBlocks;
+    uint64_t na = (count_a + kThreads - 1) / kThreads, nb = (count_b + kThreads - 1) / kThreads;
+    if (na + nb > most) {
+        const uint64_t share = std::max<uint64_t>(most * na / (na + nb), na ? 1 : 0);
+        nb = std::min(nb, std::max<uint64_t>(most - share, nb ? 1 : 0));
+        na = share;
+    }
+    const int blocks = (int)(na + nb);
+    *a = CountRows{partials, (int)na, nullptr};
+    *b = CountRows{partials + na * kSlots, (int)nb, nullptr};
+    if (g.rng == kRngPhilox)
+        return mix ? launch_pair_rng<true, kRngPhilox>(g, blocks, (int)na, count_a, count_b, seed, partials, s)
+                   : launch_pair_rng<false, kRngPhilox>(g, blocks, (int)na, count_a, count_b, seed, partials, s);
+    return mix ? launch_pair_rng<true, kRngSplitMix>(g, blocks, (int)na, count_a, count_b, seed, partials, s)
+               : launch_pair_rng<false, kRngSplitMix>(g, blocks, (int)na, count_a, count_b, seed, partials, s);
 }
 
 template <int T>
