@@ -556,8 +556,12 @@ __global__ void k_slot_alias_fill(uint64_t nnz, const uint4 *__restrict__ vert, 
 
 // ---------------------------------------------------- vertex (seed) tables ---
 constexpr int kSeedThreads = 256;
-constexpr int kSeedRounds = 16;                              // items per thread per block
-constexpr uint32_t kSeedChunk = kSeedThreads * kSeedRounds;  // items per block
+// items per thread per block: 16, or 4 where 16 would leave most SMs without
+// a block (n = 100,000, two levels of two tables: 100 blocks of 16 dependent
+// rounds each; with 4 the count went from 20 to 8 us, the placement from 20 to
+// 9; n = 5,003: 13 to 6 and 15 to 7).  At n = 1M 16 rounds fill the chip.
+constexpr int kSeedRoundsMost = 16, kSeedRoundsFew = 4;
+constexpr uint32_t kSeedFewMost = 1u << 19;   // n up to which chunks are small
 
 struct SeedSplit {
     uint32_t nl, nh;
@@ -660,80 +664,74 @@ __device__ __forceinline__ void block_scan_counts(uint32_t cl, uint32_t ch, u128
     __syncthreads();
 }
 
-// floor(thr 2^64 / W) for thr < W by binary long division
-__device__ __noinline__ uint64_t quantize64_long(u128 thr, u128 W) {
-    uint64_t qq = 0;
-    u128 r = thr;
+// floor(thr 2^64 / W) for thr < W, exactly, in integer arithmetic: W is the
+// same for every column of a level, so its reciprocal is formed once per
+// block and each quotient is two 64 x 64 -> 128 products and at most two
+// corrections (Moller and Granlund, "Improved division by invariant
+// integers", IEEE Trans. Computers 2011: algorithms 4 (3 by 2 words) and 6
+// (its reciprocal)).  A quotient through doubles, as before, costs several
+// FP64 divisions at 1/64 of the integer rate (k_seed_fill over 2 x 2M columns
+// 239 -> 141 us, over 2 x 200,000 33 -> 17 us).
+struct Reciprocal {
+    uint64_t d1, d0;   // W shifted so that its top bit is set
+    uint64_t v;        // floor((2^192 - 1) / (d1 2^64 + d0)) - 2^64
+    int shift;
+};
+
+__device__ __forceinline__ Reciprocal reciprocal_of(u128 W) {   // W > 0
+    Reciprocal r;
+    const uint64_t hi = (uint64_t)(W >> 64);
+    r.shift = hi ? __clzll((long long)hi) : 64 + __clzll((long long)(uint64_t)W);
+    W <<= r.shift;
+    r.d1 = (uint64_t)(W >> 64);
+    r.d0 = (uint64_t)W;
+    // floor((2^128 - 1) / d1) - 2^64 by binary long division of ~d1 : ~0
+    uint64_t rem = ~r.d1, v = 0;
     for (int i = 0; i < 64; ++i) {
-        const bool carry = (uint64_t)(r >> 127) != 0;
-        r <<= 1;
-        qq <<= 1;
-        if (carry || r >= W) { r -= W; qq |= 1; }
-    }
-    return qq;
-}
-
-__device__ __forceinline__ double u128_to_double(u128 x) {
-    return (double)(uint64_t)(x >> 64) * 18446744073709551616.0 + (double)(uint64_t)x;
-}
-
-// thr 2^64 - q W as a signed 192-bit number: (hi, lo), hi's sign its sign
-__device__ __forceinline__ void quantize_rem(u128 thr, u128 W, uint64_t q, int64_t &hi, u128 &lo) {
-    const u128 p0 = (u128)q * (uint64_t)W, p1 = (u128)q * (uint64_t)(W >> 64);
-    const u128 blo = p0 + (p1 << 64);
-    const uint64_t bhi = (uint64_t)(p1 >> 64) + (blo < p0 ? 1u : 0u);
-    const u128 alo = (u128)(uint64_t)thr << 64;
-    const uint64_t ahi = (uint64_t)(thr >> 64);
-    lo = alo - blo;
-    hi = (int64_t)(ahi - bhi - (alo < blo ? 1u : 0u));
-}
-
-// floor(thr 2^64 / W) for thr <= W, saturated: a double estimate (53 good
-// bits), one correction from the exact remainder, then at most a few unit
-// steps -- the long division when they do not settle
-__device__ __forceinline__ uint64_t quantize64(u128 thr, u128 W) {
-    if (W == 0) return 0;
-    if (thr >= W) return ~0ULL;
-    const double dw = u128_to_double(W);
-    const double est = u128_to_double(thr) / dw * 18446744073709551616.0;
-    uint64_t q = est >= 18446744073709549568.0 ? ~0ULL : (uint64_t)est;
-    int64_t hi;
-    u128 lo;
-    quantize_rem(thr, W, q, hi, lo);
-    // the remainder is a few thousand W at most: its quotient by W in
-    // doubles, from its magnitude (the two halves of a negative one would
-    // cancel in a double)
-    double rem;
-    if (hi < 0) {
-        const u128 nlo = ~lo + 1;
-        const uint64_t nhi = ~(uint64_t)hi + (nlo == 0 ? 1u : 0u);
-        rem = -((double)nhi * 340282366920938463463374607431768211456.0 + u128_to_double(nlo));
-    } else {
-        rem = (double)hi * 340282366920938463463374607431768211456.0 + u128_to_double(lo);
-    }
-    const double delta = rem / dw;
-    if (delta > -1e6 && delta < 1e6) {
-        const int64_t step = (int64_t)floor(delta);
-        if (step < 0) q = (uint64_t)(-step) > q ? 0 : q - (uint64_t)(-step);
-        else q = (uint64_t)step > ~q ? ~0ULL : q + (uint64_t)step;
-        quantize_rem(thr, W, q, hi, lo);
-        for (int it = 0; it < 4; ++it) {
-            if (hi < 0) {   // remainder below 0: one W too many
-                --q;
-                const u128 nlo = lo + W;
-                hi += nlo < lo ? 1 : 0;
-                lo = nlo;
-            } else if (hi > 0 || lo >= W) {   // at least W left
-                ++q;
-                const u128 nlo = lo - W;
-                hi -= nlo > lo ? 1 : 0;
-                lo = nlo;
-            } else {
-                return q;
-            }
+        const bool carry = rem >> 63;
+        rem = (rem << 1) | 1u;
+        v <<= 1;
+        if (carry || rem >= r.d1) {
+            rem -= r.d1;
+            v |= 1u;
         }
     }
-    return quantize64_long(thr, W);
+    // the low word's share
+    uint64_t p = r.d1 * v + r.d0;
+    if (p < r.d0) {
+        --v;
+        if (p >= r.d1) {
+            --v;
+            p -= r.d1;
+        }
+        p -= r.d1;
+    }
+    const uint64_t t1 = __umul64hi(v, r.d0), t0 = v * r.d0;
+    p += t1;
+    if (p < t1) {
+        --v;
+        if (p > r.d1 || (p == r.d1 && t0 >= r.d0)) --v;
+    }
+    r.v = v;
+    return r;
+}
+
+// floor(thr 2^64 / W) for thr <= W, saturated; r the reciprocal of W
+__device__ __forceinline__ uint64_t quantize64(u128 thr, u128 W, const Reciprocal &r) {
+    if (thr >= W) return W == 0 ? 0 : ~0ULL;
+    const u128 u = thr << r.shift, d = ((u128)r.d1 << 64) | r.d0;
+    const uint64_t u2 = (uint64_t)(u >> 64), u1 = (uint64_t)u;
+    const u128 q = (u128)r.v * u2 + u;
+    uint64_t q1 = (uint64_t)(q >> 64);
+    const uint64_t q0 = (uint64_t)q;
+    u128 rem = ((u128)(u1 - q1 * r.d1) << 64) - (u128)r.d0 * q1 - d;
+    ++q1;
+    if ((uint64_t)(rem >> 64) >= q0) {
+        --q1;
+        rem += d;
+    }
+    if (rem >= d) ++q1;
+    return q1;
 }
 
 // ---- the split into levels (per table): heavy iff w_v >= ceil(W / 2^split)
@@ -755,6 +753,7 @@ __device__ __forceinline__ u128 heavy_cut(u128 W, int split) {
 
 // per-chunk count and weight of the heavy vertices (and the overflow check
 // of the whole table: w_v n must fit 128 bits)
+template <int ROUNDS>
 __global__ void __launch_bounds__(kSeedThreads) k_level_count(uint32_t n, const DevTotals *tot, LevelTasks tasks,
                                                              int split, uint32_t *flags) {
     const LevelTask &T = tasks.t[blockIdx.y];
@@ -762,11 +761,11 @@ __global__ void __launch_bounds__(kSeedThreads) k_level_count(uint32_t n, const 
     if (blockIdx.x == 0 && threadIdx.x == 0 && n > 1 && W > (~(u128)0) / n) atomicOr(flags, kErrOverflow);
     if (W == 0) return;
     const u128 cut = heavy_cut(W, split);
-    const uint64_t base = (uint64_t)blockIdx.x * kSeedChunk;
+    const uint64_t base = (uint64_t)blockIdx.x * (kSeedThreads * ROUNDS);
     // each thread's count and weight over its rounds, then one block sum
     uint32_t nh = 0;
     u128 E = 0;
-    for (int r = 0; r < kSeedRounds; ++r) {
+    for (int r = 0; r < ROUNDS; ++r) {
         const uint64_t j = base + (uint64_t)r * kSeedThreads + threadIdx.x;
         if (j < n) {
             const u128 w = T.w[j];
@@ -839,19 +838,20 @@ __global__ void __launch_bounds__(kSeedThreads) k_level_offsets(uint32_t chunks,
         L.nh = run_h;
         L.WH = run_E;
         L.WL = W - run_E;
-        L.tl = run_h ? quantize64(W - run_E, W) : 0;
+        L.tl = run_h ? quantize64(W - run_E, W, reciprocal_of(W)) : 0;
     }
 }
 
 // column order: every heavy vertex at its rank among the heavies, every light
 // one at nh + its rank among the lights (a table of total 0: the identity)
+template <int ROUNDS>
 __global__ void __launch_bounds__(kSeedThreads) k_level_place(uint32_t n, const DevTotals *tot, LevelTasks tasks,
                                                              int split) {
     const LevelTask &T = tasks.t[blockIdx.y];
     const u128 W = tot->gamma[T.which];
-    const uint64_t base = (uint64_t)blockIdx.x * kSeedChunk;
+    const uint64_t base = (uint64_t)blockIdx.x * (kSeedThreads * ROUNDS);
     if (W == 0) {
-        for (int r = 0; r < kSeedRounds; ++r) {
+        for (int r = 0; r < ROUNDS; ++r) {
             const uint64_t j = base + (uint64_t)r * kSeedThreads + threadIdx.x;
             if (j < n) T.perm[j] = (uint32_t)j;
         }
@@ -862,7 +862,7 @@ __global__ void __launch_bounds__(kSeedThreads) k_level_place(uint32_t n, const 
     uint32_t before = T.agg[blockIdx.x].nh;   // heavies in earlier chunks
     __shared__ uint32_t s_w[2][kSeedThreads / kWarp];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int r = 0; r < kSeedRounds; ++r) {
+    for (int r = 0; r < ROUNDS; ++r) {
         const uint64_t j = base + (uint64_t)r * kSeedThreads + threadIdx.x;
         const bool heavy = j < n && T.w[j] >= cut;
         // rank among the round's heavies: a ballot per warp, the warps'
@@ -886,6 +886,7 @@ __global__ void __launch_bounds__(kSeedThreads) k_level_place(uint32_t n, const 
 
 // ---- the alias table of each level, in four phases (closed form of the sweep)
 // phase 1: per-chunk aggregates
+template <int ROUNDS>
 __global__ void __launch_bounds__(kSeedThreads) k_seed_count(uint32_t n, const DevTotals *tot, SeedTasks tasks,
                                                             uint32_t *flags) {
     const SeedTask &T = tasks.t[blockIdx.y];
@@ -894,11 +895,11 @@ __global__ void __launch_bounds__(kSeedThreads) k_seed_count(uint32_t n, const D
     if (flags && blockIdx.x == 0 && threadIdx.x == 0 && n > 1 && W > (~(u128)0) / n) atomicOr(flags, kErrOverflow);
     if (W == 0) return;
     const uint32_t m = task_items(T, tot, n), b0 = task_base(T, tot);
-    const uint64_t base = (uint64_t)blockIdx.x * kSeedChunk;
+    const uint64_t base = (uint64_t)blockIdx.x * (kSeedThreads * ROUNDS);
     // each thread's counts and deficit/excess sums, then one block sum
     uint32_t cl = 0, ch = 0;
     u128 sD = 0, sE = 0;
-    for (int r = 0; r < kSeedRounds; ++r) {
+    for (int r = 0; r < ROUNDS; ++r) {
         bool light, heavy;
         u128 D, E;
         seed_item(T, base + (uint64_t)r * kSeedThreads + threadIdx.x, m, b0, W, light, heavy, D, E);
@@ -975,17 +976,18 @@ __global__ void __launch_bounds__(kSeedThreads) k_seed_offsets(uint32_t chunks, 
 }
 
 // phase 3: place every item at its split position with its prefix
+template <int ROUNDS>
 __global__ void __launch_bounds__(kSeedThreads) k_seed_place(uint32_t n, const DevTotals *tot, SeedTasks tasks) {
     const SeedTask &T = tasks.t[blockIdx.y];
     const u128 W = task_total(T, tot);
     if (W == 0) return;
     const uint32_t m = task_items(T, tot, n), b0 = task_base(T, tot);
-    // thread t takes kSeedRounds consecutive items of the chunk: its counts
+    // thread t takes ROUNDS consecutive items of the chunk: its counts
     // and sums, one block scan of them, then the items again in order
-    const uint64_t first = (uint64_t)blockIdx.x * kSeedChunk + (uint64_t)threadIdx.x * kSeedRounds;
+    const uint64_t first = ((uint64_t)blockIdx.x * kSeedThreads + threadIdx.x) * ROUNDS;
     uint32_t cl = 0, ch = 0;
     u128 sD = 0, sE = 0;
-    for (int r = 0; r < kSeedRounds; ++r) {
+    for (int r = 0; r < ROUNDS; ++r) {
         bool light, heavy;
         u128 D, E;
         seed_item(T, first + r, m, b0, W, light, heavy, D, E);
@@ -1001,7 +1003,7 @@ __global__ void __launch_bounds__(kSeedThreads) k_seed_place(uint32_t n, const D
     const SeedAgg off = T.agg[blockIdx.x];
     uint32_t rl = off.nl + xl, rh = off.nh + xh;
     u128 A = off.D + xD, P = off.E + xE;
-    for (int r = 0; r < kSeedRounds; ++r) {
+    for (int r = 0; r < ROUNDS; ++r) {
         const uint64_t j = first + r;
         bool light, heavy;
         u128 D, E;
@@ -1031,6 +1033,10 @@ __global__ void k_seed_fill(uint32_t n, const DevTotals *tot, SeedTasks tasks) {
     const u128 *pre = T.pre;
     const uint32_t nl = T.split->nl, nh = T.split->nh;
     const u128 Ptot = T.split->total;
+    __shared__ Reciprocal s_rec;
+    if (threadIdx.x == 0 && W != 0) s_rec = reciprocal_of(W);
+    __syncthreads();
+    const Reciprocal rec = s_rec;
     for (uint64_t p = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; p < m; p += (uint64_t)gridDim.x * blockDim.x) {
         if (W == 0) {   // a level without weight is never drawn
             const uint32_t v = task_vertex(T, b0 + (uint32_t)p);
@@ -1067,7 +1073,7 @@ __global__ void k_seed_fill(uint32_t n, const DevTotals *tot, SeedTasks tasks) {
                 alias = j;
             }
         }
-        const uint64_t Tq = quantize64(thr, W);
+        const uint64_t Tq = quantize64(thr, W, rec);
         const uint32_t av = task_vertex(T, b0 + alias), sv = task_vertex(T, b0 + j);
         T.seed[2 * (uint64_t)(b0 + j)] = make_uint4((uint32_t)Tq, (uint32_t)(Tq >> 32), av, sv);
         T.seed[2 * (uint64_t)(b0 + j) + 1] = T.vrec[av];
@@ -1401,8 +1407,14 @@ cudaError_t launch_sigma_alias(uint32_t n, uint64_t nnz, const uint4 *vert, cons
     return cudaGetLastError();
 }
 
+static int seed_rounds(uint32_t n) { return n <= kSeedFewMost ? kSeedRoundsFew : kSeedRoundsMost; }
+static uint32_t seed_chunks(uint32_t n) {
+    const uint64_t chunk = (uint64_t)kSeedThreads * seed_rounds(n);
+    return (uint32_t)((n + chunk - 1) / chunk);
+}
+
 uint64_t seed_scratch_bytes(uint32_t n) {
-    const uint64_t chunks = ((uint64_t)n + kSeedChunk - 1) / kSeedChunk;
+    const uint64_t chunks = seed_chunks(n);
     // per table: the column order and the split's chunk aggregates; per level:
     // the split order, its prefixes, its totals and chunk aggregates
     const uint64_t table = (uint64_t)n * 4 + 256 + chunks * sizeof(SeedAgg) + 256;
@@ -1411,12 +1423,34 @@ uint64_t seed_scratch_bytes(uint32_t n) {
     return 3 * (table + 2 * level);
 }
 
+// the level split (two levels) and the first three phases of the tables
+template <int ROUNDS>
+static cudaError_t launch_seed_split(uint32_t n, uint32_t chunks, DevTotals *tot, const LevelTasks &lt,
+                                     const SeedTasks &tasks, int ntables, int nt, bool one_level, uint32_t *flags,
+                                     int split, cudaStream_t s) {
+    cudaError_t e;
+    if (!one_level) {
+        k_level_count<ROUNDS><<<dim3(chunks, ntables), kSeedThreads, 0, s>>>(n, tot, lt, split, flags);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        k_level_offsets<<<ntables, kSeedThreads, 0, s>>>(chunks, tot, lt);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        k_level_place<ROUNDS><<<dim3(chunks, ntables), kSeedThreads, 0, s>>>(n, tot, lt, split);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
+    k_seed_count<ROUNDS><<<dim3(chunks, nt), kSeedThreads, 0, s>>>(n, tot, tasks, one_level ? flags : nullptr);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    k_seed_offsets<<<nt, kSeedThreads, 0, s>>>(chunks, tot, tasks);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    k_seed_place<ROUNDS><<<dim3(chunks, nt), kSeedThreads, 0, s>>>(n, tot, tasks);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_seed_alias(uint32_t n, DevTotals *tot, int ntables, const int *which, u128 *const *w,
                               uint4 *const *seed, const uint4 *const *vrec, void *scratch, uint32_t *flags, int split,
                               cudaStream_t s) {
     if (ntables < 1 || ntables > 3 || split < 0 || split > 64) return cudaErrorInvalidValue;
     const bool one_level = split == 64;   // one table over all vertices, in id order
-    const uint32_t chunks = (uint32_t)(((uint64_t)n + kSeedChunk - 1) / kSeedChunk);
+    const uint32_t chunks = seed_chunks(n);
     LevelTasks lt = {};
     SeedTasks tasks = {};
     uint8_t *p = static_cast<uint8_t *>(scratch);
@@ -1447,21 +1481,10 @@ cudaError_t launch_seed_alias(uint32_t n, DevTotals *tot, int ntables, const int
         }
     }
     const int nt = per * ntables;
-    cudaError_t e = cudaSuccess;
-    if (!one_level) {
-        k_level_count<<<dim3(chunks, ntables), kSeedThreads, 0, s>>>(n, tot, lt, split, flags);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        k_level_offsets<<<ntables, kSeedThreads, 0, s>>>(chunks, tot, lt);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        k_level_place<<<dim3(chunks, ntables), kSeedThreads, 0, s>>>(n, tot, lt, split);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    }
-    k_seed_count<<<dim3(chunks, nt), kSeedThreads, 0, s>>>(n, tot, tasks, one_level ? flags : nullptr);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    k_seed_offsets<<<nt, kSeedThreads, 0, s>>>(chunks, tot, tasks);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    k_seed_place<<<dim3(chunks, nt), kSeedThreads, 0, s>>>(n, tot, tasks);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    const bool few = seed_rounds(n) == kSeedRoundsFew;
+    const cudaError_t e = few ? launch_seed_split<kSeedRoundsFew>(n, chunks, tot, lt, tasks, ntables, nt, one_level, flags, split, s)
+                              : launch_seed_split<kSeedRoundsMost>(n, chunks, tot, lt, tasks, ntables, nt, one_level, flags, split, s);
+    if (e != cudaSuccess) return e;
     const int threads = 256;
     uint64_t blocks = ((uint64_t)n + threads - 1) / threads;
     if (blocks > 4096) blocks = 4096;
