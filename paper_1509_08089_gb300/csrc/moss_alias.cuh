@@ -12,6 +12,8 @@
 // and each thread merges a run of about d / NT entries.
 #pragma once
 
+#include <type_traits>
+
 #include "moss_internal.cuh"
 
 namespace moss {
@@ -192,6 +194,132 @@ __device__ void block_alias(uint32_t d, T W, Weight weight, uint32_t *idx, T *pr
         }
     }
     __syncthreads();   // idx / pre are reused by the block's next list
+}
+
+// ------------------------------------------------------------ short lists --
+// Lists of at most kShortList entries, most lists of a power-law graph, go to
+// groups of 8, 16 or 32 lanes, an entry per lane, so one warp builds four, two
+// or one of them at a time.  A warp per list leaves most lanes idle: the
+// passes over 1M lists of mean length 16 were bound by the instructions of
+// their half-empty warps, not by the ~60 bytes an entry moves.  Measured there (us):
+// k_slots 174 -> 79, k_sigma_alias 428 -> 195 with the alias's fields filled in
+// the same pass (the fill 169 -> 107), k_rank_warp 372 -> 154, k_min_alias with
+// the short lists' slot and pick records 780 + 283 + 172 -> 525 + 177 + 108,
+// k_owner 72 -> 27.
+constexpr uint32_t kShortList = 32;
+
+// Walks every vertex v < n: a warp takes TILE consecutive records and hands
+// their lists of 1..kShortList entries to small(G, v, rec, j, valid) -- a
+// group of G.value lanes per list, lane j of it entry j when valid; all 32
+// lanes call, groups without a list with valid false -- and empty ones to
+// empty(v, rec), one lane each; and, of TILE records a stride apart (so that
+// long lists which lie together spread over the warps), the longer lists one
+// by one to large(v, rec), the whole warp each.
+template <int TILE, typename Small, typename Empty, typename Large>
+__device__ __forceinline__ void for_lists(uint32_t n, const uint4 *rec, Small small, Empty empty, Large large) {
+    const int lane = threadIdx.x & 31;
+    const uint64_t tiles = ((uint64_t)n + TILE - 1) / TILE;
+    const uint64_t warps = (uint64_t)gridDim.x * (blockDim.x >> 5);
+    for (uint64_t t = (uint64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); t < tiles; t += warps) {
+        const uint64_t v0 = t * TILE, vs = t + (uint64_t)lane * tiles;
+        const bool here = lane < TILE && v0 + lane < n;
+        const uint4 r = here ? rec[v0 + lane] : make_uint4(0u, 0u, 0u, 0u);
+        const uint4 rs = lane < TILE && vs < n ? rec[vs] : make_uint4(0u, 0u, 0u, 0u);
+        if (here && r.y == 0) empty((uint32_t)(v0 + lane), r);
+        auto pass = [&](auto G, uint32_t mask) {
+            constexpr int g = decltype(G)::value;
+            while (mask) {   // warp-uniform
+                int src = -1;
+#pragma unroll
+                for (int k = 0; k < 32 / g; ++k) {   // group k takes the mask's next list
+                    if (lane / g == k && mask) src = __ffs(mask) - 1;
+                    mask &= mask - 1;
+                }
+                const int from = src < 0 ? 0 : src;
+                uint4 q;
+                q.x = __shfl_sync(0xffffffffu, r.x, from);
+                q.y = __shfl_sync(0xffffffffu, r.y, from);
+                q.z = __shfl_sync(0xffffffffu, r.z, from);
+                q.w = __shfl_sync(0xffffffffu, r.w, from);
+                const uint32_t j = lane & (g - 1);
+                small(G, (uint32_t)(v0 + from), q, j, src >= 0 && j < q.y);
+            }
+        };
+        pass(std::integral_constant<int, 8>{}, __ballot_sync(0xffffffffu, r.y >= 1 && r.y <= 8));
+        pass(std::integral_constant<int, 16>{}, __ballot_sync(0xffffffffu, r.y > 8 && r.y <= 16));
+        pass(std::integral_constant<int, 32>{}, __ballot_sync(0xffffffffu, r.y > 16 && r.y <= kShortList));
+        for (uint32_t mask = __ballot_sync(0xffffffffu, rs.y > kShortList); mask; mask &= mask - 1) {
+            const int src = __ffs(mask) - 1;
+            uint4 q;
+            q.x = __shfl_sync(0xffffffffu, rs.x, src);
+            q.y = __shfl_sync(0xffffffffu, rs.y, src);
+            q.z = __shfl_sync(0xffffffffu, rs.z, src);
+            q.w = __shfl_sync(0xffffffffu, rs.w, src);
+            large((uint32_t)(t + (uint64_t)src * tiles), q);
+        }
+    }
+}
+
+// records per warp: enough lists to fill the groups, but a warp for every
+// scheduler first
+template <typename F>
+inline void with_tile(uint32_t n, F f) {
+    if (n >= (1u << 18)) f(std::integral_constant<int, 32>{});
+    else f(std::integral_constant<int, 8>{});
+}
+// blocks of THREADS threads that cover n records in tiles, at most per_sm an SM
+inline unsigned tile_blocks(uint32_t n, int tile, int threads, int sms, int per_sm) {
+    const uint64_t tiles = ((uint64_t)n + tile - 1) / tile, b = (tiles + threads / 32 - 1) / (threads / 32);
+    const uint64_t cap = (uint64_t)sms * per_sm;
+    return (unsigned)(b < 1 ? 1 : (b < cap ? b : cap));
+}
+
+// inclusive sum over the lanes of a group of G
+template <int G>
+__device__ __forceinline__ uint64_t group_scan(uint64_t x, uint32_t j) {
+#pragma unroll
+    for (int d = 1; d < G; d <<= 1) {
+        const uint64_t t = __shfl_up_sync(0xffffffffu, x, d, G);
+        if (j >= (uint32_t)d) x += t;
+    }
+    return x;
+}
+
+// The alias table of a list held by a group of G lanes, lane j with q_j = w_j d
+// (closed form as above): the prefixes of deficits and excesses stay in the
+// lanes and, being monotone over them, are searched there by shuffles.
+template <int G>
+__device__ __forceinline__ void group_alias(bool valid, uint64_t q, uint64_t W, uint32_t j, uint64_t &thr,
+                                            uint32_t &alias) {
+    const int lane = threadIdx.x & 31;
+    const bool light = valid && q < W, heavy = valid && !light;
+    const uint32_t group = G == 32 ? 0xffffffffu : (1u << (G & 31)) - 1u;
+    const uint32_t heavies = __ballot_sync(0xffffffffu, heavy) >> (lane & ~(G - 1)) & group;
+    const uint64_t D = light ? W - q : 0;
+    const uint64_t A = group_scan<G>(D, j) - D;                  // exclusive deficits
+    const uint64_t P = group_scan<G>(heavy ? q - W : 0, j);      // inclusive excesses
+    const uint64_t total = __shfl_sync(0xffffffffu, P, G - 1, G);
+    // light: the first lane whose P reaches A; heavy: the first whose A exceeds P
+    uint32_t at = 0;
+#pragma unroll
+    for (int step = G / 2; step > 0; step >>= 1) {
+        const uint64_t Pe = __shfl_sync(0xffffffffu, P, at + step - 1, G);
+        const uint64_t Ae = __shfl_sync(0xffffffffu, A, at + step - 1, G);
+        if (light ? Pe < A : Ae <= P) at += step;
+    }
+    const uint64_t Aat = __shfl_sync(0xffffffffu, A, at, G);
+    if (light) {
+        thr = q;
+        alias = __ffs(heavies >> at << at) - 1;
+    } else if (P < total) {
+        // the first light there or after has the same A (nothing in between
+        // adds a deficit); without one A ends at the total
+        thr = W + P - (Aat > P ? Aat : total);
+        alias = __ffs(heavies & ~((2u << j) - 1u)) - 1;
+    } else {
+        thr = W;
+        alias = j;
+    }
 }
 
 // Calls body(v) for every vertex v < n whose record passes pred, one vertex at

@@ -37,17 +37,33 @@ constexpr uint32_t kLongList = 256;   // longer lists: k_min_alias_long, a block
 
 __device__ __forceinline__ uint64_t order_key(uint32_t x, uint32_t dx) { return ((uint64_t)dx << 32) | x; }
 
-// lists of at most kWarpKeys * 32 entries: lane l holds entries l, l + 32, ...;
-// an entry's rank is the number of keys above its own, counted against every
-// key of the list broadcast by shuffles
+// lists of at most kWarpKeys * 32 entries: an entry's rank is the number of
+// keys above its own, counted against every key of the list broadcast by
+// shuffles.  Short lists by groups of lanes, an entry per lane; longer ones a
+// warp each, lane l holding entries l, l + 32, ...
+template <int TILE>
 __global__ void __launch_bounds__(kListThreads) k_rank_warp(uint32_t n, const uint4 *__restrict__ vert,
                                                            const uint32_t *__restrict__ col, uint2 *rlist,
                                                            uint32_t *rank) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, wpb = blockDim.x >> 5;
-    for (uint64_t v = (uint64_t)blockIdx.x * wpb + warp; v < n; v += (uint64_t)gridDim.x * wpb) {
-        const uint4 vr = vert[v];
+    const int lane = threadIdx.x & 31;
+    auto small = [&](auto G, uint32_t, uint4 vr, uint32_t i, bool valid) {
+        constexpr int g = decltype(G)::value;
+        uint32_t x = 0, dx = 0, r = 0;
+        if (valid) {
+            x = col[vr.x + i];
+            dx = vert[x].y;
+        }
+        const uint64_t key = order_key(x, dx);   // 0, below every real key, where there is no entry
+#pragma unroll 8
+        for (int j = 0; j < g; ++j) r += __shfl_sync(0xffffffffu, key, j, g) > key;
+        if (valid) {
+            rlist[vr.x + r] = make_uint2(x, dx);
+            rank[vr.x + i] = r;
+        }
+    };
+    auto large = [&](uint32_t, uint4 vr) {
         const uint32_t o = vr.x, d = vr.y;
-        if (d == 0 || d > kWarpKeys * (uint32_t)kWarp) continue;   // warp-uniform
+        if (d > kWarpKeys * (uint32_t)kWarp) return;   // k_rank_block, k_rank_long
         const int rounds = (int)((d + kWarp - 1) / kWarp);
         uint32_t x[kWarpKeys], dx[kWarpKeys], r[kWarpKeys];
         uint64_t key[kWarpKeys];
@@ -81,7 +97,8 @@ __global__ void __launch_bounds__(kListThreads) k_rank_warp(uint32_t n, const ui
                 rank[o + i] = r[k];
             }
         }
-    }
+    };
+    for_lists<TILE>(n, vert, small, [](uint32_t, uint4) {}, large);
 }
 
 __device__ __forceinline__ uint32_t pow2_at_least(uint32_t x) {
@@ -234,10 +251,13 @@ __global__ void __launch_bounds__(kSortThreads) k_rank_long(uint32_t n, const ui
     });
 }
 
-// per slot p (v -> u): {0, 0, 0, u} and {off_u, d_u, d_{v,u}, d_{u,v}}
+// per slot p (v -> u) of a list above kShortList entries: {0, 0, 0, u} and
+// {off_u, d_u, d_{v,u}, d_{u,v}} (k_min_alias forms the short lists' itself)
 __global__ void k_min_slots(uint64_t nnz, const uint4 *__restrict__ vert, const uint32_t *__restrict__ col,
-                            const uint4 *__restrict__ slot, const uint32_t *__restrict__ rank, uint4 *mslot) {
+                            const uint32_t *__restrict__ owner, const uint4 *__restrict__ slot,
+                            const uint32_t *__restrict__ rank, uint4 *mslot) {
     for (uint64_t p = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; p < nnz; p += (uint64_t)gridDim.x * blockDim.x) {
+        if (vert[owner[p]].y <= kShortList) continue;
         const uint32_t u = col[p];
         const uint4 ur = vert[u];
         const uint32_t twin = slot_twin(reinterpret_cast<const uint32_t *>(slot), p);
@@ -258,7 +278,7 @@ __device__ __forceinline__ void set_min_alias(uint32_t *m32, uint64_t p, uint64_
     m32[8 * p + 2] = alias;
 }
 
-// warp per list: Gamma-check_v, mvert, and the alias table of sigma-check^(v)
+// a list each: Gamma-check_v, mvert, and the alias table of sigma-check^(v)
 // over capacity W = Gamma-check_v.  Lights (q_j = w_j d < W) carry the deficit
 // W - q_j, heavies the excess q_j - W, both in list order; with A_i the
 // exclusive prefix of the light deficits and P_k the inclusive prefix of the
@@ -379,38 +399,95 @@ __device__ void warp_min_alias(const uint4 *mslot, uint32_t *m32, uint32_t o, ui
     }
 }
 
-__global__ void __launch_bounds__(kListThreads) k_min_alias(uint32_t n, const uint4 *__restrict__ vert, uint4 *mslot,
-                                                           uint4 *mvert, u128 *gmin, u128 *partials) {
+// A pick record (moss_internal.cuh) from a slot's record (a0 its threshold
+// and u, a1 its fields) and its alias position's u and fields; narrow lists
+// (Gamma-check_v < 2^32) whose fields fit 16 bits are marked usable.
+__device__ __forceinline__ void store_pick(uint4 *mpick, uint64_t p, bool narrow, uint4 a0, uint4 a1, uint32_t bu,
+                                           uint4 b1) {
+    constexpr uint32_t kNarrow = 0xffffu;   // fields below this fit a half word
+    const bool fits = narrow && a1.y < kNarrow && a1.z < kNarrow && a1.w < kNarrow && b1.y < kNarrow &&
+                      b1.z < kNarrow && b1.w < kNarrow;
+    mpick[2 * p] = make_uint4(a0.x, a0.w, a1.x, a1.z | a1.w << 16);
+    mpick[2 * p + 1] = make_uint4(bu, b1.x, b1.z | b1.w << 16, fits ? (a1.y | b1.y << 16) : kSlotHub);
+}
+
+// Short lists (kShortList) by groups of lanes, in one pass from the ranks to
+// the finished slot and pick records: d_{v,u} and d_{u,v}, Gamma-check_v, the
+// alias, and the alias's fields from its lane.  Longer ones a warp each, from
+// the slot records k_min_slots left; their pick records are k_min_pick's.
+template <int TILE>
+__global__ void __launch_bounds__(kListThreads) k_min_alias(uint32_t n, const uint4 *__restrict__ vert,
+                                                           const uint32_t *__restrict__ col,
+                                                           const uint4 *__restrict__ slot,
+                                                           const uint32_t *__restrict__ rank, uint4 *mslot,
+                                                           uint4 *mpick, uint4 *mvert, u128 *gmin, u128 *partials) {
     __shared__ u128 s_pre[kListThreads / kWarp][kLongList];
     __shared__ uint32_t s_idx[kListThreads / kWarp][kLongList];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, wpb = blockDim.x >> 5;
     uint32_t *m32 = reinterpret_cast<uint32_t *>(mslot);
-    u128 total = 0;
-    for (uint64_t v = (uint64_t)blockIdx.x * wpb + warp; v < n; v += (uint64_t)gridDim.x * wpb) {
-        const uint4 vr = vert[v];
+    u128 total = 0;   // of the lists whose record this lane left
+    auto leave = [&](uint32_t v, uint4 vr, uint64_t W) {
+        mvert[v] = make_uint4(vr.x, vr.y, (uint32_t)W, (uint32_t)(W >> 32));
+        gmin[v] = W;
+        total += W;
+    };
+    auto small = [&](auto G, uint32_t v, uint4 vr, uint32_t j, bool valid) {
+        constexpr int g = decltype(G)::value;
+        const uint64_t p = (uint64_t)vr.x + j;
+        uint32_t u = 0;
+        uint4 f = make_uint4(0u, 0u, 0u, 0u);   // {off_u, d_u, d_{v,u}, d_{u,v}}
+        if (valid) {
+            u = col[p];
+            const uint4 ur = vert[u];
+            const uint32_t twin = slot_twin(reinterpret_cast<const uint32_t *>(slot), p);
+            f = make_uint4(ur.x, ur.y, rank[p], rank[(uint64_t)ur.x + twin]);
+        }
+        const uint64_t w = (uint64_t)f.z * f.w;
+        const uint64_t W = __shfl_sync(0xffffffffu, group_scan<g>(w, j), g - 1, g);
+        uint64_t thr;
+        uint32_t alias;
+        group_alias<g>(valid, w * vr.y, W, j, thr, alias);   // w d < 2^32 2^5 2^5
+        if (W == 0) {   // never drawn: keep every column
+            thr = 0;
+            alias = j;
+        }
+        const uint32_t a = alias & (g - 1);
+        uint4 b;
+        b.x = __shfl_sync(0xffffffffu, f.x, a, g);
+        b.y = __shfl_sync(0xffffffffu, f.y, a, g);
+        b.z = __shfl_sync(0xffffffffu, f.z, a, g);
+        b.w = __shfl_sync(0xffffffffu, f.w, a, g);
+        const uint32_t bu = __shfl_sync(0xffffffffu, u, a, g);
+        if (valid) {
+            const uint4 head = make_uint4((uint32_t)thr, (uint32_t)(thr >> 32), alias, u);
+            mslot[2 * p] = head;
+            mslot[2 * p + 1] = f;
+            store_pick(mpick, p, W >> 32 == 0, head, f, bu, b);
+            if (j == 0) leave(v, vr, W);
+        }
+    };
+    auto large = [&](uint32_t v, uint4 vr) {
         const uint32_t o = vr.x, d = vr.y;
         uint64_t W = 0;
         for (uint32_t j = lane; j < d; j += kWarp) W += min_weight(mslot, (uint64_t)o + j);
 #pragma unroll
         for (int s = 16; s > 0; s >>= 1) W += __shfl_down_sync(0xffffffffu, W, s);
         W = __shfl_sync(0xffffffffu, W, 0);
-        if (lane == 0) {
-            mvert[v] = make_uint4(o, d, (uint32_t)W, (uint32_t)(W >> 32));
-            gmin[v] = W;
-            total += W;
-        }
-        if (d == 0 || (d > kLongList && W != 0)) continue;
-        if (W == 0) {   // never drawn: keep every column
+        if (lane == 0) leave(v, vr, W);
+        if (d > kLongList && W != 0) return;   // k_min_alias_long
+        if (W == 0) {
             for (uint32_t j = lane; j < d; j += kWarp) set_min_alias(m32, (uint64_t)o + j, 0, j);
-            continue;
+            return;
         }
         if (W < (1ull << 56))   // q = w d <= W kLongList < 2^64
             warp_min_alias<uint64_t>(mslot, m32, o, d, W, reinterpret_cast<uint64_t *>(s_pre[warp]), s_idx[warp]);
         else
             warp_min_alias<u128>(mslot, m32, o, d, W, s_pre[warp], s_idx[warp]);
         __syncwarp();
-    }
-    // block share of Gamma-check (lane 0 of each warp holds its warp's)
+    };
+    for_lists<TILE>(n, vert, small, [&](uint32_t v, uint4 vr) { leave(v, vr, 0); }, large);
+    total = warp_sum128(total);
+    // block share of Gamma-check
     __shared__ u128 sh[kListThreads / kWarp];
     if (lane == 0) sh[warp] = total;
     __syncthreads();
@@ -474,29 +551,32 @@ unsigned grid_for(uint64_t items, int per_block, int cap_per_sm) {
     return (unsigned)(b ? b : 1);
 }
 
+// blocks of k_min_alias (and rows of its partial totals)
+unsigned alias_grid(uint32_t n) {
+    unsigned b = 0;
+    with_tile(n, [&](auto T) { b = tile_blocks(n, decltype(T)::value, kListThreads, current_sms(), 8); });
+    return b;
+}
+
 struct MinScratch {
-    uint32_t *rank;   // nnz, then reused as the alias split order
+    uint32_t *rank;   // nnz
     uint64_t *a, *b;  // nnz each (long-list merges), then reused as u128 prefixes
-    uint32_t *ia, *ib;  // nnz each: list positions of the keys in a, b
+    uint32_t *ia, *ib;  // nnz each: list positions of the keys in a, b, then the alias split order
     u128 *partials;
     void *seed;       // vertex alias scratch
     uint64_t bytes;
 };
 
-// per slot p of a list with Gamma-check_v < 2^32: the pick record (layout in
-// moss_internal.cuh) from p's mslot record and its alias position's
+// per slot p of a list above kShortList entries: its pick record from p's
+// mslot record and its alias position's
 __global__ void k_min_pick(uint64_t nnz, const uint32_t *__restrict__ owner, const uint4 *__restrict__ mvert,
                            const uint4 *__restrict__ mslot, uint4 *mpick) {
-    constexpr uint32_t kNarrow = 0xffffu;   // fields below this fit a half word
     for (uint64_t p = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; p < nnz; p += (uint64_t)gridDim.x * blockDim.x) {
         const uint4 mv = mvert[owner[p]];
+        if (mv.y <= kShortList) continue;
         const uint4 a0 = mslot[2 * p], a1 = mslot[2 * p + 1];
         const uint64_t ap = (uint64_t)mv.x + a0.z;
-        const uint4 b0 = mslot[2 * ap], b1 = mslot[2 * ap + 1];
-        const bool fits = mv.w == 0 && a1.y < kNarrow && a1.z < kNarrow && a1.w < kNarrow && b1.y < kNarrow &&
-                          b1.z < kNarrow && b1.w < kNarrow;
-        mpick[2 * p] = make_uint4(a0.x, a0.w, a1.x, a1.z | a1.w << 16);
-        mpick[2 * p + 1] = make_uint4(b0.w, b1.x, b1.z | b1.w << 16, fits ? (a1.y | b1.y << 16) : kSlotHub);
+        store_pick(mpick, p, mv.w == 0, a0, a1, mslot[2 * ap].w, mslot[2 * ap + 1]);
     }
 }
 
@@ -510,7 +590,7 @@ MinScratch carve(void *base, uint32_t n, uint64_t nnz) {
         off += bytes ? bytes : 1;
         return r;
     };
-    const unsigned alias_blocks = grid_for((uint64_t)n, kListThreads / kWarp, 8);
+    const unsigned alias_blocks = alias_grid(n);
     m.rank = reinterpret_cast<uint32_t *>(take(nnz * 4));
     m.a = reinterpret_cast<uint64_t *>(take(nnz * 16));
     m.b = m.a ? m.a + nnz : nullptr;
@@ -559,14 +639,17 @@ cudaError_t launch_min_tables(uint32_t n, uint64_t nnz, const uint4 *vert, const
             k_rank_long<<<grid_for((uint64_t)n, kSortThreads, 1), kSortThreads, 0, h1>>>(n, vert, col, m.a, m.b, m.ia,
                                                                                         m.ib, rlist, m.rank);
             if (eh == cudaSuccess) eh = cudaGetLastError();
-            k_rank_warp<<<grid_for((uint64_t)n, kListThreads / kWarp, 8), kListThreads, 0, s>>>(n, vert, col, rlist,
-                                                                                                 m.rank);
+            with_tile(n, [&](auto T) {
+                constexpr int tile = decltype(T)::value;
+                k_rank_warp<tile><<<tile_blocks(n, tile, kListThreads, current_sms(), 8), kListThreads, 0, s>>>(
+                    n, vert, col, rlist, m.rank);
+            });
             e = cudaGetLastError();
         }
         join(2);
         if (e == cudaSuccess) e = eh;
         if (e != cudaSuccess) return e;
-        k_min_slots<<<grid_for(nnz, 256, 16), 256, 0, s>>>(nnz, vert, col, slot, m.rank, mslot);
+        k_min_slots<<<grid_for(nnz, 256, 16), 256, 0, s>>>(nnz, vert, col, owner, slot, m.rank, mslot);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     static std::atomic<bool> attr_set[64];
@@ -577,14 +660,18 @@ cudaError_t launch_min_tables(uint32_t n, uint64_t nnz, const uint4 *vert, const
         if (e != cudaSuccess) return e;
         if (dev >= 0 && dev < 64) attr_set[dev].store(true, std::memory_order_relaxed);
     }
-    const unsigned ab = grid_for((uint64_t)n, kListThreads / kWarp, 8);
+    const unsigned ab = alias_grid(n);
     fork(1);
     if (e != cudaSuccess) return e;
-    // the rank array is dead now: the long-list kernel reuses it (split order) with a[] (prefixes)
+    // the merges' scratch is dead now: the long-list kernel keeps its split
+    // order in ia[] and its prefixes in a[], b[] (k_min_alias still reads the ranks)
     const unsigned chunks = (unsigned)(((uint64_t)n + kWarp - 1) / kWarp);
-    k_min_alias_long<<<chunks, kListThreads, kMinSmemBytes, h0>>>(n, vert, mslot, m.rank, reinterpret_cast<u128 *>(m.a));
+    k_min_alias_long<<<chunks, kListThreads, kMinSmemBytes, h0>>>(n, vert, mslot, m.ia, reinterpret_cast<u128 *>(m.a));
     eh = cudaGetLastError();
-    k_min_alias<<<ab, kListThreads, 0, s>>>(n, vert, mslot, mvert, gmin, m.partials);
+    with_tile(n, [&](auto T) {
+        k_min_alias<decltype(T)::value><<<ab, kListThreads, 0, s>>>(n, vert, col, slot, m.rank, mslot, mpick, mvert,
+                                                                    gmin, m.partials);
+    });
     e = cudaGetLastError();
     if (aux && e == cudaSuccess) {   // the pick records need both alias passes and mvert
         e = cudaEventRecord(aux->sub_mid, s);

@@ -36,7 +36,6 @@ namespace {
 constexpr int kWarp = 32;
 constexpr int kTableThreads = 256;
 constexpr uint32_t kLongList = 256;   // longer lists get a block each in the alias passes
-constexpr int kUnroll = 1;            // chunks of 32 slots per round in k_slots
 constexpr int kLongThreads = 256;
 
 // ------------------------------------------------------------ vertices ---
@@ -54,19 +53,22 @@ __global__ void k_vertices(const IdxT *row_ptr, uint32_t n, uint64_t nnz, uint4 
 }
 
 // --------------------------------------------------------------- slots ---
-// Three passes.  k_owner: the vertex of each slot (warp per vertex, stores
-// only).  k_slot_weights: one thread per slot validates the neighbour id and
+// Three passes.  k_owner: the vertex of each slot (stores only).  k_slot_weights: one thread per slot validates the neighbour id and
 // order and gathers w = d_x - 1 into acc -- every gather of the graph in
-// flight at once.  k_slots: one warp per vertex scans its w (coalesced
-// loads) into the ACC prefix and the prefix of squares, then S_v, Q_v, the
-// three vertex weights and the block's share of the exact totals.
-__global__ void k_owner(uint32_t n, const uint4 *__restrict__ vert, uint32_t *owner) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int wpb = blockDim.x >> 5;
-    for (uint64_t v = (uint64_t)blockIdx.x * wpb + warp; v < n; v += (uint64_t)gridDim.x * wpb) {
-        const uint4 vr = vert[v];
-        for (uint32_t i = lane; i < vr.y; i += kWarp) owner[vr.x + i] = (uint32_t)v;
-    }
+// flight at once.  k_slots: the lanes of a list scan its w (coalesced loads)
+// into the ACC prefix and the prefix of squares, and leave S_v and Q_v.
+template <int TILE>
+__global__ void __launch_bounds__(kTableThreads) k_owner(uint32_t n, const uint4 *__restrict__ vert, uint32_t *owner) {
+    const int lane = threadIdx.x & 31;
+    for_lists<TILE>(
+        n, vert,
+        [&](auto, uint32_t v, uint4 r, uint32_t j, bool valid) {
+            if (valid) owner[r.x + j] = v;
+        },
+        [](uint32_t, uint4) {},
+        [&](uint32_t v, uint4 r) {
+            for (uint32_t i = lane; i < r.y; i += kWarp) owner[r.x + i] = v;
+        });
 }
 
 __global__ void k_slot_weights(uint32_t n, uint64_t nnz, const uint32_t *__restrict__ col,
@@ -142,48 +144,47 @@ __device__ __forceinline__ uint32_t warp_incl_scan32(uint32_t v, int lane) {
     return v;
 }
 
+template <int TILE>
 __global__ void __launch_bounds__(kTableThreads, 8) k_slots(uint32_t n, uint4 *vert, uint32_t *acc, uint64_t *sq,
                                                            u128 *gam2) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int wpb = blockDim.x >> 5;
-    const uint64_t stride = (uint64_t)gridDim.x * wpb;
-    uint64_t v = (uint64_t)blockIdx.x * wpb + warp;
-    uint4 next = v < n ? vert[v] : make_uint4(0u, 0u, 0u, 0u);
-    for (; v < n; v += stride) {
-        // the next vertex's record is loaded while this list is scanned
-        const uint4 vr = next;
-        if (v + stride < n) next = vert[v + stride];
-        const uint32_t o = vr.x, d = vr.y;
-        if (d > kLongList) continue;   // k_slots_long
-        uint64_t run = 0, qsum = 0;
-        // kUnroll chunks of 32 per round, their loads issued together
-        for (uint32_t base = 0; base < d; base += kWarp * kUnroll) {
-            uint32_t w[kUnroll];
-#pragma unroll
-            for (int u = 0; u < kUnroll; ++u) {
-                const uint32_t i = base + u * kWarp + lane;
-                w[u] = i < d ? acc[o + i] : 0u;
+    const int lane = threadIdx.x & 31;
+    // S_v, and Q_v until k_vertex_weights turns it into Gamma^(2)_v
+    auto leave = [&](uint32_t v, uint64_t S, uint64_t Q) {
+        vert[v].z = (uint32_t)S;
+        gam2[v] = Q;
+    };
+    for_lists<TILE>(
+        n, vert,
+        [&](auto G, uint32_t v, uint4 r, uint32_t j, bool valid) {
+            constexpr int g = decltype(G)::value;
+            const uint64_t w = valid ? acc[r.x + j] : 0u;
+            const uint64_t S = group_scan<g>(w, j), Q = group_scan<g>(w * w, j);
+            if (valid) {
+                acc[r.x + j] = (uint32_t)(S - w);
+                sq[r.x + j] = Q - w * w;
+                if (j + 1 == r.y) leave(v, S, Q);
             }
-#pragma unroll
-            for (int u = 0; u < kUnroll; ++u) {
-                if (base + u * kWarp >= d) break;   // warp-uniform
-                const uint32_t i = base + u * kWarp + lane;
-                const uint64_t w2 = (uint64_t)w[u] * w[u];
-                const uint64_t incl = warp_incl_scan32(w[u], lane);   // S_v < 2^32
+        },
+        [&](uint32_t v, uint4) { leave(v, 0, 0); },
+        [&](uint32_t v, uint4 r) {
+            const uint32_t o = r.x, d = r.y;
+            if (d > kLongList) return;   // k_slots_long
+            uint64_t run = 0, qsum = 0;
+            for (uint32_t base = 0; base < d; base += kWarp) {
+                const uint32_t i = base + lane;
+                const uint32_t w = i < d ? acc[o + i] : 0u;
+                const uint64_t w2 = (uint64_t)w * w;
+                const uint64_t incl = warp_incl_scan32(w, lane);   // S_v < 2^32
                 const uint64_t incl2 = warp_incl_scan64(w2, lane);
                 if (i < d) {
-                    acc[o + i] = (uint32_t)(run + incl - w[u]);
+                    acc[o + i] = (uint32_t)(run + incl - w);
                     sq[o + i] = qsum + incl2 - w2;
                 }
                 run += __shfl_sync(0xffffffffu, incl, 31);
                 qsum += __shfl_sync(0xffffffffu, incl2, 31);
             }
-        }
-        if (lane == 0) {   // S_v, and Q_v until k_vertex_weights turns it into Gamma^(2)_v
-            vert[v].z = (uint32_t)run;
-            gam2[v] = qsum;
-        }
-    }
+            if (lane == 0) leave(v, run, qsum);
+        });
 }
 
 // lists longer than kLongList: a block per list scans NT x 4 entries a round
@@ -399,31 +400,51 @@ __device__ __forceinline__ uint32_t acc_weight(const uint32_t *acc, uint32_t o, 
     return (p + 1 < d ? __ldg(acc + o + p + 1) : S) - __ldg(acc + o + p);
 }
 
-// A warp per list of at most kLongList entries; the split (idx, pre) of the
-// list being built lives in the warp's share of shared memory, so the
-// searches and merges of pass 2 wait on shared rather than global loads.
+// Lists of at most kLongList entries.  Short ones (kShortList) by groups of
+// lanes, which also complete the record with the alias's fields; longer ones a
+// warp each, the split (idx, pre) of the list being built in the warp's share
+// of shared memory, so the searches and merges of pass 2 wait on shared rather
+// than global loads.
+template <int TILE>
 __global__ void __launch_bounds__(kTableThreads) k_sigma_alias(uint32_t n, const uint4 *__restrict__ vert,
                                                               const uint32_t *__restrict__ acc, uint4 *slot) {
     __shared__ uint64_t s_pre[kTableThreads / kWarp][kLongList];
     __shared__ uint32_t s_idx[kTableThreads / kWarp][kLongList];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int wpb = blockDim.x >> 5;
     uint64_t *pre = s_pre[warp];
     uint32_t *idx = s_idx[warp];
+    uint32_t *slot32 = reinterpret_cast<uint32_t *>(slot);
     const uint32_t below = (1u << lane) - 1u;
-    const uint64_t stride = (uint64_t)gridDim.x * wpb;
-    uint64_t v = (uint64_t)blockIdx.x * wpb + warp;
-    uint4 next = v < n ? vert[v] : make_uint4(0u, 0u, 0u, 0u);
-    for (; v < n; v += stride) {
-        // the next list's record is loaded while this one is built
-        const uint4 vr = next;
-        if (v + stride < n) next = vert[v + stride];
+    auto small = [&](auto G, uint32_t, uint4 r, uint32_t j, bool valid) {
+        constexpr int g = decltype(G)::value;
+        const uint32_t o = r.x, d = r.y, S = r.z;
+        const uint64_t p = (uint64_t)o + j;
+        const uint32_t a = valid ? __ldg(acc + p) : S;
+        const uint32_t after = __shfl_down_sync(0xffffffffu, a, 1, g);
+        const uint32_t w = (j + 1 < d ? after : S) - a;
+        uint64_t thr;
+        uint32_t alias;
+        group_alias<g>(valid, (uint64_t)w * d, S, j, thr, alias);
+        if (S == 0) {   // never drawn (Gamma_v = 0): keep every column
+            thr = 0;
+            alias = j;
+        }
+        const uint2 cn = valid ? *reinterpret_cast<const uint2 *>(slot32 + 8 * p) : make_uint2(0u, 0u);
+        const uint32_t off = valid ? slot32[8 * p + 4] : 0u;
+        const uint32_t col = __shfl_sync(0xffffffffu, cn.x, alias & (g - 1), g);
+        const uint32_t nb = __shfl_sync(0xffffffffu, cn.y, alias & (g - 1), g);
+        const uint32_t aoff = __shfl_sync(0xffffffffu, off, alias & (g - 1), g);
+        if (valid) {
+            slot[2 * p] = make_uint4(cn.x, cn.y, (uint32_t)thr, alias);
+            slot[2 * p + 1] = make_uint4(off, col, nb, aoff);
+        }
+    };
+    auto large = [&](uint32_t, uint4 vr) {
         const uint32_t o = vr.x, d = vr.y, S = vr.z;
-        if (d == 0 || (d > kLongList && S != 0)) continue;   // long lists: k_sigma_alias_long
-        uint32_t *slot32 = reinterpret_cast<uint32_t *>(slot);
-        if (S == 0) {  // never drawn (Gamma_v = 0): keep every column
+        if (d > kLongList && S != 0) return;   // k_sigma_alias_long
+        if (S == 0) {
             for (uint32_t p = lane; p < d; p += kWarp) set_sigma(slot32, o, p, 0, p);
-            continue;
+            return;
         }
         const uint64_t W = S;
         // pass 1: split into lights (front) and heavies (back) with prefixes
@@ -509,7 +530,8 @@ __global__ void __launch_bounds__(kTableThreads) k_sigma_alias(uint32_t n, const
             }
         }
         __syncwarp();
-    }
+    };
+    for_lists<TILE>(n, vert, small, [](uint32_t, uint4) {}, large);
 }
 
 // lists longer than kLongList: a block per list (moss_alias.cuh); a list of
@@ -541,13 +563,16 @@ __global__ void __launch_bounds__(kLongThreads) k_sigma_alias_long(uint32_t n, c
         });
 }
 
-// One thread per slot: words 5..7 of each record from words 0, 1 and 4 of
-// its alias position's record (written before this launch, read only here).
+// One thread per slot of the lists above kShortList entries: words 5..7 of
+// each record from words 0, 1 and 4 of its alias position's record (written
+// before this launch, read only here).
 __global__ void k_slot_alias_fill(uint64_t nnz, const uint4 *__restrict__ vert, const uint32_t *__restrict__ owner,
                                   uint4 *slot) {
     uint32_t *s32 = reinterpret_cast<uint32_t *>(slot);
     for (uint64_t p = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; p < nnz; p += (uint64_t)gridDim.x * blockDim.x) {
-        const uint64_t a = (uint64_t)vert[owner[p]].x + s32[8 * p + 3];
+        const uint4 vr = vert[owner[p]];
+        if (vr.y <= kShortList) continue;   // k_sigma_alias wrote the whole record
+        const uint64_t a = (uint64_t)vr.x + s32[8 * p + 3];
         const uint32_t col = s32[8 * a], nb = s32[8 * a + 1], off = s32[8 * a + 4];
         s32[8 * p + 5] = col;
         *reinterpret_cast<uint2 *>(s32 + 8 * p + 6) = make_uint2(nb, off);
@@ -1273,7 +1298,9 @@ static unsigned flat_blocks(uint64_t items) {
 cudaError_t launch_slots(uint32_t n, uint64_t nnz, const uint32_t *col, uint4 *vert, uint4 *slot, uint32_t *acc,
                          uint32_t *owner, uint64_t *sq, u128 *gam0, u128 *gam1, u128 *gam2, u128 *partials,
                          int blocks, uint32_t *flags, cudaStream_t s, const AuxStreams *aux) {
-    k_owner<<<blocks, kTableThreads, 0, s>>>(n, vert, owner);
+    with_tile(n, [&](auto T) {
+        k_owner<decltype(T)::value><<<tile_blocks(n, decltype(T)::value, kTableThreads, current_sms(), 8), kTableThreads, 0, s>>>(n, vert, owner);
+    });
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     if (nnz) {
@@ -1290,7 +1317,9 @@ cudaError_t launch_slots(uint32_t n, uint64_t nnz, const uint32_t *col, uint4 *v
     cudaError_t et = cudaGetLastError();
     k_slots_long<<<long_blocks(n), kLongThreads, 0, ls>>>(n, vert, acc, sq, gam2);
     cudaError_t el = cudaGetLastError();
-    k_slots<<<blocks, kTableThreads, 0, s>>>(n, vert, acc, sq, gam2);
+    with_tile(n, [&](auto T) {
+        k_slots<decltype(T)::value><<<tile_blocks(n, decltype(T)::value, kTableThreads, current_sms(), 8), kTableThreads, 0, s>>>(n, vert, acc, sq, gam2);
+    });
     e = cudaGetLastError();
     if (forked) {
         const cudaError_t ej = aux->join(s);
@@ -1395,7 +1424,9 @@ cudaError_t launch_sigma_alias(uint32_t n, uint64_t nnz, const uint4 *vert, cons
     k_sigma_alias_long<<<chunks ? chunks : 1, kLongThreads, kLongSmemBytes, ls>>>(n, vert, acc, slot, scratch_idx,
                                                                                    scratch_pre);
     cudaError_t el = cudaGetLastError();
-    k_sigma_alias<<<table_blocks(n), kTableThreads, 0, s>>>(n, vert, acc, slot);
+    with_tile(n, [&](auto T) {
+        k_sigma_alias<decltype(T)::value><<<tile_blocks(n, decltype(T)::value, kTableThreads, current_sms(), 8), kTableThreads, 0, s>>>(n, vert, acc, slot);
+    });
     e = cudaGetLastError();
     if (aux) {
         const cudaError_t ew = aux->wait_for(s, long_stream);
