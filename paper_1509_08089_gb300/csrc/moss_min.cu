@@ -5,14 +5,14 @@
 // N_{u,v} = {x in N_u : x above v}, d_{u,v} = |N_{u,v}|.  Every list N_v is
 // stored sorted by that key, highest first (rlist), so N_{v,u} is its first
 // d_{v,u} entries and d_{v,u} is the position of u in it:
-//   * lists of at most 128 entries: a warp per list, each entry's rank is the
-//     count of keys above its own;
-//   * lists of at most kTile entries: a block per list, bitonic sort in
-//     shared memory, each key's list position moving with it;
+//   * lists of at most 128 entries: a group of lanes or a warp per list, each
+//     entry's rank is the count of keys above its own;
+//   * lists of at most kTile entries: a block per list, merge sort in shared
+//     memory, each key's list position moving with it;
 //   * longer lists: a block per list sorts tiles of kTile keys in shared
-//     memory, then merges runs pairwise in global memory, each key (with its
-//     position) placed by one binary search in the partner run (keys are
-//     distinct).
+//     memory, then merges runs pairwise in global memory.
+// A merge places each key by one binary search in the partner run (keys are
+// distinct).
 // Then per slot (v -> u): u, d_u, off_u, d_{v,u} and d_{u,v} (the rank of the
 // twin slot); per list: Gamma-check_v = sum_u d_{v,u} d_{u,v} and the alias
 // table of sigma-check^(v) (eq. 3) -- the parallel closed form of the sweep
@@ -29,7 +29,7 @@ namespace moss {
 namespace {
 
 constexpr int kWarp = 32;
-constexpr uint32_t kTile = 4096;      // keys sorted per shared-memory pass (32 KB)
+constexpr uint32_t kTile = 4096;      // keys sorted per shared-memory pass
 constexpr int kSortThreads = 512;
 constexpr int kListThreads = 256;
 constexpr uint32_t kWarpKeys = 4;     // k_rank_warp: lists up to 128 entries
@@ -101,113 +101,115 @@ __global__ void __launch_bounds__(kListThreads) k_rank_warp(uint32_t n, const ui
     for_lists<TILE>(n, vert, small, [](uint32_t, uint4) {}, large);
 }
 
-__device__ __forceinline__ uint32_t pow2_at_least(uint32_t x) {
-    uint32_t p = 1;
-    while (p < x) p <<= 1;
-    return p;
-}
-
-// keys of col[o + base, o + base + len) into k[0, P), zero padded (zero sorts
-// last), with each key's position in the list in id[]
-__device__ void load_keys(const uint4 *vert, const uint32_t *col, uint32_t o, uint32_t base, uint32_t len,
-                          uint32_t P, uint64_t *k, uint16_t *id) {
-    for (uint32_t i = threadIdx.x; i < P; i += blockDim.x) {
-        uint64_t key = 0;
+// Keys of col[o + base, o + base + len) sorted highest first, each with its
+// position in the list from base: runs of 32 ranked by counting within a warp,
+// then merged pairwise between the two halves of shared memory, every key
+// placed by one binary search -- 35 dependent steps for 1,000 keys, where
+// counting against the whole list took 1,000 and a bitonic sort 55 stages with
+// a barrier each (lists of 129..1,024 entries of the 7.9M-edge graph 370 -> 108
+// us, of the 1M-edge graph 116 -> 33).  k and id hold 2 MOST entries; returns the offset of the
+// sorted half.  The block calls it together.
+template <int THREADS, uint32_t MOST>
+__device__ uint32_t sort_keys(const uint4 *vert, const uint32_t *col, uint32_t o, uint32_t base, uint32_t len,
+                              uint64_t *k, uint16_t *id) {
+    const int lane = threadIdx.x & 31;
+    for (uint32_t i0 = threadIdx.x & ~31u; i0 < len; i0 += THREADS) {   // warp-uniform
+        const uint32_t i = i0 + lane;
+        uint64_t key = 0;   // below every real key (d_x >= 1)
         if (i < len) {
             const uint32_t x = col[o + base + i];
             key = order_key(x, vert[x].y);
         }
-        k[i] = key;
-        id[i] = (uint16_t)i;
+        uint32_t r = 0;
+#pragma unroll 8
+        for (int j = 0; j < kWarp; ++j) r += __shfl_sync(0xffffffffu, key, j) > key;
+        if (i < len) {
+            k[i0 + r] = key;
+            id[i0 + r] = (uint16_t)i;
+        }
     }
     __syncthreads();
-}
-
-// block-wide bitonic sort of k[0, P), P a power of two, highest first; id[]
-// moves with its key
-__device__ void bitonic_desc(uint64_t *k, uint16_t *id, uint32_t P) {
-    for (uint32_t size = 2; size <= P; size <<= 1)
-        for (uint32_t stride = size >> 1; stride > 0; stride >>= 1) {
-            for (uint32_t t = threadIdx.x; t < P / 2; t += blockDim.x) {
-                const uint32_t i = 2 * t - (t & (stride - 1)), j = i + stride;
-                const uint64_t a = k[i], b = k[j];
-                const bool down = (i & size) == 0;   // this run ends highest first
-                if ((a < b) == down) {
-                    k[i] = b;
-                    k[j] = a;
-                    const uint16_t t0 = id[i];
-                    id[i] = id[j];
-                    id[j] = t0;
+    uint32_t src = 0, dst = MOST;
+    for (uint32_t lg = 5; (1u << lg) < len; ++lg) {
+        const uint32_t L = 1u << lg;
+        for (uint32_t i = threadIdx.x; i < len; i += THREADS) {
+            const uint64_t key = k[src + i];
+            const uint32_t run = i >> lg, ps = (run ^ 1u) << lg;
+            uint32_t lo = ps, n = ps < len ? min(L, len - ps) : 0;   // partner keys above key
+            while (n > 0) {
+                const uint32_t half = n >> 1;
+                if (k[src + lo + half] > key) {
+                    lo += half + 1;
+                    n -= half + 1;
+                } else {
+                    n = half;
                 }
             }
-            __syncthreads();
+            const uint32_t at = dst + ((run & ~1u) << lg) + (i & (L - 1u)) + (lo - ps);
+            k[at] = key;
+            id[at] = id[src + i];
         }
+        __syncthreads();
+        const uint32_t t = src;
+        src = dst;
+        dst = t;
+    }
+    return src;
 }
 
-// a block per 32 vertex records (the scheduler spreads the lists).  A list
-// of at most kCountList entries ranks each key by counting the keys above it
-// (every thread reads the same key at a time: shared-memory broadcasts, no
-// barrier per step); a longer one sorts keys and positions together
-// (bitonic, a barrier per stage).
-constexpr uint32_t kCountList = 1024;
+// lists of kWarpKeys * 32 + 1 .. kBlockList entries, a block each
+constexpr uint32_t kBlockList = 1024;
+constexpr int kBlockThreads = 256;
 
-__global__ void __launch_bounds__(kSortThreads) k_rank_block(uint32_t n, const uint4 *__restrict__ vert,
-                                                            const uint32_t *__restrict__ col, uint2 *rlist,
-                                                            uint32_t *rank) {
-    __shared__ uint64_t k[kTile];
-    __shared__ uint16_t id[kTile];
-    for_each_vertex<kSortThreads, kWarp>(
-        n, vert, [](uint4 vr) { return vr.y > kWarpKeys * (uint32_t)kWarp && vr.y <= kTile; },
+__global__ void __launch_bounds__(kBlockThreads) k_rank_block(uint32_t n, const uint4 *__restrict__ vert,
+                                                             const uint32_t *__restrict__ col, uint2 *rlist,
+                                                             uint32_t *rank) {
+    __shared__ uint64_t k[2 * kBlockList];
+    __shared__ uint16_t id[2 * kBlockList];
+    for_each_vertex<kBlockThreads, kWarp>(
+        n, vert, [](uint4 vr) { return vr.y > kWarpKeys * (uint32_t)kWarp && vr.y <= kBlockList; },
         [&](uint32_t v) {
             const uint4 vr = vert[v];
             const uint32_t o = vr.x, d = vr.y;
-            if (d <= kCountList) {
-                for (uint32_t i = threadIdx.x; i < d; i += blockDim.x) {
-                    const uint32_t x = col[o + i];
-                    k[i] = order_key(x, vert[x].y);
-                }
-                __syncthreads();
-                for (uint32_t i = threadIdx.x; i < d; i += blockDim.x) {
-                    const uint64_t key = k[i];
-                    uint32_t r = 0;
-                    for (uint32_t j = 0; j < d; ++j) r += k[j] > key;
-                    rlist[o + r] = make_uint2((uint32_t)key, (uint32_t)(key >> 32));
-                    rank[o + i] = r;
-                }
-                __syncthreads();   // k is refilled for the next list
-                return;
-            }
-            const uint32_t P = pow2_at_least(d);
-            load_keys(vert, col, o, 0, d, P, k, id);
-            bitonic_desc(k, id, P);
-            for (uint32_t q = threadIdx.x; q < d; q += blockDim.x) {
-                const uint64_t key = k[q];
+            const uint32_t at = sort_keys<kBlockThreads, kBlockList>(vert, col, o, 0, d, k, id);
+            for (uint32_t q = threadIdx.x; q < d; q += kBlockThreads) {
+                const uint64_t key = k[at + q];
                 rlist[o + q] = make_uint2((uint32_t)key, (uint32_t)(key >> 32));
-                rank[o + id[q]] = q;
+                rank[o + id[at + q]] = q;
             }
             __syncthreads();   // k and id are refilled for the next list
         });
 }
 
-// lists longer than kTile: tiles sorted in shared memory into a[], then runs
-// of length L merged pairwise between a[] and b[] until one run is left
+// lists longer than kBlockList: up to kTile entries sorted in shared memory;
+// longer ones by tiles into a[], then runs of length L merged pairwise between
+// a[] and b[] until one run is left
+constexpr size_t kSortBytes = (size_t)2 * kTile * (sizeof(uint64_t) + sizeof(uint16_t));
 __global__ void __launch_bounds__(kSortThreads) k_rank_long(uint32_t n, const uint4 *__restrict__ vert,
                                                            const uint32_t *__restrict__ col, uint64_t *a,
                                                            uint64_t *b, uint32_t *ia, uint32_t *ib, uint2 *rlist,
                                                            uint32_t *rank) {
-    __shared__ uint64_t k[kTile];
-    __shared__ uint16_t id[kTile];
-    for_each_vertex<kSortThreads>(n, vert, [](uint4 vr) { return vr.y > kTile; }, [&](uint32_t v) {
+    extern __shared__ uint64_t k[];   // 2 kTile keys, then their positions
+    uint16_t *id = reinterpret_cast<uint16_t *>(k + 2 * kTile);
+    for_each_vertex<kSortThreads>(n, vert, [](uint4 vr) { return vr.y > kBlockList; }, [&](uint32_t v) {
         const uint4 vr = vert[v];
         const uint32_t o = vr.x, d = vr.y;
+        if (d <= kTile) {
+            const uint32_t at = sort_keys<kSortThreads, kTile>(vert, col, o, 0, d, k, id);
+            for (uint32_t q = threadIdx.x; q < d; q += kSortThreads) {
+                const uint64_t key = k[at + q];
+                rlist[o + q] = make_uint2((uint32_t)key, (uint32_t)(key >> 32));
+                rank[o + id[at + q]] = q;
+            }
+            __syncthreads();   // k and id are refilled for the next list
+            return;
+        }
         for (uint32_t base = 0; base < d; base += kTile) {
             const uint32_t len = min(kTile, d - base);
-            const uint32_t P = pow2_at_least(len);
-            load_keys(vert, col, o, base, len, P, k, id);
-            bitonic_desc(k, id, P);
+            const uint32_t at = sort_keys<kSortThreads, kTile>(vert, col, o, base, len, k, id);
             for (uint32_t i = threadIdx.x; i < len; i += blockDim.x) {
-                a[(uint64_t)o + base + i] = k[i];
-                ia[(uint64_t)o + base + i] = base + id[i];
+                a[(uint64_t)o + base + i] = k[at + i];
+                ia[(uint64_t)o + base + i] = base + id[at + i];
             }
             __syncthreads();
         }
@@ -285,27 +287,12 @@ __device__ __forceinline__ void set_min_alias(uint32_t *m32, uint64_t p, uint64_
 // heavy excesses: light i keeps q_i and aliases heavy min{k : P_k >= A_i};
 // heavy k keeps W + P_k - A_{i'} (i' = min{i : A_i > P_k}) and aliases heavy
 // k+1, or keeps W when P_k is the total.  The split (idx, pre) of the list
-// being built lives in the warp's share of shared memory; the prefixes are
-// 64-bit when d W fits (every list short enough for this kernel with W below
-// 2^56), else 128-bit.
-template <typename T>
-__device__ __forceinline__ T warp_scan_any(T v, int lane);
-template <>
-__device__ __forceinline__ uint64_t warp_scan_any<uint64_t>(uint64_t v, int lane) {
-    return warp_incl_scan64(v, lane);
-}
-template <>
-__device__ __forceinline__ u128 warp_scan_any<u128>(u128 v, int lane) {
-    return warp_incl_scan128(v, lane);
-}
-__device__ __forceinline__ uint64_t shfl_idx_any(uint64_t v, int src) { return __shfl_sync(0xffffffffu, v, src); }
-__device__ __forceinline__ u128 shfl_idx_any(u128 v, int src) { return shfl_idx_u128(v, src); }
-
+// being built lives in the warp's share of shared memory.
 // alias table of sigma-check^(v) for the list at o of d <= kLongList entries
-// with total W > 0, one warp; pre holds kLongList T, idx kLongList positions
-template <typename T>
-__device__ void warp_min_alias(const uint4 *mslot, uint32_t *m32, uint32_t o, uint32_t d, uint64_t W, T *pre,
+// with total W > 0, one warp; pre and idx hold kLongList entries
+__device__ void warp_min_alias(const uint4 *mslot, uint32_t *m32, uint32_t o, uint32_t d, uint64_t W, uint64_t *pre,
                                uint32_t *idx) {
+    typedef uint64_t T;
     const int lane = threadIdx.x & 31;
     const uint32_t below = (1u << lane) - 1u;
     // pass 1: lights to the front, heavies to the back, with their prefixes
@@ -320,8 +307,8 @@ __device__ void warp_min_alias(const uint4 *mslot, uint32_t *m32, uint32_t o, ui
         const uint32_t hmask = __ballot_sync(0xffffffffu, valid && !light);
         const T D = light ? (T)W - q : (T)0;
         const T E = valid && !light ? q - (T)W : (T)0;
-        const T Dincl = warp_scan_any<T>(D, lane);
-        const T Eincl = warp_scan_any<T>(E, lane);
+        const T Dincl = warp_incl_scan64(D, lane);
+        const T Eincl = warp_incl_scan64(E, lane);
         if (light) {
             const uint32_t r = nl + __popc(lmask & below);
             idx[r] = j;
@@ -333,8 +320,8 @@ __device__ void warp_min_alias(const uint4 *mslot, uint32_t *m32, uint32_t o, ui
         }
         nl += __popc(lmask);
         nh += __popc(hmask);
-        Arun += shfl_idx_any(Dincl, 31);
-        Prun += shfl_idx_any(Eincl, 31);
+        Arun += __shfl_sync(0xffffffffu, Dincl, 31);
+        Prun += __shfl_sync(0xffffffffu, Eincl, 31);
     }
     __syncwarp();
     const T Ptot = Prun;   // == Arun
@@ -421,7 +408,7 @@ __global__ void __launch_bounds__(kListThreads) k_min_alias(uint32_t n, const ui
                                                            const uint4 *__restrict__ slot,
                                                            const uint32_t *__restrict__ rank, uint4 *mslot,
                                                            uint4 *mpick, uint4 *mvert, u128 *gmin, u128 *partials) {
-    __shared__ u128 s_pre[kListThreads / kWarp][kLongList];
+    __shared__ uint64_t s_pre[kListThreads / kWarp][kLongList];
     __shared__ uint32_t s_idx[kListThreads / kWarp][kLongList];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, wpb = blockDim.x >> 5;
     uint32_t *m32 = reinterpret_cast<uint32_t *>(mslot);
@@ -479,10 +466,8 @@ __global__ void __launch_bounds__(kListThreads) k_min_alias(uint32_t n, const ui
             for (uint32_t j = lane; j < d; j += kWarp) set_min_alias(m32, (uint64_t)o + j, 0, j);
             return;
         }
-        if (W < (1ull << 56))   // q = w d <= W kLongList < 2^64
-            warp_min_alias<uint64_t>(mslot, m32, o, d, W, reinterpret_cast<uint64_t *>(s_pre[warp]), s_idx[warp]);
-        else
-            warp_min_alias<u128>(mslot, m32, o, d, W, s_pre[warp], s_idx[warp]);
+        // W = sum d_{v,u} d_{u,v} < d d 2^32, so q = w d <= W d < 2^56
+        warp_min_alias(mslot, m32, o, d, W, s_pre[warp], s_idx[warp]);
         __syncwarp();
     };
     for_lists<TILE>(n, vert, small, [&](uint32_t v, uint4 vr) { leave(v, vr, 0); }, large);
@@ -502,14 +487,26 @@ __global__ void __launch_bounds__(kListThreads) k_min_alias(uint32_t n, const ui
 // block forms Gamma-check_v itself (the same integer sum k_min_alias writes
 // into mvert), so the two kernels may run side by side.  A block per kWarp
 // vertex records (the scheduler spreads the long lists); the split of a list
-// of at most kMinSmemList entries in dynamic shared memory, of a longer one in
-// its range of the global scratch (idx, pre)
-constexpr uint32_t kMinSmemList = 2048;
-constexpr size_t kMinSmemBytes = (size_t)kMinSmemList * (sizeof(u128) + sizeof(uint32_t));
+// that fits it in dynamic shared memory, of a longer one in its range of the
+// global scratch (idx, pre).  The arithmetic is 64-bit where d Gamma-check_v
+// fits (every list of the workloads), else 128-bit.
+constexpr size_t kMinSmemBytes = 2048 * (sizeof(u128) + sizeof(uint32_t));
+
+template <typename T>
+__device__ __forceinline__ void long_min_alias(const uint4 *mslot, uint32_t *m32, uint32_t o, uint32_t d, uint64_t W,
+                                               u128 *smem, uint32_t *idx, u128 *pre) {
+    constexpr uint32_t most = kMinSmemBytes / (sizeof(T) + sizeof(uint32_t));
+    const bool fits = d <= most;
+    T *s_pre = reinterpret_cast<T *>(smem);
+    block_alias<T, kListThreads>(
+        d, (T)W, [&](uint32_t j) { return (T)min_weight(mslot, (uint64_t)o + j); },
+        fits ? reinterpret_cast<uint32_t *>(s_pre + most) : idx + o, fits ? s_pre : reinterpret_cast<T *>(pre + o),
+        [&](uint32_t j, T thr, uint32_t alias) { set_min_alias(m32, (uint64_t)o + j, (uint64_t)thr, alias); });
+}
 
 __global__ void __launch_bounds__(kListThreads) k_min_alias_long(uint32_t n, const uint4 *__restrict__ vert,
                                                                 uint4 *mslot, uint32_t *idx, u128 *pre) {
-    extern __shared__ u128 s_split[];   // kMinSmemList prefixes, then kMinSmemList positions
+    extern __shared__ u128 s_split[];   // the prefixes, then the positions
     __shared__ uint64_t s_w[kListThreads / kWarp];
     uint32_t *m32 = reinterpret_cast<uint32_t *>(mslot);
     for_each_vertex<kListThreads, kWarp>(
@@ -527,11 +524,8 @@ __global__ void __launch_bounds__(kListThreads) k_min_alias_long(uint32_t n, con
             for (int w = 0; w < kListThreads / kWarp; ++w) W += s_w[w];
             __syncthreads();   // s_w is refilled for the next list
             if (W == 0) return;   // block-uniform: k_min_alias keeps every column
-            const bool fits = d <= kMinSmemList;
-            block_alias<u128, kListThreads>(
-                d, (u128)W, [&](uint32_t j) { return (u128)min_weight(mslot, (uint64_t)o + j); },
-                fits ? reinterpret_cast<uint32_t *>(s_split + kMinSmemList) : idx + o, fits ? s_split : pre + o,
-                [&](uint32_t j, u128 thr, uint32_t alias) { set_min_alias(m32, (uint64_t)o + j, (uint64_t)thr, alias); });
+            if (W <= ~0ull / d) long_min_alias<uint64_t>(mslot, m32, o, d, W, s_split, idx, pre);
+            else long_min_alias<u128>(mslot, m32, o, d, W, s_split, idx, pre);
         });
 }
 
@@ -617,6 +611,16 @@ cudaError_t launch_min_tables(uint32_t n, uint64_t nnz, const uint4 *vert, const
     const MinScratch m = carve(scratch, n, nnz);
     cudaStream_t h0 = aux ? aux->a[3] : s, h1 = aux ? aux->a[4] : s;
     cudaError_t e = cudaSuccess, eh = cudaSuccess;
+    static std::atomic<bool> attr_set[64];
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev < 0 || dev >= 64 || !attr_set[dev].load(std::memory_order_relaxed)) {
+        e = cudaFuncSetAttribute(k_min_alias_long, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMinSmemBytes);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k_rank_long, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSortBytes);
+        if (e != cudaSuccess) return e;
+        if (dev >= 0 && dev < 64) attr_set[dev].store(true, std::memory_order_relaxed);
+    }
     auto fork = [&](int k) {   // h0 (and h1) wait for what is queued on s
         if (!aux) return;
         if (e == cudaSuccess) e = cudaEventRecord(aux->sub_fork, s);
@@ -634,9 +638,9 @@ cudaError_t launch_min_tables(uint32_t n, uint64_t nnz, const uint4 *vert, const
         fork(2);
         if (e == cudaSuccess) {
             const unsigned chunks = (unsigned)(((uint64_t)n + kWarp - 1) / kWarp);
-            k_rank_block<<<chunks, kSortThreads, 0, h0>>>(n, vert, col, rlist, m.rank);
+            k_rank_block<<<chunks, kBlockThreads, 0, h0>>>(n, vert, col, rlist, m.rank);
             eh = cudaGetLastError();
-            k_rank_long<<<grid_for((uint64_t)n, kSortThreads, 1), kSortThreads, 0, h1>>>(n, vert, col, m.a, m.b, m.ia,
+            k_rank_long<<<grid_for((uint64_t)n, kSortThreads, 2), kSortThreads, kSortBytes, h1>>>(n, vert, col, m.a, m.b, m.ia,
                                                                                         m.ib, rlist, m.rank);
             if (eh == cudaSuccess) eh = cudaGetLastError();
             with_tile(n, [&](auto T) {
@@ -651,14 +655,6 @@ cudaError_t launch_min_tables(uint32_t n, uint64_t nnz, const uint4 *vert, const
         if (e != cudaSuccess) return e;
         k_min_slots<<<grid_for(nnz, 256, 16), 256, 0, s>>>(nnz, vert, col, owner, slot, m.rank, mslot);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    }
-    static std::atomic<bool> attr_set[64];
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (dev < 0 || dev >= 64 || !attr_set[dev].load(std::memory_order_relaxed)) {
-        e = cudaFuncSetAttribute(k_min_alias_long, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMinSmemBytes);
-        if (e != cudaSuccess) return e;
-        if (dev >= 0 && dev < 64) attr_set[dev].store(true, std::memory_order_relaxed);
     }
     const unsigned ab = alias_grid(n);
     fork(1);
