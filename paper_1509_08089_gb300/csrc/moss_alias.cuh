@@ -260,6 +260,19 @@ __device__ __forceinline__ void for_lists(uint32_t n, const uint4 *rec, Small sm
     }
 }
 
+// Lists above kHubList entries get 1,024 threads (hub_blocks(n) blocks walk
+// them), their splits in up to kHubSmemList entries of shared memory: with 256
+// the longest list's chain of rounds was the whole pass (d_max 15,000, us:
+// sigma 255 -> 109 + 89 for the lists up to kHubList, MOSS-4Min 525 -> 197 +
+// 147; the passes that a graph's largest degree rules out are not launched).
+constexpr uint32_t kHubList = 2048;
+constexpr int kHubThreads = 1024;
+constexpr uint32_t kHubSmemList = 16384;   // 192 KB at 12 bytes an entry
+inline unsigned hub_blocks(uint32_t n) {
+    const uint64_t chunks = ((uint64_t)n + kHubThreads - 1) / kHubThreads, sms = (uint64_t)current_sms();
+    return (unsigned)(chunks < sms ? chunks : sms);
+}
+
 // records per warp: enough lists to fill the groups, but a warp for every
 // scheduler first
 template <typename F>

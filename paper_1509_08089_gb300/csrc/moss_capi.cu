@@ -657,7 +657,7 @@ static int build_min_tables(moss_graph *g, cudaStream_t s, const AuxStreams *aux
     void *scratch = nullptr;
     if ((e = pool_alloc(g->device, &scratch, min_scratch_bytes(g->n, g->nnz), s)) != cudaSuccess)
         return cuda_fail(e, "allocating scratch");
-    e = launch_min_tables(g->n, g->nnz, g->vert, g->col, g->owner, g->slot, g->mvert, g->mslot, g->mpick, g->rlist,
+    e = launch_min_tables(g->n, g->nnz, g->tot_h.d_max, g->vert, g->col, g->owner, g->slot, g->mvert, g->mslot, g->mpick, g->rlist,
                           g->gam[3], g->seed[3], g->tot, scratch, g->flags, g->vsplit_min, s, aux);
     cudaFreeAsync(scratch, s);
     if (e != cudaSuccess) return cuda_fail(e, "MOSS-4Min table kernels");
@@ -748,7 +748,7 @@ int moss_build_tables(moss_graph *g, unsigned k_mask, void *stream) {
         ev = launch_seed_alias(g->n, g->tot, nt, which, w, seed, vrec, seed_scratch, g->flags, g->vsplit, sv);
     // per-list tables
     if (e == cudaSuccess)
-        e = launch_sigma_alias(g->n, g->nnz, g->vert, g->acc, g->owner, g->slot, idx, pre, s, aux, 0);
+        e = launch_sigma_alias(g->n, g->nnz, g->tot_h.d_max, g->vert, g->acc, g->owner, g->slot, idx, pre, s, aux, 0);
     // edge hash and filter
     bool hashed = false, filtered = false;
     cudaError_t eh = cudaSuccess;

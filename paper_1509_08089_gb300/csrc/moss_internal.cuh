@@ -363,8 +363,8 @@ uint64_t hub_bytes(uint32_t n);
 cudaError_t launch_hub_tables(uint32_t n, const uint4 *vert, const uint32_t *col, void *mem, uint2 **rank_out,
                               uint32_t **bits_out, uint32_t **list_out, cudaStream_t s);
 // aux (nullable, already forked from s): the long lists go to aux->a[long_stream]
-cudaError_t launch_sigma_alias(uint32_t n, uint64_t nnz, const uint4 *vert, const uint32_t *acc, const uint32_t *owner,
-                               uint4 *slot, uint32_t *scratch_idx, uint64_t *scratch_pre, cudaStream_t s,
+cudaError_t launch_sigma_alias(uint32_t n, uint64_t nnz, uint32_t d_max, const uint4 *vert, const uint32_t *acc,
+                               const uint32_t *owner, uint4 *slot, uint32_t *scratch_idx, uint64_t *scratch_pre, cudaStream_t s,
                                const AuxStreams *aux, int long_stream);
 // two-level vertex alias tables of up to 3 weights in the same launches
 // (seed[t]: 2n uint4, vrec[t]: the n vertex records copied beside each
@@ -380,7 +380,7 @@ int slot_partial_rows(uint32_t n);   // rows of 6 u128 totals launch_slots write
 // moss_min.cu: the MOSS-4Min tables (ordered lists, d_{v,u}, Gamma-check_v,
 // the sigma-check alias tables, tot->gamma[3] and its vertex alias table)
 uint64_t min_scratch_bytes(uint32_t n, uint64_t nnz);
-cudaError_t launch_min_tables(uint32_t n, uint64_t nnz, const uint4 *vert, const uint32_t *col,
+cudaError_t launch_min_tables(uint32_t n, uint64_t nnz, uint32_t d_max, const uint4 *vert, const uint32_t *col,
                               const uint32_t *owner, const uint4 *slot, uint4 *mvert, uint4 *mslot, uint4 *mpick,
                               uint2 *rlist, u128 *gmin, uint4 *seed_min, DevTotals *tot, void *scratch,
                               uint32_t *flags, int split, cudaStream_t s, const AuxStreams *aux);

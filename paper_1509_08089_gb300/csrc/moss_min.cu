@@ -19,6 +19,7 @@
 // used for sigma^(v) in moss_tables.cu, here in 128-bit arithmetic since
 // q_j = w_j d_v can exceed 2^64; the exact total Gamma-check; and the vertex
 // alias table of pi-check through the seed-table kernels.
+#include <algorithm>
 #include <atomic>
 
 #include "moss_alias.cuh"
@@ -30,7 +31,7 @@ namespace {
 
 constexpr int kWarp = 32;
 constexpr uint32_t kTile = 4096;      // keys sorted per shared-memory pass
-constexpr int kSortThreads = 512;
+constexpr int kSortThreads = 1024;
 constexpr int kListThreads = 256;
 constexpr uint32_t kWarpKeys = 4;     // k_rank_warp: lists up to 128 entries
 constexpr uint32_t kLongList = 256;   // longer lists: k_min_alias_long, a block per list
@@ -483,51 +484,55 @@ __global__ void __launch_bounds__(kListThreads) k_min_alias(uint32_t n, const ui
     }
 }
 
-// the alias tables of lists longer than kLongList, a block per list; each
-// block forms Gamma-check_v itself (the same integer sum k_min_alias writes
-// into mvert), so the two kernels may run side by side.  A block per kWarp
-// vertex records (the scheduler spreads the long lists); the split of a list
-// that fits it in dynamic shared memory, of a longer one in its range of the
-// global scratch (idx, pre).  The arithmetic is 64-bit where d Gamma-check_v
-// fits (every list of the workloads), else 128-bit.
-constexpr size_t kMinSmemBytes = 2048 * (sizeof(u128) + sizeof(uint32_t));
+// the alias tables of lists longer than kLongList, a block per list, 256
+// threads up to kHubList entries and 1,024 above (moss_alias.cuh); each block
+// forms Gamma-check_v itself (the same integer sum k_min_alias writes into
+// mvert), so the kernels may run side by side.  The split of a list that fits
+// the smem_bytes of dynamic shared memory is kept there, of a longer one in
+// its range of the global scratch (idx, pre).  The arithmetic is 64-bit where
+// d Gamma-check_v fits (always below 2^16 entries: d_{v,u} < d, d_{u,v} < d_u
+// and S_v < 2^32), else 128-bit.
+constexpr uint32_t kMidBytes = kHubList * (sizeof(uint64_t) + sizeof(uint32_t));
+constexpr uint32_t kHubBytes = kHubSmemList * (sizeof(uint64_t) + sizeof(uint32_t));
 
-template <typename T>
+template <typename T, int NT>
 __device__ __forceinline__ void long_min_alias(const uint4 *mslot, uint32_t *m32, uint32_t o, uint32_t d, uint64_t W,
-                                               u128 *smem, uint32_t *idx, u128 *pre) {
-    constexpr uint32_t most = kMinSmemBytes / (sizeof(T) + sizeof(uint32_t));
-    const bool fits = d <= most;
+                                               u128 *smem, uint32_t smem_bytes, uint32_t *idx, u128 *pre) {
+    const bool fits = d <= smem_bytes / (sizeof(T) + sizeof(uint32_t));
     T *s_pre = reinterpret_cast<T *>(smem);
-    block_alias<T, kListThreads>(
+    block_alias<T, NT>(
         d, (T)W, [&](uint32_t j) { return (T)min_weight(mslot, (uint64_t)o + j); },
-        fits ? reinterpret_cast<uint32_t *>(s_pre + most) : idx + o, fits ? s_pre : reinterpret_cast<T *>(pre + o),
+        fits ? reinterpret_cast<uint32_t *>(s_pre + d) : idx + o, fits ? s_pre : reinterpret_cast<T *>(pre + o),
         [&](uint32_t j, T thr, uint32_t alias) { set_min_alias(m32, (uint64_t)o + j, (uint64_t)thr, alias); });
 }
 
-__global__ void __launch_bounds__(kListThreads) k_min_alias_long(uint32_t n, const uint4 *__restrict__ vert,
-                                                                uint4 *mslot, uint32_t *idx, u128 *pre) {
+template <int NT, int CH, uint32_t LO, uint32_t HI>
+__global__ void __launch_bounds__(NT) k_min_alias_long(uint32_t n, const uint4 *__restrict__ vert, uint4 *mslot,
+                                                      uint32_t *idx, u128 *pre, uint32_t smem_bytes) {
     extern __shared__ u128 s_split[];   // the prefixes, then the positions
-    __shared__ uint64_t s_w[kListThreads / kWarp];
+    __shared__ uint64_t s_w[NT / kWarp];
     uint32_t *m32 = reinterpret_cast<uint32_t *>(mslot);
-    for_each_vertex<kListThreads, kWarp>(
-        n, vert, [](uint4 vr) { return vr.y > kLongList; },
+    for_each_vertex<NT, CH>(
+        n, vert, [](uint4 vr) { return vr.y > LO && vr.y <= HI; },
         [&](uint32_t v) {
             const uint4 vr = vert[v];
             const uint32_t o = vr.x, d = vr.y;
             uint64_t W = 0;
-            for (uint32_t j = threadIdx.x; j < d; j += kListThreads) W += min_weight(mslot, (uint64_t)o + j);
+            for (uint32_t j = threadIdx.x; j < d; j += NT) W += min_weight(mslot, (uint64_t)o + j);
 #pragma unroll
             for (int sft = 16; sft > 0; sft >>= 1) W += __shfl_down_sync(0xffffffffu, W, sft);
             if ((threadIdx.x & 31) == 0) s_w[threadIdx.x >> 5] = W;
             __syncthreads();
             W = 0;
-            for (int w = 0; w < kListThreads / kWarp; ++w) W += s_w[w];
+            for (int w = 0; w < NT / kWarp; ++w) W += s_w[w];
             __syncthreads();   // s_w is refilled for the next list
             if (W == 0) return;   // block-uniform: k_min_alias keeps every column
-            if (W <= ~0ull / d) long_min_alias<uint64_t>(mslot, m32, o, d, W, s_split, idx, pre);
-            else long_min_alias<u128>(mslot, m32, o, d, W, s_split, idx, pre);
+            if (W <= ~0ull / d) long_min_alias<uint64_t, NT>(mslot, m32, o, d, W, s_split, smem_bytes, idx, pre);
+            else long_min_alias<u128, NT>(mslot, m32, o, d, W, s_split, smem_bytes, idx, pre);
         });
 }
+const auto k_min_alias_mid = k_min_alias_long<kListThreads, kWarp, kLongList, kHubList>;
+const auto k_min_alias_hub = k_min_alias_long<kHubThreads, kHubThreads, kHubList, 0xffffffffu>;
 
 __global__ void k_min_total(const u128 *partials, int blocks, DevTotals *tot) {
     const int lane = threadIdx.x;   // one warp
@@ -600,7 +605,7 @@ MinScratch carve(void *base, uint32_t n, uint64_t nnz) {
 
 uint64_t min_scratch_bytes(uint32_t n, uint64_t nnz) { return carve(nullptr, n, nnz).bytes; }
 
-cudaError_t launch_min_tables(uint32_t n, uint64_t nnz, const uint4 *vert, const uint32_t *col,
+cudaError_t launch_min_tables(uint32_t n, uint64_t nnz, uint32_t d_max, const uint4 *vert, const uint32_t *col,
                               const uint32_t *owner, const uint4 *slot, uint4 *mvert, uint4 *mslot, uint4 *mpick,
                               uint2 *rlist, u128 *gmin, uint4 *seed_min, DevTotals *tot, void *scratch,
                               uint32_t *flags, int split, cudaStream_t s, const AuxStreams *aux) {
@@ -615,7 +620,7 @@ cudaError_t launch_min_tables(uint32_t n, uint64_t nnz, const uint4 *vert, const
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev < 0 || dev >= 64 || !attr_set[dev].load(std::memory_order_relaxed)) {
-        e = cudaFuncSetAttribute(k_min_alias_long, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMinSmemBytes);
+        e = cudaFuncSetAttribute(k_min_alias_hub, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kHubBytes);
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(k_rank_long, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSortBytes);
         if (e != cudaSuccess) return e;
@@ -638,10 +643,11 @@ cudaError_t launch_min_tables(uint32_t n, uint64_t nnz, const uint4 *vert, const
         fork(2);
         if (e == cudaSuccess) {
             const unsigned chunks = (unsigned)(((uint64_t)n + kWarp - 1) / kWarp);
-            k_rank_block<<<chunks, kBlockThreads, 0, h0>>>(n, vert, col, rlist, m.rank);
+            if (d_max > kWarpKeys * kWarp) k_rank_block<<<chunks, kBlockThreads, 0, h0>>>(n, vert, col, rlist, m.rank);
             eh = cudaGetLastError();
-            k_rank_long<<<grid_for((uint64_t)n, kSortThreads, 2), kSortThreads, kSortBytes, h1>>>(n, vert, col, m.a, m.b, m.ia,
-                                                                                        m.ib, rlist, m.rank);
+            if (d_max > kBlockList)
+                k_rank_long<<<grid_for((uint64_t)n, kSortThreads, 2), kSortThreads, kSortBytes, h1>>>(
+                    n, vert, col, m.a, m.b, m.ia, m.ib, rlist, m.rank);
             if (eh == cudaSuccess) eh = cudaGetLastError();
             with_tile(n, [&](auto T) {
                 constexpr int tile = decltype(T)::value;
@@ -662,7 +668,13 @@ cudaError_t launch_min_tables(uint32_t n, uint64_t nnz, const uint4 *vert, const
     // the merges' scratch is dead now: the long-list kernel keeps its split
     // order in ia[] and its prefixes in a[], b[] (k_min_alias still reads the ranks)
     const unsigned chunks = (unsigned)(((uint64_t)n + kWarp - 1) / kWarp);
-    k_min_alias_long<<<chunks, kListThreads, kMinSmemBytes, h0>>>(n, vert, mslot, m.ia, reinterpret_cast<u128 *>(m.a));
+    u128 *pre = reinterpret_cast<u128 *>(m.a);
+    if (d_max > kHubList) {
+        const uint32_t bytes = std::min<uint64_t>(kHubBytes, (uint64_t)d_max * (sizeof(uint64_t) + sizeof(uint32_t)));
+        k_min_alias_hub<<<hub_blocks(n), kHubThreads, bytes, h0>>>(n, vert, mslot, m.ia, pre, bytes);
+    }
+    if (d_max > kLongList)
+        k_min_alias_mid<<<chunks, kListThreads, kMidBytes, h0>>>(n, vert, mslot, m.ia, pre, kMidBytes);
     eh = cudaGetLastError();
     with_tile(n, [&](auto T) {
         k_min_alias<decltype(T)::value><<<ab, kListThreads, 0, s>>>(n, vert, col, slot, m.rank, mslot, mpick, mvert,

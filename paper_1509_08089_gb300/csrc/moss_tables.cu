@@ -36,6 +36,7 @@ namespace {
 constexpr int kWarp = 32;
 constexpr int kTableThreads = 256;
 constexpr uint32_t kLongList = 256;   // longer lists get a block each in the alias passes
+constexpr size_t kSplitBytes = sizeof(uint64_t) + sizeof(uint32_t);   // per entry of a list's split
 constexpr int kLongThreads = 256;
 
 // ------------------------------------------------------------ vertices ---
@@ -534,29 +535,31 @@ __global__ void __launch_bounds__(kTableThreads) k_sigma_alias(uint32_t n, const
     for_lists<TILE>(n, vert, small, [](uint32_t, uint4) {}, large);
 }
 
-// lists longer than kLongList: a block per list (moss_alias.cuh); a list of
-// at most kLongSmemList entries keeps its split in dynamic shared memory, a
-// longer one in its range of the global scratch (idx, pre).  The grid has a
-// block per kSigmaChunk vertices, so the hardware scheduler spreads the long
-// lists over the SMs as blocks finish instead of a fixed share per block.
-constexpr uint32_t kLongSmemList = 4096;
-constexpr size_t kLongSmemBytes = (size_t)kLongSmemList * (sizeof(uint64_t) + sizeof(uint32_t));
+// lists longer than kLongList: a block per list (moss_alias.cuh), 256 threads
+// up to kHubList entries and 1,024 above, where one list's chain of scans and
+// merges would set the launch's time (a 15,000-entry list: 60 rounds of 256).
+// A list of at most smem_list entries keeps its split in dynamic shared
+// memory, a longer one in its range of the global scratch (idx, pre).  The
+// 256-thread grid has a block per kSigmaChunk vertices, so the hardware
+// scheduler spreads the lists over the SMs as blocks finish; the few hubs go
+// to a block per SM.
 constexpr int kSigmaChunk = 32;
 
-__global__ void __launch_bounds__(kLongThreads) k_sigma_alias_long(uint32_t n, const uint4 *__restrict__ vert,
-                                                                  const uint32_t *__restrict__ acc, uint4 *slot,
-                                                                  uint32_t *idx, uint64_t *pre) {
-    extern __shared__ uint64_t s_split[];   // kLongSmemList pre, then kLongSmemList idx
+template <int NT, int CH, uint32_t LO, uint32_t HI>
+__global__ void __launch_bounds__(NT) k_sigma_alias_long(uint32_t n, const uint4 *__restrict__ vert,
+                                                        const uint32_t *__restrict__ acc, uint4 *slot, uint32_t *idx,
+                                                        uint64_t *pre, uint32_t smem_list) {
+    extern __shared__ uint64_t s_split[];   // smem_list pre, then smem_list idx
     uint32_t *slot32 = reinterpret_cast<uint32_t *>(slot);
-    for_each_vertex<kLongThreads, kSigmaChunk>(
-        n, vert, [](uint4 vr) { return vr.y > kLongList && vr.z != 0; },
+    for_each_vertex<NT, CH>(
+        n, vert, [](uint4 vr) { return vr.y > LO && vr.y <= HI && vr.z != 0; },
         [&](uint32_t v) {
             const uint4 vr = vert[v];
             const uint32_t o = vr.x, d = vr.y, S = vr.z;
-            const bool fits = d <= kLongSmemList;
-            block_alias<uint64_t, kLongThreads>(
+            const bool fits = d <= smem_list;
+            block_alias<uint64_t, NT>(
                 d, (uint64_t)S, [&](uint32_t j) { return (uint64_t)acc_weight(acc, o, d, S, j); },
-                fits ? reinterpret_cast<uint32_t *>(s_split + kLongSmemList) : idx + o, fits ? s_split : pre + o,
+                fits ? reinterpret_cast<uint32_t *>(s_split + smem_list) : idx + o, fits ? s_split : pre + o,
                 [&](uint32_t j, uint64_t thr, uint32_t alias) {
                     set_sigma(slot32, o, j, (uint32_t)thr, alias);
                 });
@@ -1405,35 +1408,47 @@ cudaError_t launch_hub_tables(uint32_t n, const uint4 *vert, const uint32_t *col
     return cudaSuccess;
 }
 
-cudaError_t launch_sigma_alias(uint32_t n, uint64_t nnz, const uint4 *vert, const uint32_t *acc, const uint32_t *owner,
-                               uint4 *slot, uint32_t *scratch_idx, uint64_t *scratch_pre, cudaStream_t s,
-                               const AuxStreams *aux, int long_stream) {
+cudaError_t launch_sigma_alias(uint32_t n, uint64_t nnz, uint32_t d_max, const uint4 *vert, const uint32_t *acc,
+                               const uint32_t *owner, uint4 *slot, uint32_t *scratch_idx, uint64_t *scratch_pre,
+                               cudaStream_t s, const AuxStreams *aux, int long_stream) {
     // the short and the long lists are built side by side (long lists on
     // aux->a[long_stream], forked from s by the caller); the fill waits for both
+    const auto mid = k_sigma_alias_long<kLongThreads, kSigmaChunk, kLongList, kHubList>;
+    const auto hub = k_sigma_alias_long<kHubThreads, kHubThreads, kHubList, 0xffffffffu>;
+    const size_t mid_bytes = (size_t)kHubList * kSplitBytes;
+    const uint32_t hub_list = std::min(d_max, kHubSmemList);
     static std::atomic<bool> attr_set[64];
     int dev = 0;
     cudaGetDevice(&dev);
     cudaError_t e = cudaSuccess;
     if (dev < 0 || dev >= 64 || !attr_set[dev].load(std::memory_order_relaxed)) {
-        e = cudaFuncSetAttribute(k_sigma_alias_long, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLongSmemBytes);
+        e = cudaFuncSetAttribute(hub, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kHubSmemList * kSplitBytes));
         if (e != cudaSuccess) return e;
         if (dev >= 0 && dev < 64) attr_set[dev].store(true, std::memory_order_relaxed);
     }
-    const unsigned chunks = (unsigned)(((uint64_t)n + kSigmaChunk - 1) / kSigmaChunk);
     cudaStream_t ls = aux ? aux->a[long_stream] : s;
-    k_sigma_alias_long<<<chunks ? chunks : 1, kLongThreads, kLongSmemBytes, ls>>>(n, vert, acc, slot, scratch_idx,
-                                                                                   scratch_pre);
-    cudaError_t el = cudaGetLastError();
+    cudaError_t el = cudaSuccess;
+    if (d_max > kHubList) {
+        hub<<<hub_blocks(n), kHubThreads, hub_list * kSplitBytes, ls>>>(n, vert, acc, slot, scratch_idx, scratch_pre,
+                                                                        hub_list);
+        el = cudaGetLastError();
+    }
+    if (d_max > kLongList && el == cudaSuccess) {
+        const unsigned chunks = (unsigned)(((uint64_t)n + kSigmaChunk - 1) / kSigmaChunk);
+        mid<<<chunks, kLongThreads, mid_bytes, ls>>>(n, vert, acc, slot, scratch_idx, scratch_pre, kHubList);
+        el = cudaGetLastError();
+    }
     with_tile(n, [&](auto T) {
         k_sigma_alias<decltype(T)::value><<<tile_blocks(n, decltype(T)::value, kTableThreads, current_sms(), 8), kTableThreads, 0, s>>>(n, vert, acc, slot);
     });
     e = cudaGetLastError();
-    if (aux) {
+    if (aux && d_max > kLongList) {
         const cudaError_t ew = aux->wait_for(s, long_stream);
         if (el == cudaSuccess) el = ew;
     }
     if (e != cudaSuccess) return e;
     if (el != cudaSuccess) return el;
+    if (d_max <= kShortList) return cudaSuccess;   // every record is complete
     k_slot_alias_fill<<<flat_blocks(nnz), 256, 0, s>>>(nnz, vert, owner, slot);
     return cudaGetLastError();
 }
