@@ -196,6 +196,13 @@ __device__ void block_alias(uint32_t d, T W, Weight weight, uint32_t *idx, T *pr
     __syncthreads();   // idx / pre are reused by the block's next list
 }
 
+// The blocks that share a pass: a whole launch, or a run of its blocks when
+// passes that do not depend on each other share one.
+struct GridPart {
+    uint32_t block, blocks;
+};
+__device__ __forceinline__ GridPart whole_grid() { return GridPart{blockIdx.x, gridDim.x}; }
+
 // ------------------------------------------------------------ short lists --
 // Lists of at most kShortList entries, most lists of a power-law graph, go to
 // groups of 8, 16 or 32 lanes, an entry per lane, so one warp builds four, two
@@ -215,12 +222,14 @@ constexpr uint32_t kShortList = 32;
 // empty(v, rec), one lane each; and, of TILE records a stride apart (so that
 // long lists which lie together spread over the warps), the longer lists one
 // by one to large(v, rec), the whole warp each.
+// The walk is shared by the blocks of `grid`.
 template <int TILE, typename Small, typename Empty, typename Large>
-__device__ __forceinline__ void for_lists(uint32_t n, const uint4 *rec, Small small, Empty empty, Large large) {
+__device__ __forceinline__ void for_lists(GridPart grid, uint32_t n, const uint4 *rec, Small small, Empty empty,
+                                          Large large) {
     const int lane = threadIdx.x & 31;
     const uint64_t tiles = ((uint64_t)n + TILE - 1) / TILE;
-    const uint64_t warps = (uint64_t)gridDim.x * (blockDim.x >> 5);
-    for (uint64_t t = (uint64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); t < tiles; t += warps) {
+    const uint64_t warps = (uint64_t)grid.blocks * (blockDim.x >> 5);
+    for (uint64_t t = (uint64_t)grid.block * (blockDim.x >> 5) + (threadIdx.x >> 5); t < tiles; t += warps) {
         const uint64_t v0 = t * TILE, vs = t + (uint64_t)lane * tiles;
         const bool here = lane < TILE && v0 + lane < n;
         const uint4 r = here ? rec[v0 + lane] : make_uint4(0u, 0u, 0u, 0u);
@@ -344,12 +353,12 @@ __device__ __forceinline__ void group_alias(bool valid, uint64_t q, uint64_t W, 
 // fall into different chunks, so a graph whose long lists sit together (one
 // loaded in degree order) still spreads them over the blocks.
 template <int NT, int CH = NT, typename Pred, typename Body>
-__device__ void for_each_vertex(uint32_t n, const uint4 *rec, Pred pred, Body body) {
+__device__ __forceinline__ void for_each_vertex(GridPart grid, uint32_t n, const uint4 *rec, Pred pred, Body body) {
     static_assert(CH <= NT, "chunk larger than the block");
     __shared__ uint32_t found[CH];
     __shared__ uint32_t nfound;
     const uint64_t chunks = ((uint64_t)n + CH - 1) / CH;
-    for (uint64_t c = blockIdx.x; c < chunks; c += gridDim.x) {
+    for (uint64_t c = grid.block; c < chunks; c += grid.blocks) {
         if (threadIdx.x == 0) nfound = 0;
         __syncthreads();
         const uint64_t v = c + (uint64_t)threadIdx.x * chunks;

@@ -419,6 +419,16 @@ cudaError_t pool_alloc(int device, void **p, size_t bytes, cudaStream_t s) {
     return cudaMallocFromPoolAsync(p, bytes ? bytes : 1, pool, s);
 }
 
+// whether p is memory of this device that kernels can read in place
+bool readable_here(const void *p, size_t align, int device) {
+    cudaPointerAttributes pa;
+    if (cudaPointerGetAttributes(&pa, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return pa.type == cudaMemoryTypeDevice && pa.device == device && reinterpret_cast<uintptr_t>(p) % align == 0;
+}
+
 // Carves 256-byte aligned arrays out of one allocation (first pass: size).
 struct Carver {
     uint8_t *base = nullptr;
@@ -528,6 +538,7 @@ int moss_graph_load_csr_order(const void *row_ptr, int row_ptr_is_64, const uint
     g->pin = pin_take();
     void *rp_dev = nullptr;
     void *oscratch = nullptr;   // renumbering scratch (released before return)
+    const bool small = small_graph(n, nnz);
     const size_t rp_bytes = (size_t)(n + 1ULL) * (row_ptr_is_64 ? 8 : 4);
     cudaError_t e = cudaSuccess;
     int blocks = table_blocks(n);
@@ -577,19 +588,12 @@ int moss_graph_load_csr_order(const void *row_ptr, int row_ptr_is_64, const uint
             if (ordered) g->order = c.take<uint32_t>(n);
         }
     }
-    STEP(cudaMemcpyAsync(rp_dev, row_ptr, rp_bytes, cudaMemcpyDefault, s), "copying row_ptr");
     STEP(cudaMemsetAsync(g->flags, 0, 2 * sizeof(uint32_t), s), "clearing status");
     if (ordered) {
+        STEP(cudaMemcpyAsync(rp_dev, row_ptr, rp_bytes, cudaMemcpyDefault, s), "copying row_ptr");
         // the input lists are read in place when they are device memory of
         // this device, else copied beside the scratch first
-        bool direct = false;
-        if (nnz) {
-            cudaPointerAttributes pa;
-            if (cudaPointerGetAttributes(&pa, col) == cudaSuccess)
-                direct = pa.type == cudaMemoryTypeDevice && pa.device == device;
-            else
-                cudaGetLastError();
-        }
+        const bool direct = nnz && readable_here(col, alignof(uint32_t), device);
         const uint64_t ob = (order_scratch_bytes(n) + 255) & ~255ull;
         STEP(pool_alloc(device, &oscratch, ob + (direct ? 0 : nnz * sizeof(uint32_t)), s), "allocating order scratch");
         const uint32_t *src = col;
@@ -601,15 +605,36 @@ int moss_graph_load_csr_order(const void *row_ptr, int row_ptr_is_64, const uint
         uint32_t *rp_new = nullptr;
         STEP(launch_degree_order(rp_dev, row_ptr_is_64, src, n, nnz, g->order, g->col, oscratch, &rp_new, g->flags, s),
              "ordering kernels");
-        STEP(launch_vertices(rp_new, 0, n, nnz, g->vert, g->flags, s), "vertex kernel");
+        if (small)
+            STEP(launch_small_load(rp_new, 0, nullptr, n, nnz, g->vert, g->col, g->slot, g->acc, g->owner, g->sq,
+                                   g->gam[0], g->gam[1], g->gam[2], g->tot, g->flags, s),
+                 "load kernels");
+        else
+            STEP(launch_vertices(rp_new, 0, n, nnz, g->vert, g->flags, s), "vertex kernel");
         void *done = oscratch;
         oscratch = nullptr;
         STEP(cudaFreeAsync(done, s), "releasing order scratch");
+    } else if (small) {
+        // rows and lists in device memory are read where they are
+        const void *rp = row_ptr;
+        const uint32_t *src = col;
+        if (!readable_here(row_ptr, row_ptr_is_64 ? 8 : 4, device)) {
+            STEP(cudaMemcpyAsync(rp_dev, row_ptr, rp_bytes, cudaMemcpyDefault, s), "copying row_ptr");
+            rp = rp_dev;
+        }
+        if (nnz && !readable_here(col, alignof(uint32_t), device)) {
+            STEP(cudaMemcpyAsync(g->col, col, nnz * sizeof(uint32_t), cudaMemcpyDefault, s), "copying col");
+            src = nullptr;
+        }
+        STEP(launch_small_load(rp, row_ptr_is_64, src, n, nnz, g->vert, g->col, g->slot, g->acc, g->owner, g->sq,
+                               g->gam[0], g->gam[1], g->gam[2], g->tot, g->flags, s),
+             "load kernels");
     } else {
+        STEP(cudaMemcpyAsync(rp_dev, row_ptr, rp_bytes, cudaMemcpyDefault, s), "copying row_ptr");
         if (nnz) STEP(cudaMemcpyAsync(g->col, col, nnz * sizeof(uint32_t), cudaMemcpyDefault, s), "copying col");
         STEP(launch_vertices(rp_dev, row_ptr_is_64, n, nnz, g->vert, g->flags, s), "vertex kernel");
     }
-    {
+    if (!small) {
         u128 *tp = reinterpret_cast<u128 *>(g->partials + (uint64_t)prow * kSlots);
         STEP(launch_slots(n, nnz, g->col, g->vert, g->slot, g->acc, g->owner, g->sq, g->gam[0], g->gam[1], g->gam[2],
                           tp, blocks, g->flags, s, aux_streams()),
@@ -715,13 +740,15 @@ int moss_build_tables(moss_graph *g, unsigned k_mask, void *stream) {
     uint32_t *idx = static_cast<uint32_t *>(scratch);
     uint64_t *pre = reinterpret_cast<uint64_t *>(static_cast<uint8_t *>(scratch) + ((g->nnz * 4 + 255) & ~255ULL));
     void *seed_scratch = static_cast<uint8_t *>(scratch) + sigma_bytes;
+    const bool want_min = (k_mask & MOSS_TABLES_4MIN) != 0;
+    // a small graph's passes share launches on s
+    const bool small = small_graph(g->n, g->nnz) && g->vsplit == MOSS_VERTEX_ONE_LEVEL && !want_min && !want_filter;
     e = cudaMemsetAsync(g->flags, 0, 2 * sizeof(uint32_t), s);
-    const AuxStreams *aux = e == cudaSuccess ? aux_streams() : nullptr;
+    const AuxStreams *aux = e == cudaSuccess && !small ? aux_streams() : nullptr;
     if (aux && aux->fork(s) != cudaSuccess) {
         cudaGetLastError();
         aux = nullptr;
     }
-    const bool want_min = (k_mask & MOSS_TABLES_4MIN) != 0;
     cudaStream_t sv = aux ? aux->a[1] : s, sm = aux ? aux->a[2] : s, sh = aux && !want_min ? aux->a[2] : s;
     // MOSS-4Min tables
     bool min_built = false;
@@ -744,15 +771,22 @@ int moss_build_tables(moss_graph *g, unsigned k_mask, void *stream) {
         }
     }
     cudaError_t ev = cudaSuccess;
-    if (e == cudaSuccess && nt > 0)
-        ev = launch_seed_alias(g->n, g->tot, nt, which, w, seed, vrec, seed_scratch, g->flags, g->vsplit, sv);
-    // per-list tables
-    if (e == cudaSuccess)
-        e = launch_sigma_alias(g->n, g->nnz, g->tot_h.d_max, g->vert, g->acc, g->owner, g->slot, idx, pre, s, aux, 0);
-    // edge hash and filter
     bool hashed = false, filtered = false;
     cudaError_t eh = cudaSuccess;
-    if (e == cudaSuccess && want_hash) {
+    if (small) {
+        if (e == cudaSuccess)
+            e = launch_small_build(g->n, g->nnz, g->tot_h.d_max, g->tot, nt, which, w, seed, vrec, seed_scratch, g->flags,
+                                   g->vert, g->acc, g->col, g->owner, g->slot, idx, pre, want_hash ? g->hash : nullptr,
+                                   buckets, s);
+        hashed = want_hash && e == cudaSuccess;
+    }
+    if (e == cudaSuccess && nt > 0 && !small)
+        ev = launch_seed_alias(g->n, g->tot, nt, which, w, seed, vrec, seed_scratch, g->flags, g->vsplit, sv);
+    // per-list tables
+    if (e == cudaSuccess && !small)
+        e = launch_sigma_alias(g->n, g->nnz, g->tot_h.d_max, g->vert, g->acc, g->owner, g->slot, idx, pre, s, aux, 0);
+    // edge hash and filter
+    if (e == cudaSuccess && want_hash && !small) {
         uint32_t lg = 0;
         while ((1ULL << lg) < buckets) ++lg;
         eh = cudaMemsetAsync(g->hash, 0xFF, buckets * 8 * kBucketKeys, sh);

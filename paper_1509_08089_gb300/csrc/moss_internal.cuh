@@ -374,6 +374,20 @@ cudaError_t launch_seed_alias(uint32_t n, DevTotals *tot, int ntables, const int
                               uint4 *const *seed, const uint4 *const *vrec, void *scratch, uint32_t *flags, int split,
                               cudaStream_t s);
 uint64_t seed_scratch_bytes(uint32_t n);
+// Graphs small enough for the load and the build in shared launches: rows
+// straight from row_ptr and, unless null, lists copied from src into col; all
+// the arrays of launch_vertices, launch_slots and launch_totals.  The build
+// makes one-level vertex tables, the per-list tables and (unless hash is null)
+// the edge set.
+bool small_graph(uint32_t n, uint64_t nnz);
+cudaError_t launch_small_load(const void *row_ptr, int is64, const uint32_t *src, uint32_t n, uint64_t nnz, uint4 *vert,
+                              uint32_t *col, uint4 *slot, uint32_t *acc, uint32_t *owner, uint64_t *sq, u128 *gam0,
+                              u128 *gam1, u128 *gam2, DevTotals *tot, uint32_t *flags, cudaStream_t s);
+cudaError_t launch_small_build(uint32_t n, uint64_t nnz, uint32_t d_max, DevTotals *tot, int ntables, const int *which,
+                               u128 *const *w, uint4 *const *seed, const uint4 *const *vrec, void *seed_scratch,
+                               uint32_t *flags, const uint4 *vert, const uint32_t *acc, const uint32_t *col,
+                               const uint32_t *owner, uint4 *slot, uint32_t *scratch_idx, uint64_t *scratch_pre,
+                               unsigned long long *hash, uint64_t hash_buckets, cudaStream_t s);
 int table_blocks(uint32_t n);
 int slot_partial_rows(uint32_t n);   // rows of 6 u128 totals launch_slots writes (launch_totals sums them)
 

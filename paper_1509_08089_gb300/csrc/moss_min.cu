@@ -99,7 +99,7 @@ __global__ void __launch_bounds__(kListThreads) k_rank_warp(uint32_t n, const ui
             }
         }
     };
-    for_lists<TILE>(n, vert, small, [](uint32_t, uint4) {}, large);
+    for_lists<TILE>(whole_grid(), n, vert, small, [](uint32_t, uint4) {}, large);
 }
 
 // Keys of col[o + base, o + base + len) sorted highest first, each with its
@@ -168,7 +168,7 @@ __global__ void __launch_bounds__(kBlockThreads) k_rank_block(uint32_t n, const 
     __shared__ uint64_t k[2 * kBlockList];
     __shared__ uint16_t id[2 * kBlockList];
     for_each_vertex<kBlockThreads, kWarp>(
-        n, vert, [](uint4 vr) { return vr.y > kWarpKeys * (uint32_t)kWarp && vr.y <= kBlockList; },
+        whole_grid(), n, vert, [](uint4 vr) { return vr.y > kWarpKeys * (uint32_t)kWarp && vr.y <= kBlockList; },
         [&](uint32_t v) {
             const uint4 vr = vert[v];
             const uint32_t o = vr.x, d = vr.y;
@@ -192,7 +192,7 @@ __global__ void __launch_bounds__(kSortThreads) k_rank_long(uint32_t n, const ui
                                                            uint32_t *rank) {
     extern __shared__ uint64_t k[];   // 2 kTile keys, then their positions
     uint16_t *id = reinterpret_cast<uint16_t *>(k + 2 * kTile);
-    for_each_vertex<kSortThreads>(n, vert, [](uint4 vr) { return vr.y > kBlockList; }, [&](uint32_t v) {
+    for_each_vertex<kSortThreads>(whole_grid(), n, vert, [](uint4 vr) { return vr.y > kBlockList; }, [&](uint32_t v) {
         const uint4 vr = vert[v];
         const uint32_t o = vr.x, d = vr.y;
         if (d <= kTile) {
@@ -471,7 +471,7 @@ __global__ void __launch_bounds__(kListThreads) k_min_alias(uint32_t n, const ui
         warp_min_alias(mslot, m32, o, d, W, s_pre[warp], s_idx[warp]);
         __syncwarp();
     };
-    for_lists<TILE>(n, vert, small, [&](uint32_t v, uint4 vr) { leave(v, vr, 0); }, large);
+    for_lists<TILE>(whole_grid(), n, vert, small, [&](uint32_t v, uint4 vr) { leave(v, vr, 0); }, large);
     total = warp_sum128(total);
     // block share of Gamma-check
     __shared__ u128 sh[kListThreads / kWarp];
@@ -513,7 +513,7 @@ __global__ void __launch_bounds__(NT) k_min_alias_long(uint32_t n, const uint4 *
     __shared__ uint64_t s_w[NT / kWarp];
     uint32_t *m32 = reinterpret_cast<uint32_t *>(mslot);
     for_each_vertex<NT, CH>(
-        n, vert, [](uint4 vr) { return vr.y > LO && vr.y <= HI; },
+        whole_grid(), n, vert, [](uint4 vr) { return vr.y > LO && vr.y <= HI; },
         [&](uint32_t v) {
             const uint4 vr = vert[v];
             const uint32_t o = vr.x, d = vr.y;

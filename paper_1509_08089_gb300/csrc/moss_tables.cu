@@ -62,7 +62,7 @@ template <int TILE>
 __global__ void __launch_bounds__(kTableThreads) k_owner(uint32_t n, const uint4 *__restrict__ vert, uint32_t *owner) {
     const int lane = threadIdx.x & 31;
     for_lists<TILE>(
-        n, vert,
+        whole_grid(), n, vert,
         [&](auto, uint32_t v, uint4 r, uint32_t j, bool valid) {
             if (valid) owner[r.x + j] = v;
         },
@@ -146,8 +146,8 @@ __device__ __forceinline__ uint32_t warp_incl_scan32(uint32_t v, int lane) {
 }
 
 template <int TILE>
-__global__ void __launch_bounds__(kTableThreads, 8) k_slots(uint32_t n, uint4 *vert, uint32_t *acc, uint64_t *sq,
-                                                           u128 *gam2) {
+__device__ __forceinline__ void scan_lists(GridPart grid, uint32_t n, uint4 *vert, uint32_t *acc, uint64_t *sq,
+                                           u128 *gam2) {
     const int lane = threadIdx.x & 31;
     // S_v, and Q_v until k_vertex_weights turns it into Gamma^(2)_v
     auto leave = [&](uint32_t v, uint64_t S, uint64_t Q) {
@@ -155,7 +155,7 @@ __global__ void __launch_bounds__(kTableThreads, 8) k_slots(uint32_t n, uint4 *v
         gam2[v] = Q;
     };
     for_lists<TILE>(
-        n, vert,
+        grid, n, vert,
         [&](auto G, uint32_t v, uint4 r, uint32_t j, bool valid) {
             constexpr int g = decltype(G)::value;
             const uint64_t w = valid ? acc[r.x + j] : 0u;
@@ -188,12 +188,18 @@ __global__ void __launch_bounds__(kTableThreads, 8) k_slots(uint32_t n, uint4 *v
         });
 }
 
+template <int TILE>
+__global__ void __launch_bounds__(kTableThreads, 8) k_slots(uint32_t n, uint4 *vert, uint32_t *acc, uint64_t *sq,
+                                                           u128 *gam2) {
+    scan_lists<TILE>(whole_grid(), n, vert, acc, sq, gam2);
+}
+
 // lists longer than kLongList: a block per list scans NT x 4 entries a round
 // (each thread 4 consecutive ones, then a block scan of the thread sums)
-__global__ void __launch_bounds__(kLongThreads) k_slots_long(uint32_t n, uint4 *vert, uint32_t *acc, uint64_t *sq,
-                                                            u128 *gam2) {
+__device__ __forceinline__ void scan_long_lists(GridPart grid, uint32_t n, uint4 *vert, uint32_t *acc, uint64_t *sq,
+                                                u128 *gam2) {
     __shared__ uint64_t s_w[kLongThreads / kWarp], s_q[kLongThreads / kWarp];
-    for_each_vertex<kLongThreads>(n, vert, [](uint4 vr) { return vr.y > kLongList; }, [&](uint32_t v) {
+    for_each_vertex<kLongThreads>(grid, n, vert, [](uint4 vr) { return vr.y > kLongList; }, [&](uint32_t v) {
         const uint4 vr = vert[v];
         const uint32_t o = vr.x, d = vr.y;
         uint64_t run = 0, qsum = 0;
@@ -231,6 +237,26 @@ __global__ void __launch_bounds__(kLongThreads) k_slots_long(uint32_t n, uint4 *
     });
 }
 
+__global__ void __launch_bounds__(kLongThreads) k_slots_long(uint32_t n, uint4 *vert, uint32_t *acc, uint64_t *sq,
+                                                            u128 *gam2) {
+    scan_long_lists(whole_grid(), n, vert, acc, sq, gam2);
+}
+
+// lane 0 receives the warp's totals
+__device__ __forceinline__ void warp_sum_totals(Totals &t) {
+#pragma unroll
+    for (int k = 16; k > 0; k >>= 1) {
+        Totals o;
+        o.g0 = shfl_down_u128(t.g0, k);
+        o.g1 = shfl_down_u128(t.g1, k);
+        o.g2 = shfl_down_u128(t.g2, k);
+        o.l3 = shfl_down_u128(t.l3, k);
+        o.l4 = shfl_down_u128(t.l4, k);
+        o.dmax = __shfl_down_sync(0xffffffffu, t.dmax, k);
+        t.add(o);
+    }
+}
+
 // Gamma_v, Gamma^(1)_v, Gamma^(2)_v from d_v, S_v and Q_v (left in gam2 by
 // the list scans), one thread per vertex, and each block's share of the
 // exact totals (the 128-bit arithmetic of a vertex on one lane each, instead
@@ -244,17 +270,7 @@ __global__ void __launch_bounds__(kTableThreads) k_vertex_weights(uint32_t n, co
     }
     __shared__ Totals sh[kTableThreads / kWarp];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int k = 16; k > 0; k >>= 1) {
-        Totals o;
-        o.g0 = shfl_down_u128(t.g0, k);
-        o.g1 = shfl_down_u128(t.g1, k);
-        o.g2 = shfl_down_u128(t.g2, k);
-        o.l3 = shfl_down_u128(t.l3, k);
-        o.l4 = shfl_down_u128(t.l4, k);
-        o.dmax = __shfl_down_sync(0xffffffffu, t.dmax, k);
-        t.add(o);
-    }
+    warp_sum_totals(t);
     if (lane == 0) sh[warp] = t;
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -277,6 +293,16 @@ __device__ __forceinline__ void warp_totals(u128 (&s)[6]) {
     }
 }
 
+__device__ __forceinline__ void store_totals(DevTotals *tot, u128 g0, u128 g1, u128 g2, u128 l3, u128 l4, uint32_t dmax) {
+    tot->gamma[0] = g0;
+    tot->gamma[1] = g1;
+    tot->gamma[2] = g2;
+    tot->gamma[3] = 0;    // Gamma-check: set when the MOSS-4Min tables are built
+    tot->lambda3 = l3;
+    tot->lambda4 = l4;
+    tot->d_max = dmax;
+}
+
 __global__ void __launch_bounds__(kTotalsThreads) k_totals(const u128 *partials, int blocks, DevTotals *tot) {
     __shared__ u128 w_tot[kTotalsThreads / kWarp][6];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -293,15 +319,7 @@ __global__ void __launch_bounds__(kTotalsThreads) k_totals(const u128 *partials,
     if (warp != 0) return;
     for (int j = 0; j < 6; ++j) s[j] = w_tot[lane][j];   // kTotalsThreads / kWarp == 32 rows
     warp_totals(s);
-    if (lane == 0) {
-        tot->gamma[0] = s[0];
-        tot->gamma[1] = s[1];
-        tot->gamma[2] = s[2];
-        tot->gamma[3] = 0;    // Gamma-check: set when the MOSS-4Min tables are built
-        tot->lambda3 = s[3];
-        tot->lambda4 = s[4];
-        tot->d_max = (uint32_t)s[5];
-    }
+    if (lane == 0) store_totals(tot, s[0], s[1], s[2], s[3], s[4], (uint32_t)s[5]);
 }
 
 // --------------------------------------------------------------- twins ---
@@ -311,12 +329,14 @@ __global__ void __launch_bounds__(kTotalsThreads) k_totals(const u128 *partials,
 // twins: twin(v->x) = POS of v in N_x and twin(x->v) = POS of x in N_v.  For
 // a symmetric graph every edge is matched once, so the matched slots add up
 // to nnz; a reverse that is missing leaves the sum short.
-__global__ void k_twin(uint32_t n, uint64_t nnz, const uint4 *__restrict__ vert, const uint32_t *__restrict__ col,
-                       const uint32_t *__restrict__ owner, uint4 *slot, uint32_t *flags) {
+__device__ __forceinline__ void match_twins(GridPart grid, uint32_t n, uint64_t nnz, const uint4 *vert,
+                                            const uint32_t *__restrict__ col, const uint32_t *__restrict__ owner,
+                                            uint4 *slot, uint32_t *flags) {
     uint32_t matched = 0, err = 0;
-    for (uint64_t p = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; p < nnz; p += (uint64_t)gridDim.x * blockDim.x) {
+    for (uint64_t p = grid.block * (uint64_t)blockDim.x + threadIdx.x; p < nnz; p += (uint64_t)grid.blocks * blockDim.x) {
         const uint32_t v = owner[p], x = col[p];
-        if (x >= n || x == v) continue;  // flagged by the slot pass
+        // flagged by the slot pass; the owners of a row that was rejected are unset
+        if (x >= n || x == v || v >= n) continue;
         // {off, deg} only: k_slots may be writing S_v into the same records;
         // x's comes from words 2 and 3 of the slot record (k_slot_weights), a
         // streamed read instead of a random one
@@ -349,14 +369,20 @@ __global__ void k_twin(uint32_t n, uint64_t nnz, const uint4 *__restrict__ vert,
     if ((threadIdx.x & 31) == 0 && matched) atomicAdd(flags + 1, matched);
 }
 
+__global__ void k_twin(uint32_t n, uint64_t nnz, const uint4 *__restrict__ vert, const uint32_t *__restrict__ col,
+                       const uint32_t *__restrict__ owner, uint4 *slot, uint32_t *flags) {
+    match_twins(whole_grid(), n, nnz, vert, col, owner, slot, flags);
+}
+
 // ----------------------------------------------------- hashed edge set ---
 // One thread per slot inserts the edge {v, x} with v < x by compare-and-swap
 // into the first free slot from the home bucket on, slots of a bucket in
 // order.  The table has at least four slots per edge, so a free slot always
 // exists and the walk is bounded by the bucket count.
-__global__ void k_edge_hash(uint64_t nnz, const uint32_t *__restrict__ col, const uint32_t *__restrict__ owner,
-                            unsigned long long *table, uint32_t mask, uint32_t shift) {
-    for (uint64_t p = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; p < nnz; p += (uint64_t)gridDim.x * blockDim.x) {
+__device__ __forceinline__ void hash_edges(GridPart grid, uint64_t nnz, const uint32_t *__restrict__ col,
+                                           const uint32_t *__restrict__ owner, unsigned long long *table,
+                                           uint32_t mask, uint32_t shift) {
+    for (uint64_t p = grid.block * (uint64_t)blockDim.x + threadIdx.x; p < nnz; p += (uint64_t)grid.blocks * blockDim.x) {
         const uint32_t v = owner[p], x = col[p];
         if (x <= v) continue;
         const unsigned long long key = edge_key(v, x);
@@ -371,6 +397,11 @@ __global__ void k_edge_hash(uint64_t nnz, const uint32_t *__restrict__ col, cons
             b = (b + 1) & mask;
         }
     }
+}
+
+__global__ void k_edge_hash(uint64_t nnz, const uint32_t *__restrict__ col, const uint32_t *__restrict__ owner,
+                            unsigned long long *table, uint32_t mask, uint32_t shift) {
+    hash_edges(whole_grid(), nnz, col, owner, table, mask, shift);
 }
 
 // --------------------------------------------------------- edge filter ---
@@ -407,8 +438,8 @@ __device__ __forceinline__ uint32_t acc_weight(const uint32_t *acc, uint32_t o, 
 // of shared memory, so the searches and merges of pass 2 wait on shared rather
 // than global loads.
 template <int TILE>
-__global__ void __launch_bounds__(kTableThreads) k_sigma_alias(uint32_t n, const uint4 *__restrict__ vert,
-                                                              const uint32_t *__restrict__ acc, uint4 *slot) {
+__device__ __forceinline__ void sigma_lists(GridPart grid, uint32_t n, const uint4 *__restrict__ vert,
+                                            const uint32_t *__restrict__ acc, uint4 *slot) {
     __shared__ uint64_t s_pre[kTableThreads / kWarp][kLongList];
     __shared__ uint32_t s_idx[kTableThreads / kWarp][kLongList];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -532,7 +563,13 @@ __global__ void __launch_bounds__(kTableThreads) k_sigma_alias(uint32_t n, const
         }
         __syncwarp();
     };
-    for_lists<TILE>(n, vert, small, [](uint32_t, uint4) {}, large);
+    for_lists<TILE>(grid, n, vert, small, [](uint32_t, uint4) {}, large);
+}
+
+template <int TILE>
+__global__ void __launch_bounds__(kTableThreads) k_sigma_alias(uint32_t n, const uint4 *__restrict__ vert,
+                                                              const uint32_t *__restrict__ acc, uint4 *slot) {
+    sigma_lists<TILE>(whole_grid(), n, vert, acc, slot);
 }
 
 // lists longer than kLongList: a block per list (moss_alias.cuh), 256 threads
@@ -552,7 +589,7 @@ __global__ void __launch_bounds__(NT) k_sigma_alias_long(uint32_t n, const uint4
     extern __shared__ uint64_t s_split[];   // smem_list pre, then smem_list idx
     uint32_t *slot32 = reinterpret_cast<uint32_t *>(slot);
     for_each_vertex<NT, CH>(
-        n, vert, [](uint4 vr) { return vr.y > LO && vr.y <= HI && vr.z != 0; },
+        whole_grid(), n, vert, [](uint4 vr) { return vr.y > LO && vr.y <= HI && vr.z != 0; },
         [&](uint32_t v) {
             const uint4 vr = vert[v];
             const uint32_t o = vr.x, d = vr.y, S = vr.z;
@@ -569,10 +606,10 @@ __global__ void __launch_bounds__(NT) k_sigma_alias_long(uint32_t n, const uint4
 // One thread per slot of the lists above kShortList entries: words 5..7 of
 // each record from words 0, 1 and 4 of its alias position's record (written
 // before this launch, read only here).
-__global__ void k_slot_alias_fill(uint64_t nnz, const uint4 *__restrict__ vert, const uint32_t *__restrict__ owner,
-                                  uint4 *slot) {
+__device__ __forceinline__ void fill_slot_aliases(GridPart grid, uint64_t nnz, const uint4 *__restrict__ vert,
+                                                  const uint32_t *__restrict__ owner, uint4 *slot) {
     uint32_t *s32 = reinterpret_cast<uint32_t *>(slot);
-    for (uint64_t p = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; p < nnz; p += (uint64_t)gridDim.x * blockDim.x) {
+    for (uint64_t p = grid.block * (uint64_t)blockDim.x + threadIdx.x; p < nnz; p += (uint64_t)grid.blocks * blockDim.x) {
         const uint4 vr = vert[owner[p]];
         if (vr.y <= kShortList) continue;   // k_sigma_alias wrote the whole record
         const uint64_t a = (uint64_t)vr.x + s32[8 * p + 3];
@@ -580,6 +617,11 @@ __global__ void k_slot_alias_fill(uint64_t nnz, const uint4 *__restrict__ vert, 
         s32[8 * p + 5] = col;
         *reinterpret_cast<uint2 *>(s32 + 8 * p + 6) = make_uint2(nb, off);
     }
+}
+
+__global__ void k_slot_alias_fill(uint64_t nnz, const uint4 *__restrict__ vert, const uint32_t *__restrict__ owner,
+                                  uint4 *slot) {
+    fill_slot_aliases(whole_grid(), nnz, vert, owner, slot);
 }
 
 // ---------------------------------------------------- vertex (seed) tables ---
@@ -915,15 +957,14 @@ __global__ void __launch_bounds__(kSeedThreads) k_level_place(uint32_t n, const 
 // ---- the alias table of each level, in four phases (closed form of the sweep)
 // phase 1: per-chunk aggregates
 template <int ROUNDS>
-__global__ void __launch_bounds__(kSeedThreads) k_seed_count(uint32_t n, const DevTotals *tot, SeedTasks tasks,
-                                                            uint32_t *flags) {
-    const SeedTask &T = tasks.t[blockIdx.y];
+__device__ __forceinline__ void seed_count(uint32_t chunk, const SeedTask &T, uint32_t n, const DevTotals *tot,
+                                           uint32_t *flags) {
     const u128 W = task_total(T, tot);
     // one level: the overflow check of the table (w_v n must fit 128 bits) is here
-    if (flags && blockIdx.x == 0 && threadIdx.x == 0 && n > 1 && W > (~(u128)0) / n) atomicOr(flags, kErrOverflow);
+    if (flags && chunk == 0 && threadIdx.x == 0 && n > 1 && W > (~(u128)0) / n) atomicOr(flags, kErrOverflow);
     if (W == 0) return;
     const uint32_t m = task_items(T, tot, n), b0 = task_base(T, tot);
-    const uint64_t base = (uint64_t)blockIdx.x * (kSeedThreads * ROUNDS);
+    const uint64_t base = (uint64_t)chunk * (kSeedThreads * ROUNDS);
     // each thread's counts and deficit/excess sums, then one block sum
     uint32_t cl = 0, ch = 0;
     u128 sD = 0, sE = 0;
@@ -940,13 +981,17 @@ __global__ void __launch_bounds__(kSeedThreads) k_seed_count(uint32_t n, const D
     u128 xD, xE;
     SeedAgg t;
     block_scan_counts(cl, ch, sD, sE, xl, xh, xD, xE, t);
-    if (threadIdx.x == 0) T.agg[blockIdx.x] = t;
+    if (threadIdx.x == 0) T.agg[chunk] = t;
+}
+
+template <int ROUNDS>
+__global__ void __launch_bounds__(kSeedThreads) k_seed_count(uint32_t n, const DevTotals *tot, SeedTasks tasks,
+                                                            uint32_t *flags) {
+    seed_count<ROUNDS>(blockIdx.x, tasks.t[blockIdx.y], n, tot, flags);
 }
 
 // phase 2: exclusive scan of the chunk aggregates (one block per level)
-__global__ void __launch_bounds__(kSeedThreads) k_seed_offsets(uint32_t chunks, const DevTotals *tot,
-                                                              SeedTasks tasks) {
-    const SeedTask &T = tasks.t[blockIdx.x];
+__device__ __forceinline__ void seed_offsets(uint32_t chunks, const SeedTask &T, const DevTotals *tot) {
     if (T.level == 2 && threadIdx.x == 0) {   // one level: the record says so (no heavy vertex)
         SeedLevel &L = const_cast<DevTotals *>(tot)->level[T.which];
         L.nh = 0;
@@ -1001,6 +1046,11 @@ __global__ void __launch_bounds__(kSeedThreads) k_seed_offsets(uint32_t chunks, 
         T.split->nh = run.nh;
         T.split->total = run.E;
     }
+}
+
+__global__ void __launch_bounds__(kSeedThreads) k_seed_offsets(uint32_t chunks, const DevTotals *tot,
+                                                              SeedTasks tasks) {
+    seed_offsets(chunks, tasks.t[blockIdx.x], tot);
 }
 
 // phase 3: place every item at its split position with its prefix
@@ -1106,6 +1156,112 @@ __global__ void k_seed_fill(uint32_t n, const DevTotals *tot, SeedTasks tasks) {
         T.seed[2 * (uint64_t)(b0 + j)] = make_uint4((uint32_t)Tq, (uint32_t)(Tq >> 32), av, sv);
         T.seed[2 * (uint64_t)(b0 + j) + 1] = T.vrec[av];
     }
+}
+
+// ------------------------------------------------------------ small graphs --
+// A graph of a few thousand vertices is loaded and built in a handful of
+// microseconds of work; what it costs is launches, and events where passes run
+// side by side on several streams.  Below kSmallVertices and kSmallSlots the
+// passes that do not depend on each other share a launch instead, each with a
+// run of its blocks: load in four launches instead of eight and two forks,
+// build in four instead of eight, a memset and a fork (5,003 vertices and 20,000
+// edges, host clock: load 75 -> 57 us, build 75 -> 57 us against the separate
+// launches).  Larger graphs keep the separate ones: their passes fill the chip
+// one by one.
+constexpr uint32_t kSmallVertices = 1u << 14;   // exclusive: also where vertex tables have one level
+constexpr uint64_t kSmallSlots = 1ull << 18;
+
+// rows: vertex records (checked as k_vertices does), owners, and the lists
+// from src when they are not in place yet
+template <typename IdxT>
+__global__ void __launch_bounds__(kTableThreads) k_small_rows(const IdxT *row_ptr, const uint32_t *src, uint32_t n,
+                                                             uint64_t nnz, uint4 *vert, uint32_t *owner,
+                                                             uint32_t *col, uint32_t *flags) {
+    const int lane = threadIdx.x & 31;
+    const uint32_t warps = gridDim.x * (kTableThreads / kWarp);
+    for (uint32_t v = blockIdx.x * (kTableThreads / kWarp) + (threadIdx.x >> 5); v < n; v += warps) {
+        uint64_t a = row_ptr[v], b = row_ptr[v + 1];
+        if (b < a || b > nnz || (v == 0 && a != 0) || (v + 1 == n && b != nnz)) {
+            if (lane == 0) atomicOr(flags, kErrRowPtr);
+            a = b = 0;
+        }
+        if (lane == 0) vert[v] = make_uint4((uint32_t)a, (uint32_t)(b - a), 0u, 0u);
+        for (uint64_t p = a + lane; p < b; p += kWarp) {
+            owner[p] = v;
+            if (src) col[p] = src[p];
+        }
+    }
+}
+
+// the list scans and the twin pass (which touches none of what they write)
+__global__ void __launch_bounds__(kTableThreads) k_small_scan(uint32_t n, uint64_t nnz, uint4 *vert,
+                                                             const uint32_t *__restrict__ col,
+                                                             const uint32_t *__restrict__ owner, uint4 *slot,
+                                                             uint32_t *acc, uint64_t *sq, u128 *gam2, uint32_t *flags,
+                                                             uint32_t scan_blocks, uint32_t long_blocks) {
+    const uint32_t b = blockIdx.x;
+    if (b < scan_blocks)
+        scan_lists<8>(GridPart{b, scan_blocks}, n, vert, acc, sq, gam2);
+    else if (b < scan_blocks + long_blocks)
+        scan_long_lists(GridPart{b - scan_blocks, long_blocks}, n, vert, acc, sq, gam2);
+    else
+        match_twins(GridPart{b - scan_blocks - long_blocks, gridDim.x - scan_blocks - long_blocks}, n, nnz, vert, col,
+                    owner, slot, flags);
+}
+
+// vertex weights and the exact totals, one block
+__global__ void __launch_bounds__(kTotalsThreads) k_small_totals(uint32_t n, const uint4 *__restrict__ vert, u128 *gam0,
+                                                                u128 *gam1, u128 *gam2, DevTotals *tot) {
+    Totals t = {};
+    for (uint32_t v = threadIdx.x; v < n; v += kTotalsThreads) {
+        const uint4 r = vert[v];
+        vertex_weights(v, r.y, r.z, (uint64_t)gam2[v], gam0, gam1, gam2, t);
+    }
+    __shared__ Totals sh[kTotalsThreads / kWarp];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    warp_sum_totals(t);
+    if (lane == 0) sh[warp] = t;
+    __syncthreads();
+    if (warp != 0) return;
+    t = sh[lane];   // kTotalsThreads / kWarp == 32 rows
+    warp_sum_totals(t);
+    if (lane == 0) store_totals(tot, t.g0, t.g1, t.g2, t.l3, t.l4, t.dmax);
+}
+
+// the vertex tables' chunk sums, the per-list tables and an empty edge set
+__global__ void __launch_bounds__(kSeedThreads) k_small_build(uint32_t n, const DevTotals *tot, SeedTasks tasks, int nt,
+                                                             uint32_t chunks, uint32_t *flags,
+                                                             const uint4 *__restrict__ vert,
+                                                             const uint32_t *__restrict__ acc, uint4 *slot,
+                                                             uint4 *hash, uint64_t hash_words, uint32_t list_blocks) {
+    const uint32_t b = blockIdx.x, counts = chunks * nt;
+    if (b < counts) {
+        seed_count<kSeedRoundsFew>(b % chunks, tasks.t[b / chunks], n, tot, flags);
+    } else if (b < counts + list_blocks) {
+        sigma_lists<8>(GridPart{b - counts, list_blocks}, n, vert, acc, slot);
+    } else {
+        const uint64_t first = (uint64_t)(b - counts - list_blocks) * kSeedThreads + threadIdx.x;
+        const uint64_t stride = (uint64_t)(gridDim.x - counts - list_blocks) * kSeedThreads;
+        for (uint64_t i = first; i < hash_words; i += stride)
+            hash[i] = make_uint4(0xffffffffu, 0xffffffffu, 0xffffffffu, 0xffffffffu);
+    }
+}
+
+// the scan of the chunk sums, the alias halves of the longer lists' records
+// and the edge set
+__global__ void __launch_bounds__(kSeedThreads) k_small_build2(uint64_t nnz, const DevTotals *tot, SeedTasks tasks,
+                                                              int nt, uint32_t chunks, const uint4 *__restrict__ vert,
+                                                              const uint32_t *__restrict__ col,
+                                                              const uint32_t *__restrict__ owner, uint4 *slot,
+                                                              unsigned long long *hash, uint32_t mask, uint32_t shift,
+                                                              uint32_t fill_blocks) {
+    const uint32_t b = blockIdx.x;
+    if (b < (uint32_t)nt)
+        seed_offsets(chunks, tasks.t[b], tot);
+    else if (b < nt + fill_blocks)
+        fill_slot_aliases(GridPart{b - nt, fill_blocks}, nnz, vert, owner, slot);
+    else
+        hash_edges(GridPart{b - nt - fill_blocks, gridDim.x - nt - fill_blocks}, nnz, col, owner, hash, mask, shift);
 }
 
 // ---- hub adjacency (behind the edge filter)
@@ -1408,15 +1564,12 @@ cudaError_t launch_hub_tables(uint32_t n, const uint4 *vert, const uint32_t *col
     return cudaSuccess;
 }
 
-cudaError_t launch_sigma_alias(uint32_t n, uint64_t nnz, uint32_t d_max, const uint4 *vert, const uint32_t *acc,
-                               const uint32_t *owner, uint4 *slot, uint32_t *scratch_idx, uint64_t *scratch_pre,
-                               cudaStream_t s, const AuxStreams *aux, int long_stream) {
-    // the short and the long lists are built side by side (long lists on
-    // aux->a[long_stream], forked from s by the caller); the fill waits for both
+// the tables of lists above kLongList entries
+static cudaError_t launch_long_sigma(uint32_t n, uint32_t d_max, const uint4 *vert, const uint32_t *acc, uint4 *slot,
+                                     uint32_t *scratch_idx, uint64_t *scratch_pre, cudaStream_t s) {
+    if (d_max <= kLongList) return cudaSuccess;
     const auto mid = k_sigma_alias_long<kLongThreads, kSigmaChunk, kLongList, kHubList>;
     const auto hub = k_sigma_alias_long<kHubThreads, kHubThreads, kHubList, 0xffffffffu>;
-    const size_t mid_bytes = (size_t)kHubList * kSplitBytes;
-    const uint32_t hub_list = std::min(d_max, kHubSmemList);
     static std::atomic<bool> attr_set[64];
     int dev = 0;
     cudaGetDevice(&dev);
@@ -1426,22 +1579,27 @@ cudaError_t launch_sigma_alias(uint32_t n, uint64_t nnz, uint32_t d_max, const u
         if (e != cudaSuccess) return e;
         if (dev >= 0 && dev < 64) attr_set[dev].store(true, std::memory_order_relaxed);
     }
-    cudaStream_t ls = aux ? aux->a[long_stream] : s;
-    cudaError_t el = cudaSuccess;
-    if (d_max > kHubList) {
-        hub<<<hub_blocks(n), kHubThreads, hub_list * kSplitBytes, ls>>>(n, vert, acc, slot, scratch_idx, scratch_pre,
-                                                                        hub_list);
-        el = cudaGetLastError();
+    if (d_max > kHubList) {   // first: the longest lists set the end of the pass
+        const uint32_t list = std::min(d_max, kHubSmemList);
+        hub<<<hub_blocks(n), kHubThreads, list * kSplitBytes, s>>>(n, vert, acc, slot, scratch_idx, scratch_pre, list);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
-    if (d_max > kLongList && el == cudaSuccess) {
-        const unsigned chunks = (unsigned)(((uint64_t)n + kSigmaChunk - 1) / kSigmaChunk);
-        mid<<<chunks, kLongThreads, mid_bytes, ls>>>(n, vert, acc, slot, scratch_idx, scratch_pre, kHubList);
-        el = cudaGetLastError();
-    }
+    const unsigned chunks = (unsigned)(((uint64_t)n + kSigmaChunk - 1) / kSigmaChunk);
+    mid<<<chunks, kLongThreads, kHubList * kSplitBytes, s>>>(n, vert, acc, slot, scratch_idx, scratch_pre, kHubList);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_sigma_alias(uint32_t n, uint64_t nnz, uint32_t d_max, const uint4 *vert, const uint32_t *acc,
+                               const uint32_t *owner, uint4 *slot, uint32_t *scratch_idx, uint64_t *scratch_pre,
+                               cudaStream_t s, const AuxStreams *aux, int long_stream) {
+    // the short and the long lists are built side by side (long lists on
+    // aux->a[long_stream], forked from s by the caller); the fill waits for both
+    cudaError_t el = launch_long_sigma(n, d_max, vert, acc, slot, scratch_idx, scratch_pre,
+                                       aux ? aux->a[long_stream] : s);
     with_tile(n, [&](auto T) {
         k_sigma_alias<decltype(T)::value><<<tile_blocks(n, decltype(T)::value, kTableThreads, current_sms(), 8), kTableThreads, 0, s>>>(n, vert, acc, slot);
     });
-    e = cudaGetLastError();
+    const cudaError_t e = cudaGetLastError();
     if (aux && d_max > kLongList) {
         const cudaError_t ew = aux->wait_for(s, long_stream);
         if (el == cudaSuccess) el = ew;
@@ -1469,6 +1627,32 @@ uint64_t seed_scratch_bytes(uint32_t n) {
     return 3 * (table + 2 * level);
 }
 
+bool small_graph(uint32_t n, uint64_t nnz) { return n < kSmallVertices && nnz <= kSmallSlots; }
+
+cudaError_t launch_small_load(const void *row_ptr, int is64, const uint32_t *src, uint32_t n, uint64_t nnz, uint4 *vert,
+                              uint32_t *col, uint4 *slot, uint32_t *acc, uint32_t *owner, uint64_t *sq, u128 *gam0,
+                              u128 *gam1, u128 *gam2, DevTotals *tot, uint32_t *flags, cudaStream_t s) {
+    const unsigned rows = (n + kTableThreads / kWarp - 1) / (kTableThreads / kWarp);
+    if (is64)
+        k_small_rows<uint64_t><<<rows, kTableThreads, 0, s>>>(static_cast<const uint64_t *>(row_ptr), src, n, nnz, vert,
+                                                              owner, col, flags);
+    else
+        k_small_rows<uint32_t><<<rows, kTableThreads, 0, s>>>(static_cast<const uint32_t *>(row_ptr), src, n, nnz, vert,
+                                                              owner, col, flags);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    if (nnz) {
+        k_slot_weights<<<flat_blocks(nnz), 256, 0, s>>>(n, nnz, col, vert, owner, slot, acc, flags);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
+    const unsigned scans = tile_blocks(n, 8, kTableThreads, current_sms(), 8), longs = long_blocks(n);
+    k_small_scan<<<scans + longs + (nnz ? flat_blocks(nnz) : 0), kTableThreads, 0, s>>>(
+        n, nnz, vert, col, owner, slot, acc, sq, gam2, flags, scans, longs);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    k_small_totals<<<1, kTotalsThreads, 0, s>>>(n, vert, gam0, gam1, gam2, tot);
+    return cudaGetLastError();
+}
+
 // the level split (two levels) and the first three phases of the tables
 template <int ROUNDS>
 static cudaError_t launch_seed_split(uint32_t n, uint32_t chunks, DevTotals *tot, const LevelTasks &lt,
@@ -1491,14 +1675,9 @@ static cudaError_t launch_seed_split(uint32_t n, uint32_t chunks, DevTotals *tot
     return cudaGetLastError();
 }
 
-cudaError_t launch_seed_alias(uint32_t n, DevTotals *tot, int ntables, const int *which, u128 *const *w,
-                              uint4 *const *seed, const uint4 *const *vrec, void *scratch, uint32_t *flags, int split,
-                              cudaStream_t s) {
-    if (ntables < 1 || ntables > 3 || split < 0 || split > 64) return cudaErrorInvalidValue;
-    const bool one_level = split == 64;   // one table over all vertices, in id order
-    const uint32_t chunks = seed_chunks(n);
-    LevelTasks lt = {};
-    SeedTasks tasks = {};
+// the level and alias tasks of the tables, their scratch carved from `scratch`
+static void seed_tasks(uint32_t n, uint32_t chunks, bool one_level, int ntables, const int *which, u128 *const *w,
+                       uint4 *const *seed, const uint4 *const *vrec, void *scratch, LevelTasks &lt, SeedTasks &tasks) {
     uint8_t *p = static_cast<uint8_t *>(scratch);
     auto take = [&](uint64_t bytes) {
         uint8_t *r = p;
@@ -1526,17 +1705,64 @@ cudaError_t launch_seed_alias(uint32_t n, DevTotals *tot, int ntables, const int
             T.agg = reinterpret_cast<SeedAgg *>(take((uint64_t)chunks * sizeof(SeedAgg)));
         }
     }
-    const int nt = per * ntables;
-    const bool few = seed_rounds(n) == kSeedRoundsFew;
-    const cudaError_t e = few ? launch_seed_split<kSeedRoundsFew>(n, chunks, tot, lt, tasks, ntables, nt, one_level, flags, split, s)
-                              : launch_seed_split<kSeedRoundsMost>(n, chunks, tot, lt, tasks, ntables, nt, one_level, flags, split, s);
-    if (e != cudaSuccess) return e;
+}
+
+static cudaError_t launch_seed_fill(uint32_t n, const DevTotals *tot, const SeedTasks &tasks, int nt, cudaStream_t s) {
     const int threads = 256;
     uint64_t blocks = ((uint64_t)n + threads - 1) / threads;
     if (blocks > 4096) blocks = 4096;
     if (blocks < 1) blocks = 1;
     k_seed_fill<<<dim3((unsigned)blocks, nt), threads, 0, s>>>(n, tot, tasks);
     return cudaGetLastError();
+}
+
+cudaError_t launch_seed_alias(uint32_t n, DevTotals *tot, int ntables, const int *which, u128 *const *w,
+                              uint4 *const *seed, const uint4 *const *vrec, void *scratch, uint32_t *flags, int split,
+                              cudaStream_t s) {
+    if (ntables < 1 || ntables > 3 || split < 0 || split > 64) return cudaErrorInvalidValue;
+    const bool one_level = split == 64;   // one table over all vertices, in id order
+    const uint32_t chunks = seed_chunks(n);
+    LevelTasks lt = {};
+    SeedTasks tasks = {};
+    seed_tasks(n, chunks, one_level, ntables, which, w, seed, vrec, scratch, lt, tasks);
+    const int nt = (one_level ? 1 : 2) * ntables;
+    const bool few = seed_rounds(n) == kSeedRoundsFew;
+    const cudaError_t e = few ? launch_seed_split<kSeedRoundsFew>(n, chunks, tot, lt, tasks, ntables, nt, one_level, flags, split, s)
+                              : launch_seed_split<kSeedRoundsMost>(n, chunks, tot, lt, tasks, ntables, nt, one_level, flags, split, s);
+    if (e != cudaSuccess) return e;
+    return launch_seed_fill(n, tot, tasks, nt, s);
+}
+
+cudaError_t launch_small_build(uint32_t n, uint64_t nnz, uint32_t d_max, DevTotals *tot, int ntables, const int *which,
+                               u128 *const *w, uint4 *const *seed, const uint4 *const *vrec, void *seed_scratch,
+                               uint32_t *flags, const uint4 *vert, const uint32_t *acc, const uint32_t *col,
+                               const uint32_t *owner, uint4 *slot, uint32_t *scratch_idx, uint64_t *scratch_pre,
+                               unsigned long long *hash, uint64_t hash_buckets, cudaStream_t s) {
+    const uint32_t chunks = seed_chunks(n);
+    LevelTasks lt = {};
+    SeedTasks tasks = {};
+    seed_tasks(n, chunks, true, ntables, which, w, seed, vrec, seed_scratch, lt, tasks);
+    const uint64_t words = hash ? hash_buckets * kBucketKeys / 2 : 0;   // 16 bytes each
+    const unsigned lists = tile_blocks(n, 8, kTableThreads, current_sms(), 8);
+    const unsigned clears = words ? flat_blocks((words + 3) / 4) : 0;
+    k_small_build<<<chunks * ntables + lists + clears, kSeedThreads, 0, s>>>(
+        n, tot, tasks, ntables, chunks, flags, vert, acc, slot, reinterpret_cast<uint4 *>(hash), words, lists);
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess) e = launch_long_sigma(n, d_max, vert, acc, slot, scratch_idx, scratch_pre, s);
+    if (e != cudaSuccess) return e;
+    const unsigned fills = d_max > kShortList ? flat_blocks(nnz) : 0, inserts = hash && nnz ? flat_blocks(nnz) : 0;
+    uint32_t lg = 0;
+    while ((1ULL << lg) < hash_buckets) ++lg;
+    if (ntables + fills + inserts) {
+        k_small_build2<<<ntables + fills + inserts, kSeedThreads, 0, s>>>(nnz, tot, tasks, ntables, chunks, vert, col, owner,
+                                                                          slot, hash, (uint32_t)(hash_buckets - 1),
+                                                                          64 - lg, fills);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
+    if (ntables == 0) return cudaSuccess;
+    k_seed_place<kSeedRoundsFew><<<dim3(chunks, ntables), kSeedThreads, 0, s>>>(n, tot, tasks);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    return launch_seed_fill(n, tot, tasks, ntables, s);
 }
 
 }  // namespace moss
