@@ -325,7 +325,8 @@ int moss_batch_add_min(moss_batch *b, moss_graph *g, uint64_t budget, uint64_t b
                        int *index);
 int moss_batch_size(const moss_batch *b);
 int moss_batch_clear(moss_batch *b);
-/* Samples per tile (32 .. 2^30; default 8192). */
+/* Samples per tile (32 .. 2^30; default 8192): the most a warp takes at a time.
+ * A run whose tiles would not keep every warp busy to the end cuts them finer. */
 int moss_batch_set_tile(moss_batch *b, uint32_t tile_samples);
 uint32_t moss_batch_tile(const moss_batch *b);
 /* Run every request: results[i] (caller-owned host array of moss_batch_size

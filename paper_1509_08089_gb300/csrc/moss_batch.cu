@@ -60,6 +60,7 @@ struct moss_batch {
     cudaEvent_t ready = nullptr;
     std::vector<Req> reqs;
     uint32_t tile = 8192;
+    uint32_t unit = 8192;              // samples per piece of the current plan (batch_unit)
     int threads = 256;                 // threads per block of the persistent launch
     int per_sm = 0;                    // resident blocks per SM (0: as many as fit)
     int rngs = kBatchSplitMix;         // generators of the planned graphs (kBatch*)
@@ -105,7 +106,7 @@ int plan(moss_batch *b) {
     std::vector<const moss_graph *> gkeys;
     std::vector<BatchTask> tasks;
     std::vector<BatchRequest> reqs(nreq);
-    uint64_t tile0 = 0;
+    uint64_t samples = 0;
     for (int r = 0; r < nreq; ++r) {
         const Req &q = b->reqs[r];
         GraphInfo gi;
@@ -155,16 +156,22 @@ int plan(moss_batch *b) {
             t.seed = q.seed;
             t.first = 0;
             t.count = Ks[j];
-            t.tile0 = tile0;
             t.graph = (uint32_t)gidx;
             t.method = (uint32_t)m;
             br.task[j] = (int)tasks.size();
             tasks.push_back(t);
-            tile0 += (Ks[j] + b->tile - 1) / b->tile;
+            samples += Ks[j];
         }
     }
     b->ntasks = (int)tasks.size();
-    b->ntiles = tile0;
+    b->rngs = batch_rngs(graphs.data(), graphs.size());
+    b->blocks = batch_blocks(b->device, b->threads, b->per_sm, b->rngs);
+    b->unit = batch_unit(samples, b->tile, (uint64_t)b->blocks * b->threads / 32);
+    b->ntiles = 0;
+    for (BatchTask &t : tasks) {
+        t.tile0 = b->ntiles;
+        b->ntiles += (t.count + b->unit - 1) / b->unit;
+    }
     b->plan_tasks = tasks;
     b->plan_graphs = gkeys;
     cudaError_t e = cudaSuccess;
@@ -194,8 +201,6 @@ int plan(moss_batch *b) {
     // the host vectors die at return: wait for the copies
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return set_error(MOSS_ECUDA, "uploading the batch plan");
-    b->rngs = batch_rngs(graphs.data(), graphs.size());
-    b->blocks = batch_blocks(b->device, b->threads, b->per_sm, b->rngs);
     return MOSS_OK;
 }
 
@@ -205,9 +210,9 @@ cudaError_t enqueue(moss_batch *b) {
     const int nreq = (int)b->reqs.size();
     cudaError_t e = cudaMemsetAsync(b->d_next, 0, sizeof(unsigned long long), s);
     if (e == cudaSuccess)
-        e = launch_sample_batch(b->d_graphs, b->d_tasks, b->ntasks, b->ntiles, b->tile, b->d_next, b->d_tiles,
+        e = launch_sample_batch(b->d_graphs, b->d_tasks, b->ntasks, b->ntiles, b->unit, b->d_next, b->d_tiles,
                                 b->threads, b->blocks, b->record ? b->d_cycles : nullptr, b->rngs, s);
-    if (e == cudaSuccess) e = launch_batch_reduce(b->d_tasks, b->ntasks, b->tile, b->d_tiles, b->d_task_counts, s);
+    if (e == cudaSuccess) e = launch_batch_reduce(b->d_tasks, b->ntasks, b->unit, b->d_tiles, b->d_task_counts, s);
     if (e == cudaSuccess) e = launch_finalize_batch(b->d_reqs, nreq, b->d_task_counts, b->d_results, s);
     if (e == cudaSuccess && nreq)
         e = cudaMemcpyAsync(b->h_results, b->d_results, nreq * sizeof(moss_result), cudaMemcpyDeviceToHost, s);
@@ -431,7 +436,7 @@ int moss_batch_tune(moss_batch *b, void *stream, uint32_t *chosen) {
         for (const BatchTask &t : b->plan_tasks) {
             const moss_graph *g = b->plan_graphs[t.graph];
             const size_t gi = (size_t)(std::find(gs.begin(), gs.end(), g) - gs.begin());
-            const uint64_t nt = (t.count + b->tile - 1) / b->tile;
+            const uint64_t nt = (t.count + b->unit - 1) / b->unit;
             for (uint64_t j = 0; j < nt; ++j) c[gi] += (double)cyc[t.tile0 + j];
             n[gi] += (double)t.count;
         }

@@ -481,6 +481,17 @@ constexpr int kBatchSplitMix = 0, kBatchPhilox = 1, kBatchBoth = 2;
 cudaError_t launch_sample_batch(const DevGraph *graphs, const BatchTask *tasks, int ntasks, uint64_t ntiles,
                                 uint32_t tile_samples, unsigned long long *next_tile, uint32_t *tile_counts,
                                 int threads, int blocks, unsigned long long *tile_cycles, int rngs, cudaStream_t s);
+// Samples a warp takes at a time, at most the caller's tile: tasks differ in
+// cost per sample, so a launch ends evenly when every warp takes many pieces.
+// 64 pieces per warp of `warps`, at least 256 samples (8 rounds of a warp, so
+// that the counter's atomic and a row of counts stay a few percent).  256
+// graphs, 3.2e8 samples, pieces of 8,192 / 4,096 / 2,048 / 1,024 / 512 samples:
+// 13.3 / 11.5 / 11.0 / 10.7 / 10.7 ms.
+inline uint32_t batch_unit(uint64_t samples, uint32_t tile, uint64_t warps) {
+    const uint64_t even = samples / (warps * 64) / 32 * 32;
+    const uint64_t unit = even < 256 ? 256 : even;
+    return unit < tile ? (uint32_t)unit : tile;
+}
 // the batch generator mode of a set of graph views
 inline int batch_rngs(const DevGraph *views, size_t n) {
     bool sm = false, ph = false;

@@ -87,6 +87,7 @@ struct TickBuffers {
     BatchTask *d_tasks = nullptr;
     size_t cap_tasks = 0;
     uint32_t *d_tiles = nullptr;
+    uint32_t unit = 0;             // samples per piece of the planned tick (batch_unit)
     size_t cap_tiles = 0;
     uint64_t *d_task_counts = nullptr;
     size_t cap_tc = 0;
@@ -268,10 +269,10 @@ int enqueue_tick(moss_server *s, TickBuffers &tb, uint64_t ntiles) {
         e = cudaMemcpyAsync(tb.d_tasks, tb.tasks.data(), nt * sizeof(BatchTask), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(tb.d_next, 0, sizeof(unsigned long long), st);
     if (e == cudaSuccess)
-        e = launch_sample_batch(s->d_graphs, tb.d_tasks, (int)nt, ntiles, s->cfg.tile_samples, tb.d_next, tb.d_tiles,
+        e = launch_sample_batch(s->d_graphs, tb.d_tasks, (int)nt, ntiles, tb.unit, tb.d_next, tb.d_tiles,
                                 256, s->blocks, nullptr, s->rngs, st);
     if (e == cudaSuccess)
-        e = launch_batch_reduce(tb.d_tasks, (int)nt, s->cfg.tile_samples, tb.d_tiles, tb.d_task_counts, st);
+        e = launch_batch_reduce(tb.d_tasks, (int)nt, tb.unit, tb.d_tiles, tb.d_task_counts, st);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(tb.h_task_counts, tb.d_task_counts, nt * kSlots * sizeof(uint64_t),
                             cudaMemcpyDeviceToHost, st);
@@ -333,7 +334,7 @@ void admit(moss_server *s, double t) {
 uint64_t plan_tick(moss_server *s, TickBuffers &tb) {
     tb.tasks.clear();
     tb.owner.clear();
-    uint64_t ntiles = 0;
+    uint64_t ntiles = 0, samples = 0;
     const uint64_t tile = s->cfg.tile_samples;
     size_t open = 0;   // requests with ids left to schedule
     for (uint64_t id : s->active) {
@@ -356,16 +357,20 @@ uint64_t plan_tick(moss_server *s, TickBuffers &tb) {
             t.seed = q.seed;
             t.first = q.next[j];
             t.count = c;
-            t.tile0 = ntiles;
             t.graph = (uint32_t)q.graph;
             t.method = (uint32_t)m[j];
             tb.tasks.push_back(t);
             tb.owner.push_back({id, j});
-            ntiles += (c + tile - 1) / tile;
+            samples += c;
             q.next[j] += c;
             any = true;
         }
         if (any) ++q.ticks;
+    }
+    tb.unit = batch_unit(samples, s->cfg.tile_samples, (uint64_t)s->blocks * 256 / 32);
+    for (BatchTask &t : tb.tasks) {
+        t.tile0 = ntiles;
+        ntiles += (t.count + tb.unit - 1) / tb.unit;
     }
     return ntiles;
 }
