@@ -386,10 +386,15 @@ def moss_batch_tile(b: int) -> int:
     return load().moss_batch_tile(b)
 
 
-def moss_batch_run(b: int, stream=None) -> list:
-    n = load().moss_batch_size(b)
+def _batch_run(b: int, n: int, stream=None):
     arr = (moss_result * max(n, 1))()
     _check(load().moss_batch_run(b, _stream(stream), arr))
+    return arr
+
+
+def moss_batch_run(b: int, stream=None) -> list:
+    n = load().moss_batch_size(b)
+    arr = _batch_run(b, n, stream)
     return [arr[i] for i in range(n)]
 
 
@@ -535,6 +540,28 @@ class Server:
 
 
 # ------------------------------------------------------------ convenience --
+# moss_result as 8-byte words: where its arrays start
+_AT = {f: getattr(moss_result, f).offset // 8 for f, _ in moss_result._fields_[2:]}
+_WORDS = ctypes.sizeof(moss_result) // 8
+
+
+def result_dicts(results) -> list[dict]:
+    """result_dict of every result of a ctypes array: one copy of the memory,
+    the arrays views of it (256 results 0.3 ms, result_dict of each 1.6 ms)."""
+    own = bytearray(results)
+    f8 = np.frombuffer(own, dtype=np.float64).reshape(-1, _WORDS)
+    u8 = np.frombuffer(own, dtype=np.uint64).reshape(-1, _WORDS)
+    i4 = np.frombuffer(own, dtype=np.int32).reshape(-1, 2 * _WORDS)
+    at, n = _AT, NSLOTS
+    ks, Ks = i4[:, 0].tolist(), u8[:, at["K"]:at["K"] + 2].tolist()
+    tris = f8[:, at["triangles"]:at["triangles"] + 2].tolist()
+    hits = u8[:, at["hits"]:at["hits"] + 2 * n].reshape(-1, 2, n)
+    lam = f8[:, at["lambda_"]:at["lambda_"] + 2 * n].reshape(-1, 2, n)
+    est, var, conc = (f8[:, at[k]:at[k] + n] for k in ("est", "var", "conc"))
+    return [{"k": ks[i], "K": tuple(Ks[i]), "hits": hits[i], "est": est[i], "var": var[i], "lam": lam[i],
+             "triangles": tris[i][0], "triangles_var": tris[i][1], "conc": conc[i]} for i in range(len(ks))]
+
+
 def result_dict(r: moss_result) -> dict:
     """moss_result as plain Python/numpy values."""
     view = np.ctypeslib.as_array
@@ -558,7 +585,8 @@ class Batch:
         return moss_batch_add_min(self.handle, graph.handle, budget, budget_min, seed)
 
     def run(self, stream=None) -> list[dict]:
-        return [result_dict(r) for r in moss_batch_run(self.handle, stream)]
+        n = len(self)
+        return result_dicts(_batch_run(self.handle, n, stream))[:n]
 
     def tune(self, stream=None) -> int:
         return moss_batch_tune(self.handle, stream)
