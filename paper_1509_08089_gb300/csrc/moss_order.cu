@@ -33,8 +33,8 @@
 //   k_order_lists   in internal order, so the renumbered lists are written
 //                   in order (written scattered by list, in input order, the
 //                   pass took 2.35 ms against 1.93 on the 34M-edge graph):
-//                   the lists of degree 32 or more a warp each: up to 128
-//                   entries ranked in registers (four a lane, one pass),
+//                   the lists of degree 1,024 or more a block each, of 32
+//                   or more a warp each: up to 128 entries ranked in registers (four a lane, one pass),
 //                   longer lists by a count over the 128 key slots and a
 //                   placing pass in input order; the rest by tiles of 32,
 //                   G lanes per list (G a power of two <= 32, the tile's
@@ -367,14 +367,94 @@ __device__ __forceinline__ void list_on_warp(uint32_t d, uint64_t a, uint64_t o,
     __syncwarp();
 }
 
-// The internal vertices below *nlong (key >= 20: degree 32 or more, the
-// front of the order) take a warp each, grid-stride, so the hubs spread
-// over the warps.  The rest go by tiles of 32 consecutive internal vertices
+// One long renumbered list on the whole block: each warp counts the keys of
+// its share of the input entries (h: a row of 128 counters per warp), the
+// rows become the warps' first places by key and warp, and each warp places
+// its share in input order.
+__device__ __forceinline__ void list_on_block(uint32_t d, uint64_t a, uint64_t o, uint32_t n, uint64_t nnz,
+                                              const uint32_t *__restrict__ col_in, const uint32_t *__restrict__ inv,
+                                              const uint8_t *__restrict__ slot_of, uint32_t *col_out,
+                                              uint32_t (&s_h)[kOrderWarps][kOrderKeys], uint32_t &err) {
+    static_assert(kOrderKeys == 128 && kOrderThreads >= kOrderKeys, "a thread per key in the scan");
+    __shared__ uint32_t s_sum[kOrderKeys / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t below = (1u << lane) - 1u;
+    uint32_t *h = s_h[warp];
+    const uint32_t share = (d + kOrderWarps * 32 - 1) / (kOrderWarps * 32) * 32;
+    const uint32_t b0 = min(d, (uint32_t)warp * share), b1 = min(d, b0 + share);
+    for (int k = lane; k < kOrderKeys; k += 32) h[k] = 0;
+    __syncwarp();
+    uint32_t last = b0 > 0 && b0 < d ? col_in[a + b0 - 1] : 0u;   // the entry before this round's first
+#pragma unroll 4
+    for (uint32_t base = b0; base < b1; base += 32) {
+        const uint32_t idx = base + lane;
+        uint32_t u = 0;
+        if (idx < b1) {
+            u = col_in[a + idx];
+            if (u < n)
+                atomicAdd(&h[slot_of[u]], 1u);
+            else
+                err |= kErrRange;
+        }
+        const uint32_t up = __shfl_up_sync(kFull, u, 1);
+        const uint32_t prev = lane ? up : last;
+        if (idx < b1 && idx > 0 && prev >= u) err |= kErrOrder;
+        last = __shfl_sync(kFull, u, 31);
+    }
+    __syncthreads();
+    if (threadIdx.x < kOrderKeys) {   // exclusive prefix over (key, warp), a thread per key
+        uint32_t sum = 0;
+        for (int w = 0; w < kOrderWarps; ++w) sum += s_h[w][threadIdx.x];
+        uint32_t incl = sum;
+#pragma unroll
+        for (int dd = 1; dd < 32; dd <<= 1) {
+            const uint32_t t = __shfl_up_sync(kFull, incl, dd);
+            if (lane >= dd) incl += t;
+        }
+        if (lane == 31) s_sum[warp] = incl;
+        asm volatile("bar.sync 1, 128;" ::: "memory");   // the four warps of the scan
+        uint32_t at = incl - sum;
+        for (int w = 0; w < warp; ++w) at += s_sum[w];
+        for (int w = 0; w < kOrderWarps; ++w) {
+            const uint32_t c = s_h[w][threadIdx.x];
+            s_h[w][threadIdx.x] = at;
+            at += c;
+        }
+    }
+    __syncthreads();
+#pragma unroll 2
+    for (uint32_t base = b0; base < b1; base += 32) {
+        const uint32_t idx = base + lane;
+        uint32_t sl = (uint32_t)kOrderKeys + lane, x = 0;
+        if (idx < b1) {
+            const uint32_t u = col_in[a + idx];
+            if (u < n) {
+                sl = slot_of[u];
+                x = inv[u];
+            }
+        }
+        const bool live = sl < (uint32_t)kOrderKeys;
+        const uint32_t m = __match_any_sync(kFull, sl);
+        const uint32_t pos = live ? h[sl] + __popc(m & below) : 0u;
+        __syncwarp();
+        if (live && (m & below) == 0) h[sl] += __popc(m);
+        __syncwarp();
+        if (live && o + pos < nnz) col_out[o + pos] = x;
+    }
+    __syncthreads();   // the counters are reused by the block's next list
+}
+
+// The internal vertices below *nhub (key >= 40: degree 1,024 or more, the
+// front of the order) take a block each, those below *nlong (key >= 20: degree
+// 32 or more) a warp each, grid-stride, so they spread.  A hub on one warp was
+// the whole pass: two passes of 470 dependent rounds for 15,000 entries.
+// The rest go by tiles of 32 consecutive internal vertices
 // (their lists are written one after another): when none of a tile's lists
 // is longer than G (a power of two <= 32), each group of G lanes takes one
 // list, 32 / G lists a round; otherwise (not met: the tail's keys are below
 // 20) the warp takes the lists one by one.
 constexpr int kLongKeySlot = kOrderKeys - 1 - 19;   // first slot of the keys below 20
+constexpr int kHubKeySlot = kOrderKeys - 1 - 39;    // first slot of the keys below 40
 
 template <typename IdxT>
 __global__ void __launch_bounds__(kOrderThreads, 8) k_order_lists(const IdxT *rp, uint32_t n, uint64_t nnz,
@@ -383,14 +463,20 @@ __global__ void __launch_bounds__(kOrderThreads, 8) k_order_lists(const IdxT *rp
                                                                const uint32_t *__restrict__ col_in,
                                                                const uint32_t *__restrict__ inv,
                                                                const uint8_t *__restrict__ slot_of, uint32_t *col_out,
-                                                               const uint32_t *nlong_p, uint32_t *flags) {
+                                                               const uint32_t *nhub_p, const uint32_t *nlong_p,
+                                                               uint32_t *flags) {
     __shared__ uint32_t s_h[kOrderWarps][kOrderKeys];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint32_t *h = s_h[warp];
     uint32_t err = 0, ignored = 0;
     const uint64_t w0 = (uint64_t)blockIdx.x * kOrderWarps + warp, nw = (uint64_t)gridDim.x * kOrderWarps;
-    const uint32_t nlong = *nlong_p < n ? *nlong_p : n;
-    for (uint64_t i = w0; i < nlong; i += nw) {
+    const uint32_t nlong = *nlong_p < n ? *nlong_p : n, nhub = *nhub_p < nlong ? *nhub_p : nlong;
+    for (uint64_t i = blockIdx.x; i < nhub; i += gridDim.x) {
+        uint64_t a;
+        const uint32_t d = input_row(rp, order[i], n, nnz, a, ignored);
+        list_on_block(d, a, rp_out[i], n, nnz, col_in, inv, slot_of, col_out, s_h, err);
+    }
+    for (uint64_t i = nhub + w0; i < nlong; i += nw) {
         uint64_t a;
         const uint32_t d = input_row(rp, order[i], n, nnz, a, ignored);
         list_on_warp(d, a, rp_out[i], n, nnz, col_in, inv, slot_of, col_out, h, lane, err);
@@ -495,9 +581,10 @@ cudaError_t order_with(const IdxT *rp, const uint32_t *col_in, uint32_t n, uint6
     const uint64_t cap = (uint64_t)current_sms() * 8;
     if (blocks > cap) blocks = cap;
     // after the scan, cell (first slot of the keys below 20, chunk 0) holds
-    // the number of vertices of key 20 and up
+    // the number of vertices of key 20 and up, and so for key 40
     k_order_lists<IdxT><<<(unsigned)blocks, kOrderThreads, 0, s>>>(
-        rp, n, nnz, order, o.rp, col_in, o.inv, o.slot_of, col_out, o.cnt + (uint64_t)kLongKeySlot * o.chunks, flags);
+        rp, n, nnz, order, o.rp, col_in, o.inv, o.slot_of, col_out, o.cnt + (uint64_t)kHubKeySlot * o.chunks,
+        o.cnt + (uint64_t)kLongKeySlot * o.chunks, flags);
     return cudaGetLastError();
 }
 
