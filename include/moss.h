@@ -248,15 +248,15 @@ int moss_sample_counts(moss_graph *g, int method, uint64_t first, uint64_t count
  * latency-bound loop that cannot take the device synchronisation an
  * allocation or free may cause, or an embedding whose allocator belongs to
  * another framework.  Same arguments and result as moss_sample_counts (the
- * graph and counts_dev are allocated by the caller beforehand); the per-block
- * partial counts live in one fixed device array of 360,448 bytes (2048 rows of
- * 22 uint64) that every GPU loading the library holds until exit.  The first
+ * graph and counts_dev are allocated by the caller beforehand); the counts add
+ * up in one fixed device array of 176 bytes (22 uint64) that every GPU loading
+ * the library holds until exit.  The first
  * call on a device looks up that array's address (cudaGetSymbolAddress), so
  * make it before any stream capture; the address is kept for the life of the
  * process, so after a cudaDeviceReset of that device the entry point must not
  * be called again.  Calls share the array: calls whose work
- * overlaps on the GPU race and must be ordered by the caller.  MOSS_EOVERFLOW
- * if the device needs more than 2048 blocks.  Asynchronous on stream. */
+ * overlaps on the GPU race and must be ordered by the caller.  Asynchronous on
+ * stream. */
 int moss_sample_counts_noalloc(moss_graph *g, int method, uint64_t first, uint64_t count, uint64_t seed,
                                void *stream, uint64_t *counts_dev);
 

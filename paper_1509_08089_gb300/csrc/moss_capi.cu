@@ -279,8 +279,7 @@ struct moss_graph {
     DevTotals *tot = nullptr;
     DevTotals tot_h{};
     unsigned built = 0;          // bit l: vertex table l; bit 3: sigma tables; bit 4: edge hash; bit 5: MOSS-4Min
-    uint64_t *partials = nullptr;
-    int partial_rows = 0;
+    u128 *partials = nullptr;        // the vertex-weight totals' block sums
     uint64_t *counts = nullptr;  // 2 x 22
     moss_result *res_dev = nullptr;
     double *cov_dev = nullptr;   // 22 x 22 covariance matrix
@@ -542,12 +541,6 @@ int moss_graph_load_csr_order(const void *row_ptr, int row_ptr_is_64, const uint
     const size_t rp_bytes = (size_t)(n + 1ULL) * (row_ptr_is_64 ? 8 : 4);
     cudaError_t e = cudaSuccess;
     int blocks = table_blocks(n);
-    int prow = 0;
-    for (int m = 0; m < kMethods; ++m) {
-        int b = sample_rows(m, device);
-        prow = b > prow ? b : prow;
-    }
-    g->partial_rows = prow;
 #define STEP(call, what)                          \
     do {                                          \
         e = (call);                               \
@@ -579,7 +572,7 @@ int moss_graph_load_csr_order(const void *row_ptr, int row_ptr_is_64, const uint
                 g->tot = &st->tot;
                 g->flags = st->flags;
             }
-            g->partials = c.take<uint64_t>(2 * (uint64_t)prow * kSlots + (uint64_t)slot_partial_rows(n) * 6 * 2);
+            g->partials = c.take<u128>((uint64_t)slot_partial_rows(n) * 6);
             g->counts = c.take<uint64_t>(2 * kSlots);
             g->res_dev = c.take<moss_result>(1);
             g->cov_dev = c.take<double>(kSlots * kSlots);
@@ -635,7 +628,7 @@ int moss_graph_load_csr_order(const void *row_ptr, int row_ptr_is_64, const uint
         STEP(launch_vertices(rp_dev, row_ptr_is_64, n, nnz, g->vert, g->flags, s), "vertex kernel");
     }
     if (!small) {
-        u128 *tp = reinterpret_cast<u128 *>(g->partials + (uint64_t)prow * kSlots);
+        u128 *tp = g->partials;
         STEP(launch_slots(n, nnz, g->col, g->vert, g->slot, g->acc, g->owner, g->sq, g->gam[0], g->gam[1], g->gam[2],
                           tp, blocks, g->flags, s, aux_streams()),
              "slot kernels");
@@ -858,10 +851,9 @@ int moss_vertex_levels(const moss_graph *g, int which, uint32_t *nheavy, uint64_
     return MOSS_OK;
 }
 
-// with `pending` the reduce of the (last chunk's) rows is left to the caller
+// adds the counts to the kSlots at sums (device memory of the graph); records
 static int sample_into(moss_graph *g, int method, uint64_t first, uint64_t count, uint64_t seed, cudaStream_t s,
-                       uint64_t *partials, uint64_t *counts_dev, uint8_t *classes, uint32_t *verts,
-                       CountRows *pending = nullptr) {
+                       uint64_t *sums, uint8_t *classes, uint32_t *verts) {
     if (method < 0 || method >= kMethods) return fail(MOSS_EINVAL, "method %d", method);
     if (!method_ready(g, method)) return fail(MOSS_ESTATE, "tables for method %d not built", method);
     if (count > 0 && g->tot_h.gamma[method] == 0)
@@ -871,11 +863,7 @@ static int sample_into(moss_graph *g, int method, uint64_t first, uint64_t count
     const int blocks = sample_launch_blocks(method, g->device, dv);
     // per-warp 32-bit counters: keep each launch below 2^31 samples per warp
     const uint64_t max_chunk = (uint64_t)blocks * 8 * (1ULL << 31);
-    if (count == 0) {
-        if (pending) *pending = CountRows{};
-        else MOSS_CUDA(cudaMemsetAsync(counts_dev, 0, kSlots * sizeof(uint64_t), s), "clearing counts");
-        return MOSS_OK;
-    }
+    if (count == 0) return MOSS_OK;
     if (count > max_chunk) return fail(MOSS_EOVERFLOW, "count above %llu per call", (unsigned long long)max_chunk);
     // a large call behind the filter is grouped (the same counts) when its
     // scratch can be had; not under capture, where the call allocates nothing
@@ -884,16 +872,20 @@ static int sample_into(moss_graph *g, int method, uint64_t first, uint64_t count
     if (scratch_bytes && cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone) {
         void *scratch = nullptr;
         if (pool_alloc(g->device, &scratch, scratch_bytes, s) == cudaSuccess) {
-            const cudaError_t e = launch_counts_grouped(method, dv, first, count, seed, partials, scratch, counts_dev, s,
-                                                        pending);
+            const cudaError_t e = launch_counts_grouped(method, dv, first, count, seed, sums, scratch, s);
             cudaFreeAsync(scratch, s);
             MOSS_CUDA(e, "grouped sample kernels");
             return MOSS_OK;
         }
         cudaGetLastError();   // no memory: the general path
     }
-    MOSS_CUDA(launch_counts(method, dv, first, count, seed, partials, classes, verts, counts_dev, s, pending),
-              "sample kernels");
+    MOSS_CUDA(launch_counts(method, dv, first, count, seed, sums, classes, verts, s), "sample kernels");
+    return MOSS_OK;
+}
+
+// zeroes the graph's sums of `methods` sub-methods
+static int clear_sums(moss_graph *g, int methods, cudaStream_t s) {
+    MOSS_CUDA(cudaMemsetAsync(g->counts, 0, methods * kSlots * sizeof(uint64_t), s), "clearing counts");
     return MOSS_OK;
 }
 
@@ -901,8 +893,11 @@ int moss_sample_counts(moss_graph *g, int method, uint64_t first, uint64_t count
                        uint64_t *counts_dev) {
     if (!g || !counts_dev) return fail(MOSS_EINVAL, "NULL argument");
     DeviceGuard dg(g->device);
-    return sample_into(g, method, first, count, seed, static_cast<cudaStream_t>(stream), g->partials, counts_dev, nullptr,
-                       nullptr);
+    const cudaStream_t s = static_cast<cudaStream_t>(stream);
+    int rc = clear_sums(g, 1, s);
+    if (rc || (rc = sample_into(g, method, first, count, seed, s, g->counts, nullptr, nullptr))) return rc;
+    MOSS_CUDA(launch_copy_counts(g->counts, counts_dev, s), "copying counts");
+    return MOSS_OK;
 }
 
 int moss_sample_records(moss_graph *g, int method, uint64_t first, uint64_t count, uint64_t seed, void *stream,
@@ -910,7 +905,8 @@ int moss_sample_records(moss_graph *g, int method, uint64_t first, uint64_t coun
     if (!g || !classes_dev) return fail(MOSS_EINVAL, "NULL argument");
     DeviceGuard dg(g->device);
     const cudaStream_t s = static_cast<cudaStream_t>(stream);
-    const int rc = sample_into(g, method, first, count, seed, s, g->partials, g->counts, classes_dev, verts_dev);
+    // (the counts that go with the records are not asked for: any base will do)
+    const int rc = sample_into(g, method, first, count, seed, s, g->counts, classes_dev, verts_dev);
     if (rc || !g->order || !verts_dev) return rc;
     // vertex words of the records back to input ids (MOSS-4 and MOSS-4Min: the first four)
     MOSS_CUDA(launch_map_records(verts_dev, count, method == 1 || method == 2 ? 5 : 4, g->order, g->n, s),
@@ -918,19 +914,26 @@ int moss_sample_records(moss_graph *g, int method, uint64_t first, uint64_t coun
     return MOSS_OK;
 }
 
-// Both sub-methods of an estimate (ids from 0) up to their rows of counts:
+// Both sub-methods of an estimate (ids from 0) up to their counts (g->counts):
 // in one launch when they are small enough (same counts).
-static int sample_both(moss_graph *g, int ma, uint64_t ka, int mb, uint64_t kb, uint64_t seed, cudaStream_t s,
-                       CountRows *a, CountRows *b) {
+static int sample_both(moss_graph *g, int ma, uint64_t ka, int mb, uint64_t kb, uint64_t seed, cudaStream_t s) {
     const bool mix = ma == MOSS_METHOD_MOSS4;
+    int rc = clear_sums(g, 2, s);
+    if (rc) return rc;
     if (pair_fits(mix, ka, kb)) {
-        MOSS_CUDA(launch_pair(mix, view(g), ka, kb, seed, g->partials, a, b, s), "sample kernels");
+        MOSS_CUDA(launch_pair(mix, view(g), ka, kb, seed, g->counts, s), "sample kernels");
         return MOSS_OK;
     }
-    const int rc = sample_into(g, ma, 0, ka, seed, s, g->partials, g->counts, nullptr, nullptr, a);
-    if (rc) return rc;
-    return sample_into(g, mb, 0, kb, seed, s, g->partials + (uint64_t)g->partial_rows * kSlots, g->counts + kSlots,
-                       nullptr, nullptr, b);
+    rc = sample_into(g, ma, 0, ka, seed, s, g->counts, nullptr, nullptr);
+    return rc ? rc : sample_into(g, mb, 0, kb, seed, s, g->counts + kSlots, nullptr, nullptr);
+}
+
+// the result of the counts at g->counts
+static int finalize_sums(moss_graph *g, const FinalizeIn &in, cudaStream_t s, moss_result *out) {
+    HitsArg hits;
+    hits.dev = g->counts;
+    MOSS_CUDA(launch_finalize(in, hits, g->tot, result_target(g), nullptr, s), "finalize kernel");
+    return read_result(g, s, out);
 }
 
 int moss_sample_estimate(moss_graph *g, int k, uint64_t budget, uint64_t seed, void *stream, moss_result *out) {
@@ -941,20 +944,18 @@ int moss_sample_estimate(moss_graph *g, int k, uint64_t budget, uint64_t seed, v
     FinalizeIn in;
     in.k = k;
     in.K[0] = in.K[1] = 0;
-    CountRows a, b;
     int rc;
     if (k == 4) {
         if (!method_ready(g, 0)) return fail(MOSS_ESTATE, "tables for k=4 not built");
         in.K[0] = g->tot_h.gamma[0] ? budget : 0;
-        if ((rc = sample_into(g, 0, 0, in.K[0], seed, s, g->partials, g->counts, nullptr, nullptr, &a))) return rc;
+        if ((rc = clear_sums(g, 2, s)) || (rc = sample_into(g, 0, 0, in.K[0], seed, s, g->counts, nullptr, nullptr))) return rc;
     } else {
         if (!method_ready(g, 1) || !method_ready(g, 2)) return fail(MOSS_ESTATE, "tables for k=5 not built");
         in.K[0] = g->tot_h.gamma[1] ? budget / 2 : 0;
         in.K[1] = g->tot_h.gamma[2] ? budget - budget / 2 : 0;
-        if ((rc = sample_both(g, 1, in.K[0], 2, in.K[1], seed, s, &a, &b))) return rc;
+        if ((rc = sample_both(g, 1, in.K[0], 2, in.K[1], seed, s))) return rc;
     }
-    MOSS_CUDA(launch_reduce_finalize(in, a, b, g->tot, result_target(g), s), "finalize kernel");
-    return read_result(g, s, out);
+    return finalize_sums(g, in, s, out);
 }
 
 // Counts handed in by the caller: host memory travels as a kernel argument,
@@ -1023,11 +1024,9 @@ int moss_sample_estimate_min(moss_graph *g, uint64_t budget, uint64_t budget_min
     in.mix = 1;
     in.K[0] = g->tot_h.gamma[0] ? budget : 0;
     in.K[1] = g->tot_h.gamma[3] ? budget_min : 0;
-    CountRows a, b;
-    const int rc = sample_both(g, MOSS_METHOD_MOSS4, in.K[0], MOSS_METHOD_MOSS4MIN, in.K[1], seed, s, &a, &b);
+    const int rc = sample_both(g, MOSS_METHOD_MOSS4, in.K[0], MOSS_METHOD_MOSS4MIN, in.K[1], seed, s);
     if (rc) return rc;
-    MOSS_CUDA(launch_reduce_finalize(in, a, b, g->tot, result_target(g), s), "finalize kernel");
-    return read_result(g, s, out);
+    return finalize_sums(g, in, s, out);
 }
 
 int moss_finalize_min(moss_graph *g, const uint64_t *K, const uint64_t *hits, void *stream, double *cov_host,

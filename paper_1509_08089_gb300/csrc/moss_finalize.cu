@@ -326,34 +326,6 @@ __global__ void k_finalize(FinalizeIn in, const __grid_constant__ HitsArg hits, 
     finalize_any(in, h, h + kSlots, tot, row == 0 ? out : nullptr, cov, row);
 }
 
-// The counts of both sub-methods from their rows (thread t adds slot t %
-// kSlots of every 32nd row from row t / kSlots, the rows of both together),
-// then the finalize on the first warp: one launch for two reduces and a
-// finalize.
-__global__ void __launch_bounds__(32 * kSlots) k_reduce_finalize(FinalizeIn in, CountRows a, CountRows b,
-                                                                 const DevTotals *tot, moss_result *out) {
-    __shared__ uint64_t part[2][32][kSlots];
-    __shared__ uint64_t hits[2][kSlots];
-    const int c = threadIdx.x % kSlots, r0 = threadIdx.x / kSlots;
-    uint64_t s0 = 0, s1 = 0;
-#pragma unroll 4
-    for (int r = r0; r < a.n; r += 32) s0 += a.rows[(uint64_t)r * kSlots + c];
-#pragma unroll 4
-    for (int r = r0; r < b.n; r += 32) s1 += b.rows[(uint64_t)r * kSlots + c];
-    part[0][r0][c] = s0;
-    part[1][r0][c] = s1;
-    __syncthreads();
-    if (threadIdx.x < 2 * kSlots) {
-        const int m = threadIdx.x / kSlots;
-        const uint64_t *base = m ? b.base : a.base;
-        uint64_t t = base ? base[c] : 0;
-        for (int r = 0; r < 32; ++r) t += part[m][r][c];
-        hits[m][c] = t;
-    }
-    __syncthreads();
-    if (threadIdx.x < 32) finalize_any(in, hits[0], hits[1], tot, out);
-}
-
 // one warp per request of a batch
 constexpr int kFinalizeWarps = 4;
 __global__ void k_finalize_batch(const BatchRequest *reqs, int nreq, const uint64_t *task_counts,
@@ -371,12 +343,6 @@ __global__ void k_finalize_batch(const BatchRequest *reqs, int nreq, const uint6
 cudaError_t launch_finalize(const FinalizeIn &in, const HitsArg &hits, const DevTotals *tot, void *result, double *cov,
                             cudaStream_t s) {
     k_finalize<<<cov ? kSlots : 1, 32, 0, s>>>(in, hits, tot, static_cast<moss_result *>(result), cov);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_reduce_finalize(const FinalizeIn &in, const CountRows &a, const CountRows &b, const DevTotals *tot,
-                                   void *result_dev, cudaStream_t s) {
-    k_reduce_finalize<<<1, 32 * kSlots, 0, s>>>(in, a, b, tot, static_cast<moss_result *>(result_dev));
     return cudaGetLastError();
 }
 

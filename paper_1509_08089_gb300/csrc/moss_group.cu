@@ -176,11 +176,11 @@ constexpr int group_blocks() { return RNG == kRngPhilox ? 5 : 6; }
 
 // The samples of the entries in order, a thread each; Path-5 samples whose
 // first pair of sigma draws collides are flagged in the (zeroed) deferral
-// bitmap for the redraw stages.  Counts leave as one row per block.
+// bitmap for the redraw stages.
 template <int METHOD, int RNG>
 __global__ void __launch_bounds__(kThreads, group_blocks<RNG>())
     k_sample_group(DevGraph g, uint64_t first, uint32_t count, uint64_t seed, const uint2 *entries,
-                   uint64_t *partials) {
+                   uint64_t *sums) {
     constexpr int PM = kPmGroup;
     __shared__ uint8_t lut[kLut];
     __shared__ uint8_t lutc[METHOD == 3 ? 4096 : 1];
@@ -215,11 +215,7 @@ __global__ void __launch_bounds__(kThreads, group_blocks<RNG>())
         }
     }
     __syncthreads();
-    if (threadIdx.x < kSlots) {
-        uint64_t sum = 0;
-        for (int w = 0; w < kWarps; ++w) sum += hist[w][threadIdx.x];
-        partials[(uint64_t)blockIdx.x * kSlots + threadIdx.x] = sum;
-    }
+    add_sums<kWarps>(hist, sums);
 }
 
 uint64_t align256(uint64_t x) { return (x + 255) & ~255ull; }
@@ -241,7 +237,7 @@ Scratch carve(void *mem, uint64_t chunk) {
 
 template <int M, int RNG>
 cudaError_t run_chunk(const DevGraph &g, uint64_t first, uint32_t len, uint64_t seed, const Scratch &w,
-                      uint64_t *partials, int sms, int blocks, cudaStream_t s) {
+                      uint64_t *sums, int sms, int blocks, cudaStream_t s) {
     cudaError_t e = cudaMemsetAsync(w.cursor, 0, kGroups * 4, s);
     if (e != cudaSuccess) return e;
     constexpr int smem = kGroupTile * sizeof(uint2);
@@ -254,18 +250,18 @@ cudaError_t run_chunk(const DevGraph &g, uint64_t first, uint32_t len, uint64_t 
     k_group_place<<<sms * kGroupPerSm, kGroupThreads, smem, s>>>(len, w.v, w.cursor, w.entries);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (M == 2 && (e = cudaMemsetAsync(g.defer, 0, ((uint64_t)len + 31) / 32 * 4, s)) != cudaSuccess) return e;
-    k_sample_group<M, RNG><<<blocks, kThreads, 0, s>>>(g, first, len, seed, w.entries, partials);
+    k_sample_group<M, RNG><<<blocks, kThreads, 0, s>>>(g, first, len, seed, w.entries, sums);
     return cudaGetLastError();
 }
 
 template <int RNG>
 cudaError_t run_method(int method, const DevGraph &g, uint64_t first, uint32_t len, uint64_t seed, const Scratch &w,
-                       uint64_t *partials, int sms, int blocks, cudaStream_t s) {
+                       uint64_t *sums, int sms, int blocks, cudaStream_t s) {
     switch (method) {
-        case 0: return run_chunk<0, RNG>(g, first, len, seed, w, partials, sms, blocks, s);
-        case 1: return run_chunk<1, RNG>(g, first, len, seed, w, partials, sms, blocks, s);
-        case 2: return run_chunk<2, RNG>(g, first, len, seed, w, partials, sms, blocks, s);
-        case 3: return run_chunk<3, RNG>(g, first, len, seed, w, partials, sms, blocks, s);
+        case 0: return run_chunk<0, RNG>(g, first, len, seed, w, sums, sms, blocks, s);
+        case 1: return run_chunk<1, RNG>(g, first, len, seed, w, sums, sms, blocks, s);
+        case 2: return run_chunk<2, RNG>(g, first, len, seed, w, sums, sms, blocks, s);
+        case 3: return run_chunk<3, RNG>(g, first, len, seed, w, sums, sms, blocks, s);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -298,22 +294,19 @@ uint64_t group_bytes(int method, const DevGraph &g, bool degree_order, uint64_t 
 }
 
 cudaError_t launch_counts_grouped(int method, const DevGraph &g, uint64_t first, uint64_t count, uint64_t seed,
-                                  uint64_t *partials, void *scratch, uint64_t *counts_dev, cudaStream_t s,
-                                  CountRows *pending) {
+                                  uint64_t *sums, void *scratch, cudaStream_t s) {
     const bool philox = g.rng == kRngPhilox;
     const int sms = current_sms(), blocks = sms * (philox ? group_blocks<kRngPhilox>() : group_blocks<kRngSplitMix>());
     const uint64_t chunk = std::min(count, kGroupChunk);
     const Scratch w = carve(scratch, chunk);
-    for (uint64_t c0 = 0; c0 < count; c0 += chunk) {
+    cudaError_t e = cudaSuccess;
+    for (uint64_t c0 = 0; e == cudaSuccess && c0 < count; c0 += chunk) {
         const uint32_t len = (uint32_t)std::min(chunk, count - c0);
-        cudaError_t e = philox ? run_method<kRngPhilox>(method, g, first + c0, len, seed, w, partials, sms, blocks, s)
-                               : run_method<kRngSplitMix>(method, g, first + c0, len, seed, w, partials, sms, blocks, s);
-        if (e == cudaSuccess)
-            e = launch_tail(method, g, first + c0, len, seed, partials, blocks, nullptr, nullptr, counts_dev, c0 > 0, s,
-                            c0 + len == count ? pending : nullptr);
-        if (e != cudaSuccess) return e;
+        e = philox ? run_method<kRngPhilox>(method, g, first + c0, len, seed, w, sums, sms, blocks, s)
+                   : run_method<kRngSplitMix>(method, g, first + c0, len, seed, w, sums, sms, blocks, s);
+        if (e == cudaSuccess && method == 2) e = launch_redraws(g, first + c0, len, seed, sums, nullptr, nullptr, s);
     }
-    return cudaSuccess;
+    return e;
 }
 
 }  // namespace moss

@@ -402,42 +402,30 @@ cudaError_t launch_min_tables(uint32_t n, uint64_t nnz, uint32_t d_max, const ui
 // moss_sample.cu
 // class of each 4- and 5-vertex edge mask; c(s) of MOSS-4Min by (mask << 6 | order bits)
 void upload_luts(const uint8_t *lut4, const uint8_t *lut5, const uint8_t *lutc);
-// Counts (22 uint64 at counts_dev) of samples [first, first+count) of one
+// Counts (added to the 22 uint64 at sums) of samples [first, first+count) of one
 // method, with optional per-sample records (classes, verts: count and 5*count
-// entries); partials holds sample_rows(method) rows of 22 uint64.  Path-5 runs
-// in chunks of kDeferChunk ids: a launch that defers the samples whose first
-// sigma attempt collides, one that redoes them, and a reduce that accumulates.
-// With `pending` the last chunk's reduce is left to the caller, who gets its
-// rows (and counts_dev as the base to add when earlier chunks are in it).
-struct CountRows {
-    const uint64_t *rows = nullptr;   // n rows of kSlots partial counts
-    int n = 0;
-    const uint64_t *base = nullptr;   // kSlots counts to add, or null
-};
-cudaError_t launch_counts(int method, const DevGraph &g, uint64_t first, uint64_t count, uint64_t seed,
-                          uint64_t *partials, uint8_t *classes, uint32_t *verts, uint64_t *counts_dev,
-                          cudaStream_t s, CountRows *pending = nullptr);
-// what follows the sampler launch of one chunk: Path-5's redraw stages and the reduce
-cudaError_t launch_tail(int method, const DevGraph &g, uint64_t first, uint64_t count, uint64_t seed,
-                        uint64_t *partials, int blocks, uint8_t *classes, uint32_t *verts, uint64_t *counts_dev,
-                        bool accumulate, cudaStream_t s, CountRows *pending);
+// entries).  Path-5 runs in chunks of kDeferChunk ids: a launch that defers
+// the samples whose first sigma attempt collides and two that redraw them.
+cudaError_t launch_counts(int method, const DevGraph &g, uint64_t first, uint64_t count, uint64_t seed, uint64_t *sums,
+                          uint8_t *classes, uint32_t *verts, cudaStream_t s);
+// the redraw stages of one chunk, adding to sums
+cudaError_t launch_redraws(const DevGraph &g, uint64_t first, uint64_t count, uint64_t seed, uint64_t *sums,
+                           uint8_t *classes, uint32_t *verts, cudaStream_t s);
+cudaError_t launch_copy_counts(const uint64_t *sums, uint64_t *out, cudaStream_t s);
 // Both sub-methods of an estimate (T-5 and Path-5, or MOSS-4 and MOSS-4Min
-// when mix) in one launch, ids from 0; false when the budgets are too large
-// for it to pay.  Rows as launch_counts' pending ones.
+// when mix) in one launch, ids from 0, counts added at sums and sums + kSlots;
+// pair_fits: false when the budgets are too large for it to pay
 bool pair_fits(bool mix, uint64_t count_a, uint64_t count_b);
-cudaError_t launch_pair(bool mix, const DevGraph &g, uint64_t count_a, uint64_t count_b, uint64_t seed,
-                        uint64_t *partials, CountRows *a, CountRows *b, cudaStream_t s);
-int sample_blocks(int method, int device);   // the most blocks any variant of a sampler launches
+cudaError_t launch_pair(bool mix, const DevGraph &g, uint64_t count_a, uint64_t count_b, uint64_t seed, uint64_t *sums,
+                        cudaStream_t s);
 int sample_launch_blocks(int method, int device, const DevGraph &g);   // blocks of the variant g uses
-int sample_rows(int method, int device);     // partial-count rows launch_counts needs
 
 // moss_group.cu: large calls behind the filter, the sample ids grouped by their first vertex
 void upload_luts_group(const uint8_t *lut4, const uint8_t *lut5, const uint8_t *lutc);
 // scratch of a grouped call; 0 when the call is not one to group
 uint64_t group_bytes(int method, const DevGraph &g, bool degree_order, uint64_t count);
 cudaError_t launch_counts_grouped(int method, const DevGraph &g, uint64_t first, uint64_t count, uint64_t seed,
-                                  uint64_t *partials, void *scratch, uint64_t *counts_dev, cudaStream_t s,
-                                  CountRows *pending);
+                                  uint64_t *sums, void *scratch, cudaStream_t s);
 
 // moss_finalize.cu
 struct FinalizeIn {
@@ -453,9 +441,6 @@ struct HitsArg {
 // result (and, with cov, the 22 x 22 covariance matrix) of given counts
 cudaError_t launch_finalize(const FinalizeIn &in, const HitsArg &hits, const DevTotals *tot, void *result, double *cov,
                             cudaStream_t s);
-// the counts of both sub-methods summed from their rows, and the finalize
-cudaError_t launch_reduce_finalize(const FinalizeIn &in, const CountRows &a, const CountRows &b, const DevTotals *tot,
-                                   void *result_dev, cudaStream_t s);
 
 // ---------------------------------------------------------------- batches --
 // One task = one sub-method of one request: sample ids [first, first+count)

@@ -18,9 +18,8 @@
 // device current) and caches it; that first call should therefore come
 // before any stream capture.  The cached address lives as long as the
 // process: a cudaDeviceReset of the device makes it stale, so the entry point
-// is not to be called again after one.  All calls share the one array: each call's
-// sampling kernel overwrites every row it later reads, so nothing needs
-// clearing, but calls whose kernels overlap on the GPU (different streams,
+// is not to be called again after one.  All calls share the one array, which
+// each call clears first: calls whose kernels overlap on the GPU (different streams,
 // no ordering between them) race on the array and must be serialised by the
 // caller.
 #include <mutex>
@@ -32,12 +31,11 @@ namespace moss {
 
 namespace {
 
-constexpr int kNoAllocMaxBlocks = 2048;   // rows of 22 uint64 partial counts
-constexpr size_t kNoAllocScratchBytes = (size_t)kNoAllocMaxBlocks * kSlots * sizeof(uint64_t);  // 360,448 B
+constexpr size_t kNoAllocScratchBytes = kSlots * sizeof(uint64_t);   // 176 B
 constexpr int kMaxDevices = 64;
 
-static __device__ __align__(256) uint64_t g_noalloc_partials[kNoAllocMaxBlocks * kSlots];
-static_assert(sizeof(g_noalloc_partials) == kNoAllocScratchBytes, "the held scratch is the stated size");
+static __device__ __align__(256) uint64_t g_noalloc_sums[kSlots];
+static_assert(sizeof(g_noalloc_sums) == kNoAllocScratchBytes, "the held scratch is the stated size");
 
 std::mutex g_mutex;
 uint64_t *g_scratch[kMaxDevices] = {};
@@ -48,8 +46,8 @@ int scratch_on(int device, uint64_t **out) {
     std::lock_guard<std::mutex> lk(g_mutex);
     if (!g_scratch[device]) {
         uint64_t *p = nullptr;
-        cudaError_t e = cudaGetSymbolAddress(reinterpret_cast<void **>(&p), g_noalloc_partials);
-        if (e != cudaSuccess || !p) return set_error(MOSS_ECUDA, "cudaGetSymbolAddress of the partial-count array failed");
+        cudaError_t e = cudaGetSymbolAddress(reinterpret_cast<void **>(&p), g_noalloc_sums);
+        if (e != cudaSuccess || !p) return set_error(MOSS_ECUDA, "cudaGetSymbolAddress of the count array failed");
         g_scratch[device] = p;
     }
     *out = g_scratch[device];
@@ -78,19 +76,19 @@ extern "C" int moss_sample_counts_noalloc(moss_graph *g, int method, uint64_t fi
         return set_error(MOSS_ECUDA, "cannot make the graph's device current");
     int rc = MOSS_OK;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    uint64_t *partials = nullptr;
+    uint64_t *sums = nullptr;
     const int blocks = sample_launch_blocks(method, gi.device, gi.view);
     const uint64_t max_chunk = (uint64_t)blocks * 8 * (1ULL << 31);
-    if (sample_rows(method, gi.device) > kNoAllocMaxBlocks) {
-        rc = set_error(MOSS_EOVERFLOW, "this GPU needs more than 2048 blocks of partial counts, the fixed maximum");
-    } else if (count > max_chunk) {
+    if (count > max_chunk) {
         rc = set_error(MOSS_EOVERFLOW, "count above the per-call maximum of 2^31 samples per warp");
-    } else if ((rc = scratch_on(gi.device, &partials)) == MOSS_OK) {
+    } else if ((rc = scratch_on(gi.device, &sums)) == MOSS_OK) {
         cudaError_t e;
         if (count == 0) {
             e = cudaMemsetAsync(counts_dev, 0, kSlots * sizeof(uint64_t), s);
         } else {
-            e = launch_counts(method, gi.view, first, count, seed, partials, nullptr, nullptr, counts_dev, s);
+            e = cudaMemsetAsync(sums, 0, kSlots * sizeof(uint64_t), s);
+            if (e == cudaSuccess) e = launch_counts(method, gi.view, first, count, seed, sums, nullptr, nullptr, s);
+            if (e == cudaSuccess) e = launch_copy_counts(sums, counts_dev, s);
         }
         if (e != cudaSuccess) rc = set_error(MOSS_ECUDA, cudaGetErrorString(e));
     }

@@ -10,8 +10,7 @@
 //   (hashed edge set, or lock-step binary searches) -> edge mask -> class
 //   through a shared-memory table.
 // Counts are aggregated per warp with __match_any_sync into shared-memory
-// histograms and leave the block as one row of per-block partials; a second
-// kernel adds the rows in a fixed order.  No global atomics.
+// histograms, and each block adds its own to the launch's 22 sums.
 //
 // Word schedule (x_i = word i of the sample, output (4 s + method) 16 + i + 1
 // of SplitMix64 seeded with seed, or Philox4x32-10 block i / 2; sample_words2
@@ -57,7 +56,7 @@ constexpr int defer_bound_blocks() { return RNG == kRngPhilox ? 4 : defer_min_bl
 
 template <int METHOD, bool RECORD, bool HASH, int PM, int RNG>
 __global__ void __launch_bounds__(kThreads, min_blocks<METHOD, RNG>()) k_sample(DevGraph g, uint64_t first, uint64_t count, uint64_t seed,
-                                                     uint64_t *partials, uint8_t *classes, uint32_t *verts) {
+                                                     uint64_t *sums, uint8_t *classes, uint32_t *verts) {
     __shared__ uint8_t lut[kLut];
     __shared__ uint8_t lutc[METHOD == 3 ? 4096 : 1];
     __shared__ uint32_t hist[kWarps][kSlots];
@@ -105,11 +104,7 @@ __global__ void __launch_bounds__(kThreads, min_blocks<METHOD, RNG>()) k_sample(
         if (cls < kSlots && lane == __ffs(peers) - 1) atomicAdd(&hist[warp][cls], (uint32_t)__popc(peers));
     }
     __syncthreads();
-    if (threadIdx.x < kSlots) {
-        uint64_t sum = 0;
-        for (int w = 0; w < kWarps; ++w) sum += hist[w][threadIdx.x];
-        partials[(uint64_t)blockIdx.x * kSlots + threadIdx.x] = sum;
-    }
+    add_sums<kWarps>(hist, sums);
 }
 
 // The Path-5 samples a launch deferred, redrawn by the next stage (STAGE 1:
@@ -121,13 +116,12 @@ __global__ void __launch_bounds__(kThreads, min_blocks<METHOD, RNG>()) k_sample(
 // round but the warp's last runs with all lanes busy however sparse the
 // flags.  STAGE 1 clears the words it reads and sets the bits of re-deferred
 // samples again (plain stores: a window's words belong to one warp).  Counts
-// are aggregated as in k_sample into this launch's partial rows; STAGE 2,
-// launched with no more blocks than STAGE 1, adds into STAGE 1's rows.
+// are aggregated as in k_sample.
 constexpr uint32_t kDeferList = 1024 + 32;   // a window's ids plus the carry-over
 
 template <bool RECORD, bool HASH, int STAGE, int PM, int RNG>
 __global__ void __launch_bounds__(kThreads, defer_bound_blocks<STAGE, RNG>())
-    k_sample_deferred(DevGraph g, uint64_t first, uint64_t count, uint64_t seed, uint64_t *partials,
+    k_sample_deferred(DevGraph g, uint64_t first, uint64_t count, uint64_t seed, uint64_t *sums,
                       uint8_t *classes, uint32_t *verts) {
     static_assert(STAGE == 1 || STAGE == 2, "deferred stages are 1 and 2");
     __shared__ uint8_t lut[kLut];
@@ -212,15 +206,9 @@ __global__ void __launch_bounds__(kThreads, defer_bound_blocks<STAGE, RNG>())
     }
     if (n) round(0, n);
     __syncthreads();
-    if (threadIdx.x < kSlots) {
-        uint64_t sum = 0;
-        for (int w = 0; w < kWarps; ++w) sum += hist[w][threadIdx.x];
-        uint64_t *row = partials + (uint64_t)blockIdx.x * kSlots + threadIdx.x;
-        *row = STAGE == 1 ? sum : *row + sum;
-    }
+    add_sums<kWarps>(hist, sums);
 }
 
-// one warp per class slot: lanes stride over the block rows, then a warp sum
 // ---------------------------------------------------------------- batches --
 // Many requests on many graphs in one persistent launch.  Warps take tiles
 // (fixed-size runs of sample ids of one task) from a global counter -- one
@@ -327,33 +315,19 @@ __global__ void k_batch_reduce(const BatchTask *tasks, uint32_t tile_samples, co
     if (lane == 0) task_counts[(uint64_t)blockIdx.x * kSlots + c] = s;
 }
 
-// accumulate: add to out (later chunks of one count) instead of overwriting
-// One block of 32 x kSlots threads: thread t adds slot t % kSlots of every
-// 32nd row from row t / kSlots (consecutive threads read consecutive words),
-// then 32 partial sums per slot are added in shared memory.
-__global__ void k_reduce(const uint64_t *partials, int blocks, uint64_t *out, int accumulate) {
-    __shared__ uint64_t part[32][kSlots];
-    const int c = threadIdx.x % kSlots, r0 = threadIdx.x / kSlots;
-    uint64_t s = 0;
-    for (int b = r0; b < blocks; b += 32) s += partials[(uint64_t)b * kSlots + c];
-    part[r0][c] = s;
-    __syncthreads();
-    if (threadIdx.x < kSlots) {
-        uint64_t t = 0;
-        for (int r = 0; r < 32; ++r) t += part[r][threadIdx.x];
-        out[threadIdx.x] = accumulate ? out[threadIdx.x] + t : t;
-    }
+__global__ void k_copy_counts(const uint64_t *sums, uint64_t *out) {
+    if (threadIdx.x < kSlots) out[threadIdx.x] = sums[threadIdx.x];
 }
 
 // T-5 and Path-5 (or, MIX, MOSS-4 and MOSS-4Min) samples 0.. in one launch:
-// the first blocks_a blocks draw the first method's, the rest the second's,
-// each leaving a row of counts.  A small estimate is launches and latency, so
+// the first blocks_a blocks draw the first method's, counted at sums, the rest
+// the second's, counted at sums + kSlots.  A small estimate is launches and latency, so
 // its two sub-methods share the chip and Path-5 redraws in line (two more
 // launches otherwise, each a few long dependent chains).
 template <bool MIX, bool HASH, int PM, int RNG>
 __global__ void __launch_bounds__(kThreads, 4)
     k_sample_pair(DevGraph g, uint32_t blocks_a, uint64_t count_a, uint64_t count_b, uint64_t seed,
-                  uint64_t *partials) {
+                  uint64_t *sums) {
     __shared__ uint8_t lut[MIX ? 64 : kLut];
     __shared__ uint8_t lutc[MIX ? 4096 : 1];
     __shared__ uint32_t hist[kWarps][kSlots];
@@ -384,11 +358,7 @@ __global__ void __launch_bounds__(kThreads, 4)
         if (cls < kSlots && lane == __ffs(peers) - 1) atomicAdd(&hist[warp][cls], (uint32_t)__popc(peers));
     }
     __syncthreads();
-    if (threadIdx.x < kSlots) {
-        uint64_t sum = 0;
-        for (int w = 0; w < kWarps; ++w) sum += hist[w][threadIdx.x];
-        partials[(uint64_t)blockIdx.x * kSlots + threadIdx.x] = sum;
-    }
+    add_sums<kWarps>(hist, second ? sums + kSlots : sums);
 }
 
 // the probe variant of a launch: 0 list search, 1 hashed set, 2 filter in
@@ -400,30 +370,30 @@ int probe_variant(int method, const DevGraph &g) {
 }
 
 template <int M, bool R, int RNG>
-cudaError_t launch_one_rng(const DevGraph &g, uint64_t first, uint64_t count, uint64_t seed, uint64_t *partials,
+cudaError_t launch_one_rng(const DevGraph &g, uint64_t first, uint64_t count, uint64_t seed, uint64_t *sums,
                            int blocks, uint8_t *classes, uint32_t *verts, cudaStream_t s) {
     switch (probe_variant(M, g)) {
         case 2:
-            k_sample<M, R, true, kPmFilter, RNG><<<blocks, kThreads, 0, s>>>(g, first, count, seed, partials, classes, verts);
+            k_sample<M, R, true, kPmFilter, RNG><<<blocks, kThreads, 0, s>>>(g, first, count, seed, sums, classes, verts);
             break;
         case 3:
-            k_sample<M, R, true, kPmStream, RNG><<<blocks, kThreads, 0, s>>>(g, first, count, seed, partials, classes, verts);
+            k_sample<M, R, true, kPmStream, RNG><<<blocks, kThreads, 0, s>>>(g, first, count, seed, sums, classes, verts);
             break;
         case 1:
-            k_sample<M, R, true, kPmPlain, RNG><<<blocks, kThreads, 0, s>>>(g, first, count, seed, partials, classes, verts);
+            k_sample<M, R, true, kPmPlain, RNG><<<blocks, kThreads, 0, s>>>(g, first, count, seed, sums, classes, verts);
             break;
         default:
-            k_sample<M, R, false, kPmPlain, RNG><<<blocks, kThreads, 0, s>>>(g, first, count, seed, partials, classes, verts);
+            k_sample<M, R, false, kPmPlain, RNG><<<blocks, kThreads, 0, s>>>(g, first, count, seed, sums, classes, verts);
     }
     return cudaGetLastError();
 }
 
 template <int M, bool R>
-cudaError_t launch_one(const DevGraph &g, uint64_t first, uint64_t count, uint64_t seed, uint64_t *partials,
+cudaError_t launch_one(const DevGraph &g, uint64_t first, uint64_t count, uint64_t seed, uint64_t *sums,
                        int blocks, uint8_t *classes, uint32_t *verts, cudaStream_t s) {
     if (g.rng == kRngPhilox)
-        return launch_one_rng<M, R, kRngPhilox>(g, first, count, seed, partials, blocks, classes, verts, s);
-    return launch_one_rng<M, R, kRngSplitMix>(g, first, count, seed, partials, blocks, classes, verts, s);
+        return launch_one_rng<M, R, kRngPhilox>(g, first, count, seed, sums, blocks, classes, verts, s);
+    return launch_one_rng<M, R, kRngSplitMix>(g, first, count, seed, sums, blocks, classes, verts, s);
 }
 
 }  // namespace
@@ -480,12 +450,6 @@ int sample_per_sm(int method, int device, int variant) {
     return per[variant];
 }
 
-int sample_blocks(int method, int device) {
-    int per = 1;
-    for (int v = 0; v < kVariants; ++v) per = std::max(per, sample_per_sm(method, device, v));
-    return device_sms(device) * per;   // the most any variant launches
-}
-
 int sample_launch_blocks(int method, int device, const DevGraph &g) {
     return device_sms(device) *
            sample_per_sm(method, device, probe_variant(method, g) + (g.rng == kRngPhilox ? kProbeVariants : 0));
@@ -494,51 +458,51 @@ int sample_launch_blocks(int method, int device, const DevGraph &g) {
 namespace {
 
 cudaError_t launch_sample(int method, const DevGraph &g, uint64_t first, uint64_t count, uint64_t seed,
-                          uint64_t *partials, int blocks, uint8_t *classes, uint32_t *verts, cudaStream_t s) {
+                          uint64_t *sums, int blocks, uint8_t *classes, uint32_t *verts, cudaStream_t s) {
     const bool rec = classes != nullptr;
     switch (method * 2 + (rec ? 1 : 0)) {
-        case 0: return launch_one<0, false>(g, first, count, seed, partials, blocks, classes, verts, s);
-        case 1: return launch_one<0, true>(g, first, count, seed, partials, blocks, classes, verts, s);
-        case 2: return launch_one<1, false>(g, first, count, seed, partials, blocks, classes, verts, s);
-        case 3: return launch_one<1, true>(g, first, count, seed, partials, blocks, classes, verts, s);
-        case 4: return launch_one<2, false>(g, first, count, seed, partials, blocks, classes, verts, s);
-        case 5: return launch_one<2, true>(g, first, count, seed, partials, blocks, classes, verts, s);
-        case 6: return launch_one<3, false>(g, first, count, seed, partials, blocks, classes, verts, s);
-        case 7: return launch_one<3, true>(g, first, count, seed, partials, blocks, classes, verts, s);
+        case 0: return launch_one<0, false>(g, first, count, seed, sums, blocks, classes, verts, s);
+        case 1: return launch_one<0, true>(g, first, count, seed, sums, blocks, classes, verts, s);
+        case 2: return launch_one<1, false>(g, first, count, seed, sums, blocks, classes, verts, s);
+        case 3: return launch_one<1, true>(g, first, count, seed, sums, blocks, classes, verts, s);
+        case 4: return launch_one<2, false>(g, first, count, seed, sums, blocks, classes, verts, s);
+        case 5: return launch_one<2, true>(g, first, count, seed, sums, blocks, classes, verts, s);
+        case 6: return launch_one<3, false>(g, first, count, seed, sums, blocks, classes, verts, s);
+        case 7: return launch_one<3, true>(g, first, count, seed, sums, blocks, classes, verts, s);
         default: return cudaErrorInvalidValue;
     }
 }
 
 template <int STAGE, int RNG>
-cudaError_t launch_deferred_rng(const DevGraph &g, uint64_t first, uint64_t count, uint64_t seed, uint64_t *partials,
+cudaError_t launch_deferred_rng(const DevGraph &g, uint64_t first, uint64_t count, uint64_t seed, uint64_t *sums,
                                 int blocks, uint8_t *classes, uint32_t *verts, cudaStream_t s) {
     const bool rec = classes != nullptr;
     switch (probe_variant(2, g)) {
         case 2:
-            if (rec) k_sample_deferred<true, true, STAGE, kPmFilter, RNG><<<blocks, kThreads, 0, s>>>(g, first, count, seed, partials, classes, verts);
-            else k_sample_deferred<false, true, STAGE, kPmFilter, RNG><<<blocks, kThreads, 0, s>>>(g, first, count, seed, partials, classes, verts);
+            if (rec) k_sample_deferred<true, true, STAGE, kPmFilter, RNG><<<blocks, kThreads, 0, s>>>(g, first, count, seed, sums, classes, verts);
+            else k_sample_deferred<false, true, STAGE, kPmFilter, RNG><<<blocks, kThreads, 0, s>>>(g, first, count, seed, sums, classes, verts);
             break;
         case 3:
-            if (rec) k_sample_deferred<true, true, STAGE, kPmStream, RNG><<<blocks, kThreads, 0, s>>>(g, first, count, seed, partials, classes, verts);
-            else k_sample_deferred<false, true, STAGE, kPmStream, RNG><<<blocks, kThreads, 0, s>>>(g, first, count, seed, partials, classes, verts);
+            if (rec) k_sample_deferred<true, true, STAGE, kPmStream, RNG><<<blocks, kThreads, 0, s>>>(g, first, count, seed, sums, classes, verts);
+            else k_sample_deferred<false, true, STAGE, kPmStream, RNG><<<blocks, kThreads, 0, s>>>(g, first, count, seed, sums, classes, verts);
             break;
         case 1:
-            if (rec) k_sample_deferred<true, true, STAGE, kPmPlain, RNG><<<blocks, kThreads, 0, s>>>(g, first, count, seed, partials, classes, verts);
-            else k_sample_deferred<false, true, STAGE, kPmPlain, RNG><<<blocks, kThreads, 0, s>>>(g, first, count, seed, partials, classes, verts);
+            if (rec) k_sample_deferred<true, true, STAGE, kPmPlain, RNG><<<blocks, kThreads, 0, s>>>(g, first, count, seed, sums, classes, verts);
+            else k_sample_deferred<false, true, STAGE, kPmPlain, RNG><<<blocks, kThreads, 0, s>>>(g, first, count, seed, sums, classes, verts);
             break;
         default:
-            if (rec) k_sample_deferred<true, false, STAGE, kPmPlain, RNG><<<blocks, kThreads, 0, s>>>(g, first, count, seed, partials, classes, verts);
-            else k_sample_deferred<false, false, STAGE, kPmPlain, RNG><<<blocks, kThreads, 0, s>>>(g, first, count, seed, partials, classes, verts);
+            if (rec) k_sample_deferred<true, false, STAGE, kPmPlain, RNG><<<blocks, kThreads, 0, s>>>(g, first, count, seed, sums, classes, verts);
+            else k_sample_deferred<false, false, STAGE, kPmPlain, RNG><<<blocks, kThreads, 0, s>>>(g, first, count, seed, sums, classes, verts);
     }
     return cudaGetLastError();
 }
 
 template <int STAGE>
-cudaError_t launch_deferred(const DevGraph &g, uint64_t first, uint64_t count, uint64_t seed, uint64_t *partials,
+cudaError_t launch_deferred(const DevGraph &g, uint64_t first, uint64_t count, uint64_t seed, uint64_t *sums,
                             int blocks, uint8_t *classes, uint32_t *verts, cudaStream_t s) {
     if (g.rng == kRngPhilox)
-        return launch_deferred_rng<STAGE, kRngPhilox>(g, first, count, seed, partials, blocks, classes, verts, s);
-    return launch_deferred_rng<STAGE, kRngSplitMix>(g, first, count, seed, partials, blocks, classes, verts, s);
+        return launch_deferred_rng<STAGE, kRngPhilox>(g, first, count, seed, sums, blocks, classes, verts, s);
+    return launch_deferred_rng<STAGE, kRngSplitMix>(g, first, count, seed, sums, blocks, classes, verts, s);
 }
 
 // blocks of a deferred stage: its resident blocks per SM times the SMs
@@ -548,51 +512,36 @@ int defer_blocks(int device, int stage) {
 
 }  // namespace
 
-int sample_rows(int method, int device) {
-    return sample_blocks(method, device) + (method == 2 ? defer_blocks(device, 1) : 0);
+cudaError_t launch_redraws(const DevGraph &g, uint64_t first, uint64_t count, uint64_t seed, uint64_t *sums,
+                           uint8_t *classes, uint32_t *verts, cudaStream_t s) {
+    int dev = 0;
+    cudaGetDevice(&dev);
+    // no more blocks than there are windows of the bitmap for their warps
+    const uint64_t windows = (count + 1024ull * kWarps - 1) / (1024ull * kWarps);
+    const int d1 = (int)std::min<uint64_t>(defer_blocks(dev, 1), windows);
+    const int d2 = (int)std::min<uint64_t>(defer_blocks(dev, 2), windows);
+    const cudaError_t e = launch_deferred<1>(g, first, count, seed, sums, d1, classes, verts, s);
+    if (e != cudaSuccess) return e;
+    return launch_deferred<2>(g, first, count, seed, sums, d2, classes, verts, s);
 }
 
-cudaError_t launch_tail(int method, const DevGraph &g, uint64_t first, uint64_t count, uint64_t seed,
-                        uint64_t *partials, int blocks, uint8_t *classes, uint32_t *verts, uint64_t *counts_dev,
-                        bool accumulate, cudaStream_t s, CountRows *pending) {
-    int dev = 0, rows = blocks;
-    cudaGetDevice(&dev);
-    if (method == 2) {
-        // no more blocks than there are windows of the bitmap for their warps;
-        // the fallback stage adds into the first rows of the second-attempt stage
-        const uint64_t windows = (count + 1024ull * kWarps - 1) / (1024ull * kWarps);
-        const int d1 = (int)std::min<uint64_t>(defer_blocks(dev, 1), windows);
-        const int d2 = (int)std::min<uint64_t>(defer_blocks(dev, 2), d1);
-        uint64_t *drows = partials + (uint64_t)blocks * kSlots;
-        cudaError_t e;
-        if ((e = launch_deferred<1>(g, first, count, seed, drows, d1, classes, verts, s)) != cudaSuccess) return e;
-        if ((e = launch_deferred<2>(g, first, count, seed, drows, d2, classes, verts, s)) != cudaSuccess) return e;
-        rows += d1;
-    }
-    if (pending) {
-        *pending = CountRows{partials, rows, accumulate ? counts_dev : nullptr};
-        return cudaSuccess;
-    }
-    k_reduce<<<1, 32 * kSlots, 0, s>>>(partials, rows, counts_dev, accumulate ? 1 : 0);
+cudaError_t launch_copy_counts(const uint64_t *sums, uint64_t *out, cudaStream_t s) {
+    k_copy_counts<<<1, 32, 0, s>>>(sums, out);
     return cudaGetLastError();
 }
 
-cudaError_t launch_counts(int method, const DevGraph &g, uint64_t first, uint64_t count, uint64_t seed,
-                          uint64_t *partials, uint8_t *classes, uint32_t *verts, uint64_t *counts_dev,
-                          cudaStream_t s, CountRows *pending) {
+cudaError_t launch_counts(int method, const DevGraph &g, uint64_t first, uint64_t count, uint64_t seed, uint64_t *sums,
+                          uint8_t *classes, uint32_t *verts, cudaStream_t s) {
     int dev = 0;
     cudaGetDevice(&dev);
     const uint64_t chunk = method == 2 ? kDeferChunk : count;
     for (uint64_t c0 = 0; c0 < count; c0 += chunk) {
         const uint64_t len = std::min(chunk, count - c0);
-        // a block per 256 ids at most: every block leaves a row to add up
         const int blocks = (int)std::min<uint64_t>(sample_launch_blocks(method, dev, g), (len + kThreads - 1) / kThreads);
         uint8_t *cl = classes ? classes + c0 : nullptr;
         uint32_t *vt = verts ? verts + 5 * c0 : nullptr;
-        cudaError_t e = launch_sample(method, g, first + c0, len, seed, partials, blocks, cl, vt, s);
-        if (e == cudaSuccess)
-            e = launch_tail(method, g, first + c0, len, seed, partials, blocks, cl, vt, counts_dev, c0 > 0, s,
-                            c0 + len == count ? pending : nullptr);
+        cudaError_t e = launch_sample(method, g, first + c0, len, seed, sums, blocks, cl, vt, s);
+        if (e == cudaSuccess && method == 2) e = launch_redraws(g, first + c0, len, seed, sums, cl, vt, s);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
@@ -605,10 +554,10 @@ constexpr int kPairBlocks = 4;   // resident blocks per SM (Path-5 with its redr
 
 template <bool MIX, int RNG>
 cudaError_t launch_pair_rng(const DevGraph &g, int blocks, int blocks_a, uint64_t count_a, uint64_t count_b,
-                            uint64_t seed, uint64_t *partials, cudaStream_t s) {
-    if (!g.hash) k_sample_pair<MIX, false, kPmPlain, RNG><<<blocks, kThreads, 0, s>>>(g, blocks_a, count_a, count_b, seed, partials);
-    else if (g.filter) k_sample_pair<MIX, true, kPmFilter, RNG><<<blocks, kThreads, 0, s>>>(g, blocks_a, count_a, count_b, seed, partials);
-    else k_sample_pair<MIX, true, kPmPlain, RNG><<<blocks, kThreads, 0, s>>>(g, blocks_a, count_a, count_b, seed, partials);
+                            uint64_t seed, uint64_t *sums, cudaStream_t s) {
+    if (!g.hash) k_sample_pair<MIX, false, kPmPlain, RNG><<<blocks, kThreads, 0, s>>>(g, blocks_a, count_a, count_b, seed, sums);
+    else if (g.filter) k_sample_pair<MIX, true, kPmFilter, RNG><<<blocks, kThreads, 0, s>>>(g, blocks_a, count_a, count_b, seed, sums);
+    else k_sample_pair<MIX, true, kPmPlain, RNG><<<blocks, kThreads, 0, s>>>(g, blocks_a, count_a, count_b, seed, sums);
     return cudaGetLastError();
 }
 
@@ -627,9 +576,8 @@ bool pair_fits(bool mix, uint64_t count_a, uint64_t count_b) {
     return count_a <= most && count_b <= most;
 }
 
-cudaError_t launch_pair(bool mix, const DevGraph &g, uint64_t count_a, uint64_t count_b, uint64_t seed,
-                        uint64_t *partials, CountRows *a, CountRows *b, cudaStream_t s) {
-    *a = *b = CountRows{};
+cudaError_t launch_pair(bool mix, const DevGraph &g, uint64_t count_a, uint64_t count_b, uint64_t seed, uint64_t *sums,
+                        cudaStream_t s) {
     if (count_a + count_b == 0) return cudaSuccess;
     // a block per 256 ids, or the resident blocks split in proportion
     const uint64_t most = (uint64_t)current_sms() * kPairBlocks;
@@ -640,13 +588,11 @@ cudaError_t launch_pair(bool mix, const DevGraph &g, uint64_t count_a, uint64_t 
         na = share;
     }
     const int blocks = (int)(na + nb);
-    *a = CountRows{partials, (int)na, nullptr};
-    *b = CountRows{partials + na * kSlots, (int)nb, nullptr};
     if (g.rng == kRngPhilox)
-        return mix ? launch_pair_rng<true, kRngPhilox>(g, blocks, (int)na, count_a, count_b, seed, partials, s)
-                   : launch_pair_rng<false, kRngPhilox>(g, blocks, (int)na, count_a, count_b, seed, partials, s);
-    return mix ? launch_pair_rng<true, kRngSplitMix>(g, blocks, (int)na, count_a, count_b, seed, partials, s)
-               : launch_pair_rng<false, kRngSplitMix>(g, blocks, (int)na, count_a, count_b, seed, partials, s);
+        return mix ? launch_pair_rng<true, kRngPhilox>(g, blocks, (int)na, count_a, count_b, seed, sums, s)
+                   : launch_pair_rng<false, kRngPhilox>(g, blocks, (int)na, count_a, count_b, seed, sums, s);
+    return mix ? launch_pair_rng<true, kRngSplitMix>(g, blocks, (int)na, count_a, count_b, seed, sums, s)
+               : launch_pair_rng<false, kRngSplitMix>(g, blocks, (int)na, count_a, count_b, seed, sums, s);
 }
 
 template <int T>

@@ -658,6 +658,20 @@ __device__ __forceinline__ Sample sample_path5(const DevGraph &g, const uint8_t 
     return rest_path5<RNG, HASH, STAGE, PM>(g, lut, seed, s, first_vertex<2, RNG, PM>(g, seed, s));
 }
 
+// The block's counts (its warps' histograms) added to the launch's sums, which
+// are zero before it: whole numbers, so any order of the blocks gives the same.
+// With a row per block and a kernel to add up the rows, an estimate of 5e6
+// samples on a 2M-edge mesh took 448 us (440 like this), one of 1e4 on 8k edges
+// 40.7 (39.1): a block's 22 adds go beside other blocks' samples.
+template <int WARPS>
+__device__ __forceinline__ void add_sums(const uint32_t (&hist)[WARPS][kSlots], uint64_t *sums) {
+    if (threadIdx.x < kSlots) {
+        uint64_t sum = 0;
+        for (int w = 0; w < WARPS; ++w) sum += hist[w][threadIdx.x];
+        if (sum) atomicAdd(reinterpret_cast<unsigned long long *>(sums) + threadIdx.x, (unsigned long long)sum);
+    }
+}
+
 // the class tables of this translation unit on the current device
 inline void upload_luts_here(const uint8_t *lut4, const uint8_t *lut5, const uint8_t *lutc) {
     cudaMemcpyToSymbol(g_lut4, lut4, 64);
