@@ -176,7 +176,7 @@ constexpr int group_blocks() { return RNG == kRngPhilox ? 5 : 6; }
 
 // The samples of the entries in order, a thread each; Path-5 samples whose
 // first pair of sigma draws collides are flagged in the (zeroed) deferral
-// bitmap for the redraw stages.
+// bitmap for the redraws.
 template <int METHOD, int RNG>
 __global__ void __launch_bounds__(kThreads, group_blocks<RNG>())
     k_sample_group(DevGraph g, uint64_t first, uint32_t count, uint64_t seed, const uint2 *entries,

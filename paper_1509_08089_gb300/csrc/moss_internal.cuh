@@ -405,10 +405,10 @@ void upload_luts(const uint8_t *lut4, const uint8_t *lut5, const uint8_t *lutc);
 // Counts (added to the 22 uint64 at sums) of samples [first, first+count) of one
 // method, with optional per-sample records (classes, verts: count and 5*count
 // entries).  Path-5 runs in chunks of kDeferChunk ids: a launch that defers
-// the samples whose first sigma attempt collides and two that redraw them.
+// the samples whose first sigma attempt collides and one that redraws them.
 cudaError_t launch_counts(int method, const DevGraph &g, uint64_t first, uint64_t count, uint64_t seed, uint64_t *sums,
                           uint8_t *classes, uint32_t *verts, cudaStream_t s);
-// the redraw stages of one chunk, adding to sums
+// the redraws of one chunk, adding to sums
 cudaError_t launch_redraws(const DevGraph &g, uint64_t first, uint64_t count, uint64_t seed, uint64_t *sums,
                            uint8_t *classes, uint32_t *verts, cudaStream_t s);
 cudaError_t launch_copy_counts(const uint64_t *sums, uint64_t *out, cudaStream_t s);

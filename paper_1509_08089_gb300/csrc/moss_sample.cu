@@ -42,17 +42,15 @@ namespace {
 // memory latency, so more warps in flight help until register spills cost
 // more than they hide (measured: 6 blocks of 256 threads for every main
 // sampler; Path-5 reaches it only with its second attempt and fallback
-// deferred).  The second-attempt launch runs 5 blocks, the fallback launch 4.
-// Under Philox words the samplers and the redraw stages hold the generator's
-// state beside their records and would spill at those register budgets, so
-// they are compiled for one block fewer (4 for the redraws); the grid of a
-// main launch follows each instance's occupancy.
+// deferred).  Under Philox words they hold the generator's state beside their
+// records and would spill at that register budget, so they are compiled for
+// one block fewer; the grid of a launch follows each instance's occupancy.
 template <int METHOD, int RNG>
 constexpr int min_blocks() { return RNG == kRngPhilox ? 5 : 6; }
-template <int STAGE>
-constexpr int defer_min_blocks() { return STAGE == 1 ? 5 : 4; }
-template <int STAGE, int RNG>
-constexpr int defer_bound_blocks() { return RNG == kRngPhilox ? 4 : defer_min_blocks<STAGE>(); }
+// The redraw launch: five blocks (48 registers) where that spills nothing, four
+// with the filter's probes or the generator's state.
+template <int PM, int RNG>
+constexpr int redraw_blocks() { return PM == kPmFilter || RNG == kRngPhilox ? 4 : 5; }
 
 template <int METHOD, bool RECORD, bool HASH, int PM, int RNG>
 __global__ void __launch_bounds__(kThreads, min_blocks<METHOD, RNG>()) k_sample(DevGraph g, uint64_t first, uint64_t count, uint64_t seed,
@@ -107,77 +105,77 @@ __global__ void __launch_bounds__(kThreads, min_blocks<METHOD, RNG>()) k_sample(
     add_sums<kWarps>(hist, sums);
 }
 
-// The Path-5 samples a launch deferred, redrawn by the next stage (STAGE 1:
-// second attempt, re-deferring the samples that collide again; STAGE 2:
-// fallback).  A warp takes windows of 32 bitmap words (grid-stride); it
-// appends each window's flagged ids to a list in shared memory (a warp scan
-// of the words' popcounts places them) and draws from the list 32 at a time,
-// one per lane, keeping fewer than 32 ids over to its next window, so every
-// round but the warp's last runs with all lanes busy however sparse the
-// flags.  STAGE 1 clears the words it reads and sets the bits of re-deferred
-// samples again (plain stores: a window's words belong to one warp).  Counts
-// are aggregated as in k_sample.
+// The Path-5 samples a launch deferred: their second attempt and, for those
+// that collide again, the fallback.  A warp takes windows of `window` (up to
+// 32) bitmap words, grid-stride; it appends each window's flagged ids to a
+// list in shared memory (a warp scan of the words' popcounts places them) and
+// draws from the list 32 at a time, one per lane, keeping fewer than 32 ids
+// over to its next window; ids that collide again go to a second list, drawn
+// in the same way.  So every round but the warp's last ones runs with all
+// lanes busy however sparse the flags.  Bound by the rounds' chains of
+// dependent gathers, with few warps' rounds in flight.  As two launches with
+// 32-word windows (the fallback after every second attempt) it took 62 us of a
+// 2M-edge mesh's estimate of 5e6 samples and 136 us of a 1M-edge graph's of
+// 1e8; the estimates as a whole, two launches -> this one: 449 -> 433 us and
+// 4.031 -> 4.013 ms.
 constexpr uint32_t kDeferList = 1024 + 32;   // a window's ids plus the carry-over
+constexpr uint32_t kAgainList = 64;          // fewer than 32 waiting plus a round's
 
-template <bool RECORD, bool HASH, int STAGE, int PM, int RNG>
-__global__ void __launch_bounds__(kThreads, defer_bound_blocks<STAGE, RNG>())
-    k_sample_deferred(DevGraph g, uint64_t first, uint64_t count, uint64_t seed, uint64_t *sums,
+template <bool RECORD, bool HASH, int PM, int RNG>
+__global__ void __launch_bounds__(kThreads, redraw_blocks<PM, RNG>())
+    k_sample_deferred(DevGraph g, uint64_t first, uint64_t count, uint32_t window, uint64_t seed, uint64_t *sums,
                       uint8_t *classes, uint32_t *verts) {
-    static_assert(STAGE == 1 || STAGE == 2, "deferred stages are 1 and 2");
     __shared__ uint8_t lut[kLut];
     __shared__ uint32_t hist[kWarps][kSlots];
-    __shared__ uint32_t list[kWarps][kDeferList];   // ids relative to the chunk's first
+    __shared__ uint32_t list[kWarps][kDeferList], again[kWarps][kAgainList];   // ids relative to the chunk's first
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int i = threadIdx.x; i < kLut; i += kThreads) lut[i] = g_lut5[i];
     for (int i = threadIdx.x; i < kWarps * kSlots; i += kThreads) (&hist[0][0])[i] = 0;
     __syncthreads();
     const uint64_t words = (count + 31) / 32;
-    const uint64_t stride = (uint64_t)gridDim.x * kWarps * 32;
-    uint32_t *lst = list[warp];
-    // draws lst[k0 + lane] for lane < cnt (warp-uniform arguments)
-    auto round = [&](uint32_t k0, uint32_t cnt) {
-        int cls = kSlots;
-        bool again = false;
-        uint64_t i = 0;
-        if ((uint32_t)lane < cnt) {
-            i = lst[k0 + lane];   // < count: only drawn ids are flagged
-            const Sample sm = sample_path5<RNG, HASH, STAGE, PM>(g, lut, seed, first + i);
-            again = STAGE == 1 && sm.cls == kDeferred;
-            if (!again) {
-                cls = sm.cls;
-                if (RECORD) {
-                    classes[i] = (uint8_t)sm.cls;
-                    if (verts) {
+    const uint64_t stride = (uint64_t)gridDim.x * kWarps * window;
+    uint32_t *lst = list[warp], *agn = again[warp];
+    // counts (and records) the lanes' samples; kDeferred ones are left out
+    auto put = [&](bool drawn, uint32_t i, const Sample &sm) {
+        const int cls = drawn && sm.cls != kDeferred ? sm.cls : kSlots;
+        if (RECORD && cls < kSlots) {
+            classes[i] = (uint8_t)cls;
+            if (verts) {
 #pragma unroll
-                        for (int k = 0; k < 5; ++k) verts[5 * i + k] = sm.v[k];
-                    }
-                }
+                for (int k = 0; k < 5; ++k) verts[5ull * i + k] = sm.v[k];
             }
-        }
-        if (STAGE == 1 && __any_sync(0xffffffffu, again)) {
-            // OR of the re-deferred bits per word; the first lane of each word stores it
-            const uint64_t wi = again ? i >> 5 : ~0ull;
-            const uint32_t bit = again ? 1u << (i & 31) : 0u;
-            uint32_t bits = 0, first_lane = 32;
-            for (int l = 0; l < 32; ++l) {
-                const uint64_t wl = __shfl_sync(0xffffffffu, wi, l);
-                const uint32_t bl = __shfl_sync(0xffffffffu, bit, l);
-                if (wl == wi) {
-                    bits |= bl;
-                    first_lane = min(first_lane, (uint32_t)l);
-                }
-            }
-            if (again && first_lane == (uint32_t)lane) g.defer[wi] |= bits;
-            __syncwarp();
         }
         const uint32_t peers = __match_any_sync(0xffffffffu, cls);
         if (cls < kSlots && lane == __ffs(peers) - 1) atomicAdd(&hist[warp][cls], (uint32_t)__popc(peers));
     };
-    uint32_t n = 0;   // ids waiting in the list (warp-uniform, < 32 between windows)
-    for (uint64_t w0 = ((uint64_t)blockIdx.x * kWarps + warp) * 32; w0 < words; w0 += stride) {
+    // the fallback of agn[from + lane] for lane < cnt (warp-uniform arguments)
+    auto fallback = [&](uint32_t from, uint32_t cnt) {
+        const bool mine = (uint32_t)lane < cnt;
+        const uint32_t i = mine ? agn[from + lane] : 0u;   // < count: only drawn ids are flagged
+        Sample sm;
+        if (mine) sm = sample_path5<RNG, HASH, 2, PM>(g, lut, seed, first + i);
+        put(mine, i, sm);
+        __syncwarp();   // the places are free again
+    };
+    uint32_t m = 0;   // ids waiting in agn (warp-uniform, < 32 between rounds)
+    // the second attempt of lst[from + lane] for lane < cnt
+    auto attempt = [&](uint32_t from, uint32_t cnt) {
+        const bool mine = (uint32_t)lane < cnt;
+        const uint32_t i = mine ? lst[from + lane] : 0u;
+        Sample sm;
+        if (mine) sm = sample_path5<RNG, HASH, 1, PM>(g, lut, seed, first + i);
+        put(mine, i, sm);
+        const bool back = mine && sm.cls == kDeferred;
+        const uint32_t bits = __ballot_sync(0xffffffffu, back);
+        if (back) agn[m + __popc(bits & ((1u << lane) - 1u))] = i;
+        __syncwarp();
+        m += __popc(bits);
+        if (m >= 32) fallback(m -= 32, 32);
+    };
+    uint32_t n = 0;   // ids waiting in lst (warp-uniform, < 32 between windows)
+    for (uint64_t w0 = ((uint64_t)blockIdx.x * kWarps + warp) * window; w0 < words; w0 += stride) {
         const uint64_t w = w0 + lane;
-        uint32_t bits = w < words ? __ldcs(g.defer + w) : 0u;
-        if (STAGE == 1 && bits) g.defer[w] = 0u;   // re-deferred ids are set again by round()
+        uint32_t bits = (uint32_t)lane < window && w < words ? __ldcs(g.defer + w) : 0u;
         const uint32_t c = __popc(bits);
         uint32_t incl = c;
 #pragma unroll
@@ -194,7 +192,7 @@ __global__ void __launch_bounds__(kThreads, defer_bound_blocks<STAGE, RNG>())
         n += total;
         __syncwarp();
         uint32_t done = 0;
-        for (; n - done >= 32; done += 32) round(done, 32);
+        for (; n - done >= 32; done += 32) attempt(done, 32);
         if (done) {   // move the remainder (< 32 ids) to the front
             const uint32_t rem = n - done;
             const uint32_t x = (uint32_t)lane < rem ? lst[done + lane] : 0u;
@@ -204,7 +202,8 @@ __global__ void __launch_bounds__(kThreads, defer_bound_blocks<STAGE, RNG>())
             n = rem;
         }
     }
-    if (n) round(0, n);
+    if (n) attempt(0, n);
+    if (m) fallback(0, m);
     __syncthreads();
     add_sums<kWarps>(hist, sums);
 }
@@ -473,56 +472,39 @@ cudaError_t launch_sample(int method, const DevGraph &g, uint64_t first, uint64_
     }
 }
 
-template <int STAGE, int RNG>
-cudaError_t launch_deferred_rng(const DevGraph &g, uint64_t first, uint64_t count, uint64_t seed, uint64_t *sums,
-                                int blocks, uint8_t *classes, uint32_t *verts, cudaStream_t s) {
-    const bool rec = classes != nullptr;
-    switch (probe_variant(2, g)) {
-        case 2:
-            if (rec) k_sample_deferred<true, true, STAGE, kPmFilter, RNG><<<blocks, kThreads, 0, s>>>(g, first, count, seed, sums, classes, verts);
-            else k_sample_deferred<false, true, STAGE, kPmFilter, RNG><<<blocks, kThreads, 0, s>>>(g, first, count, seed, sums, classes, verts);
-            break;
-        case 3:
-            if (rec) k_sample_deferred<true, true, STAGE, kPmStream, RNG><<<blocks, kThreads, 0, s>>>(g, first, count, seed, sums, classes, verts);
-            else k_sample_deferred<false, true, STAGE, kPmStream, RNG><<<blocks, kThreads, 0, s>>>(g, first, count, seed, sums, classes, verts);
-            break;
-        case 1:
-            if (rec) k_sample_deferred<true, true, STAGE, kPmPlain, RNG><<<blocks, kThreads, 0, s>>>(g, first, count, seed, sums, classes, verts);
-            else k_sample_deferred<false, true, STAGE, kPmPlain, RNG><<<blocks, kThreads, 0, s>>>(g, first, count, seed, sums, classes, verts);
-            break;
-        default:
-            if (rec) k_sample_deferred<true, false, STAGE, kPmPlain, RNG><<<blocks, kThreads, 0, s>>>(g, first, count, seed, sums, classes, verts);
-            else k_sample_deferred<false, false, STAGE, kPmPlain, RNG><<<blocks, kThreads, 0, s>>>(g, first, count, seed, sums, classes, verts);
-    }
+template <bool HASH, int PM, int RNG>
+cudaError_t launch_deferred(const DevGraph &g, uint64_t first, uint64_t count, uint64_t seed, uint64_t *sums,
+                            uint8_t *classes, uint32_t *verts, cudaStream_t s) {
+    // windows of 32 words, or smaller ones that give every resident warp one:
+    // a warp draws its window's ids one round of 32 after the other
+    const uint64_t warps = (uint64_t)current_sms() * redraw_blocks<PM, RNG>() * kWarps, words = (count + 31) / 32;
+    const uint32_t window = (uint32_t)std::min<uint64_t>(32, (words + warps - 1) / warps);
+    const uint64_t windows = (words + window - 1) / window;
+    const int blocks = (int)std::min<uint64_t>(warps / kWarps, (windows + kWarps - 1) / kWarps);
+    if (classes)
+        k_sample_deferred<true, HASH, PM, RNG><<<blocks, kThreads, 0, s>>>(g, first, count, window, seed, sums, classes, verts);
+    else
+        k_sample_deferred<false, HASH, PM, RNG><<<blocks, kThreads, 0, s>>>(g, first, count, window, seed, sums, classes, verts);
     return cudaGetLastError();
 }
 
-template <int STAGE>
-cudaError_t launch_deferred(const DevGraph &g, uint64_t first, uint64_t count, uint64_t seed, uint64_t *sums,
-                            int blocks, uint8_t *classes, uint32_t *verts, cudaStream_t s) {
-    if (g.rng == kRngPhilox)
-        return launch_deferred_rng<STAGE, kRngPhilox>(g, first, count, seed, sums, blocks, classes, verts, s);
-    return launch_deferred_rng<STAGE, kRngSplitMix>(g, first, count, seed, sums, blocks, classes, verts, s);
-}
-
-// blocks of a deferred stage: its resident blocks per SM times the SMs
-int defer_blocks(int device, int stage) {
-    return device_sms(device) * (stage == 1 ? defer_min_blocks<1>() : defer_min_blocks<2>());
+template <int RNG>
+cudaError_t launch_deferred_rng(const DevGraph &g, uint64_t first, uint64_t count, uint64_t seed, uint64_t *sums,
+                                uint8_t *classes, uint32_t *verts, cudaStream_t s) {
+    switch (probe_variant(2, g)) {
+        case 2: return launch_deferred<true, kPmFilter, RNG>(g, first, count, seed, sums, classes, verts, s);
+        case 3: return launch_deferred<true, kPmStream, RNG>(g, first, count, seed, sums, classes, verts, s);
+        case 1: return launch_deferred<true, kPmPlain, RNG>(g, first, count, seed, sums, classes, verts, s);
+        default: return launch_deferred<false, kPmPlain, RNG>(g, first, count, seed, sums, classes, verts, s);
+    }
 }
 
 }  // namespace
 
 cudaError_t launch_redraws(const DevGraph &g, uint64_t first, uint64_t count, uint64_t seed, uint64_t *sums,
                            uint8_t *classes, uint32_t *verts, cudaStream_t s) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    // no more blocks than there are windows of the bitmap for their warps
-    const uint64_t windows = (count + 1024ull * kWarps - 1) / (1024ull * kWarps);
-    const int d1 = (int)std::min<uint64_t>(defer_blocks(dev, 1), windows);
-    const int d2 = (int)std::min<uint64_t>(defer_blocks(dev, 2), windows);
-    const cudaError_t e = launch_deferred<1>(g, first, count, seed, sums, d1, classes, verts, s);
-    if (e != cudaSuccess) return e;
-    return launch_deferred<2>(g, first, count, seed, sums, d2, classes, verts, s);
+    if (g.rng == kRngPhilox) return launch_deferred_rng<kRngPhilox>(g, first, count, seed, sums, classes, verts, s);
+    return launch_deferred_rng<kRngSplitMix>(g, first, count, seed, sums, classes, verts, s);
 }
 
 cudaError_t launch_copy_counts(const uint64_t *sums, uint64_t *out, cudaStream_t s) {
