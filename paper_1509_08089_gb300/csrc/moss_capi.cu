@@ -853,7 +853,7 @@ int moss_vertex_levels(const moss_graph *g, int which, uint32_t *nheavy, uint64_
 
 // adds the counts to the kSlots at sums (device memory of the graph); records
 static int sample_into(moss_graph *g, int method, uint64_t first, uint64_t count, uint64_t seed, cudaStream_t s,
-                       uint64_t *sums, uint8_t *classes, uint32_t *verts) {
+                       uint64_t *sums, uint8_t *classes, uint32_t *verts, bool early = false) {
     if (method < 0 || method >= kMethods) return fail(MOSS_EINVAL, "method %d", method);
     if (!method_ready(g, method)) return fail(MOSS_ESTATE, "tables for method %d not built", method);
     if (count > 0 && g->tot_h.gamma[method] == 0)
@@ -879,7 +879,7 @@ static int sample_into(moss_graph *g, int method, uint64_t first, uint64_t count
         }
         cudaGetLastError();   // no memory: the general path
     }
-    MOSS_CUDA(launch_counts(method, dv, first, count, seed, sums, classes, verts, s), "sample kernels");
+    MOSS_CUDA(launch_counts(method, dv, first, count, seed, sums, classes, verts, s, early), "sample kernels");
     return MOSS_OK;
 }
 
@@ -896,7 +896,7 @@ int moss_sample_counts(moss_graph *g, int method, uint64_t first, uint64_t count
     const cudaStream_t s = static_cast<cudaStream_t>(stream);
     int rc = clear_sums(g, 1, s);
     if (rc || (rc = sample_into(g, method, first, count, seed, s, g->counts, nullptr, nullptr))) return rc;
-    MOSS_CUDA(launch_copy_counts(g->counts, counts_dev, s), "copying counts");
+    MOSS_CUDA(launch_copy_counts(g->counts, counts_dev, count > 0, s), "copying counts");
     return MOSS_OK;
 }
 
@@ -924,15 +924,19 @@ static int sample_both(moss_graph *g, int ma, uint64_t ka, int mb, uint64_t kb, 
         MOSS_CUDA(launch_pair(mix, view(g), ka, kb, seed, g->counts, s), "sample kernels");
         return MOSS_OK;
     }
+    // the second method's blocks come in as the first's leave (after a grouped
+    // launch, whose scratch is being given back, they start in order)
     rc = sample_into(g, ma, 0, ka, seed, s, g->counts, nullptr, nullptr);
-    return rc ? rc : sample_into(g, mb, 0, kb, seed, s, g->counts + kSlots, nullptr, nullptr);
+    const bool early = ka != 0 && group_bytes(ma, view(g), g->order != nullptr, ka) == 0;
+    return rc ? rc : sample_into(g, mb, 0, kb, seed, s, g->counts + kSlots, nullptr, nullptr, early);
 }
 
 // the result of the counts at g->counts
 static int finalize_sums(moss_graph *g, const FinalizeIn &in, cudaStream_t s, moss_result *out) {
+    const bool drawn = in.K[0] || in.K[1];   // the launch before is a kernel
     HitsArg hits;
     hits.dev = g->counts;
-    MOSS_CUDA(launch_finalize(in, hits, g->tot, result_target(g), nullptr, s), "finalize kernel");
+    MOSS_CUDA(launch_finalize(in, hits, g->tot, result_target(g), nullptr, s, drawn), "finalize kernel");
     return read_result(g, s, out);
 }
 

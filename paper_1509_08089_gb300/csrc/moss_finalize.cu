@@ -322,6 +322,7 @@ __device__ void finalize_any(const FinalizeIn &in, const uint64_t *hits0, const 
 __global__ void k_finalize(FinalizeIn in, const __grid_constant__ HitsArg hits, const DevTotals *tot, moss_result *out,
                            double *cov) {
     const int row = blockIdx.x;
+    await_previous();
     const uint64_t *h = hits.dev ? hits.dev : hits.h;
     finalize_any(in, h, h + kSlots, tot, row == 0 ? out : nullptr, cov, row);
 }
@@ -341,9 +342,8 @@ __global__ void k_finalize_batch(const BatchRequest *reqs, int nreq, const uint6
 }  // namespace
 
 cudaError_t launch_finalize(const FinalizeIn &in, const HitsArg &hits, const DevTotals *tot, void *result, double *cov,
-                            cudaStream_t s) {
-    k_finalize<<<cov ? kSlots : 1, 32, 0, s>>>(in, hits, tot, static_cast<moss_result *>(result), cov);
-    return cudaGetLastError();
+                            cudaStream_t s, bool early) {
+    return launch_early(early, k_finalize, cov ? kSlots : 1, 32, s, in, hits, tot, static_cast<moss_result *>(result), cov);
 }
 
 cudaError_t launch_finalize_batch(const BatchRequest *reqs, int nreq, const uint64_t *task_counts, void *results,

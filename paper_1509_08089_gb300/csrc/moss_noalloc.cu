@@ -88,7 +88,7 @@ extern "C" int moss_sample_counts_noalloc(moss_graph *g, int method, uint64_t fi
         } else {
             e = cudaMemsetAsync(sums, 0, kSlots * sizeof(uint64_t), s);
             if (e == cudaSuccess) e = launch_counts(method, gi.view, first, count, seed, sums, nullptr, nullptr, s);
-            if (e == cudaSuccess) e = launch_copy_counts(sums, counts_dev, s);
+            if (e == cudaSuccess) e = launch_copy_counts(sums, counts_dev, true, s);
         }
         if (e != cudaSuccess) rc = set_error(MOSS_ECUDA, cudaGetErrorString(e));
     }

@@ -58,6 +58,7 @@ __global__ void __launch_bounds__(kThreads, min_blocks<METHOD, RNG>()) k_sample(
     __shared__ uint8_t lut[kLut];
     __shared__ uint8_t lutc[METHOD == 3 ? 4096 : 1];
     __shared__ uint32_t hist[kWarps][kSlots];
+    let_next_begin();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint8_t *src = (METHOD == 0 || METHOD == 3) ? g_lut4 : g_lut5;
     const int lut_n = (METHOD == 0 || METHOD == 3) ? 64 : 1024;
@@ -102,6 +103,7 @@ __global__ void __launch_bounds__(kThreads, min_blocks<METHOD, RNG>()) k_sample(
         if (cls < kSlots && lane == __ffs(peers) - 1) atomicAdd(&hist[warp][cls], (uint32_t)__popc(peers));
     }
     __syncthreads();
+    await_previous();
     add_sums<kWarps>(hist, sums);
 }
 
@@ -128,10 +130,12 @@ __global__ void __launch_bounds__(kThreads, redraw_blocks<PM, RNG>())
     __shared__ uint8_t lut[kLut];
     __shared__ uint32_t hist[kWarps][kSlots];
     __shared__ uint32_t list[kWarps][kDeferList], again[kWarps][kAgainList];   // ids relative to the chunk's first
+    let_next_begin();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int i = threadIdx.x; i < kLut; i += kThreads) lut[i] = g_lut5[i];
     for (int i = threadIdx.x; i < kWarps * kSlots; i += kThreads) (&hist[0][0])[i] = 0;
     __syncthreads();
+    await_previous();
     const uint64_t words = (count + 31) / 32;
     const uint64_t stride = (uint64_t)gridDim.x * kWarps * window;
     uint32_t *lst = list[warp], *agn = again[warp];
@@ -315,6 +319,7 @@ __global__ void k_batch_reduce(const BatchTask *tasks, uint32_t tile_samples, co
 }
 
 __global__ void k_copy_counts(const uint64_t *sums, uint64_t *out) {
+    await_previous();
     if (threadIdx.x < kSlots) out[threadIdx.x] = sums[threadIdx.x];
 }
 
@@ -330,6 +335,7 @@ __global__ void __launch_bounds__(kThreads, 4)
     __shared__ uint8_t lut[MIX ? 64 : kLut];
     __shared__ uint8_t lutc[MIX ? 4096 : 1];
     __shared__ uint32_t hist[kWarps][kSlots];
+    let_next_begin();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int i = threadIdx.x; i < (MIX ? 64 : kLut); i += kThreads) lut[i] = MIX ? g_lut4[i] : g_lut5[i];
     if (MIX)
@@ -369,30 +375,24 @@ int probe_variant(int method, const DevGraph &g) {
 }
 
 template <int M, bool R, int RNG>
-cudaError_t launch_one_rng(const DevGraph &g, uint64_t first, uint64_t count, uint64_t seed, uint64_t *sums,
-                           int blocks, uint8_t *classes, uint32_t *verts, cudaStream_t s) {
+cudaError_t launch_one_rng(const DevGraph &g, uint64_t first, uint64_t count, uint64_t seed, uint64_t *sums, int blocks,
+                           uint8_t *classes, uint32_t *verts, cudaStream_t s, bool early) {
+    auto *k = &k_sample<M, R, false, kPmPlain, RNG>;
     switch (probe_variant(M, g)) {
-        case 2:
-            k_sample<M, R, true, kPmFilter, RNG><<<blocks, kThreads, 0, s>>>(g, first, count, seed, sums, classes, verts);
-            break;
-        case 3:
-            k_sample<M, R, true, kPmStream, RNG><<<blocks, kThreads, 0, s>>>(g, first, count, seed, sums, classes, verts);
-            break;
-        case 1:
-            k_sample<M, R, true, kPmPlain, RNG><<<blocks, kThreads, 0, s>>>(g, first, count, seed, sums, classes, verts);
-            break;
-        default:
-            k_sample<M, R, false, kPmPlain, RNG><<<blocks, kThreads, 0, s>>>(g, first, count, seed, sums, classes, verts);
+        case 2: k = &k_sample<M, R, true, kPmFilter, RNG>; break;
+        case 3: k = &k_sample<M, R, true, kPmStream, RNG>; break;
+        case 1: k = &k_sample<M, R, true, kPmPlain, RNG>; break;
+        default: break;
     }
-    return cudaGetLastError();
+    return launch_early(early, k, blocks, kThreads, s, g, first, count, seed, sums, classes, verts);
 }
 
 template <int M, bool R>
-cudaError_t launch_one(const DevGraph &g, uint64_t first, uint64_t count, uint64_t seed, uint64_t *sums,
-                       int blocks, uint8_t *classes, uint32_t *verts, cudaStream_t s) {
+cudaError_t launch_one(const DevGraph &g, uint64_t first, uint64_t count, uint64_t seed, uint64_t *sums, int blocks,
+                       uint8_t *classes, uint32_t *verts, cudaStream_t s, bool early) {
     if (g.rng == kRngPhilox)
-        return launch_one_rng<M, R, kRngPhilox>(g, first, count, seed, sums, blocks, classes, verts, s);
-    return launch_one_rng<M, R, kRngSplitMix>(g, first, count, seed, sums, blocks, classes, verts, s);
+        return launch_one_rng<M, R, kRngPhilox>(g, first, count, seed, sums, blocks, classes, verts, s, early);
+    return launch_one_rng<M, R, kRngSplitMix>(g, first, count, seed, sums, blocks, classes, verts, s, early);
 }
 
 }  // namespace
@@ -457,17 +457,17 @@ int sample_launch_blocks(int method, int device, const DevGraph &g) {
 namespace {
 
 cudaError_t launch_sample(int method, const DevGraph &g, uint64_t first, uint64_t count, uint64_t seed,
-                          uint64_t *sums, int blocks, uint8_t *classes, uint32_t *verts, cudaStream_t s) {
+                          uint64_t *sums, int blocks, uint8_t *classes, uint32_t *verts, cudaStream_t s, bool early) {
     const bool rec = classes != nullptr;
     switch (method * 2 + (rec ? 1 : 0)) {
-        case 0: return launch_one<0, false>(g, first, count, seed, sums, blocks, classes, verts, s);
-        case 1: return launch_one<0, true>(g, first, count, seed, sums, blocks, classes, verts, s);
-        case 2: return launch_one<1, false>(g, first, count, seed, sums, blocks, classes, verts, s);
-        case 3: return launch_one<1, true>(g, first, count, seed, sums, blocks, classes, verts, s);
-        case 4: return launch_one<2, false>(g, first, count, seed, sums, blocks, classes, verts, s);
-        case 5: return launch_one<2, true>(g, first, count, seed, sums, blocks, classes, verts, s);
-        case 6: return launch_one<3, false>(g, first, count, seed, sums, blocks, classes, verts, s);
-        case 7: return launch_one<3, true>(g, first, count, seed, sums, blocks, classes, verts, s);
+        case 0: return launch_one<0, false>(g, first, count, seed, sums, blocks, classes, verts, s, early);
+        case 1: return launch_one<0, true>(g, first, count, seed, sums, blocks, classes, verts, s, early);
+        case 2: return launch_one<1, false>(g, first, count, seed, sums, blocks, classes, verts, s, early);
+        case 3: return launch_one<1, true>(g, first, count, seed, sums, blocks, classes, verts, s, early);
+        case 4: return launch_one<2, false>(g, first, count, seed, sums, blocks, classes, verts, s, early);
+        case 5: return launch_one<2, true>(g, first, count, seed, sums, blocks, classes, verts, s, early);
+        case 6: return launch_one<3, false>(g, first, count, seed, sums, blocks, classes, verts, s, early);
+        case 7: return launch_one<3, true>(g, first, count, seed, sums, blocks, classes, verts, s, early);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -481,11 +481,8 @@ cudaError_t launch_deferred(const DevGraph &g, uint64_t first, uint64_t count, u
     const uint32_t window = (uint32_t)std::min<uint64_t>(32, (words + warps - 1) / warps);
     const uint64_t windows = (words + window - 1) / window;
     const int blocks = (int)std::min<uint64_t>(warps / kWarps, (windows + kWarps - 1) / kWarps);
-    if (classes)
-        k_sample_deferred<true, HASH, PM, RNG><<<blocks, kThreads, 0, s>>>(g, first, count, window, seed, sums, classes, verts);
-    else
-        k_sample_deferred<false, HASH, PM, RNG><<<blocks, kThreads, 0, s>>>(g, first, count, window, seed, sums, classes, verts);
-    return cudaGetLastError();
+    auto *k = classes ? &k_sample_deferred<true, HASH, PM, RNG> : &k_sample_deferred<false, HASH, PM, RNG>;
+    return launch_early(true, k, blocks, kThreads, s, g, first, count, window, seed, sums, classes, verts);
 }
 
 template <int RNG>
@@ -507,13 +504,12 @@ cudaError_t launch_redraws(const DevGraph &g, uint64_t first, uint64_t count, ui
     return launch_deferred_rng<kRngSplitMix>(g, first, count, seed, sums, classes, verts, s);
 }
 
-cudaError_t launch_copy_counts(const uint64_t *sums, uint64_t *out, cudaStream_t s) {
-    k_copy_counts<<<1, 32, 0, s>>>(sums, out);
-    return cudaGetLastError();
+cudaError_t launch_copy_counts(const uint64_t *sums, uint64_t *out, bool early, cudaStream_t s) {
+    return launch_early(early, k_copy_counts, 1, 32, s, sums, out);
 }
 
 cudaError_t launch_counts(int method, const DevGraph &g, uint64_t first, uint64_t count, uint64_t seed, uint64_t *sums,
-                          uint8_t *classes, uint32_t *verts, cudaStream_t s) {
+                          uint8_t *classes, uint32_t *verts, cudaStream_t s, bool early) {
     int dev = 0;
     cudaGetDevice(&dev);
     const uint64_t chunk = method == 2 ? kDeferChunk : count;
@@ -522,7 +518,7 @@ cudaError_t launch_counts(int method, const DevGraph &g, uint64_t first, uint64_
         const int blocks = (int)std::min<uint64_t>(sample_launch_blocks(method, dev, g), (len + kThreads - 1) / kThreads);
         uint8_t *cl = classes ? classes + c0 : nullptr;
         uint32_t *vt = verts ? verts + 5 * c0 : nullptr;
-        cudaError_t e = launch_sample(method, g, first + c0, len, seed, sums, blocks, cl, vt, s);
+        cudaError_t e = launch_sample(method, g, first + c0, len, seed, sums, blocks, cl, vt, s, early && c0 == 0);
         if (e == cudaSuccess && method == 2) e = launch_redraws(g, first + c0, len, seed, sums, cl, vt, s);
         if (e != cudaSuccess) return e;
     }
