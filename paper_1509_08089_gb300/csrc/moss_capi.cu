@@ -319,12 +319,30 @@ void release(moss_graph *g) {
     delete g;
 }
 
-// buckets of the hashed edge set: the next power of two >= nnz / 2, so at
-// least 4 slots per undirected edge (nnz / 2 edges, kBucketKeys slots each)
-uint64_t hash_buckets_for(uint64_t nnz) {
+// Buckets of the hashed edge set, a power of two.  Four to eight slots per
+// undirected edge (nnz / 2 edges, kBucketKeys slots each) while the set takes
+// 32 MiB at most, and behind the filter, where few pairs reach it; two to four
+// otherwise: beside 32 bytes of slot record per list entry, a set of 64 MiB no
+// longer stays in the L2, and its misses cost more than the buckets that
+// overflow.  1e7 samples, ms, four to eight slots -> two to four (MOSS-4, T-5,
+// Path-5, MOSS-4Min): power-law graph, 2.5M entries 0.35 -> 0.27, 0.45 -> 0.39,
+// 0.59 -> 0.47, 0.34 -> 0.30; 4.1M 0.40 -> 0.32, 0.43 -> 0.51, 0.68 -> 0.61,
+// 0.40 -> 0.37; mesh, 2.3M 0.33 -> 0.28, 0.48 -> 0.39, 0.64 -> 0.48, 0.38 ->
+// 0.30; 3.9M 0.43 -> 0.32, 0.62 -> 0.48, 0.80 -> 0.64, 0.52 -> 0.42; larger ones
+// with the hash asked for gain 10-40%.  On 1.95M entries, all of it in the L2,
+// 16 MiB instead of 32 cost 25%; behind the filter the halves gain up to 15% on
+// meshes of 6-13M entries and cost 1-8% on power-law graphs of that size.
+constexpr uint64_t kRoomyBuckets = 1ull << 20;
+
+uint64_t roomy_buckets(uint64_t nnz) {
     uint64_t b = 2;
     while (b < (nnz + 1) / 2) b <<= 1;
     return b;
+}
+
+uint64_t hash_buckets_for(uint64_t nnz, bool filter) {
+    const uint64_t b = roomy_buckets(nnz);
+    return filter || b <= kRoomyBuckets ? b : b / 2;
 }
 
 // words of the edge filter: the largest power of two <= nnz / 8 (4 to 8 bits per edge)
@@ -336,7 +354,7 @@ uint64_t filter_words_for(uint64_t nnz) {
 
 int effective_probe(const moss_graph *g) {
     if (g->probe != MOSS_PROBE_AUTO) return g->probe;
-    return hash_buckets_for(g->nnz) * 8 * kBucketKeys > (64ull << 20) ? MOSS_PROBE_FILTER : MOSS_PROBE_HASH;
+    return roomy_buckets(g->nnz) * 8 * kBucketKeys > (64ull << 20) ? MOSS_PROBE_FILTER : MOSS_PROBE_HASH;
 }
 
 DevGraph view_with(const moss_graph *g, int eff) {
@@ -702,13 +720,12 @@ int moss_build_tables(moss_graph *g, unsigned k_mask, void *stream) {
     g->built = 0;
     const int eff = effective_probe(g);
     const bool want_hash = eff != MOSS_PROBE_SEARCH, want_filter = eff == MOSS_PROBE_FILTER;
-    const uint64_t buckets = hash_buckets_for(g->nnz), words = filter_words_for(g->nnz);
+    // (a set that is there keeps its place and size under another probe: planned
+    // batches and servers hold its address)
+    const uint64_t buckets = g->hash ? g->hash_buckets : hash_buckets_for(g->nnz, want_filter);
+    const uint64_t words = filter_words_for(g->nnz);
     if (want_hash && buckets > (1ULL << 32)) return fail(MOSS_EOVERFLOW, "edge hash above 2^32 buckets");
     // allocations first, on s, so that every chain may use them after the fork
-    if (want_hash && g->hash && g->hash_buckets != buckets) {
-        cudaFreeAsync(g->hash, s);
-        g->hash = nullptr;
-    }
     if (want_hash && !g->hash) {
         if ((e = pool_alloc(g->device, reinterpret_cast<void **>(&g->hash), buckets * 8 * kBucketKeys, s)) !=
             cudaSuccess)

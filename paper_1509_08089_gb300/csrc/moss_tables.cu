@@ -377,7 +377,7 @@ __global__ void k_twin(uint32_t n, uint64_t nnz, const uint4 *__restrict__ vert,
 // ----------------------------------------------------- hashed edge set ---
 // One thread per slot inserts the edge {v, x} with v < x by compare-and-swap
 // into the first free slot from the home bucket on, slots of a bucket in
-// order.  The table has at least four slots per edge, so a free slot always
+// order.  The table has at least two slots per edge, so a free slot always
 // exists and the walk is bounded by the bucket count.
 __device__ __forceinline__ void hash_edges(GridPart grid, uint64_t nnz, const uint32_t *__restrict__ col,
                                            const uint32_t *__restrict__ owner, unsigned long long *table,
