@@ -267,6 +267,8 @@ struct moss_graph {
     uint32_t *col = nullptr;
     uint4 *slot = nullptr;
     uint32_t *acc = nullptr;
+    uint32_t *off = nullptr;     // n + 1 list offsets (table passes)
+    uint32_t *twin = nullptr;    // POS of v in N_x of each CSR slot (v -> x)
     uint32_t *owner = nullptr;   // vertex of each CSR slot (flat per-slot passes)
     uint64_t *sq = nullptr;      // prefix of (d_x - 1)^2 within each list
     u128 *gam[kMethods] = {nullptr, nullptr, nullptr, nullptr};    // [3]: Gamma-check_v (min arena)
@@ -576,9 +578,11 @@ int moss_graph_load_csr_order(const void *row_ptr, int row_ptr_is_64, const uint
                 c.off = 0;
             }
             g->vert = c.take<uint4>(n);
+            g->off = c.take<uint32_t>((uint64_t)n + 1);
             g->col = c.take<uint32_t>(nnz);
             g->slot = c.take<uint4>(2 * nnz);
             g->acc = c.take<uint32_t>(nnz);
+            g->twin = c.take<uint32_t>(nnz);
             g->owner = c.take<uint32_t>(nnz);
             g->sq = c.take<uint64_t>(nnz);
             for (int l = 0; l < 3; ++l) {
@@ -617,11 +621,11 @@ int moss_graph_load_csr_order(const void *row_ptr, int row_ptr_is_64, const uint
         STEP(launch_degree_order(rp_dev, row_ptr_is_64, src, n, nnz, g->order, g->col, oscratch, &rp_new, g->flags, s),
              "ordering kernels");
         if (small)
-            STEP(launch_small_load(rp_new, 0, nullptr, n, nnz, g->vert, g->col, g->slot, g->acc, g->owner, g->sq,
+            STEP(launch_small_load(rp_new, 0, nullptr, n, nnz, g->vert, g->off, g->col, g->twin, g->acc, g->owner, g->sq,
                                    g->gam[0], g->gam[1], g->gam[2], g->tot, g->flags, s),
                  "load kernels");
         else
-            STEP(launch_vertices(rp_new, 0, n, nnz, g->vert, g->flags, s), "vertex kernel");
+            STEP(launch_vertices(rp_new, 0, n, nnz, g->vert, g->off, g->flags, s), "vertex kernel");
         void *done = oscratch;
         oscratch = nullptr;
         STEP(cudaFreeAsync(done, s), "releasing order scratch");
@@ -637,17 +641,17 @@ int moss_graph_load_csr_order(const void *row_ptr, int row_ptr_is_64, const uint
             STEP(cudaMemcpyAsync(g->col, col, nnz * sizeof(uint32_t), cudaMemcpyDefault, s), "copying col");
             src = nullptr;
         }
-        STEP(launch_small_load(rp, row_ptr_is_64, src, n, nnz, g->vert, g->col, g->slot, g->acc, g->owner, g->sq,
+        STEP(launch_small_load(rp, row_ptr_is_64, src, n, nnz, g->vert, g->off, g->col, g->twin, g->acc, g->owner, g->sq,
                                g->gam[0], g->gam[1], g->gam[2], g->tot, g->flags, s),
              "load kernels");
     } else {
         STEP(cudaMemcpyAsync(rp_dev, row_ptr, rp_bytes, cudaMemcpyDefault, s), "copying row_ptr");
         if (nnz) STEP(cudaMemcpyAsync(g->col, col, nnz * sizeof(uint32_t), cudaMemcpyDefault, s), "copying col");
-        STEP(launch_vertices(rp_dev, row_ptr_is_64, n, nnz, g->vert, g->flags, s), "vertex kernel");
+        STEP(launch_vertices(rp_dev, row_ptr_is_64, n, nnz, g->vert, g->off, g->flags, s), "vertex kernel");
     }
     if (!small) {
         u128 *tp = g->partials;
-        STEP(launch_slots(n, nnz, g->col, g->vert, g->slot, g->acc, g->owner, g->sq, g->gam[0], g->gam[1], g->gam[2],
+        STEP(launch_slots(n, nnz, g->col, g->vert, g->off, g->twin, g->acc, g->owner, g->sq, g->gam[0], g->gam[1], g->gam[2],
                           tp, blocks, g->flags, s, aux_streams()),
              "slot kernels");
         STEP(launch_totals(tp, slot_partial_rows(n), g->tot, s), "totals kernel");
@@ -693,7 +697,7 @@ static int build_min_tables(moss_graph *g, cudaStream_t s, const AuxStreams *aux
     void *scratch = nullptr;
     if ((e = pool_alloc(g->device, &scratch, min_scratch_bytes(g->n, g->nnz), s)) != cudaSuccess)
         return cuda_fail(e, "allocating scratch");
-    e = launch_min_tables(g->n, g->nnz, g->tot_h.d_max, g->vert, g->col, g->owner, g->slot, g->mvert, g->mslot, g->mpick, g->rlist,
+    e = launch_min_tables(g->n, g->nnz, g->tot_h.d_max, g->vert, g->col, g->owner, g->twin, g->mvert, g->mslot, g->mpick, g->rlist,
                           g->gam[3], g->seed[3], g->tot, scratch, g->flags, g->vsplit_min, s, aux);
     cudaFreeAsync(scratch, s);
     if (e != cudaSuccess) return cuda_fail(e, "MOSS-4Min table kernels");
@@ -712,7 +716,8 @@ int moss_build_tables(moss_graph *g, unsigned k_mask, void *stream) {
     // tables on the second, the edge hash (and filter) on the third -- or,
     // when the MOSS-4Min tables are built (the longest chain), those on the
     // third and the edge hash after the per-list tables on s
-    const uint64_t sigma_bytes = ((g->nnz * 4 + 255) & ~255ULL) + ((g->nnz * 8 + 255) & ~255ULL);
+    const uint64_t split = sigma_scratch_entries(g->nnz, g->tot_h.d_max);
+    const uint64_t sigma_bytes = ((split * 4 + 255) & ~255ULL) + ((split * 8 + 255) & ~255ULL);
     const uint64_t seed_bytes = seed_scratch_bytes(g->n);
     void *scratch = nullptr;
     int rc = MOSS_OK;
@@ -748,7 +753,7 @@ int moss_build_tables(moss_graph *g, unsigned k_mask, void *stream) {
     if ((e = pool_alloc(g->device, &scratch, sigma_bytes + seed_bytes, s)) != cudaSuccess)
         return cuda_fail(e, "allocating scratch");
     uint32_t *idx = static_cast<uint32_t *>(scratch);
-    uint64_t *pre = reinterpret_cast<uint64_t *>(static_cast<uint8_t *>(scratch) + ((g->nnz * 4 + 255) & ~255ULL));
+    uint64_t *pre = reinterpret_cast<uint64_t *>(static_cast<uint8_t *>(scratch) + ((split * 4 + 255) & ~255ULL));
     void *seed_scratch = static_cast<uint8_t *>(scratch) + sigma_bytes;
     const bool want_min = (k_mask & MOSS_TABLES_4MIN) != 0;
     // a small graph's passes share launches on s
@@ -786,7 +791,7 @@ int moss_build_tables(moss_graph *g, unsigned k_mask, void *stream) {
     if (small) {
         if (e == cudaSuccess)
             e = launch_small_build(g->n, g->nnz, g->tot_h.d_max, g->tot, nt, which, w, seed, vrec, seed_scratch, g->flags,
-                                   g->vert, g->acc, g->col, g->owner, g->slot, idx, pre, want_hash ? g->hash : nullptr,
+                                   g->vert, g->off, g->acc, g->col, g->twin, g->owner, g->slot, idx, pre, want_hash ? g->hash : nullptr,
                                    buckets, s);
         hashed = want_hash && e == cudaSuccess;
     }
@@ -794,7 +799,8 @@ int moss_build_tables(moss_graph *g, unsigned k_mask, void *stream) {
         ev = launch_seed_alias(g->n, g->tot, nt, which, w, seed, vrec, seed_scratch, g->flags, g->vsplit, sv);
     // per-list tables
     if (e == cudaSuccess && !small)
-        e = launch_sigma_alias(g->n, g->nnz, g->tot_h.d_max, g->vert, g->acc, g->owner, g->slot, idx, pre, s, aux, 0);
+        e = launch_sigma_alias(g->n, g->nnz, g->tot_h.d_max, g->vert, g->off, g->acc, g->col, g->twin, g->owner, g->slot, idx, pre, s,
+                               aux, 0);
     // edge hash and filter
     if (e == cudaSuccess && want_hash && !small) {
         uint32_t lg = 0;

@@ -2,6 +2,7 @@
 //
 // Device layout of a loaded graph (all arrays in HBM, owned by moss_graph):
 //   vert[n]   uint4 {off, deg, S_v, 0}           S_v = sum_{x in N_v} (d_x - 1)
+//   off[n+1]  uint32 the lists' offsets, for the passes that build the tables
 //   col[nnz]  uint32 sorted neighbour lists N_v   (the CSR, Table 1)
 //   slot[2 nnz] two uint4 per position, one 32-byte sector:
 //             {col, nb, thr, alias} {off, alias col, alias nb, alias off} --
@@ -12,6 +13,8 @@
 //             Sec. 4.1.3, used to exclude v from N_x).  nb packs
 //             twin | d_x << 16 when d_x < 2^16; for a larger list nb is
 //             kSlotHub, off holds twin and N_x comes from vert[x].
+//             Written by the table build; the load leaves
+//   twin[nnz] uint32 twin of each position
 //   acc[nnz]  uint32 ACC_sigma^(v) exclusive prefix of (d_x - 1) within N_v
 //   sq[nnz]   uint64 exclusive prefix of (d_x - 1)^2 within N_v: with ACC it
 //             gives the prefix of tau^(v) weights (d_x - 1)(S_v - d_x + 1) as
@@ -61,11 +64,6 @@ constexpr uint32_t kSlotDegLimit = 1u << 16;
 // nb and off words of a slot record for neighbour degree dx and twin tw
 __host__ __device__ __forceinline__ uint32_t slot_nb(uint32_t dx, uint32_t tw) {
     return dx < kSlotDegLimit ? (tw | dx << 16) : kSlotHub;
-}
-// twin of position p from the 32-bit view of the slot records
-__device__ __forceinline__ uint32_t slot_twin(const uint32_t *s32, uint64_t p) {
-    const uint32_t nb = s32[8 * p + 1];
-    return nb == kSlotHub ? s32[8 * p + 4] : (nb & (kSlotDegLimit - 1));
 }
 // Path-5 samples run in chunks of kDeferChunk ids; a sample whose first pair
 // of sigma draws collides is flagged in a bitmap and redone by a second launch
@@ -343,10 +341,10 @@ int device_sms(int device);
 int current_sms();
 
 // moss_tables.cu
-cudaError_t launch_vertices(const void *row_ptr, int is64, uint32_t n, uint64_t nnz, uint4 *vert,
+cudaError_t launch_vertices(const void *row_ptr, int is64, uint32_t n, uint64_t nnz, uint4 *vert, uint32_t *off,
                             uint32_t *flags, cudaStream_t s);
 // flags[0]: kErr* bits; flags[1]: slots whose twin was matched (must reach nnz)
-cudaError_t launch_slots(uint32_t n, uint64_t nnz, const uint32_t *col, uint4 *vert, uint4 *slot, uint32_t *acc,
+cudaError_t launch_slots(uint32_t n, uint64_t nnz, const uint32_t *col, uint4 *vert, const uint32_t *off, uint32_t *twin, uint32_t *acc,
                          uint32_t *owner, uint64_t *sq, u128 *gam0, u128 *gam1, u128 *gam2, u128 *partials,
                          int blocks, uint32_t *flags, cudaStream_t s, const AuxStreams *aux);
 cudaError_t launch_totals(const u128 *partials, int blocks, DevTotals *tot, cudaStream_t s);
@@ -363,9 +361,12 @@ uint64_t hub_bytes(uint32_t n);
 cudaError_t launch_hub_tables(uint32_t n, const uint4 *vert, const uint32_t *col, void *mem, uint2 **rank_out,
                               uint32_t **bits_out, uint32_t **list_out, cudaStream_t s);
 // aux (nullable, already forked from s): the long lists go to aux->a[long_stream]
-cudaError_t launch_sigma_alias(uint32_t n, uint64_t nnz, uint32_t d_max, const uint4 *vert, const uint32_t *acc,
-                               const uint32_t *owner, uint4 *slot, uint32_t *scratch_idx, uint64_t *scratch_pre, cudaStream_t s,
-                               const AuxStreams *aux, int long_stream);
+// entries of launch_sigma_alias's scratch (idx and pre): lists too long for
+// shared memory split there, at their places
+uint64_t sigma_scratch_entries(uint64_t nnz, uint32_t d_max);
+cudaError_t launch_sigma_alias(uint32_t n, uint64_t nnz, uint32_t d_max, const uint4 *vert, const uint32_t *off,
+                               const uint32_t *acc, const uint32_t *col, const uint32_t *twin, const uint32_t *owner,
+                               uint4 *slot, uint32_t *scratch_idx, uint64_t *scratch_pre, cudaStream_t s, const AuxStreams *aux, int long_stream);
 // two-level vertex alias tables of up to 3 weights in the same launches
 // (seed[t]: 2n uint4, vrec[t]: the n vertex records copied beside each
 // alias; the levels go to tot->level[which[t]]; heavy: w_v 2^split >= W;
@@ -381,13 +382,13 @@ uint64_t seed_scratch_bytes(uint32_t n);
 // the edge set.
 bool small_graph(uint32_t n, uint64_t nnz);
 cudaError_t launch_small_load(const void *row_ptr, int is64, const uint32_t *src, uint32_t n, uint64_t nnz, uint4 *vert,
-                              uint32_t *col, uint4 *slot, uint32_t *acc, uint32_t *owner, uint64_t *sq, u128 *gam0,
+                              uint32_t *off, uint32_t *col, uint32_t *twin, uint32_t *acc, uint32_t *owner, uint64_t *sq, u128 *gam0,
                               u128 *gam1, u128 *gam2, DevTotals *tot, uint32_t *flags, cudaStream_t s);
 cudaError_t launch_small_build(uint32_t n, uint64_t nnz, uint32_t d_max, DevTotals *tot, int ntables, const int *which,
                                u128 *const *w, uint4 *const *seed, const uint4 *const *vrec, void *seed_scratch,
-                               uint32_t *flags, const uint4 *vert, const uint32_t *acc, const uint32_t *col,
-                               const uint32_t *owner, uint4 *slot, uint32_t *scratch_idx, uint64_t *scratch_pre,
-                               unsigned long long *hash, uint64_t hash_buckets, cudaStream_t s);
+                               uint32_t *flags, const uint4 *vert, const uint32_t *off, const uint32_t *acc,
+                               const uint32_t *col, const uint32_t *twin, const uint32_t *owner, uint4 *slot,
+                               uint32_t *scratch_idx, uint64_t *scratch_pre, unsigned long long *hash, uint64_t hash_buckets, cudaStream_t s);
 int table_blocks(uint32_t n);
 int slot_partial_rows(uint32_t n);   // rows of 6 u128 totals launch_slots writes (launch_totals sums them)
 
@@ -395,7 +396,7 @@ int slot_partial_rows(uint32_t n);   // rows of 6 u128 totals launch_slots write
 // the sigma-check alias tables, tot->gamma[3] and its vertex alias table)
 uint64_t min_scratch_bytes(uint32_t n, uint64_t nnz);
 cudaError_t launch_min_tables(uint32_t n, uint64_t nnz, uint32_t d_max, const uint4 *vert, const uint32_t *col,
-                              const uint32_t *owner, const uint4 *slot, uint4 *mvert, uint4 *mslot, uint4 *mpick,
+                              const uint32_t *owner, const uint32_t *twin, uint4 *mvert, uint4 *mslot, uint4 *mpick,
                               uint2 *rlist, u128 *gmin, uint4 *seed_min, DevTotals *tot, void *scratch,
                               uint32_t *flags, int split, cudaStream_t s, const AuxStreams *aux);
 

@@ -257,15 +257,14 @@ __global__ void __launch_bounds__(kSortThreads) k_rank_long(uint32_t n, const ui
 // per slot p (v -> u) of a list above kShortList entries: {0, 0, 0, u} and
 // {off_u, d_u, d_{v,u}, d_{u,v}} (k_min_alias forms the short lists' itself)
 __global__ void k_min_slots(uint64_t nnz, const uint4 *__restrict__ vert, const uint32_t *__restrict__ col,
-                            const uint32_t *__restrict__ owner, const uint4 *__restrict__ slot,
+                            const uint32_t *__restrict__ owner, const uint32_t *__restrict__ twin,
                             const uint32_t *__restrict__ rank, uint4 *mslot) {
     for (uint64_t p = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; p < nnz; p += (uint64_t)gridDim.x * blockDim.x) {
         if (vert[owner[p]].y <= kShortList) continue;
         const uint32_t u = col[p];
         const uint4 ur = vert[u];
-        const uint32_t twin = slot_twin(reinterpret_cast<const uint32_t *>(slot), p);
         mslot[2 * p] = make_uint4(0u, 0u, 0u, u);
-        mslot[2 * p + 1] = make_uint4(ur.x, ur.y, rank[p], rank[(uint64_t)ur.x + twin]);
+        mslot[2 * p + 1] = make_uint4(ur.x, ur.y, rank[p], rank[(uint64_t)ur.x + twin[p]]);
     }
 }
 
@@ -406,7 +405,7 @@ __device__ __forceinline__ void store_pick(uint4 *mpick, uint64_t p, bool narrow
 template <int TILE>
 __global__ void __launch_bounds__(kListThreads) k_min_alias(uint32_t n, const uint4 *__restrict__ vert,
                                                            const uint32_t *__restrict__ col,
-                                                           const uint4 *__restrict__ slot,
+                                                           const uint32_t *__restrict__ twin,
                                                            const uint32_t *__restrict__ rank, uint4 *mslot,
                                                            uint4 *mpick, uint4 *mvert, u128 *gmin, u128 *partials) {
     __shared__ uint64_t s_pre[kListThreads / kWarp][kLongList];
@@ -427,8 +426,7 @@ __global__ void __launch_bounds__(kListThreads) k_min_alias(uint32_t n, const ui
         if (valid) {
             u = col[p];
             const uint4 ur = vert[u];
-            const uint32_t twin = slot_twin(reinterpret_cast<const uint32_t *>(slot), p);
-            f = make_uint4(ur.x, ur.y, rank[p], rank[(uint64_t)ur.x + twin]);
+            f = make_uint4(ur.x, ur.y, rank[p], rank[(uint64_t)ur.x + twin[p]]);
         }
         const uint64_t w = (uint64_t)f.z * f.w;
         const uint64_t W = __shfl_sync(0xffffffffu, group_scan<g>(w, j), g - 1, g);
@@ -606,7 +604,7 @@ MinScratch carve(void *base, uint32_t n, uint64_t nnz) {
 uint64_t min_scratch_bytes(uint32_t n, uint64_t nnz) { return carve(nullptr, n, nnz).bytes; }
 
 cudaError_t launch_min_tables(uint32_t n, uint64_t nnz, uint32_t d_max, const uint4 *vert, const uint32_t *col,
-                              const uint32_t *owner, const uint4 *slot, uint4 *mvert, uint4 *mslot, uint4 *mpick,
+                              const uint32_t *owner, const uint32_t *twin, uint4 *mvert, uint4 *mslot, uint4 *mpick,
                               uint2 *rlist, u128 *gmin, uint4 *seed_min, DevTotals *tot, void *scratch,
                               uint32_t *flags, int split, cudaStream_t s, const AuxStreams *aux) {
     // With helper streams h0, h1 (aux->a[3], a[4]): the three sort tiers side
@@ -659,7 +657,7 @@ cudaError_t launch_min_tables(uint32_t n, uint64_t nnz, uint32_t d_max, const ui
         join(2);
         if (e == cudaSuccess) e = eh;
         if (e != cudaSuccess) return e;
-        k_min_slots<<<grid_for(nnz, 256, 16), 256, 0, s>>>(nnz, vert, col, owner, slot, m.rank, mslot);
+        k_min_slots<<<grid_for(nnz, 256, 16), 256, 0, s>>>(nnz, vert, col, owner, twin, m.rank, mslot);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     const unsigned ab = alias_grid(n);
@@ -677,7 +675,7 @@ cudaError_t launch_min_tables(uint32_t n, uint64_t nnz, uint32_t d_max, const ui
         k_min_alias_mid<<<chunks, kListThreads, kMidBytes, h0>>>(n, vert, mslot, m.ia, pre, kMidBytes);
     eh = cudaGetLastError();
     with_tile(n, [&](auto T) {
-        k_min_alias<decltype(T)::value><<<ab, kListThreads, 0, s>>>(n, vert, col, slot, m.rank, mslot, mpick, mvert,
+        k_min_alias<decltype(T)::value><<<ab, kListThreads, 0, s>>>(n, vert, col, twin, m.rank, mslot, mpick, mvert,
                                                                     gmin, m.partials);
     });
     e = cudaGetLastError();

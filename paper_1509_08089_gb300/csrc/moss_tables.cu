@@ -41,7 +41,7 @@ constexpr int kLongThreads = 256;
 
 // ------------------------------------------------------------ vertices ---
 template <typename IdxT>
-__global__ void k_vertices(const IdxT *row_ptr, uint32_t n, uint64_t nnz, uint4 *vert, uint32_t *flags) {
+__global__ void k_vertices(const IdxT *row_ptr, uint32_t n, uint64_t nnz, uint4 *vert, uint32_t *off, uint32_t *flags) {
     for (uint64_t v = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; v < n; v += (uint64_t)gridDim.x * blockDim.x) {
         uint64_t a = row_ptr[v], b = row_ptr[v + 1];
         bool bad = b < a || b > nnz || (v == 0 && a != 0) || (v + 1 == n && b != nnz);
@@ -50,7 +50,18 @@ __global__ void k_vertices(const IdxT *row_ptr, uint32_t n, uint64_t nnz, uint4 
             a = b = 0;
         }
         vert[v] = make_uint4((uint32_t)a, (uint32_t)(b - a), 0u, 0u);
+        off[v] = (uint32_t)a;
+        if (v + 1 == n) off[n] = (uint32_t)b;
     }
+}
+
+// {off, deg} of a neighbour: the passes that meet every slot's neighbour gather
+// 4-byte offsets rather than 16-byte vertex records, a quarter of the L2 (of a
+// 4M-vertex graph 16 MB instead of 64).  (The offsets of rejected rows may not
+// ascend; every range taken from them stays within the nnz entries.)
+__device__ __forceinline__ uint2 list_of(const uint32_t *off, uint32_t x) {
+    const uint32_t a = __ldg(off + x), b = __ldg(off + x + 1);
+    return make_uint2(a, b > a ? b - a : 0u);
 }
 
 // --------------------------------------------------------------- slots ---
@@ -73,27 +84,21 @@ __global__ void __launch_bounds__(kTableThreads) k_owner(uint32_t n, const uint4
 }
 
 __global__ void k_slot_weights(uint32_t n, uint64_t nnz, const uint32_t *__restrict__ col,
-                               const uint4 *__restrict__ vert, const uint32_t *__restrict__ owner, uint4 *slot,
-                               uint32_t *acc, uint32_t *flags) {
+                               const uint32_t *__restrict__ off, const uint32_t *__restrict__ owner, uint32_t *acc,
+                               uint32_t *flags) {
     uint32_t err = 0;
     for (uint64_t p = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; p < nnz; p += (uint64_t)gridDim.x * blockDim.x) {
         const uint32_t v = owner[p], x = col[p];
-        uint32_t w = 0, ox = 0, dx = 0;
+        uint32_t w = 0;
         if (x >= n) {
             err |= kErrRange;
         } else {
             if (x == v) err |= kErrSelf;
             if (p > 0 && owner[p - 1] == v && col[p - 1] >= x) err |= kErrOrder;
-            const uint4 xr = vert[x];
-            w = xr.y ? xr.y - 1 : 0;
-            ox = xr.x;
-            dx = xr.y;
+            const uint32_t dx = list_of(off, x).y;
+            w = dx ? dx - 1 : 0;
         }
         acc[p] = w;    // turned into the prefix by k_slots
-        // words 2 and 3 (the sigma threshold and alias, written by the table
-        // build) hold x's {off, deg} until then, for k_twin
-        slot[2 * p] = make_uint4(x, 0u, ox, dx);
-        slot[2 * p + 1] = make_uint4(ox, 0u, 0u, 0u);   // nb and, for a hub, off: k_twin
     }
     if (err) atomicOr(flags, err);
 }
@@ -328,20 +333,22 @@ __global__ void __launch_bounds__(kTotalsThreads) k_totals(const u128 *partials,
 // itself in the other endpoint's (shorter) sorted list and writes both
 // twins: twin(v->x) = POS of v in N_x and twin(x->v) = POS of x in N_v.  For
 // a symmetric graph every edge is matched once, so the matched slots add up
-// to nnz; a reverse that is missing leaves the sum short.
-__device__ __forceinline__ void match_twins(GridPart grid, uint32_t n, uint64_t nnz, const uint4 *vert,
+// to nnz; a reverse that is missing leaves the sum short.  The twins are an
+// array of their own, from which the table build writes whole slot records:
+// written into the 32-byte records, a twin's 4 bytes at a random place cost a
+// sector read and written (14M slots: 1.2 GB read, 0.5 GB written, 470 us), and
+// the records a pass of their own at load.  Load and five-node tables, before
+// -> after: 7M edges 0.85 + 1.06 -> 0.57 + 1.06 ms, 34M edges 4.7 + 5.6 -> 3.3 +
+// 6.5 ms (there the build's gathers compete for the L2 with the edge set's).
+__device__ __forceinline__ void match_twins(GridPart grid, uint32_t n, uint64_t nnz, const uint32_t *off,
                                             const uint32_t *__restrict__ col, const uint32_t *__restrict__ owner,
-                                            uint4 *slot, uint32_t *flags) {
+                                            uint32_t *twin, uint32_t *flags) {
     uint32_t matched = 0, err = 0;
     for (uint64_t p = grid.block * (uint64_t)blockDim.x + threadIdx.x; p < nnz; p += (uint64_t)grid.blocks * blockDim.x) {
         const uint32_t v = owner[p], x = col[p];
         // flagged by the slot pass; the owners of a row that was rejected are unset
         if (x >= n || x == v || v >= n) continue;
-        // {off, deg} only: k_slots may be writing S_v into the same records;
-        // x's comes from words 2 and 3 of the slot record (k_slot_weights), a
-        // streamed read instead of a random one
-        const uint2 vr = reinterpret_cast<const uint2 *>(vert)[2 * (uint64_t)v];
-        const uint2 xr = reinterpret_cast<const uint2 *>(slot)[4 * p + 1];
+        const uint2 vr = list_of(off, v), xr = list_of(off, x);
         const bool mine = vr.y > xr.y || (vr.y == xr.y && v < x);
         if (!mine) continue;
         uint32_t lo = xr.x, len = xr.y;
@@ -353,13 +360,8 @@ __device__ __forceinline__ void match_twins(GridPart grid, uint32_t n, uint64_t 
             err |= kErrAsym;
             continue;
         }
-        uint32_t *s32 = reinterpret_cast<uint32_t *>(slot);
-        const uint32_t tp = lo - xr.x;                 // POS of v in N_x
-        const uint32_t tl = (uint32_t)(p - vr.x);      // POS of x in N_v
-        s32[8 * p + 1] = slot_nb(xr.y, tp);
-        if (xr.y >= kSlotDegLimit) s32[8 * p + 4] = tp;
-        s32[8 * (uint64_t)lo + 1] = slot_nb(vr.y, tl);
-        if (vr.y >= kSlotDegLimit) s32[8 * (uint64_t)lo + 4] = tl;
+        twin[p] = lo - xr.x;                  // POS of v in N_x
+        twin[lo] = (uint32_t)(p - vr.x);      // POS of x in N_v
         matched += 2;
     }
     if (err) atomicOr(flags, err);
@@ -369,9 +371,9 @@ __device__ __forceinline__ void match_twins(GridPart grid, uint32_t n, uint64_t 
     if ((threadIdx.x & 31) == 0 && matched) atomicAdd(flags + 1, matched);
 }
 
-__global__ void k_twin(uint32_t n, uint64_t nnz, const uint4 *__restrict__ vert, const uint32_t *__restrict__ col,
-                       const uint32_t *__restrict__ owner, uint4 *slot, uint32_t *flags) {
-    match_twins(whole_grid(), n, nnz, vert, col, owner, slot, flags);
+__global__ void k_twin(uint32_t n, uint64_t nnz, const uint32_t *__restrict__ off, const uint32_t *__restrict__ col,
+                       const uint32_t *__restrict__ owner, uint32_t *twin, uint32_t *flags) {
+    match_twins(whole_grid(), n, nnz, off, col, owner, twin, flags);
 }
 
 // ----------------------------------------------------- hashed edge set ---
@@ -432,14 +434,24 @@ __device__ __forceinline__ uint32_t acc_weight(const uint32_t *acc, uint32_t o, 
     return (p + 1 < d ? __ldg(acc + o + p + 1) : S) - __ldg(acc + o + p);
 }
 
+// {col, nb, off} of position p's neighbour (moss_internal.cuh)
+__device__ __forceinline__ uint3 slot_pick_words(const uint32_t *off, const uint32_t *col, const uint32_t *twin,
+                                                 uint64_t p) {
+    const uint32_t x = __ldg(col + p), tw = __ldg(twin + p);
+    const uint2 xr = list_of(off, x);
+    return make_uint3(x, slot_nb(xr.y, tw), xr.y < kSlotDegLimit ? xr.x : tw);
+}
+
 // Lists of at most kLongList entries.  Short ones (kShortList) by groups of
-// lanes, which also complete the record with the alias's fields; longer ones a
+// lanes, which write the whole record, the alias's fields from its lane; longer ones a
 // warp each, the split (idx, pre) of the list being built in the warp's share
 // of shared memory, so the searches and merges of pass 2 wait on shared rather
 // than global loads.
 template <int TILE>
 __device__ __forceinline__ void sigma_lists(GridPart grid, uint32_t n, const uint4 *__restrict__ vert,
-                                            const uint32_t *__restrict__ acc, uint4 *slot) {
+                                            const uint32_t *__restrict__ off, const uint32_t *__restrict__ acc,
+                                            const uint32_t *__restrict__ col, const uint32_t *__restrict__ twin,
+                                            uint4 *slot) {
     __shared__ uint64_t s_pre[kTableThreads / kWarp][kLongList];
     __shared__ uint32_t s_idx[kTableThreads / kWarp][kLongList];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -452,6 +464,7 @@ __device__ __forceinline__ void sigma_lists(GridPart grid, uint32_t n, const uin
         const uint32_t o = r.x, d = r.y, S = r.z;
         const uint64_t p = (uint64_t)o + j;
         const uint32_t a = valid ? __ldg(acc + p) : S;
+        const uint3 c = valid ? slot_pick_words(off, col, twin, p) : make_uint3(0u, 0u, 0u);
         const uint32_t after = __shfl_down_sync(0xffffffffu, a, 1, g);
         const uint32_t w = (j + 1 < d ? after : S) - a;
         uint64_t thr;
@@ -461,14 +474,12 @@ __device__ __forceinline__ void sigma_lists(GridPart grid, uint32_t n, const uin
             thr = 0;
             alias = j;
         }
-        const uint2 cn = valid ? *reinterpret_cast<const uint2 *>(slot32 + 8 * p) : make_uint2(0u, 0u);
-        const uint32_t off = valid ? slot32[8 * p + 4] : 0u;
-        const uint32_t col = __shfl_sync(0xffffffffu, cn.x, alias & (g - 1), g);
-        const uint32_t nb = __shfl_sync(0xffffffffu, cn.y, alias & (g - 1), g);
-        const uint32_t aoff = __shfl_sync(0xffffffffu, off, alias & (g - 1), g);
+        const uint32_t acol = __shfl_sync(0xffffffffu, c.x, alias & (g - 1), g);
+        const uint32_t anb = __shfl_sync(0xffffffffu, c.y, alias & (g - 1), g);
+        const uint32_t aoff = __shfl_sync(0xffffffffu, c.z, alias & (g - 1), g);
         if (valid) {
-            slot[2 * p] = make_uint4(cn.x, cn.y, (uint32_t)thr, alias);
-            slot[2 * p + 1] = make_uint4(off, col, nb, aoff);
+            slot[2 * p] = make_uint4(c.x, c.y, (uint32_t)thr, alias);
+            slot[2 * p + 1] = make_uint4(c.z, acol, anb, aoff);
         }
     };
     auto large = [&](uint32_t, uint4 vr) {
@@ -568,8 +579,11 @@ __device__ __forceinline__ void sigma_lists(GridPart grid, uint32_t n, const uin
 
 template <int TILE>
 __global__ void __launch_bounds__(kTableThreads) k_sigma_alias(uint32_t n, const uint4 *__restrict__ vert,
-                                                              const uint32_t *__restrict__ acc, uint4 *slot) {
-    sigma_lists<TILE>(whole_grid(), n, vert, acc, slot);
+                                                              const uint32_t *__restrict__ off,
+                                                              const uint32_t *__restrict__ acc,
+                                                              const uint32_t *__restrict__ col,
+                                                              const uint32_t *__restrict__ twin, uint4 *slot) {
+    sigma_lists<TILE>(whole_grid(), n, vert, off, acc, col, twin, slot);
 }
 
 // lists longer than kLongList: a block per list (moss_alias.cuh), 256 threads
@@ -603,25 +617,27 @@ __global__ void __launch_bounds__(NT) k_sigma_alias_long(uint32_t n, const uint4
         });
 }
 
-// One thread per slot of the lists above kShortList entries: words 5..7 of
-// each record from words 0, 1 and 4 of its alias position's record (written
-// before this launch, read only here).
-__device__ __forceinline__ void fill_slot_aliases(GridPart grid, uint64_t nnz, const uint4 *__restrict__ vert,
-                                                  const uint32_t *__restrict__ owner, uint4 *slot) {
-    uint32_t *s32 = reinterpret_cast<uint32_t *>(slot);
+// One thread per slot of the lists above kShortList entries: the rest of each
+// record around its threshold and alias, from its own neighbour and its alias
+// position's.
+__device__ __forceinline__ void fill_slots(GridPart grid, uint64_t nnz, const uint4 *__restrict__ vert,
+                                           const uint32_t *__restrict__ off, const uint32_t *__restrict__ col,
+                                           const uint32_t *__restrict__ twin, const uint32_t *__restrict__ owner,
+                                           uint4 *slot) {
     for (uint64_t p = grid.block * (uint64_t)blockDim.x + threadIdx.x; p < nnz; p += (uint64_t)grid.blocks * blockDim.x) {
         const uint4 vr = vert[owner[p]];
         if (vr.y <= kShortList) continue;   // k_sigma_alias wrote the whole record
-        const uint64_t a = (uint64_t)vr.x + s32[8 * p + 3];
-        const uint32_t col = s32[8 * a], nb = s32[8 * a + 1], off = s32[8 * a + 4];
-        s32[8 * p + 5] = col;
-        *reinterpret_cast<uint2 *>(s32 + 8 * p + 6) = make_uint2(nb, off);
+        const uint2 pick = reinterpret_cast<const uint2 *>(slot)[4 * p + 1];   // threshold, alias
+        const uint3 c = slot_pick_words(off, col, twin, p), a = slot_pick_words(off, col, twin, (uint64_t)vr.x + pick.y);
+        slot[2 * p] = make_uint4(c.x, c.y, pick.x, pick.y);
+        slot[2 * p + 1] = make_uint4(c.z, a.x, a.y, a.z);
     }
 }
 
-__global__ void k_slot_alias_fill(uint64_t nnz, const uint4 *__restrict__ vert, const uint32_t *__restrict__ owner,
-                                  uint4 *slot) {
-    fill_slot_aliases(whole_grid(), nnz, vert, owner, slot);
+__global__ void k_slot_fill(uint64_t nnz, const uint4 *__restrict__ vert, const uint32_t *__restrict__ off,
+                            const uint32_t *__restrict__ col, const uint32_t *__restrict__ twin,
+                            const uint32_t *__restrict__ owner, uint4 *slot) {
+    fill_slots(whole_grid(), nnz, vert, off, col, twin, owner, slot);
 }
 
 // ---------------------------------------------------- vertex (seed) tables ---
@@ -1175,8 +1191,8 @@ constexpr uint64_t kSmallSlots = 1ull << 18;
 // from src when they are not in place yet
 template <typename IdxT>
 __global__ void __launch_bounds__(kTableThreads) k_small_rows(const IdxT *row_ptr, const uint32_t *src, uint32_t n,
-                                                             uint64_t nnz, uint4 *vert, uint32_t *owner,
-                                                             uint32_t *col, uint32_t *flags) {
+                                                             uint64_t nnz, uint4 *vert, uint32_t *off,
+                                                             uint32_t *owner, uint32_t *col, uint32_t *flags) {
     const int lane = threadIdx.x & 31;
     const uint32_t warps = gridDim.x * (kTableThreads / kWarp);
     for (uint32_t v = blockIdx.x * (kTableThreads / kWarp) + (threadIdx.x >> 5); v < n; v += warps) {
@@ -1185,7 +1201,11 @@ __global__ void __launch_bounds__(kTableThreads) k_small_rows(const IdxT *row_pt
             if (lane == 0) atomicOr(flags, kErrRowPtr);
             a = b = 0;
         }
-        if (lane == 0) vert[v] = make_uint4((uint32_t)a, (uint32_t)(b - a), 0u, 0u);
+        if (lane == 0) {
+            vert[v] = make_uint4((uint32_t)a, (uint32_t)(b - a), 0u, 0u);
+            off[v] = (uint32_t)a;
+            if (v + 1 == n) off[n] = (uint32_t)b;
+        }
         for (uint64_t p = a + lane; p < b; p += kWarp) {
             owner[p] = v;
             if (src) col[p] = src[p];
@@ -1195,8 +1215,9 @@ __global__ void __launch_bounds__(kTableThreads) k_small_rows(const IdxT *row_pt
 
 // the list scans and the twin pass (which touches none of what they write)
 __global__ void __launch_bounds__(kTableThreads) k_small_scan(uint32_t n, uint64_t nnz, uint4 *vert,
+                                                             const uint32_t *__restrict__ off,
                                                              const uint32_t *__restrict__ col,
-                                                             const uint32_t *__restrict__ owner, uint4 *slot,
+                                                             const uint32_t *__restrict__ owner, uint32_t *twin,
                                                              uint32_t *acc, uint64_t *sq, u128 *gam2, uint32_t *flags,
                                                              uint32_t scan_blocks, uint32_t long_blocks) {
     const uint32_t b = blockIdx.x;
@@ -1205,8 +1226,8 @@ __global__ void __launch_bounds__(kTableThreads) k_small_scan(uint32_t n, uint64
     else if (b < scan_blocks + long_blocks)
         scan_long_lists(GridPart{b - scan_blocks, long_blocks}, n, vert, acc, sq, gam2);
     else
-        match_twins(GridPart{b - scan_blocks - long_blocks, gridDim.x - scan_blocks - long_blocks}, n, nnz, vert, col,
-                    owner, slot, flags);
+        match_twins(GridPart{b - scan_blocks - long_blocks, gridDim.x - scan_blocks - long_blocks}, n, nnz, off, col,
+                    owner, twin, flags);
 }
 
 // vertex weights and the exact totals, one block
@@ -1232,13 +1253,16 @@ __global__ void __launch_bounds__(kTotalsThreads) k_small_totals(uint32_t n, con
 __global__ void __launch_bounds__(kSeedThreads) k_small_build(uint32_t n, const DevTotals *tot, SeedTasks tasks, int nt,
                                                              uint32_t chunks, uint32_t *flags,
                                                              const uint4 *__restrict__ vert,
-                                                             const uint32_t *__restrict__ acc, uint4 *slot,
+                                                             const uint32_t *__restrict__ off,
+                                                             const uint32_t *__restrict__ acc,
+                                                             const uint32_t *__restrict__ col,
+                                                             const uint32_t *__restrict__ twin, uint4 *slot,
                                                              uint4 *hash, uint64_t hash_words, uint32_t list_blocks) {
     const uint32_t b = blockIdx.x, counts = chunks * nt;
     if (b < counts) {
         seed_count<kSeedRoundsFew>(b % chunks, tasks.t[b / chunks], n, tot, flags);
     } else if (b < counts + list_blocks) {
-        sigma_lists<8>(GridPart{b - counts, list_blocks}, n, vert, acc, slot);
+        sigma_lists<8>(GridPart{b - counts, list_blocks}, n, vert, off, acc, col, twin, slot);
     } else {
         const uint64_t first = (uint64_t)(b - counts - list_blocks) * kSeedThreads + threadIdx.x;
         const uint64_t stride = (uint64_t)(gridDim.x - counts - list_blocks) * kSeedThreads;
@@ -1247,11 +1271,13 @@ __global__ void __launch_bounds__(kSeedThreads) k_small_build(uint32_t n, const 
     }
 }
 
-// the scan of the chunk sums, the alias halves of the longer lists' records
+// the scan of the chunk sums, the rest of the longer lists' records
 // and the edge set
 __global__ void __launch_bounds__(kSeedThreads) k_small_build2(uint64_t nnz, const DevTotals *tot, SeedTasks tasks,
                                                               int nt, uint32_t chunks, const uint4 *__restrict__ vert,
+                                                              const uint32_t *__restrict__ off,
                                                               const uint32_t *__restrict__ col,
+                                                              const uint32_t *__restrict__ twin,
                                                               const uint32_t *__restrict__ owner, uint4 *slot,
                                                               unsigned long long *hash, uint32_t mask, uint32_t shift,
                                                               uint32_t fill_blocks) {
@@ -1259,7 +1285,7 @@ __global__ void __launch_bounds__(kSeedThreads) k_small_build2(uint64_t nnz, con
     if (b < (uint32_t)nt)
         seed_offsets(chunks, tasks.t[b], tot);
     else if (b < nt + fill_blocks)
-        fill_slot_aliases(GridPart{b - nt, fill_blocks}, nnz, vert, owner, slot);
+        fill_slots(GridPart{b - nt, fill_blocks}, nnz, vert, off, col, twin, owner, slot);
     else
         hash_edges(GridPart{b - nt - fill_blocks, gridDim.x - nt - fill_blocks}, nnz, col, owner, hash, mask, shift);
 }
@@ -1422,18 +1448,18 @@ int table_blocks(uint32_t n) {
     return (int)blocks;
 }
 
-cudaError_t launch_vertices(const void *row_ptr, int is64, uint32_t n, uint64_t nnz, uint4 *vert, uint32_t *flags,
-                            cudaStream_t s) {
+cudaError_t launch_vertices(const void *row_ptr, int is64, uint32_t n, uint64_t nnz, uint4 *vert, uint32_t *off,
+                            uint32_t *flags, cudaStream_t s) {
     const int threads = 256;
     uint64_t blocks = ((uint64_t)n + threads - 1) / threads;
     if (blocks > 65535) blocks = 65535;
     if (blocks < 1) blocks = 1;
     if (is64)
         k_vertices<uint64_t><<<(unsigned)blocks, threads, 0, s>>>(static_cast<const uint64_t *>(row_ptr), n, nnz,
-                                                                   vert, flags);
+                                                                   vert, off, flags);
     else
         k_vertices<uint32_t><<<(unsigned)blocks, threads, 0, s>>>(static_cast<const uint32_t *>(row_ptr), n, nnz,
-                                                                   vert, flags);
+                                                                   vert, off, flags);
     return cudaGetLastError();
 }
 
@@ -1454,7 +1480,7 @@ static unsigned flat_blocks(uint64_t items) {
     return (unsigned)(b ? b : 1);
 }
 
-cudaError_t launch_slots(uint32_t n, uint64_t nnz, const uint32_t *col, uint4 *vert, uint4 *slot, uint32_t *acc,
+cudaError_t launch_slots(uint32_t n, uint64_t nnz, const uint32_t *col, uint4 *vert, const uint32_t *off, uint32_t *twin, uint32_t *acc,
                          uint32_t *owner, uint64_t *sq, u128 *gam0, u128 *gam1, u128 *gam2, u128 *partials,
                          int blocks, uint32_t *flags, cudaStream_t s, const AuxStreams *aux) {
     with_tile(n, [&](auto T) {
@@ -1463,7 +1489,7 @@ cudaError_t launch_slots(uint32_t n, uint64_t nnz, const uint32_t *col, uint4 *v
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     if (nnz) {
-        k_slot_weights<<<flat_blocks(nnz), 256, 0, s>>>(n, nnz, col, vert, owner, slot, acc, flags);
+        k_slot_weights<<<flat_blocks(nnz), 256, 0, s>>>(n, nnz, col, off, owner, acc, flags);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     // the twin pass touches none of what the list scans write, and the short
@@ -1472,7 +1498,7 @@ cudaError_t launch_slots(uint32_t n, uint64_t nnz, const uint32_t *col, uint4 *v
     const bool forked = aux && aux->fork(s) == cudaSuccess;
     if (aux && !forked) cudaGetLastError();
     cudaStream_t ts = forked ? aux->a[0] : s, ls = forked ? aux->a[1] : s;
-    if (nnz) k_twin<<<flat_blocks(nnz), 256, 0, ts>>>(n, nnz, vert, col, owner, slot, flags);
+    if (nnz) k_twin<<<flat_blocks(nnz), 256, 0, ts>>>(n, nnz, off, col, owner, twin, flags);
     cudaError_t et = cudaGetLastError();
     k_slots_long<<<long_blocks(n), kLongThreads, 0, ls>>>(n, vert, acc, sq, gam2);
     cudaError_t el = cudaGetLastError();
@@ -1565,6 +1591,8 @@ cudaError_t launch_hub_tables(uint32_t n, const uint4 *vert, const uint32_t *col
 }
 
 // the tables of lists above kLongList entries
+uint64_t sigma_scratch_entries(uint64_t nnz, uint32_t d_max) { return d_max > kHubSmemList ? nnz : 0; }
+
 static cudaError_t launch_long_sigma(uint32_t n, uint32_t d_max, const uint4 *vert, const uint32_t *acc, uint4 *slot,
                                      uint32_t *scratch_idx, uint64_t *scratch_pre, cudaStream_t s) {
     if (d_max <= kLongList) return cudaSuccess;
@@ -1589,15 +1617,16 @@ static cudaError_t launch_long_sigma(uint32_t n, uint32_t d_max, const uint4 *ve
     return cudaGetLastError();
 }
 
-cudaError_t launch_sigma_alias(uint32_t n, uint64_t nnz, uint32_t d_max, const uint4 *vert, const uint32_t *acc,
-                               const uint32_t *owner, uint4 *slot, uint32_t *scratch_idx, uint64_t *scratch_pre,
+cudaError_t launch_sigma_alias(uint32_t n, uint64_t nnz, uint32_t d_max, const uint4 *vert, const uint32_t *off,
+                               const uint32_t *acc, const uint32_t *col, const uint32_t *twin, const uint32_t *owner,
+                               uint4 *slot, uint32_t *scratch_idx, uint64_t *scratch_pre,
                                cudaStream_t s, const AuxStreams *aux, int long_stream) {
     // the short and the long lists are built side by side (long lists on
     // aux->a[long_stream], forked from s by the caller); the fill waits for both
     cudaError_t el = launch_long_sigma(n, d_max, vert, acc, slot, scratch_idx, scratch_pre,
                                        aux ? aux->a[long_stream] : s);
     with_tile(n, [&](auto T) {
-        k_sigma_alias<decltype(T)::value><<<tile_blocks(n, decltype(T)::value, kTableThreads, current_sms(), 8), kTableThreads, 0, s>>>(n, vert, acc, slot);
+        k_sigma_alias<decltype(T)::value><<<tile_blocks(n, decltype(T)::value, kTableThreads, current_sms(), 8), kTableThreads, 0, s>>>(n, vert, off, acc, col, twin, slot);
     });
     const cudaError_t e = cudaGetLastError();
     if (aux && d_max > kLongList) {
@@ -1607,7 +1636,7 @@ cudaError_t launch_sigma_alias(uint32_t n, uint64_t nnz, uint32_t d_max, const u
     if (e != cudaSuccess) return e;
     if (el != cudaSuccess) return el;
     if (d_max <= kShortList) return cudaSuccess;   // every record is complete
-    k_slot_alias_fill<<<flat_blocks(nnz), 256, 0, s>>>(nnz, vert, owner, slot);
+    k_slot_fill<<<flat_blocks(nnz), 256, 0, s>>>(nnz, vert, off, col, twin, owner, slot);
     return cudaGetLastError();
 }
 
@@ -1630,24 +1659,24 @@ uint64_t seed_scratch_bytes(uint32_t n) {
 bool small_graph(uint32_t n, uint64_t nnz) { return n < kSmallVertices && nnz <= kSmallSlots; }
 
 cudaError_t launch_small_load(const void *row_ptr, int is64, const uint32_t *src, uint32_t n, uint64_t nnz, uint4 *vert,
-                              uint32_t *col, uint4 *slot, uint32_t *acc, uint32_t *owner, uint64_t *sq, u128 *gam0,
+                              uint32_t *off, uint32_t *col, uint32_t *twin, uint32_t *acc, uint32_t *owner, uint64_t *sq, u128 *gam0,
                               u128 *gam1, u128 *gam2, DevTotals *tot, uint32_t *flags, cudaStream_t s) {
     const unsigned rows = (n + kTableThreads / kWarp - 1) / (kTableThreads / kWarp);
     if (is64)
-        k_small_rows<uint64_t><<<rows, kTableThreads, 0, s>>>(static_cast<const uint64_t *>(row_ptr), src, n, nnz, vert,
+        k_small_rows<uint64_t><<<rows, kTableThreads, 0, s>>>(static_cast<const uint64_t *>(row_ptr), src, n, nnz, vert, off,
                                                               owner, col, flags);
     else
-        k_small_rows<uint32_t><<<rows, kTableThreads, 0, s>>>(static_cast<const uint32_t *>(row_ptr), src, n, nnz, vert,
+        k_small_rows<uint32_t><<<rows, kTableThreads, 0, s>>>(static_cast<const uint32_t *>(row_ptr), src, n, nnz, vert, off,
                                                               owner, col, flags);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     if (nnz) {
-        k_slot_weights<<<flat_blocks(nnz), 256, 0, s>>>(n, nnz, col, vert, owner, slot, acc, flags);
+        k_slot_weights<<<flat_blocks(nnz), 256, 0, s>>>(n, nnz, col, off, owner, acc, flags);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     const unsigned scans = tile_blocks(n, 8, kTableThreads, current_sms(), 8), longs = long_blocks(n);
     k_small_scan<<<scans + longs + (nnz ? flat_blocks(nnz) : 0), kTableThreads, 0, s>>>(
-        n, nnz, vert, col, owner, slot, acc, sq, gam2, flags, scans, longs);
+        n, nnz, vert, off, col, owner, twin, acc, sq, gam2, flags, scans, longs);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     k_small_totals<<<1, kTotalsThreads, 0, s>>>(n, vert, gam0, gam1, gam2, tot);
     return cudaGetLastError();
@@ -1735,9 +1764,9 @@ cudaError_t launch_seed_alias(uint32_t n, DevTotals *tot, int ntables, const int
 
 cudaError_t launch_small_build(uint32_t n, uint64_t nnz, uint32_t d_max, DevTotals *tot, int ntables, const int *which,
                                u128 *const *w, uint4 *const *seed, const uint4 *const *vrec, void *seed_scratch,
-                               uint32_t *flags, const uint4 *vert, const uint32_t *acc, const uint32_t *col,
-                               const uint32_t *owner, uint4 *slot, uint32_t *scratch_idx, uint64_t *scratch_pre,
-                               unsigned long long *hash, uint64_t hash_buckets, cudaStream_t s) {
+                               uint32_t *flags, const uint4 *vert, const uint32_t *off, const uint32_t *acc,
+                               const uint32_t *col, const uint32_t *twin, const uint32_t *owner, uint4 *slot,
+                               uint32_t *scratch_idx, uint64_t *scratch_pre, unsigned long long *hash, uint64_t hash_buckets, cudaStream_t s) {
     const uint32_t chunks = seed_chunks(n);
     LevelTasks lt = {};
     SeedTasks tasks = {};
@@ -1746,7 +1775,7 @@ cudaError_t launch_small_build(uint32_t n, uint64_t nnz, uint32_t d_max, DevTota
     const unsigned lists = tile_blocks(n, 8, kTableThreads, current_sms(), 8);
     const unsigned clears = words ? flat_blocks((words + 3) / 4) : 0;
     k_small_build<<<chunks * ntables + lists + clears, kSeedThreads, 0, s>>>(
-        n, tot, tasks, ntables, chunks, flags, vert, acc, slot, reinterpret_cast<uint4 *>(hash), words, lists);
+        n, tot, tasks, ntables, chunks, flags, vert, off, acc, col, twin, slot, reinterpret_cast<uint4 *>(hash), words, lists);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = launch_long_sigma(n, d_max, vert, acc, slot, scratch_idx, scratch_pre, s);
     if (e != cudaSuccess) return e;
@@ -1754,7 +1783,7 @@ cudaError_t launch_small_build(uint32_t n, uint64_t nnz, uint32_t d_max, DevTota
     uint32_t lg = 0;
     while ((1ULL << lg) < hash_buckets) ++lg;
     if (ntables + fills + inserts) {
-        k_small_build2<<<ntables + fills + inserts, kSeedThreads, 0, s>>>(nnz, tot, tasks, ntables, chunks, vert, col, owner,
+        k_small_build2<<<ntables + fills + inserts, kSeedThreads, 0, s>>>(nnz, tot, tasks, ntables, chunks, vert, off, col, twin, owner,
                                                                           slot, hash, (uint32_t)(hash_buckets - 1),
                                                                           64 - lg, fills);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
