@@ -367,6 +367,54 @@ def launches_per_step(k: int, budget: int, mix: bool, filtered: bool = False, tw
     return n
 
 
+def device_launches(rp, k: int, budget: int, mix: bool, probe: str, two_level: bool, two_level_min: bool,
+                    order: str, grouped=()) -> int:
+    """Kernels that one step launches, by the library's rules (launches_per_step
+    counts the passes as they were when each was a launch and summed its rows in
+    another).  Graphs below 2^14 vertices and 2^18 entries load in 4 and build
+    in 4 launches and those of the longer lists; `grouped`: the sub-methods
+    whose calls are grouped by first vertex."""
+    from paper_1509_08089_gb300.dist import sub_budgets
+    deg = np.diff(np.asarray(rp).astype(np.int64))
+    n, nnz, d_max = len(deg), int(deg.sum()), int(deg.max(initial=0))
+    long = (d_max > 256) + (d_max > 2048)           # the alias passes of long lists
+    small = n < 1 << 14 and nnz <= 1 << 18 and not (two_level or mix or probe == "filter")
+    total = 4 if order == "degree" else 0
+    if small:
+        total += 4 + 4 + long
+    else:
+        total += 8 + 1 + long + (d_max > 32) + 4 + (3 if two_level else 0)
+        total += (1 if probe != "search" else 0) + (7 if probe == "filter" else 0)
+    if mix:   # the sort tiers, records, alias passes, picks, total and vertex table
+        total += 1 + (d_max > 128) + (d_max > 1024) + 1 + 1 + long + 1 + 1 + 4 + (3 if two_level_min else 0)
+    subs = sub_budgets(k, budget, mix)
+    together = len(subs) == 2 and all(K <= (1 << 19 if mix else 1 << 21) for _, K in subs)
+    if together:
+        total += 1
+    else:
+        for m, K in subs:
+            chunks = -(-K // DEFER_CHUNK) if m == 2 or m in grouped else 1
+            total += chunks * ((4 if m in grouped else 1) + (m == 2))
+    return total + 1   # the finalize
+
+
+def grouped_methods(h, subs, probe: str, order: str):
+    """The sub-methods of `subs` whose calls the library groups by first vertex:
+    behind the filter from 2^22 ids, in degree order from 2^24 and, but for
+    Path-5, where the vertex table has no level of at most 4,096 heavy columns."""
+    import paper_1509_08089_gb300 as moss
+    out = []
+    for m, K in subs:
+        least = 1 << 24 if order == "degree" else 1 << 22
+        if probe != "filter" or K < least:
+            continue
+        heavy = moss.moss_vertex_levels(h, m)[0]
+        if order == "degree" and m != 2 and 0 < heavy <= 4096:
+            continue
+        out.append(m)
+    return out
+
+
 def peaks_file() -> dict:
     path = os.path.join(ROOT, "MEASURED_PEAKS.json")
     return json.load(open(path)) if os.path.exists(path) else {}
@@ -376,8 +424,8 @@ def sampler_tables_bytes(rp, probe: str, methods) -> int:
     """Bytes of the device tables a sampling call reads, by the library's
     layout: 32 B slot records and 4 B ids per list entry, 16 B vertex records
     and a 32 B vertex alias record per vertex and method, and the hashed edge
-    set (32 B buckets, the next power of two >= nnz / 2) or the edge filter in
-    front of it (4 B words, the largest power of two <= nnz / 8) with the
+    set (32 B buckets, the next power of two >= nnz / 2, without the filter half
+    of that above 2^20) or the edge filter in front of it (4 B words, the largest power of two <= nnz / 8) with the
     hubs' rank table (8 B per 32 vertices) and adjacency bits (H^2,
     H = min(8192, max(16, n / 16)))."""
     n, nnz = len(rp) - 1, int(rp[-1])
@@ -386,6 +434,8 @@ def sampler_tables_bytes(rp, probe: str, methods) -> int:
         b = 2
         while b < (nnz + 1) // 2:
             b <<= 1
+        if probe == "hash" and b > 1 << 20:
+            b //= 2
         total += 32 * b
     if probe == "filter":
         w = 1
@@ -420,7 +470,7 @@ def small_case_traffic(workload: str, key: str, samples: int):
         else:
             rec[a] = b
     src = b"".join(open(os.path.join(ROOT, "paper_1509_08089_gb300", "csrc", f), "rb").read()
-                   for f in ("moss_sample.cu", "moss_internal.cuh"))
+                   for f in ("moss_sample.cu", "moss_sampler.cuh", "moss_group.cu", "moss_internal.cuh"))
     if hashlib.sha256(src).hexdigest()[:16] != rec.get("source_sha") or not pts:
         return None, None
     if len(pts) == 1:
@@ -651,6 +701,7 @@ def run_gpu(args):
         if args.vertex_split >= 0:
             moss.moss_set_vertex_split(h, args.vertex_split)
         moss.moss_build_tables(h, kmask, stream)
+        grouped = grouped_methods(h, sub_budgets(k, args.budget, mix), probe_name, order_main)
         times = time_calls(moss, torch, h, k, args.budget, mix, args.seed, stream, l2_flush)
     finally:
         moss.moss_graph_free(h)
@@ -668,8 +719,8 @@ def run_gpu(args):
                 "d2h_bytes_per_step": d2h},
         "roofline": roof,
         "clocks": clk,
-        "gpu_launches": launches_per_step(k, args.budget, mix, probe_name == "filter", *two_levels(args, len(rp) - 1),
-                                          ordered=order_main == "degree") * args.steps,
+        "gpu_launches": device_launches(rp, k, args.budget, mix, probe_name, *two_levels(args, len(rp) - 1), order_main,
+                                        grouped) * args.steps,
         "wall_s_timed": t_wall,
         "step_ms": step_ms,
     }
@@ -695,6 +746,7 @@ def run_gpu(args):
             moss.moss_set_probe(h, probe)
             moss.moss_set_rng(h, rng)
             moss.moss_build_tables(h, 1 << 5, stream)
+            g3 = grouped_methods(h, sub_budgets(5, B3, False), p3, o3)
             t3 = time_calls(moss, torch, h, 5, B3, False, args.seed, stream, l2_flush, reps=2)
         finally:
             moss.moss_graph_free(h)
@@ -708,7 +760,7 @@ def run_gpu(args):
                        "l2": "flushed (512 MB write) before every timed step; tables larger than the L2"},
             "roofline": roofline(data_key("cl_n4m", o3), rp3, p3, t3, [1, 2], l2_bytes, gather, peaks),
             "clocks": clk3,
-            "gpu_launches": launches_per_step(5, B3, False, p3 == "filter", True, ordered=o3 == "degree") * args.steps}
+            "gpu_launches": device_launches(rp3, 5, B3, False, p3, True, False, o3, g3) * args.steps}
         out["batched"] = measure_batched(moss, torch, [f.result() for f in futures["batched"]],
                                          batch_specs(args.graphs)[1], args.steps, args.warmup, stream, rng)
         out["served"] = measure_served(moss, [f.result() for f in futures["served"]], args.rate,

@@ -290,7 +290,7 @@ def moss_sample_counts(g: int, method: int, first: int, count: int, seed: int, c
 
 def moss_sample_counts_noalloc(g: int, method: int, first: int, count: int, seed: int, counts_dev, stream=None):
     """moss_sample_counts for callers that may not allocate device memory:
-    the per-block partial counts live in a fixed array inside the library."""
+    the counts add up in a fixed array inside the library."""
     _check(load().moss_sample_counts_noalloc(g, method, first, count, seed, _stream(stream), _ptr(counts_dev)))
 
 

@@ -421,9 +421,9 @@ __global__ void k_edge_filter(uint64_t nnz, const uint32_t *__restrict__ col, co
 // ------------------------------------------------ per-list sigma tables ---
 // Slot record (32 bytes) of position j of N_v: {col, nb, thr, alias} {off,
 // alias col, alias nb, alias off}, so a draw that takes the alias needs no
-// second load.  col, nb and off were set at load; the alias passes write thr
-// and alias (one 8-byte store), and k_slot_alias_fill then copies col, nb
-// and off of the alias position into words 5..7.
+// second load.  Lists up to kShortList entries are written whole; in longer ones
+// the alias passes write thr and alias (one 8-byte store), and k_slot_fill then
+// the rest.
 __device__ __forceinline__ void set_sigma(uint32_t *slot32, uint32_t o, uint32_t j, uint32_t thr, uint32_t alias) {
     *reinterpret_cast<uint2 *>(slot32 + 8 * (uint64_t)(o + j) + 2) = make_uint2(thr, alias);
 }
