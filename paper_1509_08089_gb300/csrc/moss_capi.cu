@@ -282,6 +282,7 @@ struct moss_graph {
     DevTotals tot_h{};
     unsigned built = 0;          // bit l: vertex table l; bit 3: sigma tables; bit 4: edge hash; bit 5: MOSS-4Min
     u128 *partials = nullptr;        // the vertex-weight totals' block sums
+    uint64_t *sums = nullptr;        // counts of the sampling calls, both sub-methods
     uint64_t *counts = nullptr;  // 2 x 22
     moss_result *res_dev = nullptr;
     double *cov_dev = nullptr;   // 22 x 22 covariance matrix
@@ -595,6 +596,7 @@ int moss_graph_load_csr_order(const void *row_ptr, int row_ptr_is_64, const uint
                 g->flags = st->flags;
             }
             g->partials = c.take<u128>((uint64_t)slot_partial_rows(n) * 6);
+            g->sums = c.take<uint64_t>(2 * kSlots);
             g->counts = c.take<uint64_t>(2 * kSlots);
             g->res_dev = c.take<moss_result>(1);
             g->cov_dev = c.take<double>(kSlots * kSlots);
@@ -908,7 +910,7 @@ static int sample_into(moss_graph *g, int method, uint64_t first, uint64_t count
 
 // zeroes the graph's sums of `methods` sub-methods
 static int clear_sums(moss_graph *g, int methods, cudaStream_t s) {
-    MOSS_CUDA(cudaMemsetAsync(g->counts, 0, methods * kSlots * sizeof(uint64_t), s), "clearing counts");
+    MOSS_CUDA(cudaMemsetAsync(g->sums, 0, methods * kSlots * sizeof(uint64_t), s), "clearing counts");
     return MOSS_OK;
 }
 
@@ -918,8 +920,8 @@ int moss_sample_counts(moss_graph *g, int method, uint64_t first, uint64_t count
     DeviceGuard dg(g->device);
     const cudaStream_t s = static_cast<cudaStream_t>(stream);
     int rc = clear_sums(g, 1, s);
-    if (rc || (rc = sample_into(g, method, first, count, seed, s, g->counts, nullptr, nullptr))) return rc;
-    MOSS_CUDA(launch_copy_counts(g->counts, counts_dev, count > 0, s), "copying counts");
+    if (rc || (rc = sample_into(g, method, first, count, seed, s, g->sums, nullptr, nullptr))) return rc;
+    MOSS_CUDA(launch_copy_counts(g->sums, counts_dev, count > 0, s), "copying counts");
     return MOSS_OK;
 }
 
@@ -929,7 +931,7 @@ int moss_sample_records(moss_graph *g, int method, uint64_t first, uint64_t coun
     DeviceGuard dg(g->device);
     const cudaStream_t s = static_cast<cudaStream_t>(stream);
     // (the counts that go with the records are not asked for: any base will do)
-    const int rc = sample_into(g, method, first, count, seed, s, g->counts, classes_dev, verts_dev);
+    const int rc = sample_into(g, method, first, count, seed, s, g->sums, classes_dev, verts_dev);
     if (rc || !g->order || !verts_dev) return rc;
     // vertex words of the records back to input ids (MOSS-4 and MOSS-4Min: the first four)
     MOSS_CUDA(launch_map_records(verts_dev, count, method == 1 || method == 2 ? 5 : 4, g->order, g->n, s),
@@ -937,28 +939,28 @@ int moss_sample_records(moss_graph *g, int method, uint64_t first, uint64_t coun
     return MOSS_OK;
 }
 
-// Both sub-methods of an estimate (ids from 0) up to their counts (g->counts):
+// Both sub-methods of an estimate (ids from 0) up to their counts (g->sums):
 // in one launch when they are small enough (same counts).
 static int sample_both(moss_graph *g, int ma, uint64_t ka, int mb, uint64_t kb, uint64_t seed, cudaStream_t s) {
     const bool mix = ma == MOSS_METHOD_MOSS4;
     int rc = clear_sums(g, 2, s);
     if (rc) return rc;
     if (pair_fits(mix, ka, kb)) {
-        MOSS_CUDA(launch_pair(mix, view(g), ka, kb, seed, g->counts, s), "sample kernels");
+        MOSS_CUDA(launch_pair(mix, view(g), ka, kb, seed, g->sums, s), "sample kernels");
         return MOSS_OK;
     }
     // the second method's blocks come in as the first's leave (after a grouped
     // launch, whose scratch is being given back, they start in order)
-    rc = sample_into(g, ma, 0, ka, seed, s, g->counts, nullptr, nullptr);
+    rc = sample_into(g, ma, 0, ka, seed, s, g->sums, nullptr, nullptr);
     const bool early = ka != 0 && group_bytes(ma, view(g), g->order != nullptr, ka) == 0;
-    return rc ? rc : sample_into(g, mb, 0, kb, seed, s, g->counts + kSlots, nullptr, nullptr, early);
+    return rc ? rc : sample_into(g, mb, 0, kb, seed, s, g->sums + kSlots, nullptr, nullptr, early);
 }
 
-// the result of the counts at g->counts
+// the result of the counts at g->sums
 static int finalize_sums(moss_graph *g, const FinalizeIn &in, cudaStream_t s, moss_result *out) {
     const bool drawn = in.K[0] || in.K[1];   // the launch before is a kernel
     HitsArg hits;
-    hits.dev = g->counts;
+    hits.dev = g->sums;
     MOSS_CUDA(launch_finalize(in, hits, g->tot, result_target(g), nullptr, s, drawn), "finalize kernel");
     return read_result(g, s, out);
 }
@@ -975,7 +977,7 @@ int moss_sample_estimate(moss_graph *g, int k, uint64_t budget, uint64_t seed, v
     if (k == 4) {
         if (!method_ready(g, 0)) return fail(MOSS_ESTATE, "tables for k=4 not built");
         in.K[0] = g->tot_h.gamma[0] ? budget : 0;
-        if ((rc = clear_sums(g, 2, s)) || (rc = sample_into(g, 0, 0, in.K[0], seed, s, g->counts, nullptr, nullptr))) return rc;
+        if ((rc = clear_sums(g, 2, s)) || (rc = sample_into(g, 0, 0, in.K[0], seed, s, g->sums, nullptr, nullptr))) return rc;
     } else {
         if (!method_ready(g, 1) || !method_ready(g, 2)) return fail(MOSS_ESTATE, "tables for k=5 not built");
         in.K[0] = g->tot_h.gamma[1] ? budget / 2 : 0;

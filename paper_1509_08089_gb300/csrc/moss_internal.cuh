@@ -422,7 +422,9 @@ cudaError_t launch_early(bool early, void (*kernel)(P...), int blocks, int threa
     cfg.stream = s;
     cfg.attrs = &attr;
     cfg.numAttrs = early ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+    if (e != cudaSuccess) cudaGetLastError();   // reported here, not by a later call
+    return e;
 }
 __device__ __forceinline__ void let_next_begin() { cudaTriggerProgrammaticLaunchCompletion(); }
 __device__ __forceinline__ void await_previous() { cudaGridDependencySynchronize(); }

@@ -91,3 +91,21 @@ def test_many_graphs_alive_and_released():
         if g.handle:
             assert np.array_equal(g.estimate(5, 1000, 5)["hits"], ref["hits"])
             g.close()
+
+
+def test_finalize_beside_a_sampling_call():
+    """Counts handed to a finalize on one stream leave those of a sampling call
+    in flight on another alone."""
+    rp, col = GRAPHS["cl_n20k"]()
+    K = 200_000_000
+    with moss.Graph(rp, col) as g:
+        ref = counts(g, 1, K, 2)
+        hits = torch.ones((2, 22), dtype=torch.int64, device="cuda")
+        out, res, Ks = torch.zeros(22, dtype=torch.int64, device="cuda"), moss.moss_result(), np.asarray([50, 50], np.uint64)
+        side = torch.cuda.Stream()
+        torch.cuda.synchronize()
+        moss.moss_sample_counts(g.handle, 1, 0, K, 2, out, side)
+        moss._check(moss.load().moss_finalize(g.handle, 5, moss._ptr(Ks), moss._ptr(hits), moss._stream(None), res))
+        side.synchronize()
+        assert np.array_equal(out.cpu().numpy().astype(np.uint64), ref)
+        assert (moss.result_dict(res)["hits"] == 1).all()
