@@ -388,7 +388,7 @@ def device_launches(rp, k: int, budget: int, mix: bool, probe: str, two_level: b
     if mix:   # the sort tiers, records, alias passes, picks, total and vertex table
         total += 1 + (d_max > 128) + (d_max > 1024) + 1 + 1 + long + 1 + 1 + 4 + (3 if two_level_min else 0)
     subs = sub_budgets(k, budget, mix)
-    together = len(subs) == 2 and all(K <= (1 << 19 if mix else 1 << 21) for _, K in subs)
+    together = len(subs) == 2 and all(K <= (1 << 16 if mix else 1 << 19) for _, K in subs)
     if together:
         total += 1
     else:

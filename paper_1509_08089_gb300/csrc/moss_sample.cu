@@ -541,16 +541,15 @@ cudaError_t launch_pair_rng(const DevGraph &g, int blocks, int blocks_a, uint64_
 
 }  // namespace
 
-// At four resident blocks per SM against the single launches' six, the pair
-// stops paying once the chip is full for long: k = 5 (us, two sampler launches
-// and two redraw stages -> one launch, 8k-edge graph / 2M-edge mesh / 1M-edge
-// power-law graph): budget 1e5 93 -> 42 / 94 -> 47 / 79 -> 44, 2e6 160 -> 128 /
-// 245 -> 203 / 155 -> 132, 5e6 269 -> 256 / 439 -> 431 / 267 -> 264, 1e7 455 ->
-// 466 / 766 -> 796 / 450 -> 485; the mix, which saves one launch, 1e5 52 -> 45 /
-// 54 -> 45 / 53 -> 45, 1e6 78 -> 68 / 119 -> 116 / 86 -> 79, 2e6 101 -> 92 / 167
-// -> 178 / 111 -> 109.
+// At four resident blocks per SM against the single launches' six, and without
+// their overlap, the pair stops paying once the chip is full for long.  Whole
+// estimates, us, launches of their own -> one launch (20k-edge graph / 2M-edge
+// mesh / 1M-edge power-law graph): k = 5, budget 1e5 55 -> 41 / 59 -> 44 / 52 ->
+// 40, 1e6 87 -> 82 / 122 -> 119 / 92 -> 86, 2e6 117 -> 120 / 173 -> 188 / 126 ->
+// 129; the mix, which has no redraws to save, 1e5 42 -> 40 / 45 -> 42 / 43 -> 40,
+// 5e5 51 -> 51 / 68 -> 78 / 54 -> 57.
 bool pair_fits(bool mix, uint64_t count_a, uint64_t count_b) {
-    const uint64_t most = mix ? 1ull << 19 : 1ull << 21;
+    const uint64_t most = mix ? 1ull << 16 : 1ull << 19;
     return count_a <= most && count_b <= most;
 }
 

@@ -13,7 +13,7 @@ torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
 MASK = (1 << 4) | (1 << 5) | moss.TABLES_4MIN
-K5_MOST, MIX_MOST = 1 << 21, 1 << 19     # ids per sub-method up to which both share a launch
+K5_MOST, MIX_MOST = 1 << 19, 1 << 16     # ids per sub-method up to which both share a launch
 
 GRAPHS = {
     "complete5": lambda: synth.complete(5),                                # Path-5 falls back often
