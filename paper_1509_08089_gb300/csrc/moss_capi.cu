@@ -987,14 +987,15 @@ int moss_sample_estimate(moss_graph *g, int k, uint64_t budget, uint64_t seed, v
     return finalize_sums(g, in, s, out);
 }
 
-// Counts handed in by the caller: host memory travels as a kernel argument,
-// device memory is read where it is copied to.
+// Counts handed in by the caller: pageable host memory travels as a kernel
+// argument; page-locked, managed and device memory, which earlier work on the
+// stream may still write, is copied in stream order.
 static int counts_arg(moss_graph *g, const uint64_t *hits, cudaStream_t s, HitsArg *arg) {
     cudaPointerAttributes pa;
     const bool known = cudaPointerGetAttributes(&pa, hits) == cudaSuccess;
     if (!known) cudaGetLastError();
     arg->dev = nullptr;
-    if (!known || pa.type == cudaMemoryTypeUnregistered || pa.type == cudaMemoryTypeHost) {
+    if (!known || pa.type == cudaMemoryTypeUnregistered) {
         memcpy(arg->h, hits, sizeof(arg->h));
         return MOSS_OK;
     }

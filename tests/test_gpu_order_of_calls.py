@@ -1,0 +1,48 @@
+"""What a call reads and writes follows its stream, whatever is in flight: counts
+in page-locked memory are read after the copy that fills them, and a call that
+is refused or draws nothing leaves the counts of another stream's call alone."""
+from __future__ import annotations
+
+import ctypes
+
+import numpy as np
+import pytest
+
+import synth
+import paper_1509_08089_gb300 as moss
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+MASK = (1 << 4) | (1 << 5) | moss.TABLES_4MIN
+LONG = 200_000_000   # samples of a call that is still running when the next one is made
+
+
+@pytest.fixture(scope="module")
+def graph():
+    rp, col = synth.chung_lu(20_000, 2.2, 12.0, 900.0, seed=3)
+    with moss.Graph(rp, col, k_mask=MASK) as g:
+        yield g
+
+
+@pytest.mark.parametrize("call", ["finalize", "covariance", "finalize_min"])
+def test_page_locked_counts_are_read_in_stream_order(graph, call):
+    lib, side = moss.load(), torch.cuda.Stream()
+    K = np.asarray([500, 500], dtype=np.uint64)
+    src = torch.full((2, 22), 3, dtype=torch.int64, device="cuda")
+    hits = torch.zeros((2, 22), dtype=torch.int64).pin_memory()
+    busy = torch.zeros(22, dtype=torch.int64, device="cuda")
+    cov, res = np.zeros((22, 22)), moss.moss_result()
+    torch.cuda.synchronize()
+    moss.moss_sample_counts(graph.handle, 1, 0, LONG, 2, busy, side)
+    with torch.cuda.stream(side):
+        hits.copy_(src, non_blocking=True)
+    assert not side.query()
+    h, s, out = ctypes.c_void_p(hits.data_ptr()), side.cuda_stream, ctypes.byref(res)
+    if call == "finalize":
+        moss._check(lib.moss_finalize(graph.handle, 5, moss._ptr(K), h, s, out))
+    elif call == "covariance":
+        moss._check(lib.moss_covariance(graph.handle, 5, moss._ptr(K), h, s, moss._ptr(cov), out))
+    else:
+        moss._check(lib.moss_finalize_min(graph.handle, moss._ptr(K), h, s, None, out))
+    assert (moss.result_dict(res)["hits"] == 3).all()
