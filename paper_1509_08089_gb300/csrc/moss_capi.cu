@@ -876,20 +876,25 @@ int moss_vertex_levels(const moss_graph *g, int which, uint32_t *nheavy, uint64_
     return MOSS_OK;
 }
 
-// adds the counts to the kSlots at sums (device memory of the graph); records
-static int sample_into(moss_graph *g, int method, uint64_t first, uint64_t count, uint64_t seed, cudaStream_t s,
-                       uint64_t *sums, uint8_t *classes, uint32_t *verts, bool early = false) {
+// whether samples first .. first + count - 1 of a method can be drawn; queues nothing
+static int check_samples(const moss_graph *g, int method, uint64_t first, uint64_t count) {
     if (method < 0 || method >= kMethods) return fail(MOSS_EINVAL, "method %d", method);
     if (!method_ready(g, method)) return fail(MOSS_ESTATE, "tables for method %d not built", method);
     if (count > 0 && g->tot_h.gamma[method] == 0)
         return fail(MOSS_EINVAL, "method %d has total weight 0 on this graph: no sample exists", method);
     if (first + count < first) return fail(MOSS_EOVERFLOW, "sample range wraps");
-    const DevGraph dv = view(g);
-    const int blocks = sample_launch_blocks(method, g->device, dv);
     // per-warp 32-bit counters: keep each launch below 2^31 samples per warp
-    const uint64_t max_chunk = (uint64_t)blocks * 8 * (1ULL << 31);
-    if (count == 0) return MOSS_OK;
+    const uint64_t max_chunk = (uint64_t)sample_launch_blocks(method, g->device, view(g)) * 8 * (1ULL << 31);
     if (count > max_chunk) return fail(MOSS_EOVERFLOW, "count above %llu per call", (unsigned long long)max_chunk);
+    return MOSS_OK;
+}
+
+// adds the counts of samples that check_samples admits to the kSlots at sums
+// (device memory of the graph); records
+static int sample_into(moss_graph *g, int method, uint64_t first, uint64_t count, uint64_t seed, cudaStream_t s,
+                       uint64_t *sums, uint8_t *classes, uint32_t *verts, bool early = false) {
+    if (count == 0) return MOSS_OK;
+    const DevGraph dv = view(g);
     // a large call behind the filter is grouped (the same counts) when its
     // scratch can be had; not under capture, where the call allocates nothing
     const uint64_t scratch_bytes = classes ? 0 : group_bytes(method, dv, g->order != nullptr, count);
@@ -908,7 +913,9 @@ static int sample_into(moss_graph *g, int method, uint64_t first, uint64_t count
     return MOSS_OK;
 }
 
-// zeroes the graph's sums of `methods` sub-methods
+// zeroes the graph's sums of `methods` sub-methods, for a call that is sure to
+// draw samples: one that is refused or empty leaves the sums to a call that
+// another stream may still be running
 static int clear_sums(moss_graph *g, int methods, cudaStream_t s) {
     MOSS_CUDA(cudaMemsetAsync(g->sums, 0, methods * kSlots * sizeof(uint64_t), s), "clearing counts");
     return MOSS_OK;
@@ -919,9 +926,15 @@ int moss_sample_counts(moss_graph *g, int method, uint64_t first, uint64_t count
     if (!g || !counts_dev) return fail(MOSS_EINVAL, "NULL argument");
     DeviceGuard dg(g->device);
     const cudaStream_t s = static_cast<cudaStream_t>(stream);
-    int rc = clear_sums(g, 1, s);
-    if (rc || (rc = sample_into(g, method, first, count, seed, s, g->sums, nullptr, nullptr))) return rc;
-    MOSS_CUDA(launch_copy_counts(g->sums, counts_dev, count > 0, s), "copying counts");
+    int rc = check_samples(g, method, first, count);
+    if (rc) return rc;
+    if (count == 0) {
+        MOSS_CUDA(cudaMemsetAsync(counts_dev, 0, kSlots * sizeof(uint64_t), s), "clearing counts");
+        return MOSS_OK;
+    }
+    if ((rc = clear_sums(g, 1, s)) || (rc = sample_into(g, method, first, count, seed, s, g->sums, nullptr, nullptr)))
+        return rc;
+    MOSS_CUDA(launch_copy_counts(g->sums, counts_dev, true, s), "copying counts");
     return MOSS_OK;
 }
 
@@ -931,7 +944,8 @@ int moss_sample_records(moss_graph *g, int method, uint64_t first, uint64_t coun
     DeviceGuard dg(g->device);
     const cudaStream_t s = static_cast<cudaStream_t>(stream);
     // (the counts that go with the records are not asked for: any base will do)
-    const int rc = sample_into(g, method, first, count, seed, s, g->sums, classes_dev, verts_dev);
+    int rc = check_samples(g, method, first, count);
+    if (!rc) rc = sample_into(g, method, first, count, seed, s, g->sums, classes_dev, verts_dev);
     if (rc || !g->order || !verts_dev) return rc;
     // vertex words of the records back to input ids (MOSS-4 and MOSS-4Min: the first four)
     MOSS_CUDA(launch_map_records(verts_dev, count, method == 1 || method == 2 ? 5 : 4, g->order, g->n, s),
@@ -943,8 +957,8 @@ int moss_sample_records(moss_graph *g, int method, uint64_t first, uint64_t coun
 // in one launch when they are small enough (same counts).
 static int sample_both(moss_graph *g, int ma, uint64_t ka, int mb, uint64_t kb, uint64_t seed, cudaStream_t s) {
     const bool mix = ma == MOSS_METHOD_MOSS4;
-    int rc = clear_sums(g, 2, s);
-    if (rc) return rc;
+    int rc = check_samples(g, ma, 0, ka);
+    if (rc || (rc = check_samples(g, mb, 0, kb)) || !(ka || kb) || (rc = clear_sums(g, 2, s))) return rc;
     if (pair_fits(mix, ka, kb)) {
         MOSS_CUDA(launch_pair(mix, view(g), ka, kb, seed, g->sums, s), "sample kernels");
         return MOSS_OK;
@@ -956,11 +970,11 @@ static int sample_both(moss_graph *g, int ma, uint64_t ka, int mb, uint64_t kb, 
     return rc ? rc : sample_into(g, mb, 0, kb, seed, s, g->sums + kSlots, nullptr, nullptr, early);
 }
 
-// the result of the counts at g->sums
+// the result of the counts at g->sums (of none where nothing is drawn)
 static int finalize_sums(moss_graph *g, const FinalizeIn &in, cudaStream_t s, moss_result *out) {
     const bool drawn = in.K[0] || in.K[1];   // the launch before is a kernel
-    HitsArg hits;
-    hits.dev = g->sums;
+    HitsArg hits = {};
+    hits.dev = drawn ? g->sums : nullptr;
     MOSS_CUDA(launch_finalize(in, hits, g->tot, result_target(g), nullptr, s, drawn), "finalize kernel");
     return read_result(g, s, out);
 }
@@ -977,7 +991,10 @@ int moss_sample_estimate(moss_graph *g, int k, uint64_t budget, uint64_t seed, v
     if (k == 4) {
         if (!method_ready(g, 0)) return fail(MOSS_ESTATE, "tables for k=4 not built");
         in.K[0] = g->tot_h.gamma[0] ? budget : 0;
-        if ((rc = clear_sums(g, 2, s)) || (rc = sample_into(g, 0, 0, in.K[0], seed, s, g->sums, nullptr, nullptr))) return rc;
+        if ((rc = check_samples(g, 0, 0, in.K[0]))) return rc;
+        if (in.K[0] && ((rc = clear_sums(g, 2, s)) ||
+                        (rc = sample_into(g, 0, 0, in.K[0], seed, s, g->sums, nullptr, nullptr))))
+            return rc;
     } else {
         if (!method_ready(g, 1) || !method_ready(g, 2)) return fail(MOSS_ESTATE, "tables for k=5 not built");
         in.K[0] = g->tot_h.gamma[1] ? budget / 2 : 0;

@@ -46,3 +46,40 @@ def test_page_locked_counts_are_read_in_stream_order(graph, call):
     else:
         moss._check(lib.moss_finalize_min(graph.handle, moss._ptr(K), h, s, None, out))
     assert (moss.result_dict(res)["hits"] == 3).all()
+
+
+def refused(g, out):
+    for method, first, count in ((-1, 0, 5), (7, 0, 5), (1, 2**64 - 1, 2), (2, 0, 2**63)):
+        with pytest.raises(moss.MossError):
+            moss.moss_sample_counts(g.handle, method, first, count, 2, out)
+    with pytest.raises(moss.MossError):
+        g.estimate(4, 2**63, 2)
+    with pytest.raises(moss.MossError):
+        g.estimate_min(5, 2**63, 2)
+
+
+def empty(g, out):
+    moss.moss_sample_counts(g.handle, 1, 9, 0, 2, out)
+    for r in (g.estimate(4, 0, 2), g.estimate(5, 0, 2), g.estimate_min(0, 0, 2)):
+        assert not r["hits"].any()
+    torch.cuda.current_stream().synchronize()
+    assert not out.any()
+
+
+@pytest.mark.parametrize("other", [refused, empty])
+@pytest.mark.parametrize("method", [1, 2])
+def test_a_call_that_draws_nothing_leaves_another_streams_counts(graph, method, other):
+    def counts(stream=None):
+        moss.moss_sample_counts(graph.handle, method, 0, LONG, 2, out, stream)
+
+    out, none = (torch.full((22,), -1, dtype=torch.int64, device="cuda") for _ in range(2))
+    counts()
+    torch.cuda.synchronize()
+    ref = out.clone()
+    side = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    counts(side)
+    assert not side.query()
+    other(graph, none)
+    side.synchronize()
+    assert torch.equal(out, ref)
