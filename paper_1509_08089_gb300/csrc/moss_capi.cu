@@ -328,11 +328,13 @@ void release(moss_graph *g) {
 // otherwise: beside 32 bytes of slot record per list entry, a set of 64 MiB no
 // longer stays in the L2, and its misses cost more than the buckets that
 // overflow.  1e7 samples, ms, four to eight slots -> two to four (MOSS-4, T-5,
-// Path-5, MOSS-4Min): power-law graph, 2.5M entries 0.35 -> 0.27, 0.45 -> 0.39,
-// 0.59 -> 0.47, 0.34 -> 0.30; 4.1M 0.40 -> 0.32, 0.43 -> 0.51, 0.68 -> 0.61,
-// 0.40 -> 0.37; mesh, 2.3M 0.33 -> 0.28, 0.48 -> 0.39, 0.64 -> 0.48, 0.38 ->
-// 0.30; 3.9M 0.43 -> 0.32, 0.62 -> 0.48, 0.80 -> 0.64, 0.52 -> 0.42; larger ones
-// with the hash asked for gain 10-40%.  On 1.95M entries, all of it in the L2,
+// Path-5, MOSS-4Min): power-law graph, 2.6M entries 0.34 -> 0.28, 0.45 -> 0.38,
+// 0.63 -> 0.48, 0.36 -> 0.30; 4.0M 0.44 -> 0.32, 0.46 -> 0.44, 0.79 -> 0.54,
+// 0.40 -> 0.34; mesh, 2.6M 0.35 -> 0.28, 0.51 -> 0.39, 0.65 -> 0.48, 0.41 ->
+// 0.30; 4.0M 0.45 -> 0.34, 0.62 -> 0.45, 0.81 -> 0.58, 0.54 -> 0.39; larger ones
+// with the hash asked for gain 10-40%.  The skew matters to T-5 alone, which on
+// power-law graphs of 3.6-4.0M entries gains 7% to loses 3% (it reads few slot
+// records from outside the L2, so it has little to win).  On 1.95M entries, all of it in the L2,
 // 16 MiB instead of 32 cost 25%; behind the filter the halves gain up to 15% on
 // meshes of 6-13M entries and cost 1-8% on power-law graphs of that size.
 constexpr uint64_t kRoomyBuckets = 1ull << 20;
