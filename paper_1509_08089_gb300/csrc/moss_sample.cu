@@ -227,13 +227,13 @@ constexpr int kBatchBlocks = 4;   // resident blocks per SM (Path-5 bound)
 template <bool HASH, int RNG>
 __device__ __forceinline__ int sample_any(const DevGraph &g, const uint8_t *lut4, const uint8_t *lut5,
                                           const uint8_t *lutc, uint32_t method, uint64_t seed, uint64_t s) {
-    if (method == 0) return sample_moss4<RNG, HASH>(g, lut4, seed, s).cls;
-    if (method == 1) return sample_t5<RNG, HASH>(g, lut5, seed, s).cls;
+    if (method == 0) return sample_moss4<RNG, HASH, kPmBatch>(g, lut4, seed, s).cls;
+    if (method == 1) return sample_t5<RNG, HASH, kPmBatch>(g, lut5, seed, s).cls;
     if (method == 3) {
-        const Sample sm = sample_min<RNG, HASH>(g, lut4, lutc, seed, s);
+        const Sample sm = sample_min<RNG, HASH, kPmBatch>(g, lut4, lutc, seed, s);
         return min_slot(sm.cls, sm.v[4]);
     }
-    return sample_path5<RNG, HASH, 3>(g, lut5, seed, s).cls;
+    return sample_path5<RNG, HASH, 3, kPmBatch>(g, lut5, seed, s).cls;
 }
 
 // Persistent sampler over a batch: warps take tiles of `tile_samples` ids of

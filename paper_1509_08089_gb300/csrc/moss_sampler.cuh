@@ -38,9 +38,31 @@ __device__ __forceinline__ uint32_t ld1(const uint32_t *p) { return __ldg(p); }
 // kPmGroup is kPmFilter for samples grouped by their first vertex v
 // (moss_group.cu): its neighbours in the group read v's slot records again, so
 // those are not read evict-first.
-constexpr int kPmPlain = 0, kPmFilter = 1, kPmStream = 2, kPmGroup = 3;
+constexpr int kPmPlain = 0, kPmFilter = 1, kPmStream = 2, kPmGroup = 3, kPmBatch = 4;
 constexpr uint32_t kStreamHeavy = 4096;   // heavy columns (32 B each) that kPmStream keeps in L1
 __host__ __device__ constexpr bool behind_filter(int pm) { return pm == kPmFilter || pm == kPmGroup; }
+
+// How a sample's pairs walk the edge set: in rounds over all of them, one bucket
+// each; by lanes, each lane its own next pair, from the first bucket on; or the
+// home buckets of all of them together and the full ones' pairs by lanes.
+//   Without the filter, a set of two slots an edge sends 14% of the pairs past
+// their home bucket, and with another round over all pairs nearly every p has
+// some lane waiting.  1.7e7 samples, ms, rounds -> home then lanes: power-law
+// graph of 4M entries T-5 0.79 -> 0.74, Path-5 1.02 -> 0.88, mesh of 4M 0.82 ->
+// 0.74 and 1.13 -> 1.00; roomier sets 0-1% either way, and the redraws, which
+// would spill, stay with rounds.
+//   Behind the filter few pairs reach the set.  Grouped samples go by lanes (the
+// 34M-edge step 70.4 ms, 73.2 with the home buckets first).  Ungrouped ones by
+// lanes / in rounds, ms: Path-5 1.02 / 1.05 (7M edges, degree order), 1.19 / 1.24
+// (4M), but T-5 1.94 / 1.80 (34M edges), 1.04 / 1.00 (4M), MOSS-4Min 0.99 / 0.95
+// (7M).  Batches (kPmBatch, otherwise as kPmPlain) keep the rounds: 13.7 ms for
+// 256 graphs, 13.9 with the home buckets first.
+constexpr int kRounds = 0, kLanes = 1, kHomeThenLanes = 2;
+__host__ __device__ constexpr int walk_of(int pm, int method, int stage = 0) {
+    if (behind_filter(pm) || pm == kPmBatch)
+        return kHubProbes[method] && (pm != kPmFilter || method == 2) ? kLanes : kRounds;
+    return stage == 1 || stage == 2 ? kRounds : kHomeThenLanes;
+}
 
 // a vertex record without L1 allocation
 __device__ __forceinline__ uint4 ld4_na(const uint4 *p) {
@@ -252,6 +274,33 @@ __device__ __forceinline__ bool holds(const Sector &e, uint64_t key) {
            (e.hi.z == lo && e.hi.w == hi);
 }
 
+// The pairs of `pending` in the set from bucket `first` after their home on, each
+// lane its own next one: where few pairs are left, at different p in the lanes
+// of a warp, the warp makes as many rounds of dependent loads as its busiest
+// lane has buckets to see, not one for every p.  Returns the pairs found.
+template <int P, int PM>
+__device__ __forceinline__ uint32_t probe_lanes(const DevGraph &g, const uint32_t (&a)[P], const uint32_t (&b)[P],
+                                                uint32_t pending, uint32_t first) {
+    uint32_t found = 0, step = first;
+    while (pending != 0) {   // (a set has two buckets at least: hash_mask >= 1)
+        const uint32_t p = __ffs(pending) - 1;
+        uint32_t x = a[0], y = b[0];
+#pragma unroll
+        for (int q = 1; q < P; ++q) {
+            x = p == q ? a[q] : x;
+            y = p == q ? b[q] : y;
+        }
+        const uint64_t key = edge_key(x, y);
+        const Sector e = ld8s<PM>(g.hash + 2 * (uint64_t)((edge_bucket(key, g.hash_shift) + step) & g.hash_mask));
+        const bool hit = holds(e, key);
+        const bool last = hit || (e.hi.z == 0xffffffffu && e.hi.w == 0xffffffffu) || step == g.hash_mask;
+        found |= (uint32_t)hit << p;
+        pending &= ~((uint32_t)last << p);
+        step = last ? first : step + 1;
+    }
+    return found;
+}
+
 // Membership tests through the hashed edge set: one 32-byte bucket load per
 // pair in the common case, all P loads issued together.  kPmFilter (behind
 // the filter): the filter rules out most pairs; the set is far larger than the
@@ -260,7 +309,7 @@ __device__ __forceinline__ bool holds(const Sector &e, uint64_t key) {
 // the ends' rank-table entries come first (one 8-byte load per vertex, all
 // together), and a pair of two hubs is answered by one bit of the hubs'
 // adjacency bitmap, loaded beside the other pairs' filter words.
-template <int P, int PM, bool HUB>
+template <int P, int PM, bool HUB, int WALK>
 __device__ __forceinline__ uint32_t probe_hash(const DevGraph &g, const uint32_t (&a)[P], const uint32_t (&b)[P]) {
     uint32_t found = 0, pending = (1u << P) - 1u;
     if (g.filter) {   // warp-uniform: only pairs the filter cannot rule out go to the set
@@ -297,64 +346,42 @@ __device__ __forceinline__ uint32_t probe_hash(const DevGraph &g, const uint32_t
                 if ((word[p] & m) != m) pending &= ~(1u << p);
             }
         }
-        if (HUB) {
-            // few pairs are left, at different p in the lanes of a warp: each lane
-            // takes its own next one, so the warp makes as many rounds of dependent
-            // loads as its busiest lane has pairs, not one for every p
-            uint32_t step = 0;
-            while (pending != 0) {
-                const uint32_t p = __ffs(pending) - 1;
-                uint32_t x = a[0], y = b[0];
-    #pragma unroll
-                for (int q = 1; q < P; ++q) {
-                    x = p == q ? a[q] : x;
-                    y = p == q ? b[q] : y;
+        if constexpr (WALK == kLanes) return found | probe_lanes<P, PM>(g, a, b, pending, 0);
+    }
+    if constexpr (WALK != kHomeThenLanes) {
+        uint32_t bk[P];
+#pragma unroll
+        for (int p = 0; p < P; ++p) bk[p] = edge_bucket(edge_key(a[p], b[p]), g.hash_shift);
+        for (uint32_t it = 0; pending != 0 && it <= g.hash_mask; ++it) {
+#pragma unroll
+            for (int p = 0; p < P; ++p) {
+                if (pending >> p & 1u) {
+                    const Sector e = ld8s<PM>(g.hash + 2 * (uint64_t)bk[p]);
+                    if (holds(e, edge_key(a[p], b[p]))) {
+                        found |= 1u << p;
+                        pending &= ~(1u << p);
+                    } else if (e.hi.z == 0xffffffffu && e.hi.w == 0xffffffffu) {   // last slot empty
+                        pending &= ~(1u << p);
+                    } else {
+                        bk[p] = (bk[p] + 1) & g.hash_mask;
+                    }
                 }
-                const uint64_t key = edge_key(x, y);
-                const Sector e = ld8s<PM>(g.hash + 2 * (uint64_t)((edge_bucket(key, g.hash_shift) + step) & g.hash_mask));
-                const bool hit = holds(e, key);
-                const bool last = hit || (e.hi.z == 0xffffffffu && e.hi.w == 0xffffffffu) || step == g.hash_mask;
-                found |= (uint32_t)hit << p;
-                pending &= ~((uint32_t)last << p);
-                step = last ? 0 : step + 1;
             }
-            return found;
         }
-    }
-    // the home buckets of all pairs together
+        return found;
+    } else {
 #pragma unroll
-    for (int p = 0; p < P; ++p) {
-        if (pending >> p & 1u) {
-            const uint64_t key = edge_key(a[p], b[p]);
-            const Sector e = ld8s<PM>(g.hash + 2 * (uint64_t)edge_bucket(key, g.hash_shift));
-            const bool hit = holds(e, key);
-            found |= (uint32_t)hit << p;
-            if (hit || (e.hi.z == 0xffffffffu && e.hi.w == 0xffffffffu)) pending &= ~(1u << p);
+        for (int p = 0; p < P; ++p) {
+            if (pending >> p & 1u) {
+                const uint64_t key = edge_key(a[p], b[p]);
+                const Sector e = ld8s<PM>(g.hash + 2 * (uint64_t)edge_bucket(key, g.hash_shift));
+                const bool hit = holds(e, key);
+                found |= (uint32_t)hit << p;
+                if (hit || (e.hi.z == 0xffffffffu && e.hi.w == 0xffffffffu)) pending &= ~(1u << p);
+            }
         }
+        return found | probe_lanes<P, PM>(g, a, b, pending, 1);
     }
-    // Pairs whose home bucket is full go on, each lane with its own next one.  A
-    // set of two slots an edge has 14% of them: with another round over all pairs
-    // nearly every p had some lane waiting, and T-5 of 1.7e7 samples took 0.79 ms
-    // on a power-law graph of 4M entries (0.71 with a set twice as large, 0.72
-    // like this; Path-5 1.03 -> 0.87, on a mesh of 4M entries 1.14 -> 0.97).
-    uint32_t step = 1;
-    while (pending != 0 && step <= g.hash_mask) {
-        const uint32_t p = __ffs(pending) - 1;
-        uint32_t x = a[0], y = b[0];
-#pragma unroll
-        for (int q = 1; q < P; ++q) {
-            x = p == q ? a[q] : x;
-            y = p == q ? b[q] : y;
-        }
-        const uint64_t key = edge_key(x, y);
-        const Sector e = ld8s<PM>(g.hash + 2 * (uint64_t)((edge_bucket(key, g.hash_shift) + step) & g.hash_mask));
-        const bool hit = holds(e, key);
-        const bool last = hit || (e.hi.z == 0xffffffffu && e.hi.w == 0xffffffffu) || step == g.hash_mask;
-        found |= (uint32_t)hit << p;
-        pending &= ~((uint32_t)last << p);
-        step = last ? 1 : step + 1;
-    }
-    return found;
 }
 
 struct Sample {
@@ -397,7 +424,7 @@ __device__ __forceinline__ Sample rest_moss4(const DevGraph &g, const uint8_t *l
     const uint32_t A[3] = {v, pu.id, w}, B[3] = {r, w, r};
     uint32_t f;
     if (HASH) {
-        f = probe_hash<3, PM, kHubProbes[0]>(g, A, B);
+        f = probe_hash<3, PM, kHubProbes[0], walk_of(PM, 0)>(g, A, B);
     } else {
         const uint4 ur = make_uint4(pu.off, pu.deg, 0u, 0u), wr = ld4(g.vert + w), rr = ld4(g.vert + r);
         const uint4 ra[3] = {vr, ur, wr}, rb[3] = {rr, wr, rr};
@@ -438,7 +465,7 @@ __device__ __forceinline__ Sample rest_t5(const DevGraph &g, const uint8_t *lut,
     const uint32_t A[6] = {pu.id, pu.id, w, v, w, r}, B[6] = {w, r, r, t, t, t};
     uint32_t f;
     if (HASH) {
-        f = probe_hash<6, PM, kHubProbes[1]>(g, A, B);
+        f = probe_hash<6, PM, kHubProbes[1], walk_of(PM, 1)>(g, A, B);
     } else {
         const uint4 ur = make_uint4(pu.off, pu.deg, 0u, 0u);
         const uint4 wr = ld4(g.vert + w), rr = ld4(g.vert + r), tr = ld4(g.vert + t);
@@ -527,7 +554,7 @@ __device__ __forceinline__ Sample rest_min(const DevGraph &g, const uint8_t *lut
     const uint32_t A[3] = {v, u, w}, B[3] = {r, w, r};
     uint32_t f;
     if (HASH) {
-        f = probe_hash<3, PM, kHubProbes[3]>(g, A, B);
+        f = probe_hash<3, PM, kHubProbes[3], walk_of(PM, 3)>(g, A, B);
     } else {
         const uint4 vr = make_uint4(mv.x, mv.y, 0u, 0u), ur = make_uint4(sb.x, sb.y, 0u, 0u);
         const uint4 wr = ld4(g.vert + w), rr = ld4(g.vert + r);
@@ -648,7 +675,7 @@ __device__ __forceinline__ Sample rest_path5(const DevGraph &g, const uint8_t *l
     const uint32_t A[6] = {v, v, u, u, w, r}, B[6] = {r, t, w, t, r, t};
     uint32_t f;
     if (HASH) {
-        f = probe_hash<6, PM, kHubProbes[2]>(g, A, B);
+        f = probe_hash<6, PM, kHubProbes[2], walk_of(PM, 2, STAGE)>(g, A, B);
     } else {
         const uint4 ur = make_uint4(pu.off, pu.deg, 0u, 0u), wr = make_uint4(pw.off, pw.deg, 0u, 0u);
         const uint4 rr = ld4(g.vert + r), tr = ld4(g.vert + t);
