@@ -449,9 +449,19 @@ int sample_per_sm(int method, int device, int variant) {
     return per[variant];
 }
 
+// Blocks of a sampling launch: as many as fit, but for MOSS-4 behind the filter
+// at most the 6 an SM that every sampler is compiled for.  Its registers would
+// let 8 in, and their reads push one another's lines out of the L2 where no
+// small heavy level holds most of the draws: 1.7e7 samples, ms, 8 -> 6 an SM:
+// mesh of 2.3M edges 0.99 -> 0.93, 8M edges, 2M vertices 0.79 -> 0.76, 34M edges
+// 1.44 -> 1.42.  With a heavy level of at most kStreamHeavy columns 8 stay (3.5M
+// edges, degree order, 0.56 -> 0.60 with 6; 7M 0.59 -> 0.61).
 int sample_launch_blocks(int method, int device, const DevGraph &g) {
-    return device_sms(device) *
-           sample_per_sm(method, device, probe_variant(method, g) + (g.rng == kRngPhilox ? kProbeVariants : 0));
+    const int variant = probe_variant(method, g);
+    int per = sample_per_sm(method, device, variant + (g.rng == kRngPhilox ? kProbeVariants : 0));
+    const bool few_heavy = g.nheavy[method] != 0 && g.nheavy[method] <= kStreamHeavy;
+    if (method == 0 && variant == 2 && !few_heavy) per = std::min(per, min_blocks<0, kRngSplitMix>());
+    return device_sms(device) * per;
 }
 
 namespace {
