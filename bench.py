@@ -399,20 +399,25 @@ def device_launches(rp, k: int, budget: int, mix: bool, probe: str, two_level: b
 
 
 def grouped_methods(h, subs, probe: str, order: str):
-    """The sub-methods of `subs` whose calls the library groups by first vertex:
-    behind the filter from 2^22 ids, in degree order from 2^24 and, but for
-    Path-5, where the vertex table has no level of at most 4,096 heavy columns."""
+    """The sub-methods of `subs` whose calls the library groups by first vertex
+    (its rule on the list entries, the vertex table's heavy columns and the ids)."""
     import paper_1509_08089_gb300 as moss
-    out = []
-    for m, K in subs:
-        least = 1 << 24 if order == "degree" else 1 << 22
-        if probe != "filter" or K < least:
-            continue
-        heavy = moss.moss_vertex_levels(h, m)[0]
-        if order == "degree" and m != 2 and 0 < heavy <= 4096:
-            continue
-        out.append(m)
-    return out
+    nnz = int(moss.moss_graph_stats(h).nnz)
+    return [m for m, K in subs if groups(m, nnz, moss.moss_vertex_levels(h, m)[0], K, probe, order)]
+
+
+def groups(m: int, nnz: int, heavy: int, K: int, probe: str, order: str) -> bool:
+    if probe != "filter":
+        return False
+    few, many = 0 < heavy <= 4096, heavy > 4096
+    if order == "degree":
+        if (few and m != 2) or (many and nnz < {0: 1 << 25, 2: 1 << 24}.get(m, 0)):
+            return False
+        return K >= 1 << 24
+    if few and m <= 1 and nnz < 1 << 23:
+        return False
+    late = nnz < 1 << 24 if m == 0 else (few or m == 3) and nnz < 3 << 22
+    return K >= (1 << 23 if late else 1 << 22)
 
 
 def peaks_file() -> dict:

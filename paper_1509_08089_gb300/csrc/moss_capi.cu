@@ -899,7 +899,7 @@ static int sample_into(moss_graph *g, int method, uint64_t first, uint64_t count
     const DevGraph dv = view(g);
     // a large call behind the filter is grouped (the same counts) when its
     // scratch can be had; not under capture, where the call allocates nothing
-    const uint64_t scratch_bytes = classes ? 0 : group_bytes(method, dv, g->order != nullptr, count);
+    const uint64_t scratch_bytes = classes ? 0 : group_bytes(method, dv, g->order != nullptr, g->nnz, count);
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusActive;
     if (scratch_bytes && cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone) {
         void *scratch = nullptr;
@@ -968,7 +968,7 @@ static int sample_both(moss_graph *g, int ma, uint64_t ka, int mb, uint64_t kb, 
     // the second method's blocks come in as the first's leave (after a grouped
     // launch, whose scratch is being given back, they start in order)
     rc = sample_into(g, ma, 0, ka, seed, s, g->sums, nullptr, nullptr);
-    const bool early = ka != 0 && group_bytes(ma, view(g), g->order != nullptr, ka) == 0;
+    const bool early = ka != 0 && group_bytes(ma, view(g), g->order != nullptr, g->nnz, ka) == 0;
     return rc ? rc : sample_into(g, mb, 0, kb, seed, s, g->sums + kSlots, nullptr, nullptr, early);
 }
 

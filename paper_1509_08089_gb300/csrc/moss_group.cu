@@ -275,22 +275,45 @@ void upload_luts_group(const uint8_t *lut4, const uint8_t *lut5, const uint8_t *
 // Which calls are grouped: those behind the filter (the tables exceed the
 // L2; on the 1M-edge graph, whose tables fit it, grouping cost 6-18%) with
 // enough ids to pay for the draw and placement passes and their scattered
-// scratch.  Measured per 1e6 ids of each call, ungrouped / grouped ms:
-//   input ids, 34M edges:  2M 0.18 / 0.20 (MOSS-4), 4M 0.34 / 0.32, 0.44 / 0.32
-//     (T-5), 0.52 / 0.50 (Path-5), 0.39 / 0.35 (MOSS-4Min)     -> from 2^22
-//   degree order, 34M edges: 8M 0.44 / 0.49, 0.52 / 0.51, 0.73 / 0.81, 0.60 /
-//     0.54; 16M 0.86 / 0.81, 0.99 / 0.93, 1.40 / 1.36, 1.17 / 0.99 -> from 2^24
-//   degree order, 7M edges (587, 367, 661 heavy vertices, the MOSS-4Min table
-//     one level): 16M 0.54 / 0.59, 0.80 / 0.83, 0.98 / 0.95, 0.82 / 0.71.  The
-//     few heavy vertices' lists lie together and stay in the L2 anyway, so
-//     only Path-5, with two slot records of v per sample, and tables without
-//     a heavy level gain.
-uint64_t group_bytes(int method, const DevGraph &g, bool degree_order, uint64_t count) {
-    if (!g.hash || !g.filter) return 0;
+// scratch.  What it gains grows with the tables; it gains least where few heavy
+// vertices hold most draws (the table's heavy level has kStreamHeavy columns at
+// most), as their lists stay in the L2 anyway, and in degree order, where those
+// lists lie together besides.  Grouped / ungrouped time of MOSS-4, T-5, Path-5,
+// MOSS-4Min (power-law graphs unless a mesh; entries):
+//   input ids, few heavy    2^22 ids                 2^23                     2^26
+//     4.4M               1.28 1.13 1.05 1.05      1.19 1.13 1.01 0.99      1.13 1.08 0.96 0.93
+//     6.9M               1.17 1.03 0.96 1.01      1.06 1.01 0.89 0.96      0.97 0.99 0.83 0.94
+//     9.0M               1.13 1.04 0.95 0.99      0.99 1.01 0.89 0.94      0.89 0.98 0.85 0.91
+//     14M                0.97 0.95 0.83 0.93      0.84 0.90 0.78 0.88      0.74 0.88 0.72 0.84
+//   input ids, others
+//     4.7M (mesh)        0.98 0.92 0.90 0.97      0.87 0.85 0.84 0.89      0.85 0.82 0.82 0.85
+//     16M                1.04 0.89 0.95 1.02      0.95 0.87 0.91 0.96      0.89 0.85 0.89 0.95
+//     24M                0.94 0.95 0.82 0.92      0.84 0.92 0.76 0.84      0.76 0.89 0.71 0.81
+//     67M                0.82 0.75 0.83 0.89      0.76 0.72 0.79 0.84      0.72 0.70 0.75 0.82
+//   degree order            2^23                     2^24                     2^26
+//     4.4M, few heavy    1.23 1.00 0.88 1.03      1.21 0.98 0.84 0.97      1.18 0.97 0.82 0.94
+//     14M, few heavy     1.09 0.99 0.98 0.87      1.08 0.98 0.97 0.86      1.06 0.96 0.97 0.86
+//     4.7M (mesh)        0.88 0.88 0.84 0.91      0.86 0.88 0.82 0.89      0.86 0.89 0.82 0.90
+//     16M                1.08 0.97 1.04 0.98      1.04 0.96 1.04 0.97      1.01 0.94 1.04 0.98
+//     24M                1.09 0.99 1.01 1.00      1.05 0.97 0.99 0.96      1.03 0.96 0.97 0.95
+//     47M                1.02 0.99 0.90 0.94      0.98 0.98 0.86 0.92      0.95 0.97 0.84 0.91
+//     67M                0.93 0.95 0.85 0.90      0.89 0.93 0.77 0.87      0.86 0.91 0.73 0.85
+static bool groups(int method, const DevGraph &g, bool degree_order, uint64_t nnz, uint64_t count) {
+    if (!g.hash || !g.filter) return false;
     const bool few_heavy = g.nheavy[method] != 0 && g.nheavy[method] <= kStreamHeavy;
-    if (degree_order && few_heavy && method != 2) return 0;
-    if (count < (degree_order ? 1ull << 24 : 1ull << 22)) return 0;
-    return scratch_bytes(std::min(count, kGroupChunk));
+    const bool many_heavy = g.nheavy[method] > kStreamHeavy;
+    if (degree_order) {
+        if (few_heavy && method != 2) return false;
+        if (many_heavy && nnz < (method == 0 ? 1ull << 25 : method == 2 ? 1ull << 24 : 0)) return false;
+        return count >= 1ull << 24;
+    }
+    if (few_heavy && method <= 1 && nnz < 1ull << 23) return false;
+    const bool late = method == 0 ? nnz < 1ull << 24 : (few_heavy || method == 3) && nnz < 3ull << 22;
+    return count >= (late ? 1ull << 23 : 1ull << 22);
+}
+
+uint64_t group_bytes(int method, const DevGraph &g, bool degree_order, uint64_t nnz, uint64_t count) {
+    return groups(method, g, degree_order, nnz, count) ? scratch_bytes(std::min(count, kGroupChunk)) : 0;
 }
 
 cudaError_t launch_counts_grouped(int method, const DevGraph &g, uint64_t first, uint64_t count, uint64_t seed,

@@ -454,7 +454,7 @@ int sample_launch_blocks(int method, int device, const DevGraph &g);   // blocks
 // moss_group.cu: large calls behind the filter, the sample ids grouped by their first vertex
 void upload_luts_group(const uint8_t *lut4, const uint8_t *lut5, const uint8_t *lutc);
 // scratch of a grouped call; 0 when the call is not one to group
-uint64_t group_bytes(int method, const DevGraph &g, bool degree_order, uint64_t count);
+uint64_t group_bytes(int method, const DevGraph &g, bool degree_order, uint64_t nnz, uint64_t count);
 cudaError_t launch_counts_grouped(int method, const DevGraph &g, uint64_t first, uint64_t count, uint64_t seed,
                                   uint64_t *sums, void *scratch, cudaStream_t s);
 
