@@ -175,6 +175,8 @@ void build_host_luts() {
     }
 }
 
+void make_pins();   // host staging, below
+
 int ensure_luts(int device) {
     std::lock_guard<std::mutex> lk(g_lut_mutex);
     build_host_luts();
@@ -183,6 +185,7 @@ int ensure_luts(int device) {
         upload_luts(g_lut4_h, g_lut5_h, g_lutc_h);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return cuda_fail(e, "uploading class tables");
+        make_pins();
         g_lut_ready[device] = true;
     }
     return MOSS_OK;
@@ -197,9 +200,9 @@ struct DevStatus {
     uint32_t flags[2];
 };
 
-// Page-locked host memory of one graph: kernels write results straight into
-// it and totals are copied to it without staging (a copy into ordinary memory
-// costs the caller about 10 us each).
+// Page-locked host memory of one synchronous call: kernels write results
+// straight into it and totals are copied to it without staging (a copy into
+// ordinary memory costs the caller about 10 us each).
 struct Pinned {
     moss_result res;
     double cov[kSlots * kSlots];
@@ -207,55 +210,47 @@ struct Pinned {
 };
 
 namespace {
-// Slots of page-locked memory, kPinBatch per allocation (one costs tens of
-// us); an allocation with no slot in use is given back unless it is the only
-// one, so what is held follows the number of graphs alive.
-constexpr int kPinBatch = 32;
-struct PinBatch {
-    Pinned *mem = nullptr;
-    uint32_t used = 0;   // bit i: slot i taken
-};
+// Slots of page-locked memory that calls borrow until they return: one block of
+// kPinSlots (190 KB), made at the first load and kept like the class tables.
+// Nothing is allocated or freed later, which would wait for the device or, when
+// another thread captures a stream in global mode, fail and end its capture; a
+// call that finds no slot reads back through copies.
+constexpr int kPinSlots = 32;
 std::mutex g_pin_mutex;
-std::vector<PinBatch> g_pins;
+Pinned *g_pins = nullptr;
+uint32_t g_pins_used = 0;   // bit i: slot i lent
 
-Pinned *pin_take() {
-    std::lock_guard<std::mutex> lk(g_pin_mutex);
-    for (PinBatch &b : g_pins)
-        for (int i = 0; i < kPinBatch; ++i)
-            if (!(b.used >> i & 1u)) {
-                b.used |= 1u << i;
-                return b.mem + i;
-            }
-    try {
-        g_pins.reserve(g_pins.size() + 1);
-    } catch (...) {
-        return nullptr;
-    }
-    PinBatch b;
-    if (cudaHostAlloc(reinterpret_cast<void **>(&b.mem), kPinBatch * sizeof(Pinned),
-                      cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
+// (callers hold g_lut_mutex)
+void make_pins() {
+    if (g_pins) return;
+    void *p = nullptr;
+    if (cudaHostAlloc(&p, kPinSlots * sizeof(Pinned), cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
         cudaGetLastError();
-        return nullptr;
-    }
-    b.used = 1;
-    g_pins.push_back(b);
-    return b.mem;
-}
-
-void pin_give(Pinned *p) {
-    if (!p) return;
-    std::lock_guard<std::mutex> lk(g_pin_mutex);
-    for (size_t k = 0; k < g_pins.size(); ++k) {
-        PinBatch &b = g_pins[k];
-        if (p < b.mem || p >= b.mem + kPinBatch) continue;
-        b.used &= ~(1u << (p - b.mem));
-        if (!b.used && g_pins.size() > 1) {
-            cudaFreeHost(b.mem);
-            g_pins.erase(g_pins.begin() + k);
-        }
         return;
     }
+    std::lock_guard<std::mutex> lk(g_pin_mutex);
+    g_pins = static_cast<Pinned *>(p);
 }
+
+// a slot for the scope of one call; at is null when there is none.  The call
+// waits for its stream before it returns, so nothing writes the slot after it.
+struct PinLease {
+    Pinned *at = nullptr;
+    PinLease() {
+        std::lock_guard<std::mutex> lk(g_pin_mutex);
+        if (!g_pins || g_pins_used == 0xFFFFFFFFu) return;
+        const int i = __builtin_ctz(~g_pins_used);
+        g_pins_used |= 1u << i;
+        at = g_pins + i;
+    }
+    ~PinLease() {
+        if (!at) return;
+        std::lock_guard<std::mutex> lk(g_pin_mutex);
+        g_pins_used &= ~(1u << (at - g_pins));
+    }
+    PinLease(const PinLease &) = delete;
+    PinLease &operator=(const PinLease &) = delete;
+};
 }  // namespace
 
 // ------------------------------------------------------------ graph object --
@@ -302,8 +297,6 @@ struct moss_graph {
     uint32_t *hub_bits = nullptr;
     uint32_t *hub_list = nullptr;
     uint32_t *order = nullptr;   // input id of each internal vertex (MOSS_ORDER_DEGREE), else null
-    Pinned *pin = nullptr;       // what the device hands back (null: res_host through a copy)
-    moss_result res_host{};
     uint32_t flags_host[2] = {0, 0};
 };
 
@@ -318,7 +311,6 @@ void release(moss_graph *g) {
     if (g->filter) cudaFreeAsync(g->filter, 0);
     if (g->hub_mem) cudaFreeAsync(g->hub_mem, 0);
     if (g->min_arena) cudaFreeAsync(g->min_arena, 0);
-    pin_give(g->pin);
     delete g;
 }
 
@@ -466,8 +458,9 @@ struct Carver {
 
 // totals and status flags of the work queued on s (waits for it)
 int read_status(moss_graph *g, cudaStream_t s) {
+    const PinLease pin;
     DevStatus here;
-    DevStatus *to = g->pin ? &g->pin->status : &here;
+    DevStatus *to = pin.at ? &pin.at->status : &here;
     MOSS_CUDA(cudaMemcpyAsync(to, g->tot, sizeof(DevStatus), cudaMemcpyDeviceToHost, s), "reading totals");
     MOSS_CUDA(cudaStreamSynchronize(s), "synchronising stream");
     g->tot_h = to->tot;
@@ -476,13 +469,13 @@ int read_status(moss_graph *g, cudaStream_t s) {
 }
 
 // where a kernel on s leaves the result, and its arrival in *out (waits for s)
-moss_result *result_target(moss_graph *g) { return g->pin ? &g->pin->res : g->res_dev; }
-int read_result(moss_graph *g, cudaStream_t s, moss_result *out) {
-    if (!g->pin)
-        MOSS_CUDA(cudaMemcpyAsync(&g->res_host, g->res_dev, sizeof(moss_result), cudaMemcpyDeviceToHost, s),
-                  "reading result");
+moss_result *result_target(moss_graph *g, const PinLease &pin) { return pin.at ? &pin.at->res : g->res_dev; }
+int read_result(moss_graph *g, cudaStream_t s, const PinLease &pin, moss_result *out) {
+    moss_result here;
+    if (!pin.at)
+        MOSS_CUDA(cudaMemcpyAsync(&here, g->res_dev, sizeof(moss_result), cudaMemcpyDeviceToHost, s), "reading result");
     MOSS_CUDA(cudaStreamSynchronize(s), "synchronising stream");
-    if (out) memcpy(out, g->pin ? &g->pin->res : &g->res_host, sizeof(moss_result));
+    if (out) memcpy(out, pin.at ? &pin.at->res : &here, sizeof(moss_result));
     return MOSS_OK;
 }
 
@@ -557,7 +550,6 @@ int moss_graph_load_csr_order(const void *row_ptr, int row_ptr_is_64, const uint
                                 : (n >= (1u << 14) ? MOSS_VERTEX_SPLIT_MID : MOSS_VERTEX_ONE_LEVEL);
     g->vsplit_min = n >= (1u << 20) ? MOSS_VERTEX_SPLIT_DEFAULT : MOSS_VERTEX_ONE_LEVEL;
     g->nnz = nnz;
-    g->pin = pin_take();
     void *rp_dev = nullptr;
     void *oscratch = nullptr;   // renumbering scratch (released before return)
     const bool small = small_graph(n, nnz);
@@ -886,6 +878,7 @@ static int check_samples(const moss_graph *g, int method, uint64_t first, uint64
         return fail(MOSS_EINVAL, "method %d has total weight 0 on this graph: no sample exists", method);
     if (first + count < first) return fail(MOSS_EOVERFLOW, "sample range wraps");
     // per-warp 32-bit counters: keep each launch below 2^31 samples per warp
+    if (count <= 8ULL << 31) return MOSS_OK;   // of one block's 8 warps
     const uint64_t max_chunk = (uint64_t)sample_launch_blocks(method, g->device, view(g)) * 8 * (1ULL << 31);
     if (count > max_chunk) return fail(MOSS_EOVERFLOW, "count above %llu per call", (unsigned long long)max_chunk);
     return MOSS_OK;
@@ -975,10 +968,12 @@ static int sample_both(moss_graph *g, int ma, uint64_t ka, int mb, uint64_t kb, 
 // the result of the counts at g->sums (of none where nothing is drawn)
 static int finalize_sums(moss_graph *g, const FinalizeIn &in, cudaStream_t s, moss_result *out) {
     const bool drawn = in.K[0] || in.K[1];   // the launch before is a kernel
-    HitsArg hits = {};
+    HitsArg hits;
     hits.dev = drawn ? g->sums : nullptr;
-    MOSS_CUDA(launch_finalize(in, hits, g->tot, result_target(g), nullptr, s, drawn), "finalize kernel");
-    return read_result(g, s, out);
+    if (!drawn) memset(hits.h, 0, sizeof(hits.h));
+    const PinLease pin;
+    MOSS_CUDA(launch_finalize(in, hits, g->tot, result_target(g, pin), nullptr, s, drawn), "finalize kernel");
+    return read_result(g, s, pin, out);
 }
 
 int moss_sample_estimate(moss_graph *g, int k, uint64_t budget, uint64_t seed, void *stream, moss_result *out) {
@@ -1028,13 +1023,14 @@ static int finalize_given(moss_graph *g, const FinalizeIn &in, const uint64_t *h
     HitsArg arg;
     const int rc = counts_arg(g, hits, s, &arg);
     if (rc) return rc;
-    double *cov = cov_host ? (g->pin ? g->pin->cov : g->cov_dev) : nullptr;
-    MOSS_CUDA(launch_finalize(in, arg, g->tot, result_target(g), cov, s), "finalize kernel");
-    if (cov_host && !g->pin)
-        MOSS_CUDA(cudaMemcpyAsync(cov_host, g->cov_dev, sizeof(g->pin->cov), cudaMemcpyDeviceToHost, s),
+    const PinLease pin;
+    double *cov = cov_host ? (pin.at ? pin.at->cov : g->cov_dev) : nullptr;
+    MOSS_CUDA(launch_finalize(in, arg, g->tot, result_target(g, pin), cov, s), "finalize kernel");
+    if (cov_host && !pin.at)
+        MOSS_CUDA(cudaMemcpyAsync(cov_host, g->cov_dev, sizeof(pin.at->cov), cudaMemcpyDeviceToHost, s),
                   "reading covariance");
-    const int rr = read_result(g, s, out);
-    if (!rr && cov_host && g->pin) memcpy(cov_host, g->pin->cov, sizeof(g->pin->cov));
+    const int rr = read_result(g, s, pin, out);
+    if (!rr && cov_host && pin.at) memcpy(cov_host, pin.at->cov, sizeof(pin.at->cov));
     return rr;
 }
 

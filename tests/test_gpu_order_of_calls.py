@@ -1,6 +1,7 @@
 """What a call reads and writes follows its stream, whatever is in flight: counts
 in page-locked memory are read after the copy that fills them, and a call that
-is refused or draws nothing leaves the counts of another stream's call alone."""
+is refused or draws nothing leaves the counts of another stream's call alone, and
+freeing graphs waits for nobody's work."""
 from __future__ import annotations
 
 import ctypes
@@ -83,3 +84,39 @@ def test_a_call_that_draws_nothing_leaves_another_streams_counts(graph, method, 
     other(graph, none)
     side.synchronize()
     assert torch.equal(out, ref)
+
+
+def test_freeing_graphs_does_not_wait_for_the_device(graph):
+    rp, col = synth.complete(5)
+    graphs = [moss.Graph(rp, col) for _ in range(70)]
+    out, side = torch.zeros(22, dtype=torch.int64, device="cuda"), torch.cuda.Stream()
+    torch.cuda.synchronize()
+    moss.moss_sample_counts(graph.handle, 1, 0, 20 * LONG, 2, out, side)
+    for g in graphs:
+        g.close()
+    assert not side.query()
+    side.synchronize()
+    assert int(out.sum()) == 20 * LONG
+
+
+def test_calls_of_many_threads(graph):
+    """More calls at a time than there are page-locked slots to lend."""
+    from concurrent.futures import ThreadPoolExecutor
+    rp, col = synth.complete(5)
+    graphs = [moss.Graph(rp, col) for _ in range(48)]
+    hits = np.ones((2, 22), dtype=np.uint64)
+    ref = moss.moss_covariance(graphs[0].handle, 5, np.array([50, 50], np.uint64), hits)
+
+    want = graphs[0].estimate(5, 1000, 5)["hits"]
+
+    def use(g):
+        for _ in range(10):
+            assert np.array_equal(g.estimate(5, 1000, 5)["hits"], want)
+            cov, r = moss.moss_covariance(g.handle, 5, np.array([50, 50], np.uint64), hits)
+            assert np.array_equal(cov, ref[0]) and np.array_equal(r["est"], ref[1]["est"])
+        return True
+
+    with ThreadPoolExecutor(48) as pool:
+        assert all(pool.map(use, graphs))
+    for g in graphs:
+        g.close()
