@@ -30,6 +30,7 @@ int fail(int code, const char *fmt, ...) {
 }
 
 int cuda_fail(cudaError_t e, const char *what) {
+    cudaGetLastError();   // reported here, not by the next call's launches
     return fail(e == cudaErrorMemoryAllocation ? MOSS_ENOMEM : MOSS_ECUDA, "%s: %s", what, cudaGetErrorString(e));
 }
 
