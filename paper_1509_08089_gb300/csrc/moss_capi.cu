@@ -10,6 +10,8 @@
 #include <new>
 #include <vector>
 
+#include <cuda.h>
+
 #include "../../include/moss.h"
 #include "moss_internal.cuh"
 #include "moss_order.cuh"
@@ -434,14 +436,31 @@ cudaError_t pool_alloc(int device, void **p, size_t bytes, cudaStream_t s) {
     return cudaMallocFromPoolAsync(p, bytes ? bytes : 1, pool, s);
 }
 
-// whether p is memory of this device that kernels can read in place
-bool readable_here(const void *p, size_t align, int device) {
+// whether p is memory of this device whose `bytes` bytes kernels can read in
+// place; when its allocation ends before, the caller's copy refuses it
+bool readable_here(const void *p, size_t bytes, size_t align, int device) {
     cudaPointerAttributes pa;
     if (cudaPointerGetAttributes(&pa, p) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
-    return pa.type == cudaMemoryTypeDevice && pa.device == device && reinterpret_cast<uintptr_t>(p) % align == 0;
+    if (pa.type != cudaMemoryTypeDevice || pa.device != device || reinterpret_cast<uintptr_t>(p) % align) return false;
+    typedef CUresult (*RangeFn)(CUdeviceptr *, size_t *, CUdeviceptr);
+    static const RangeFn range = [] {
+        void *fn = nullptr;
+        cudaDriverEntryPointQueryResult found = cudaDriverEntryPointSymbolNotFound;
+        if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &fn, 12000, cudaEnableDefault, &found) !=
+                cudaSuccess ||
+            found != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            fn = nullptr;
+        }
+        return reinterpret_cast<RangeFn>(fn);
+    }();
+    CUdeviceptr base = 0;
+    size_t size = 0;
+    const CUdeviceptr at = reinterpret_cast<CUdeviceptr>(p);
+    return range && range(&base, &size, at) == CUDA_SUCCESS && at - base <= size && bytes <= size - (at - base);
 }
 
 // Carves 256-byte aligned arrays out of one allocation (first pass: size).
@@ -605,7 +624,7 @@ int moss_graph_load_csr_order(const void *row_ptr, int row_ptr_is_64, const uint
         STEP(cudaMemcpyAsync(rp_dev, row_ptr, rp_bytes, cudaMemcpyDefault, s), "copying row_ptr");
         // the input lists are read in place when they are device memory of
         // this device, else copied beside the scratch first
-        const bool direct = nnz && readable_here(col, alignof(uint32_t), device);
+        const bool direct = nnz && readable_here(col, nnz * sizeof(uint32_t), alignof(uint32_t), device);
         const uint64_t ob = (order_scratch_bytes(n) + 255) & ~255ull;
         STEP(pool_alloc(device, &oscratch, ob + (direct ? 0 : nnz * sizeof(uint32_t)), s), "allocating order scratch");
         const uint32_t *src = col;
@@ -630,11 +649,11 @@ int moss_graph_load_csr_order(const void *row_ptr, int row_ptr_is_64, const uint
         // rows and lists in device memory are read where they are
         const void *rp = row_ptr;
         const uint32_t *src = col;
-        if (!readable_here(row_ptr, row_ptr_is_64 ? 8 : 4, device)) {
+        if (!readable_here(row_ptr, rp_bytes, row_ptr_is_64 ? 8 : 4, device)) {
             STEP(cudaMemcpyAsync(rp_dev, row_ptr, rp_bytes, cudaMemcpyDefault, s), "copying row_ptr");
             rp = rp_dev;
         }
-        if (nnz && !readable_here(col, alignof(uint32_t), device)) {
+        if (nnz && !readable_here(col, nnz * sizeof(uint32_t), alignof(uint32_t), device)) {
             STEP(cudaMemcpyAsync(g->col, col, nnz * sizeof(uint32_t), cudaMemcpyDefault, s), "copying col");
             src = nullptr;
         }

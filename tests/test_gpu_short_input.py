@@ -1,5 +1,5 @@
-"""A CSR array that is shorter than the call says is refused, and the
-next call does not report it again."""
+"""A CSR array that is shorter than the call says is refused, whether it would be
+copied or read in place."""
 from __future__ import annotations
 
 import ctypes
@@ -22,8 +22,8 @@ def device_copy(rt, a, nbytes):
     return p
 
 
-@pytest.mark.parametrize("order", [moss.ORDER_INPUT])
-@pytest.mark.parametrize("n", [20_000])
+@pytest.mark.parametrize("order", [moss.ORDER_INPUT, moss.ORDER_DEGREE])
+@pytest.mark.parametrize("n", [10_000, 20_000])     # read in place; copied
 @pytest.mark.parametrize("short", ["none", "row_ptr", "col"])
 def test_short_device_arrays(short, n, order):
     rp, col = synth.chung_lu(n, 2.5, 8.0, 200.0, seed=2)
