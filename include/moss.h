@@ -342,7 +342,7 @@ int moss_batch_set_launch(moss_batch *b, int threads_per_block, int blocks_per_s
  * graph lacks the tables the strategy needs.  Counts do not depend on it. */
 int moss_batch_set_graph_probe(moss_batch *b, const moss_graph *g, int strategy);
 typedef struct {
-    uint32_t tile_samples;     /* samples per tile: one warp's unit of work      */
+    uint32_t tile_samples;     /* the most a warp takes at a time (moss_batch_set_tile) */
     int threads_per_block;     /* 128, 256 or 512                                 */
     int blocks_per_sm;         /* resident blocks of the persistent launch per SM */
     int tuned;                 /* 1 once moss_batch_tune has run                   */
@@ -356,9 +356,10 @@ typedef struct {
  * (1) each graph's probe strategy, from the SM cycles per sample of its
  * tiles in one run with every graph on list search, one on the hashed set
  * and one on the filtered set (each where its tables exist); (2) the tile
- * size among 1,024 .. 65,536 samples; (3) the block shape among 128, 256 and
- * 512 threads at 1/2, 3/4 and all of the resident blocks that fit; (4) the
- * tile size again under that shape.  *chosen (nullable) receives the tile.
+ * size among 1,024 .. 65,536 samples (of those that cut the run the same way
+ * the smallest); (3) the block shape among 128, 256 and 512 threads at 1/2, 3/4
+ * and all of the resident blocks that fit; (4) the tile size again under that
+ * shape.  *chosen (nullable) receives the tile.
  * Every setting leaves each request's result unchanged. */
 int moss_batch_tune(moss_batch *b, void *stream, uint32_t *chosen);
 /* The settings in force (and what the last tuning chose). */
@@ -382,7 +383,8 @@ void moss_batch_free(moss_batch *b);
 typedef struct {
     int max_active;            /* requests sampled concurrently (slots)           */
     uint64_t tick_samples;     /* samples per launch over all active requests    */
-    uint32_t tile_samples;     /* tile of the persistent launch                   */
+    uint32_t tile_samples;     /* the most a warp takes at a time; a tick whose tiles would
+                                  not keep every warp busy to the end is cut finer */
     uint64_t pilot_samples;    /* first chunk of a target-error request           */
     uint64_t min_budget;       /* clamp of a budget derived from a target         */
     uint64_t max_budget;

@@ -61,6 +61,7 @@ struct moss_batch {
     std::vector<Req> reqs;
     uint32_t tile = 8192;
     uint32_t unit = 8192;              // samples per piece of the current plan (batch_unit)
+    uint64_t samples = 0;              // samples of the current plan
     int threads = 256;                 // threads per block of the persistent launch
     int per_sm = 0;                    // resident blocks per SM (0: as many as fit)
     int rngs = kBatchSplitMix;         // generators of the planned graphs (kBatch*)
@@ -166,6 +167,7 @@ int plan(moss_batch *b) {
     b->ntasks = (int)tasks.size();
     b->rngs = batch_rngs(graphs.data(), graphs.size());
     b->blocks = batch_blocks(b->device, b->threads, b->per_sm, b->rngs);
+    b->samples = samples;
     b->unit = batch_unit(samples, b->tile, (uint64_t)b->blocks * b->threads / 32);
     b->ntiles = 0;
     for (BatchTask &t : tasks) {
@@ -466,10 +468,14 @@ int moss_batch_tune(moss_batch *b, void *stream, uint32_t *chosen) {
     double best_t = 1e300;
     auto try_tiles = [&]() -> int {
         uint32_t best = b->tile;
+        bool timed = false;
         for (uint32_t c : tiles) {
+            // (a tile beyond the pieces that keep the warps busy is the plan just timed)
+            if (timed && batch_unit(b->samples, c, (uint64_t)b->blocks * b->threads / 32) == b->unit) continue;
             int r = moss_batch_set_tile(b, c);
             double t;
             if (r || (r = timed_runs(b, stream, tmp, 2, &t))) return r;
+            timed = true;
             if (t < best_t) {
                 best_t = t;
                 best = c;
