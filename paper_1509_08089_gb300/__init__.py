@@ -545,10 +545,22 @@ _AT = {f: getattr(moss_result, f).offset // 8 for f, _ in moss_result._fields_[2
 _WORDS = ctypes.sizeof(moss_result) // 8
 
 
+_SHARE = 64
+
+
 def result_dicts(results) -> list[dict]:
-    """result_dict of every result of a ctypes array: one copy of the memory,
-    the arrays views of it (256 results 0.3 ms, result_dict of each 1.6 ms)."""
-    own = bytearray(results)
+    """result_dict of every result of a ctypes array.  _SHARE results at a time
+    are one copy of their memory, the arrays views of it (256 results 0.3 ms,
+    result_dict of each 1.6 ms), so a result that is kept holds the memory of
+    _SHARE, not of all of them."""
+    raw, step = memoryview(results).cast("B"), _SHARE * ctypes.sizeof(moss_result)
+    out = []
+    for i in range(0, len(raw), step):
+        out += _result_dicts(bytearray(raw[i:i + step]))
+    return out
+
+
+def _result_dicts(own: bytearray) -> list[dict]:
     f8 = np.frombuffer(own, dtype=np.float64).reshape(-1, _WORDS)
     u8 = np.frombuffer(own, dtype=np.uint64).reshape(-1, _WORDS)
     i4 = np.frombuffer(own, dtype=np.int32).reshape(-1, 2 * _WORDS)
