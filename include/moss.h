@@ -228,7 +228,8 @@ int moss_vertex_levels(const moss_graph *g, int which, uint32_t *nheavy, uint64_
  * K1 = floor(budget/2) and Path-5 with K2 = budget - K1 (K1 = K2, Sec. 5.1.5).
  * A sub-method whose total weight is 0 draws nothing (its classes cannot
  * occur and are estimated as exactly 0).  Sample ids are 0..K-1 per
- * sub-method.  out is caller-owned host memory.  Synchronous on stream. */
+ * sub-method.  out is caller-owned host memory.  Large calls may borrow device
+ * scratch (see moss_sample_counts).  Synchronous on stream. */
 int moss_sample_estimate(moss_graph *g, int k, uint64_t budget, uint64_t seed, void *stream,
                          moss_result *out);
 
@@ -237,8 +238,14 @@ int moss_sample_estimate(moss_graph *g, int k, uint64_t budget, uint64_t seed, v
  * (MOSS_METHOD_MOSS4MIN: its (class, c) slots).  Asynchronous on stream.
  * Shards of a sample range sum exactly.  A call of 2^22 ids or more behind the
  * edge filter may borrow up to 12 bytes per id (at most 805 MB) of device
- * scratch from the library's pool, returned on the stream; without it (no
- * memory, stream capture) the same counts come from the slower path. */
+ * scratch from the library's pool; so may each sub-method of
+ * moss_sample_estimate and moss_sample_estimate_min.  The call gives it back to
+ * the pool on the stream, and the pool keeps it, as it keeps the memory of freed
+ * graphs, for the next call: cudaMemGetInfo, other processes and a server's
+ * reserve_bytes see it taken, while an allocation of this process that needs
+ * the memory gets it (the driver releases what a pool does not use).  Without
+ * scratch (no memory, stream capture) the same counts come from the slower
+ * path; moss_sample_counts_noalloc never takes any. */
 int moss_sample_counts(moss_graph *g, int method, uint64_t first, uint64_t count, uint64_t seed,
                        void *stream, uint64_t *counts_dev);
 
