@@ -22,7 +22,7 @@
 //             Q_v = sum (d_x - 1)^2 is the list's total (Gamma^(2)_v = S_v^2 - Q_v)
 //   gam[l][n] u128 vertex weights Gamma_v, Gamma^(1)_v, Gamma^(2)_v
 //   seed[l][2n] two uint4 per column c, one 32-byte sector: {T lo, T hi,
-//             alias, 0} -- vertex alias table of weight l, keep the column when
+//             alias, the column's own vertex} -- vertex alias table of weight l, keep the column when
 //             x < T for a 64-bit word x -- and a copy of the alias's vertex
 //             record (vert, or mvert for MOSS-4Min), so that a draw that takes
 //             the alias (most draws for skewed weights) needs no second load.

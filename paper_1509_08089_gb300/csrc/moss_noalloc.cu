@@ -5,11 +5,11 @@
 // running -- a service that reserves its whole device-memory budget at start
 // and forbids growth, a latency-critical loop that cannot afford the device
 // synchronisation cudaMalloc/cudaFree may imply, or a host whose allocator
-// is owned by another framework.  The ordinary moss_sample_counts uses
-// per-block partial counts held by the graph object; this variant keeps
-// them in one fixed array of this file instead, so the call itself touches
-// no allocator (the graph, its tables and the output buffer are the caller's
-// inputs and outputs, allocated earlier).
+// is owned by another framework.  The ordinary moss_sample_counts adds its
+// counts up in 22 sums held by the graph object and may borrow scratch for a
+// large call; this variant keeps the sums in one fixed array of this file and
+// never groups, so the call itself touches no allocator (the graph, its tables
+// and the output buffer are the caller's inputs and outputs, allocated earlier).
 //
 // The array is a file-scope __device__ object: every GPU that loads the
 // library holds it (kNoAllocScratchBytes) until the process exits.  Host code
