@@ -12,19 +12,21 @@
 // lists together are a few MB and stay in the L2.
 //
 // Bound: the sampling pass by DRAM lines and L1-to-L2 requests as before, at
-// fewer of the former (34M-edge graph, degree order, ncu: T-5 349 -> 219,
-// MOSS-4 304 -> 193, Path-5 480 -> 408 B of DRAM reads per sample); the draw
-// by its ~130 instructions per id, the placement by its 12 B per id and the
-// shared-memory atomics (0.27 + 0.28 ms per 2^26 ids).  Calls of 2e8 ids, ms,
-// ungrouped -> grouped, same run:
+// fewer of the former.  34M-edge graph, chunks of 2^26 ids, ncu: DRAM reads per
+// sample and the pass's DRAM rate (a copy runs at 6.8 TB/s, random lines at 5.2),
+// MOSS-4 / T-5 / Path-5: degree order 202 / 184 / 294 B, 5.7 / 4.0 / 5.7 TB/s
+// (ungrouped 304 / 349 / 480 B); input ids 204 / 193 / 344 B, 4.6 / 3.6 / 4.8.
+// The draw is bound by its ~130 instructions per id (0.29-0.31 ms per 2^26 ids),
+// the placement by its 12 B per id and the shared-memory atomics (0.29 ms).
+// Calls of 2e8 ids, ms, ungrouped -> grouped, same run:
 //              34M edges, degree order   34M edges, input ids
-//   MOSS-4         10.3 -> 8.8               15.6 -> 10.5
-//   T-5            12.0 -> 10.8              20.5 -> 12.4
-//   Path-5         16.9 -> 13.9              23.6 -> 17.3
-//   MOSS-4Min      14.2 -> 11.8              18.0 -> 14.2
+//   MOSS-4          9.9 -> 8.7               15.2 -> 10.4
+//   T-5            11.9 -> 10.9              19.3 -> 12.2
+//   Path-5         15.9 -> 12.0              22.8 -> 16.1
+//   MOSS-4Min      13.4 -> 10.9              17.5 -> 13.4
 // Reads in the grouped pass must not skip L1 allocation: with
-// ld.global.nc.L1::no_allocate the L2 gave the lines up early (T-5 533 B of
-// DRAM reads per sample).  Groups: 512 or 2,048 measured 2-4% slower than
+// ld.global.nc.L1::no_allocate the L2 gave the lines up early (T-5's DRAM reads
+// per sample more than doubled).  Groups: 512 or 2,048 measured 2-4% slower than
 // 1,024; chunks of 2^25 ids 4% slower than 2^26.
 #include <algorithm>
 
