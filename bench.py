@@ -511,7 +511,7 @@ def time_calls(moss, torch, h, k, budget, mix, seed, stream, l2_flush, reps=3):
 NAMES = {0: "MOSS4", 1: "T5", 2: "PATH5", 3: "MOSS4MIN"}
 
 
-def roofline(workload, rp, probe_name, times, methods, l2_bytes, gather, peaks):
+def roofline(workload, rp, probe_name, times, methods, l2_bytes, gather, peaks, grouped=()):
     """The roofline object of the slowest sampling call.  Its achieved rate
     is algorithmic sectors per sample (tests/golden/sectors_<workload>.json)
     x 32 B x samples per call / the call's CUDA-event time.  When the tables
@@ -536,7 +536,7 @@ def roofline(workload, rp, probe_name, times, methods, l2_bytes, gather, peaks):
     ws = sampler_tables_bytes(rp, probe_name, methods)
     l2_rate, hbm_rate = gather
     tb, how = small_case_traffic(workload, key, K)
-    out = {"kernel": f"k_sample<{dom}> ({NAMES[dom]}, {probe_name} probes)", "achieved": ach, "unit": "GB/s",
+    out = {"kernel": f"k_sample{'_group' if dom in grouped else ''}<{dom}> ({NAMES[dom]}, {probe_name} probes)", "achieved": ach, "unit": "GB/s",
            "traffic": tb, "traffic_scaling": how, "algorithmic_bytes_per_sample": spb * 32.0,
            "samples_per_launch": K, "launch_ms": tms, "kernel_times_ms": {NAMES[m]: times[m][1] for m in times},
            "tables_bytes": ws, "l2_bytes": l2_bytes,
@@ -713,7 +713,7 @@ def run_gpu(args):
     gather = (moss.moss_gather_rate(64 << 20, dev, stream) * 32.0 / 1e9,
               moss.moss_gather_rate(4 << 30, dev, stream) * 32.0 / 1e9)
     roof = roofline(data_key(args.workload, order_main), rp, probe_name, times, methods_main, l2_bytes, gather,
-                    peaks)
+                    peaks, grouped)
 
     out = {
         "metric": METRIC, "value": value, "unit": "samples/s", "n_gpus": world, "steps": args.steps,
@@ -763,7 +763,7 @@ def run_gpu(args):
             "config": {"workload": describe("cl_n4m", 5)[1], "budget": B3, "seed": args.seed, "probe": p3,
                        "rng": args.rng, "vertex_order": o3,
                        "l2": "flushed (512 MB write) before every timed step; tables larger than the L2"},
-            "roofline": roofline(data_key("cl_n4m", o3), rp3, p3, t3, [1, 2], l2_bytes, gather, peaks),
+            "roofline": roofline(data_key("cl_n4m", o3), rp3, p3, t3, [1, 2], l2_bytes, gather, peaks, g3),
             "clocks": clk3,
             "gpu_launches": device_launches(rp3, 5, B3, False, p3, True, False, o3, g3) * args.steps}
         out["batched"] = measure_batched(moss, torch, [f.result() for f in futures["batched"]],
